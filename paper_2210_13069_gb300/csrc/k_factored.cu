@@ -295,63 +295,6 @@ cudaError_t launch_build_K(int n, int P, const double* d_C, const double* d_w, d
   return e;
 }
 
-// Mode product on a tensor viewed as (I, n, Kd): out[i][a][k] = sum_m C[a][m] in[i][m][k].
-// If acc_w != 0, out = (first ? 0 : out) + acc_w * result.
-__global__ void k_mode(int64_t I, int n, int64_t Kd, const double* __restrict__ Cm, const double* __restrict__ in,
-                       double* __restrict__ out, double acc_w, int accumulate, int first) {
-  const int64_t total = I * n * Kd;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t k = t % Kd;
-    const int a = (int)((t / Kd) % n);
-    const int64_t i = t / Kd / n;
-    const double* src = in + (size_t)i * n * Kd + k;
-    const double* c = Cm + (size_t)a * n;
-    double acc = 0.0;
-    for (int m = 0; m < n; ++m) acc += c[m] * src[(size_t)m * Kd];
-    if (accumulate)
-      out[t] = (first ? 0.0 : out[t]) + acc_w * acc;
-    else
-      out[t] = acc;
-  }
-}
-
-__global__ void k_axpy_w(int64_t count, const double* __restrict__ w, int p, const double* __restrict__ x,
-                         double* __restrict__ y, int first) {
-  const double wp = w[p];
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < count; t += (int64_t)gridDim.x * blockDim.x)
-    y[t] = (first ? 0.0 : y[t]) + wp * x[t];
-}
-
-static void launch_axpy_w(int64_t count, const double* w, int p, const double* x, double* y, int first, cudaStream_t st) {
-  int64_t blocks = (count + 255) / 256;
-  if (blocks > 152 * 64) blocks = 152 * 64;
-  count_launch();
-  k_axpy_w<<<(unsigned)blocks, 256, 0, st>>>(count, w, p, x, y, first);
-}
-
-void launch_kron_apply(int n, int P, const double* d_C, const double* d_w, const double* d_X, double* d_Y,
-                       int64_t ncol, double* d_t1, double* d_t2, cudaStream_t st) {
-  // X, Y: ncol rows of length n^3 (cube index (m1, m2, m3), m3 fastest).
-  const int64_t n3 = (int64_t)n * n * n;
-  const int64_t total = ncol * n3;
-  int64_t blocks = (total + 255) / 256;
-  if (blocks > 152 * 64) blocks = 152 * 64;
-  const size_t nn = (size_t)n * n;
-  for (int p = 0; p < P; ++p) {
-    const double* cx = d_C + ((size_t)0 * P + p) * nn;
-    const double* cy = d_C + ((size_t)1 * P + p) * nn;
-    const double* cz = d_C + ((size_t)2 * P + p) * nn;
-    count_launch();
-    k_mode<<<(unsigned)blocks, 256, 0, st>>>(ncol, n, (int64_t)n * n, cx, d_X, d_t1, 0.0, 0, 0);
-    count_launch();
-    k_mode<<<(unsigned)blocks, 256, 0, st>>>(ncol * n, n, n, cy, d_t1, d_t2, 0.0, 0, 0);
-    // mode 3, then Y += w_p * result (the weight is read on the device)
-    count_launch();
-    k_mode<<<(unsigned)blocks, 256, 0, st>>>(ncol * nn, n, 1, cz, d_t2, d_t1, 0.0, 0, 0);
-    launch_axpy_w(total, d_w, p, d_t1, d_Y, p == 0, st);
-  }
-}
-
 // One block per unique pair r = (mu, nu); writes full rows mu*N_b+nu and nu*N_b+mu.
 // The column walk of one B row: col = t, t + step, ... with (ka, la) = (col / N_b, col % N_b)
 // advanced by additions (no 64-bit division per element), the non-finite test on the bit pattern

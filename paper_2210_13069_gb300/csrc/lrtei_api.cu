@@ -627,6 +627,9 @@ lrtei_status ensure_T(lrtei_plan* pl, cudaStream_t st) {
 }
 
 bool is_split(const lrtei_plan* pl);
+// A_d^(p)(a, b) = 0 for odd a + b: the kernel on boxes about one centre is even under inversion.  The
+// Khatri-Rao projection mixes the degrees.
+bool has_parity(const lrtei_plan* pl) { return pl->kr_rank == 0; }
 
 lrtei_status ensure_F64(lrtei_plan* pl, cudaStream_t st) {
   if (pl->d_F) return LRTEI_OK;
@@ -1049,9 +1052,6 @@ lrtei_status bu_adaptive(lrtei_plan* pl, double* Bu, cudaStream_t st) {
     }
     return finish_launch("adaptive B (tensor cores)");
   }
-  double *t1, *t2;
-  LRTEI_TRY(sc.get(&t1, (size_t)maxr * n3));
-  LRTEI_TRY(sc.get(&t2, (size_t)maxr * n3));
   for (int t = 0; t < np; ++t) {
     const int64_t nt = ar.off[t + 1] - ar.off[t];
     for (int s = 0; s <= t; ++s) {
@@ -1059,8 +1059,8 @@ lrtei_status bu_adaptive(lrtei_plan* pl, double* Bu, cudaStream_t st) {
       if (ns == 0 || nt == 0) continue;
       {  // rows of G = F_s K_{st}: K_{ts} applied to each row of F_s by mode products
         ProfScope ps("kron", st);
-        launch_kron_apply(n, P, pl->d_C + (size_t)(t * np + s) * cblk, pl->d_w, ar.Fp + ar.off[s] * n3, G, ns, t1, t2,
-                          st);
+        LRTEI_CUDA(launch_kron_apply(n, P, pl->d_C + (size_t)(t * np + s) * cblk, pl->d_w, ar.Fp + ar.off[s] * n3, 1, 0,
+                                     G, ns, true, st));
       }
       {
         ProfScope ps("gemm_fp64", st);
@@ -1082,14 +1082,12 @@ lrtei_status jbuild_adaptive(lrtei_plan* pl, const double* d_D, int R, double* d
   Scratch sc(st);
   AdaptiveRows ar;
   LRTEI_TRY(adaptive_rows(pl, sc, ar, true, st));
-  double *Du, *Dp, *X, *Yp, *Y, *t1, *t2, *Jp, *Ju;
+  double *Du, *Dp, *X, *Yp, *Y, *Jp, *Ju;
   LRTEI_TRY(sc.get(&Du, (size_t)npair * R));
   LRTEI_TRY(sc.get(&Dp, (size_t)npair * R));
   LRTEI_TRY(sc.get(&X, (size_t)np * R * n3));
   LRTEI_TRY(sc.get(&Yp, (size_t)np * R * n3));
   LRTEI_TRY(sc.get(&Y, (size_t)R * n3));
-  LRTEI_TRY(sc.get(&t1, (size_t)R * n3));
-  LRTEI_TRY(sc.get(&t2, (size_t)R * n3));
   LRTEI_TRY(sc.get(&Jp, (size_t)npair * R));
   LRTEI_TRY(sc.get(&Ju, (size_t)npair * R));
   launch_pack_density(nbf, R, d_D, Du, st);
@@ -1104,8 +1102,8 @@ lrtei_status jbuild_adaptive(lrtei_plan* pl, const double* d_D, int R, double* d
     const int64_t ns = ar.off[s + 1] - ar.off[s];
     for (int t = 0; t < np; ++t) {  // K_{st} X_t, rows of X_t^T: A_{st} by mode products
       ProfScope ps("kron", st);
-      launch_kron_apply(n, P, pl->d_C + (size_t)(s * np + t) * cblk, pl->d_w, X + (size_t)t * R * n3,
-                        Yp + (size_t)t * R * n3, R, t1, t2, st);
+      LRTEI_CUDA(launch_kron_apply(n, P, pl->d_C + (size_t)(s * np + t) * cblk, pl->d_w, X + (size_t)t * R * n3, 1, 0,
+                                   Yp + (size_t)t * R * n3, R, true, st));
     }
     launch_reduce_splits(Yp, np, (int64_t)R * n3, R, n3, n3, Y, n3, st);
     {
@@ -1197,13 +1195,11 @@ lrtei_status bu_rows(lrtei_plan* pl, int form, int64_t r0, int64_t r1, double* o
   // factored: G = kron(F rows), B_u rows = pref * G F^T
   LRTEI_TRY(ensure_F64(pl, st));
   Scratch sc(st);
-  double *G, *t1, *t2;
+  double* G;
   LRTEI_TRY(sc.get(&G, (size_t)nr * n3));
-  LRTEI_TRY(sc.get(&t1, (size_t)nr * n3));
-  LRTEI_TRY(sc.get(&t2, (size_t)nr * n3));
   {
     ProfScope ps("kron", st);
-    launch_kron_apply(n, P, pl->d_C, pl->d_w, pl->d_F + r0 * n3, G, nr, t1, t2, st);
+    LRTEI_CUDA(launch_kron_apply(n, P, pl->d_C, pl->d_w, pl->d_F + r0 * n3, 1, 0, G, nr, has_parity(pl), st));
   }
   if (pl->prec == LRTEI_FP32) {
     LRTEI_TRY(ensure_F32(pl, st));
@@ -1570,9 +1566,6 @@ lrtei_status lrtei_exchange(lrtei_plan* plan, const double* d_Q, int norb, doubl
                         plan->d_status, st));
     }
   } else {
-    double *t1, *t2;
-    LRTEI_TRY(sc.get(&t1, (size_t)ob * rowlen));
-    LRTEI_TRY(sc.get(&t2, (size_t)ob * rowlen));
     const int64_t kc = 32768;  // split-K chunk of the last product (an N_b x N_b output)
     const int64_t maxk = (int64_t)ob * n3, nchunk = (maxk + kc - 1) / kc;
     double* part;
@@ -1585,7 +1578,7 @@ lrtei_status lrtei_exchange(lrtei_plan* plan, const double* d_Q, int norb, doubl
       }
       {
         ProfScope ps("kron", st);
-        launch_kron_apply(n, P, plan->d_C, plan->d_w, X, Y, (int64_t)nj * nbf, t1, t2, st);
+        LRTEI_CUDA(launch_kron_apply(n, P, plan->d_C, plan->d_w, X, 1, 0, Y, (int64_t)nj * nbf, has_parity(plan), st));
       }
       launch_perm_orbital_rows(nbf, n3, nj, X, Xp, st);
       launch_perm_orbital_rows(nbf, n3, nj, Y, Yp, st);
@@ -1741,12 +1734,10 @@ static lrtei_status jbuild_streamed(lrtei_plan* plan, const double* d_D, int R, 
   rb = std::max<int64_t>(1, std::min(rb, npair));
   const int64_t nblk = (npair + rb - 1) / rb;
   Scratch sc(st);
-  double *Du, *Xt, *Yt, *t1, *t2, *Ju, *Fb;
+  double *Du, *Xt, *Yt, *Ju, *Fb;
   LRTEI_TRY(sc.get(&Du, (size_t)npair * R));
   LRTEI_TRY(sc.get(&Xt, (size_t)R * n3));
   LRTEI_TRY(sc.get(&Yt, (size_t)R * n3));
-  LRTEI_TRY(sc.get(&t1, (size_t)R * n3));
-  LRTEI_TRY(sc.get(&t2, (size_t)R * n3));
   LRTEI_TRY(sc.get(&Ju, (size_t)npair * R));
   LRTEI_TRY(sc.get(&Fb, (size_t)rb * n3));
   launch_pack_density(nbf, R, d_D, Du, st);
@@ -1759,7 +1750,7 @@ static lrtei_status jbuild_streamed(lrtei_plan* plan, const double* d_D, int R, 
     }
     {
       ProfScope ps("kron", st);
-      launch_kron_apply(n, P, plan->d_C, plan->d_w, Xt, Yt, R, t1, t2, st);
+      LRTEI_CUDA(launch_kron_apply(n, P, plan->d_C, plan->d_w, Xt, 1, 0, Yt, R, has_parity(plan), st));
     }
     for (int64_t r0 = 0; r0 < npair; r0 += rb) {  // J_b = F_b Y
       const int64_t nr = std::min(npair, r0 + rb) - r0;
@@ -1803,7 +1794,7 @@ static lrtei_status jbuild_streamed(lrtei_plan* plan, const double* d_D, int R, 
   launch_reduce_splits(Xparts, (int)nblk, R * n3, R, n3, n3, Xt, n3, st);
   {
     ProfScope ps("kron", st);
-    launch_kron_apply(n, P, plan->d_C, plan->d_w, Xt, Yt, R, t1, t2, st);
+    LRTEI_CUDA(launch_kron_apply(n, P, plan->d_C, plan->d_w, Xt, 1, 0, Yt, R, has_parity(plan), st));
   }
   {
     ProfScope ps("split", st);
@@ -1892,15 +1883,13 @@ lrtei_status lrtei_jbuild_apply_x(lrtei_plan* plan, const double* d_X, int R, in
   if (nr == 0) return LRTEI_OK;
   ProfScope ps_all("jbuild", st);
   Scratch sc(st);
-  double *Y, *t1, *t2, *Fb, *Ju;
+  double *Y, *Fb, *Ju;
   LRTEI_TRY(sc.get(&Y, (size_t)R * n3));
-  LRTEI_TRY(sc.get(&t1, (size_t)R * n3));
-  LRTEI_TRY(sc.get(&t2, (size_t)R * n3));
   LRTEI_TRY(sc.get(&Fb, (size_t)nr * n3));
   LRTEI_TRY(sc.get(&Ju, (size_t)nr * R));
   {
     ProfScope ps("kron", st);
-    launch_kron_apply(n, P, plan->d_C, plan->d_w, d_X, Y, R, t1, t2, st);
+    LRTEI_CUDA(launch_kron_apply(n, P, plan->d_C, plan->d_w, d_X, 1, 0, Y, R, has_parity(plan), st));
   }
   launch_build_F<double>(plan->t, n, plan->d_S, pair_begin, pair_end, Fb, n3, st);
   if (!is_split(plan)) {
@@ -1961,29 +1950,29 @@ static lrtei_status jbuild_direct(lrtei_plan* plan, const double* d_D, int R, do
   const int64_t npair = plan->t.npair, n3 = (int64_t)n * n * n;
   const double pref = plan->omega / sqrt(kPi);
   Scratch sc(st);
-  double *Du, *Xt, *Yt, *t1, *t2, *Ju;
-  LRTEI_TRY(sc.get(&Du, (size_t)npair * R));
-  LRTEI_TRY(sc.get(&Xt, (size_t)R * n3));
-  LRTEI_TRY(sc.get(&Yt, (size_t)R * n3));
-  LRTEI_TRY(sc.get(&t1, (size_t)R * n3));
-  LRTEI_TRY(sc.get(&t2, (size_t)R * n3));
-  LRTEI_TRY(sc.get(&Ju, (size_t)npair * R));
-  launch_pack_density(nbf, R, d_D, Du, st);
   LRTEI_TRY(ensure_F64(plan, st));
-  // Xt = Du^T F  (R x n^3); Yt = kron(Xt); Ju = F Yt^T (npair x R)
+  double *part, *X, *Y;
+  int ns = jx_splits(npair, n3);
+  LRTEI_TRY(sc.get(&part, (size_t)ns * R * n3));
+  LRTEI_TRY(sc.get(&Y, (size_t)R * n3));
   {
     ProfScope ps("gemm_fp64", st);
-    gemm_cuda_core<double>(true, false, R, n3, npair, 1.0, Du, R, plan->d_F, n3, 0.0, Xt, n3, st);
+    ns = launch_jx(plan->t, nbf, n3, R, ns, d_D, plan->d_F, part, st);
+  }
+  X = part;
+  if (ns > 8) {  // many partial sums: added once here, not by every CTA of the node sum
+    LRTEI_TRY(sc.get(&X, (size_t)R * n3));
+    launch_reduce_splits(part, ns, R * n3, R, n3, n3, X, n3, st);
+    ns = 1;
   }
   {
     ProfScope ps("kron", st);
-    launch_kron_apply(n, P, plan->d_C, plan->d_w, Xt, Yt, R, t1, t2, st);
+    LRTEI_CUDA(launch_kron_apply(n, P, plan->d_C, plan->d_w, X, ns, R * n3, Y, R, has_parity(plan), st));
   }
   {
     ProfScope ps("gemm_fp64", st);
-    gemm_cuda_core<double>(false, true, npair, R, n3, 1.0, plan->d_F, n3, Yt, n3, 0.0, Ju, R, st);
+    launch_jy(plan->t, nbf, n3, R, plan->d_F, Y, pref, d_J, plan->d_status, st);
   }
-  launch_unpack_J(nbf, R, Ju, pref, d_J, plan->d_status, st);
   return finish_launch("jbuild");
 }
 

@@ -179,9 +179,18 @@ void launch_build_F_pairs(const PairTable& t, int n, const double* d_S, int64_t 
 // Dense K = sum_p w_p C_x^p (x) C_y^p (x) C_z^p  (n^3 x n^3), FP64.
 cudaError_t launch_build_K(int n, int P, const double* d_C, const double* d_w, double scale, double* d_K,
                            cudaStream_t st);
-// Y = sum_p w_p (C_x^p (x) C_y^p (x) C_z^p) X, X/Y: n^3 x ncol (column index fastest).
-void launch_kron_apply(int n, int P, const double* d_C, const double* d_w, const double* d_X, double* d_Y,
-                       int64_t ncol, double* d_t1, double* d_t2, cudaStream_t st);
+// Y = sum_p w_p (C_x^p (x) C_y^p (x) C_z^p) X on ncol rows of n^3 (cube index m3 fastest; k_jfp64.cu).
+// X comes as nsplit partial sums split_stride apart.  parity: C_d^p(a, b) = 0 for odd a + b (every plan
+// but a compressed one), so those terms are skipped.
+cudaError_t launch_kron_apply(int n, int P, const double* d_C, const double* d_w, const double* d_X, int nsplit,
+                              int64_t split_stride, double* d_Y, int64_t ncol, bool parity, cudaStream_t st);
+// FP64 CUDA-core J-build products: partial sums of X = F_u^T u from the densities D (at most nsplit
+// of them; returns how many, part[s][q][m]), and J from Y, scaled, both halves stored.
+int jx_splits(int64_t npair, int64_t n3);
+int launch_jx(const PairTable& t, int nbf, int64_t n3, int R, int nsplit, const double* d_D, const double* d_F,
+              double* d_part, cudaStream_t st);
+void launch_jy(const PairTable& t, int nbf, int64_t n3, int R, const double* d_F, const double* d_Y, double scale,
+               double* d_J, int* d_status, cudaStream_t st);
 // Expand the unique-pair square B_u (npair x npair, ld) into full B (N_b^2 x N_b^2, ldB), times scale.
 // The expansion and unpacking kernels latch kDevNonFinite into *d_status if they store a NaN or an
 // infinity (a warp vote per store loop; no extra memory traffic).
