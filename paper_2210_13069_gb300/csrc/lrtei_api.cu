@@ -118,6 +118,10 @@ struct lrtei_plan {
   bool have_Fsp = false, have_Ksp = false, have_FTsp = false;
   HadOperands had;            // tensor-core Hadamard form (one primitive pair per unique pair)
   bool have_had = false;
+  // FP64 plans on the tensor cores: digit planes of F_u, F_u^T and K in parity-class order
+  ParityClasses pc;
+  int* d_perm = nullptr;  // [pc.cols] natural column of each permuted one (-1: padding)
+  OzMatrix ozF, ozFT, ozK;
   std::vector<void*> allocs;
   size_t bytes = 0;
 
@@ -1117,6 +1121,184 @@ lrtei_status jbuild_adaptive(lrtei_plan* pl, const double* d_D, int R, double* d
   return finish_launch("adaptive J-build");
 }
 
+// ---- FP64 plans on the tensor cores (k_ozaki.cu) ---------------------------------------------
+// Parity classes of the plan's columns and the permutation on the device.
+lrtei_status ensure_classes(lrtei_plan* pl, cudaStream_t st) {
+  if (pl->d_perm) return LRTEI_OK;
+  ParityClasses& pc = pl->pc;
+  const int n = pl->n;
+  pc = ParityClasses();
+  pc.n = n;
+  pc.par = has_parity(pl) ? 1 : 0;
+  pc.cnt[0] = (n + 1) / 2;
+  pc.cnt[1] = n / 2;
+  pc.nclass = pc.par ? 8 : 1;
+  for (int c = 0; c < pc.nclass; ++c) {
+    pc.size[c] = pc.par ? pc.cnt[(c >> 2) & 1] * pc.cnt[(c >> 1) & 1] * pc.cnt[c & 1] : n * n * n;
+    pc.off[c] = pc.cols;
+    pc.row0[c] = pc.rows;
+    const int k = (pc.size[c] + 63) / 64 * 64;
+    pc.cols += k;
+    pc.rows += (pc.size[c] + 127) / 128 * 128;
+    pc.kmax = std::max(pc.kmax, k);
+  }
+  std::vector<int> perm((size_t)pc.cols, -1);
+  for (int m1 = 0, m = 0; m1 < n; ++m1)
+    for (int m2 = 0; m2 < n; ++m2)
+      for (int m3 = 0; m3 < n; ++m3, ++m) perm[pc.off[pc.cls(m1, m2, m3)] + pc.index(m1, m2, m3)] = m;
+  int* d = nullptr;
+  LRTEI_TRY(pl->alloc(&d, perm.size()));
+  LRTEI_CUDA(cudaMemcpyAsync(d, perm.data(), sizeof(int) * perm.size(), cudaMemcpyHostToDevice, st));
+  pl->d_perm = d;
+  return LRTEI_OK;
+}
+
+lrtei_status alloc_oz(lrtei_plan* pl, OzMatrix& m, int64_t rows, int64_t kpad) {
+  OzMatrix q;
+  q.rows = rows;
+  q.kpad = kpad;
+  LRTEI_TRY(pl->alloc(&q.d, (size_t)kOzSlices * rows * kpad));
+  LRTEI_TRY(pl->alloc(&q.expo, (size_t)rows));
+  m = q;
+  return LRTEI_OK;
+}
+void release_oz(lrtei_plan* pl, OzMatrix& m) {
+  pl->release(m.d, sizeof(uint16_t) * kOzSlices * (size_t)m.rows * m.kpad);
+  pl->release(m.expo, sizeof(int) * (size_t)m.rows);
+  m = OzMatrix();
+}
+lrtei_status scratch_oz(Scratch& sc, OzMatrix& m, int64_t rows, int64_t kpad) {
+  m.rows = rows;
+  m.kpad = kpad;
+  LRTEI_TRY(sc.get(&m.d, (size_t)kOzSlices * rows * kpad));
+  return sc.get(&m.expo, (size_t)rows);
+}
+
+lrtei_status ensure_ozF(lrtei_plan* pl, cudaStream_t st) {
+  if (pl->ozF.d) return LRTEI_OK;
+  LRTEI_TRY(ensure_classes(pl, st));
+  LRTEI_TRY(ensure_F64(pl, st));
+  const int64_t n3 = (int64_t)pl->n * pl->n * pl->n;
+  OzMatrix m;
+  LRTEI_TRY(alloc_oz(pl, m, pl->t.npair, pl->pc.cols));
+  ProfScope ps("split", st);
+  launch_oz_split(pl->d_F, n3, n3, nullptr, pl->d_perm, m, st);
+  pl->ozF = m;
+  return finish_launch("digits of F");
+}
+lrtei_status ensure_ozFT(lrtei_plan* pl, cudaStream_t st) {
+  if (pl->ozFT.d) return LRTEI_OK;
+  LRTEI_TRY(ensure_classes(pl, st));
+  LRTEI_TRY(ensure_F64(pl, st));
+  const int64_t n3 = (int64_t)pl->n * pl->n * pl->n, npair = pl->t.npair;
+  Scratch sc(st);
+  double* FT;
+  LRTEI_TRY(sc.get(&FT, (size_t)n3 * npair));
+  launch_transpose(pl->d_F, npair, n3, n3, FT, npair, st);
+  OzMatrix m;
+  LRTEI_TRY(alloc_oz(pl, m, pl->pc.cols, (npair + 63) / 64 * 64));
+  ProfScope ps("split", st);
+  launch_oz_split(FT, npair, npair, pl->d_perm, nullptr, m, st);
+  pl->ozFT = m;
+  return finish_launch("digits of F^T");
+}
+// K carries the prefactor omega / sqrt(pi).
+lrtei_status ensure_ozK(lrtei_plan* pl, cudaStream_t st) {
+  if (pl->ozK.d) return LRTEI_OK;
+  LRTEI_TRY(ensure_classes(pl, st));
+  const ParityClasses& pc = pl->pc;
+  Scratch sc(st);
+  double* K;
+  LRTEI_TRY(sc.get(&K, (size_t)pc.rows * pc.kmax));
+  LRTEI_CUDA(cudaMemsetAsync(K, 0, sizeof(double) * (size_t)pc.rows * pc.kmax, st));
+  {
+    ProfScope ps("build_K", st);
+    launch_oz_build_K(pl->n, pl->P, has_parity(pl), pc, pl->d_C, pl->d_w, pl->omega / sqrt(kPi), K, pc.kmax, st);
+  }
+  OzMatrix m;
+  LRTEI_TRY(alloc_oz(pl, m, pc.rows, pc.kmax));
+  ProfScope ps("split", st);
+  launch_oz_split(K, pc.kmax, pc.kmax, nullptr, nullptr, m, st);
+  pl->ozK = m;
+  return finish_launch("digits of K");
+}
+
+// Whether `bytes` more fit in sixty percent of the free device memory (small needs are not asked about).
+bool fits(double bytes) {
+  if (bytes < 1e9) return true;
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return bytes <= 0.6 * (double)free_b;
+}
+
+// Estimated seconds of the FP64 FMAs of a CUDA-core form (2 FMAs per clock and SM), of the K build, and
+// whether the digit products are cheaper for nr rows of B_u: 21 products at about half the FP16 peak plus
+// 0.4 ms of launches and slicing.  Measured at 60 functions, n = 24: 153 against 3 ms; the line lies near
+// 15 functions.  The memory they need decides too (digit planes are 12 bytes per element).
+constexpr double kFmaRate = 0.6e12;
+double node_fmas(const lrtei_plan* pl, double rows) {
+  const double n = pl->n;
+  return rows * (has_parity(pl) ? 1.5 : 3.0) * pl->P * n * n * n * n;
+}
+double K_elems(const lrtei_plan* pl) {
+  const double n = pl->n, n6 = n * n * n * n * n * n;
+  return has_parity(pl) ? n6 / 8 : n6;
+}
+// Operands cannot be built while the caller captures the stream.
+bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
+  return cap != cudaStreamCaptureStatusNone;
+}
+bool oz_rows_ok(const lrtei_plan* pl, int64_t nr, cudaStream_t st) {
+  if (pl->prec != LRTEI_FP64 || pl->npart > 0 || (!(pl->ozF.d && pl->ozK.d) && capturing(st))) return false;
+  const double n3 = (double)pl->n * pl->n * pl->n, np = (double)pl->t.npair;
+  const double cuda = ((double)nr * np * n3 + node_fmas(pl, (double)nr)) / kFmaRate;
+  const double build = pl->ozK.d ? 0.0 : K_elems(pl) * pl->P / kFmaRate;
+  if (cuda <= build + 42.0 * (double)nr * np * n3 / 0.9e15 + 4e-4) return false;
+  const double need = (pl->ozF.d ? 0.0 : 12 * np * n3) + (pl->d_F ? 0.0 : 8 * np * n3) +
+                      (pl->ozK.d ? 0.0 : 21 * K_elems(pl)) + nr * (20 * n3 + 8 * np);
+  return fits(need);
+}
+// J-builds: R >= 2 densities (one is as fast through FP64 F_u, 8 bytes an element against 12), orders up
+// to 32 unless K is there (its build grows as n^6), and enough work to pay for a dozen launches.
+bool oz_jbuild_ok(const lrtei_plan* pl, int R, cudaStream_t st) {
+  if (pl->prec != LRTEI_FP64 || pl->npart > 0 || R < 2 || (pl->n > 32 && !pl->ozK.d)) return false;
+  const double n3 = (double)pl->n * pl->n * pl->n, np = (double)pl->t.npair;
+  const double cuda = (2 * np * n3 * R + node_fmas(pl, R)) / kFmaRate;
+  if (cuda <= (24 * np * n3 + 12 * K_elems(pl)) / 5e12 + 8e-5) return false;
+  if (pl->ozF.d && pl->ozFT.d && pl->ozK.d) return true;
+  if (capturing(st)) return false;
+  return fits(np * n3 * (pl->d_F ? 32 : 40) + 21 * K_elems(pl));
+}
+
+lrtei_status bu_rows_oz(lrtei_plan* pl, int64_t r0, int64_t r1, double* out, int64_t ld, cudaStream_t st) {
+  const int64_t npair = pl->t.npair, nr = r1 - r0;
+  LRTEI_TRY(ensure_ozF(pl, st));
+  LRTEI_TRY(ensure_ozK(pl, st));
+  const ParityClasses& pc = pl->pc;
+  Scratch sc(st);
+  double* G;
+  LRTEI_TRY(sc.get(&G, (size_t)nr * pc.cols));
+  std::vector<OzSegment> seg;
+  for (int c = 0; c < pc.nclass; ++c) {
+    const int k = (pc.size[c] + 63) / 64 * 64;  // the padding columns of G come out as zeros
+    if (k > 0) seg.push_back({r0, pc.row0[c], nr, k, pc.off[c], pc.off[c], 0, k});
+  }
+  LRTEI_TRY(oz_gemm(pl->ozF, pl->ozK, seg, G, pc.cols, false, false, nr, pc.cols, pl->d_status, st));
+  OzMatrix Gs;
+  LRTEI_TRY(scratch_oz(sc, Gs, nr, pc.cols));
+  {
+    ProfScope ps("split", st);
+    launch_oz_split(G, pc.cols, pc.cols, nullptr, nullptr, Gs, st);
+  }
+  const bool sym = r0 == 0 && r1 == npair;
+  return oz_gemm(Gs, pl->ozF, {{0, 0, nr, npair, 0, 0, 0, pc.cols}}, out, ld, false, sym, nr, npair, pl->d_status, st);
+}
+
 // The tensor-core Hadamard form covers six-product split plans whose unique pairs each hold one
 // primitive pair (uncontracted bases), n <= 64, with the plain moments of one box.
 bool hadamard_tc_ok(const lrtei_plan* pl) {
@@ -1191,6 +1373,10 @@ lrtei_status bu_rows(lrtei_plan* pl, int form, int64_t r0, int64_t r1, double* o
       launch_hadamard_rows(pl->t, n, P, pl->d_S, pl->d_T, pl->d_w, pref, r0, r1, out, ld, st);
     }
     return finish_launch("hadamard_rows");
+  }
+  if (oz_rows_ok(pl, nr, st)) {
+    LRTEI_TRY(bu_rows_oz(pl, r0, r1, out, ld, st));
+    return finish_launch("factored B rows (digit products)");
   }
   // factored: G = kron(F rows), B_u rows = pref * G F^T
   LRTEI_TRY(ensure_F64(pl, st));
@@ -1294,7 +1480,14 @@ lrtei_status batched_graph_run(lrtei_plan* const* plans, int nmol, const double*
   // operands of every molecule exist before capture (their set-up allocates and synchronises)
   for (int m = 0; m < nmol; ++m) {
     if (is_split(plans[m])) LRTEI_TRY(ensure_jbuild_operands(plans[m], st));
-    else LRTEI_TRY(ensure_F64(plans[m], st));
+    else {
+      LRTEI_TRY(ensure_F64(plans[m], st));
+      if (oz_jbuild_ok(plans[m], R[m], st)) {
+        LRTEI_TRY(ensure_ozFT(plans[m], st));
+        LRTEI_TRY(ensure_ozF(plans[m], st));
+        LRTEI_TRY(ensure_ozK(plans[m], st));
+      }
+    }
   }
   std::vector<uintptr_t> key;
   key.push_back((uintptr_t)nmol);
@@ -1421,6 +1614,10 @@ lrtei_status lrtei_assemble_B(lrtei_plan* plan, lrtei_form form, double* d_B, in
   }
   rb = std::min(rb, npair);
   if (is_split(plan)) rb = npair;  // one symmetric tensor-core pass over the whole B_u
+  else if (f == LRTEI_FORM_FACTORED) {  // the same in digit products, or bands of 4096 rows, where they fit
+    if (oz_rows_ok(plan, npair, st)) rb = npair;
+    else if (npair > 4096 && oz_rows_ok(plan, 4096, st)) rb = 4096;
+  }
   Scratch sc(st);
   double* blk;
   LRTEI_TRY(sc.get(&blk, (size_t)rb * npair));
@@ -1667,6 +1864,11 @@ lrtei_status lrtei_plan_compress(lrtei_plan* plan, double eps, int max_rank, dou
   if (plan->have_Fsp) { release_split(plan, plan->Fsp); plan->have_Fsp = false; }
   if (plan->have_Ksp) { release_split(plan, plan->Ksp); plan->have_Ksp = false; }
   if (plan->have_FTsp) { release_split(plan, plan->FTsp); plan->have_FTsp = false; }
+  release_oz(plan, plan->ozF);
+  release_oz(plan, plan->ozFT);
+  release_oz(plan, plan->ozK);
+  plan->release(plan->d_perm, sizeof(int) * (size_t)plan->pc.cols);
+  plan->d_perm = nullptr;
   plan->release(plan->d_S, sizeof(double) * 3 * (size_t)nrows * n);
   plan->release(plan->d_C, sizeof(double) * 3 * (size_t)P * n * n);
   plan->release(V, sizeof(double) * 3 * (size_t)n * n);
@@ -1939,6 +2141,42 @@ static int64_t jbuild_stream_block(const lrtei_plan* plan) {
 
 }  // extern "C"
 
+// FP64 J-build through digit products: X = F_u^T u, Y = K X by parity class, J_u = F_u Y, the rows of
+// X and Y in parity-class order.
+static lrtei_status jbuild_oz(lrtei_plan* plan, const double* d_D, int R, double* d_J, cudaStream_t st) {
+  const int nbf = plan->basis.nbf;
+  const int64_t npair = plan->t.npair;
+  LRTEI_TRY(ensure_ozFT(plan, st));
+  LRTEI_TRY(ensure_ozF(plan, st));
+  LRTEI_TRY(ensure_ozK(plan, st));
+  const ParityClasses& pc = plan->pc;
+  Scratch sc(st);
+  double *u, *X, *Y, *Ju;
+  LRTEI_TRY(sc.get(&u, (size_t)npair * R));
+  LRTEI_TRY(sc.get(&X, (size_t)R * pc.cols));
+  LRTEI_TRY(sc.get(&Y, (size_t)R * pc.cols));
+  LRTEI_TRY(sc.get(&Ju, (size_t)npair * R));
+  OzMatrix us, Xs, Ys;
+  LRTEI_TRY(scratch_oz(sc, us, R, plan->ozFT.kpad));
+  LRTEI_TRY(scratch_oz(sc, Xs, R, pc.cols));
+  LRTEI_TRY(scratch_oz(sc, Ys, R, pc.cols));
+  launch_oz_pack(plan->t, nbf, R, d_D, u, st);
+  launch_oz_split(u, npair, npair, nullptr, nullptr, us, st);
+  LRTEI_TRY(oz_gemm(plan->ozFT, us, {{0, 0, pc.cols, R, 0, 0, 0, (int)us.kpad}}, X, pc.cols, true, false, R, pc.cols,
+                    plan->d_status, st));
+  launch_oz_split(X, pc.cols, pc.cols, nullptr, nullptr, Xs, st);
+  std::vector<OzSegment> seg;
+  for (int c = 0; c < pc.nclass; ++c) {
+    const int k = (pc.size[c] + 63) / 64 * 64;
+    if (k > 0) seg.push_back({pc.row0[c], 0, k, R, pc.off[c], 0, pc.off[c], k});
+  }
+  LRTEI_TRY(oz_gemm(plan->ozK, Xs, seg, Y, pc.cols, true, false, R, pc.cols, plan->d_status, st));
+  launch_oz_split(Y, pc.cols, pc.cols, nullptr, nullptr, Ys, st);
+  LRTEI_TRY(oz_gemm(plan->ozF, Ys, {{0, 0, npair, R, 0, 0, 0, pc.cols}}, Ju, R, false, false, npair, R, plan->d_status, st));
+  launch_unpack_J(nbf, R, Ju, 1.0, d_J, plan->d_status, st);
+  return finish_launch("jbuild (digit products)");
+}
+
 // One J-build launched kernel by kernel (also what a captured graph replays).
 static lrtei_status jbuild_direct(lrtei_plan* plan, const double* d_D, int R, double* d_J, cudaStream_t st) {
   ProfScope ps_all("jbuild", st);
@@ -1946,6 +2184,7 @@ static lrtei_status jbuild_direct(lrtei_plan* plan, const double* d_D, int R, do
   const int64_t rb = jbuild_stream_block(plan);
   if (rb > 0) return jbuild_streamed(plan, d_D, R, d_J, rb, st);
   if (is_split(plan)) return jbuild_tc(plan, d_D, R, d_J, st);
+  if (oz_jbuild_ok(plan, R, st)) return jbuild_oz(plan, d_D, R, d_J, st);
   const int nbf = plan->basis.nbf, n = plan->n, P = plan->P;
   const int64_t npair = plan->t.npair, n3 = (int64_t)n * n * n;
   const double pref = plan->omega / sqrt(kPi);

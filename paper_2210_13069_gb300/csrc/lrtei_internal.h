@@ -249,6 +249,49 @@ void gemm_cuda_core(bool transA, bool transB, int64_t M, int64_t N, int64_t K, T
 void convert_f64_to_f32(const double* in, float* out, int64_t count, cudaStream_t st);
 void convert_f32_to_f64(const float* in, double* out, int64_t count, cudaStream_t st);
 
+// ---------------------------------------------------------------- FP64 on the tensor cores (k_ozaki.cu)
+// The columns (m1, m2, m3) of F_u and the rows and columns of K in classes of the degrees' parities: K
+// couples equal parities only (A_d^(p)(a, b) = 0 for odd a + b), so it is block diagonal in them.
+// Without that symmetry (compressed plans) there is one class in the natural order.
+struct ParityClasses {
+  int n = 0, nclass = 0, par = 0;
+  int cnt[2] = {0, 0};     // even and odd degrees below n
+  int size[8] = {};        // columns of each class
+  int off[8] = {};         // first column of each class in the permuted order, a multiple of 64
+  int64_t row0[8] = {};    // first row of each class in K, a multiple of 128
+  int cols = 0;            // permuted columns, padding included
+  int64_t rows = 0;        // rows of K, padding included
+  int kmax = 0;            // columns of K (the largest class, a multiple of 64)
+  __host__ __device__ int cls(int m1, int m2, int m3) const {
+    return par ? (m1 & 1) * 4 + (m2 & 1) * 2 + (m3 & 1) : 0;
+  }
+  __host__ __device__ int index(int m1, int m2, int m3) const {  // inside the class
+    return par ? ((m1 >> 1) * cnt[m2 & 1] + (m2 >> 1)) * cnt[m3 & 1] + (m3 >> 1) : (m1 * n + m2) * n + m3;
+  }
+  __host__ __device__ int64_t row(int m1, int m2, int m3) const { return row0[cls(m1, m2, m3)] + index(m1, m2, m3); }
+};
+constexpr int kOzSlices = 6;      // base-512 digits of an FP64 element
+constexpr int kOzBad = 1 << 20;   // exponent of a row that holds a NaN or an infinity
+struct OzMatrix {                 // rows x kpad (a multiple of 64), kOzSlices digit planes
+  int64_t rows = 0, kpad = 0;
+  uint16_t* d = nullptr;
+  int* expo = nullptr;
+};
+void launch_oz_split(const double* d_src, int64_t k, int64_t ld, const int* d_rowinv, const int* d_colinv, OzMatrix& m,
+                     cudaStream_t st);
+// K (pc.rows x ldK, zero-filled by the caller) by parity class.
+void launch_oz_build_K(int n, int P, bool parity, const ParityClasses& pc, const double* d_C, const double* d_w,
+                       double scale, double* d_K, int64_t ldK, cudaStream_t st);
+void launch_oz_pack(const PairTable& t, int nbf, int R, const double* d_D, double* d_u, cudaStream_t st);
+struct OzSegment {  // rows [a_row0, a_row0 + M) of A times rows [b_row0, b_row0 + N) of B over k (a multiple
+  int64_t a_row0, b_row0, M, N, c_off;  // of 64) columns from a_k0 and b_k0, written at C + c_off
+  int a_k0, b_k0, k;
+};
+// C = A B^T of the segments (C^T with transpose_out); c_rows x c_cols is the stored output's shape.
+// symmetric: one segment of a square C, computed in the upper triangle and mirrored.
+lrtei_status oz_gemm(const OzMatrix& A, const OzMatrix& B, const std::vector<OzSegment>& segs, double* d_C, int64_t ldc,
+                     bool transpose_out, bool symmetric, int64_t c_rows, int64_t c_cols, int* d_status, cudaStream_t st);
+
 // ---------------------------------------------------------------- tensor cores (tcgen05)
 struct SplitMatrix {  // row-major rows x kpad, three FP16 integer slices + per-row scale exponent
   int64_t rows = 0, kpad = 0;

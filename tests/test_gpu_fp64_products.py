@@ -65,3 +65,47 @@ def test_jbuild_fp64_nonfinite_density_is_reported(lib):
     ref = oracle.Oracle.from_molecule(m).jbuild_factored(D[[0, 2]])
     assert rel_fro(J[[0, 2]], ref) <= 1e-12 and not np.isfinite(J[1]).any()
     pl.close()
+
+
+# The FP64 path on the tensor cores (digit products).  Sizes that reach it: ragged last tiles of the pairs (120 and
+# 465 pairs against 128-row tiles), orders whose classes fill and miss 64 columns, one to three 32-column density tiles.
+@pytest.mark.parametrize("n,P,natoms", [(24, 32, 2), (21, 40, 3), (17, 24, 4)])
+def test_B_fp64_digit_products_against_oracle_rows(lib, n, P, natoms):
+    m = molecule(n, P, natoms=natoms)
+    o = oracle.Oracle.from_molecule(m)
+    pl = lib.Plan(m, "fp64")
+    lib.lrtei_profile_enable(True)
+    lib.lrtei_profile_reset()
+    B = pl.assemble_B("factored")
+    assert lib.lrtei_profile_get("kron")[1] == 0, "the CUDA-core node sum ran: the size does not reach the digit products"
+    lib.lrtei_profile_enable(False)
+    pl.status()
+    nb2 = m.nbf ** 2
+    rows = [0, m.nbf + 2, nb2 // 2 + 1, nb2 - 1]
+    B = B.cpu().numpy()
+    assert np.array_equal(B, B.T)
+    assert rel_fro(B[rows], o.B_rows(rows)) <= 1e-12
+    pl.close()
+
+
+@pytest.mark.parametrize("R", [6, 31, 32, 33, 70])
+def test_jbuild_fp64_digit_products(lib, R):
+    import torch
+    m = molecule(19, 21, natoms=4)
+    D = synth.random_densities(6, m.nbf, R)
+    pl = lib.Plan(m, "fp64")
+    Dd = torch.as_tensor(D, device="cuda")
+    lib.lrtei_profile_enable(True)
+    lib.lrtei_profile_reset()
+    J = pl.jbuild(Dd).cpu().numpy()
+    assert lib.lrtei_profile_get("kron")[1] == 0
+    lib.lrtei_profile_enable(False)
+    pl.status()
+    assert rel_fro(J, oracle.Oracle.from_molecule(m).jbuild_factored(D)) <= 1e-12
+    D[1, 2, 3] = D[1, 3, 2] = np.nan  # a density that is not a number spoils its own J only, and is reported
+    Jn = pl.jbuild(torch.as_tensor(D, device="cuda")).cpu().numpy()
+    with pytest.raises(lib.LrteiError) as ei:
+        pl.status()
+    assert ei.value.status == 5
+    assert np.isnan(Jn[1]).all() and np.array_equal(Jn[0], J[0]) and np.array_equal(Jn[2:], J[2:])
+    pl.close()
