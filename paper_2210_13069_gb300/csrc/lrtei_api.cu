@@ -1157,20 +1157,21 @@ lrtei_status alloc_oz(lrtei_plan* pl, OzMatrix& m, int64_t rows, int64_t kpad) {
   OzMatrix q;
   q.rows = rows;
   q.kpad = kpad;
-  LRTEI_TRY(pl->alloc(&q.d, (size_t)kOzSlices * rows * kpad));
+  LRTEI_TRY(pl->alloc(&q.d, (size_t)q.count()));
   LRTEI_TRY(pl->alloc(&q.expo, (size_t)rows));
   m = q;
   return LRTEI_OK;
 }
 void release_oz(lrtei_plan* pl, OzMatrix& m) {
-  pl->release(m.d, sizeof(uint16_t) * kOzSlices * (size_t)m.rows * m.kpad);
+  pl->release(m.d, sizeof(uint16_t) * (size_t)m.count());
   pl->release(m.expo, sizeof(int) * (size_t)m.rows);
   m = OzMatrix();
 }
-lrtei_status scratch_oz(Scratch& sc, OzMatrix& m, int64_t rows, int64_t kpad) {
+lrtei_status scratch_oz(Scratch& sc, OzMatrix& m, int64_t rows, int64_t kpad, int tile) {
   m.rows = rows;
   m.kpad = kpad;
-  LRTEI_TRY(sc.get(&m.d, (size_t)kOzSlices * rows * kpad));
+  m.tile = tile;
+  LRTEI_TRY(sc.get(&m.d, (size_t)m.count()));
   return sc.get(&m.expo, (size_t)rows);
 }
 
@@ -1290,7 +1291,7 @@ lrtei_status bu_rows_oz(lrtei_plan* pl, int64_t r0, int64_t r1, double* out, int
   }
   LRTEI_TRY(oz_gemm(pl->ozF, pl->ozK, seg, G, pc.cols, false, false, nr, pc.cols, pl->d_status, st));
   OzMatrix Gs;
-  LRTEI_TRY(scratch_oz(sc, Gs, nr, pc.cols));
+  LRTEI_TRY(scratch_oz(sc, Gs, nr, pc.cols, 128));
   {
     ProfScope ps("split", st);
     launch_oz_split(G, pc.cols, pc.cols, nullptr, nullptr, Gs, st);
@@ -2156,10 +2157,11 @@ static lrtei_status jbuild_oz(lrtei_plan* plan, const double* d_D, int R, double
   LRTEI_TRY(sc.get(&X, (size_t)R * pc.cols));
   LRTEI_TRY(sc.get(&Y, (size_t)R * pc.cols));
   LRTEI_TRY(sc.get(&Ju, (size_t)npair * R));
+  const int tw = R <= 32 ? 32 : 128;  // rows of the right operands' tiles: the skinny product's or the wide one's
   OzMatrix us, Xs, Ys;
-  LRTEI_TRY(scratch_oz(sc, us, R, plan->ozFT.kpad));
-  LRTEI_TRY(scratch_oz(sc, Xs, R, pc.cols));
-  LRTEI_TRY(scratch_oz(sc, Ys, R, pc.cols));
+  LRTEI_TRY(scratch_oz(sc, us, R, plan->ozFT.kpad, tw));
+  LRTEI_TRY(scratch_oz(sc, Xs, R, pc.cols, tw));
+  LRTEI_TRY(scratch_oz(sc, Ys, R, pc.cols, tw));
   launch_oz_pack(plan->t, nbf, R, d_D, u, st);
   launch_oz_split(u, npair, npair, nullptr, nullptr, us, st);
   LRTEI_TRY(oz_gemm(plan->ozFT, us, {{0, 0, pc.cols, R, 0, 0, 0, (int)us.kpad}}, X, pc.cols, true, false, R, pc.cols,

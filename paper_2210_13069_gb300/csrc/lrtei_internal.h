@@ -272,8 +272,10 @@ struct ParityClasses {
 };
 constexpr int kOzSlices = 6;      // base-512 digits of an FP64 element
 constexpr int kOzBad = 1 << 20;   // exponent of a row that holds a NaN or an infinity
-struct OzMatrix {                 // rows x kpad (a multiple of 64), kOzSlices digit planes
-  int64_t rows = 0, kpad = 0;
+struct OzMatrix {                 // rows x kpad (a multiple of 64), kOzSlices digit planes, in tiles of
+  int64_t rows = 0, kpad = 0;     // `tile` rows x 32 columns (128; 32 for the B operand of skinny products)
+  int tile = 128;
+  int64_t count() const { return (rows + tile - 1) / tile * tile * kpad * kOzSlices; }
   uint16_t* d = nullptr;
   int* expo = nullptr;
 };

@@ -85,6 +85,12 @@ def test_B_fp64_digit_products_against_oracle_rows(lib, n, P, natoms):
     B = B.cpu().numpy()
     assert np.array_equal(B, B.T)
     assert rel_fro(B[rows], o.B_rows(rows)) <= 1e-12
+    # a band that starts and ends inside 128-row tiles (B row of the unique pair (0, nu) is nu)
+    r0, r1 = 13, min(pl.npair - 3, 400)
+    band = pl.Bu_rows(r0, r1, "factored").cpu().numpy()
+    cols = [ka * m.nbf + la for ka in range(m.nbf) for la in range(ka, m.nbf)]
+    assert rel_fro(band[:m.nbf - r0], B[r0:m.nbf][:, cols]) <= 1e-13
+    assert rel_fro(band, B[cols[r0:r1]][:, cols]) <= 1e-13
     pl.close()
 
 
