@@ -41,18 +41,20 @@ void launch_gather_MT(int nbf, int64_t n3, const double* d_F, int64_t ldF, doubl
   k_gather_MT<<<grid, block, 0, st>>>(nbf, n3, d_F, ldF, d_MT);
 }
 
-// Zp[mu][j n3 + m] = Z[(j nbf + mu) n3 + m]; one block per (j, mu) row.
-__global__ void k_perm_orbital_rows(int nbf, int64_t n3, int nj, const double* __restrict__ Z, double* __restrict__ Zp) {
+// Zp[mu][j n3 + m] = Z[(j nbf + mu) ld + map[m]] (map NULL: m); one block per (j, mu) row.
+__global__ void k_perm_orbital_rows(int nbf, int64_t n3, int nj, const double* __restrict__ Z, int64_t ld,
+                                    const int* __restrict__ map, double* __restrict__ Zp) {
   const int64_t row = blockIdx.x;  // j nbf + mu
   const int j = (int)(row / nbf), mu = (int)(row % nbf);
-  const double* src = Z + row * n3;
+  const double* src = Z + row * ld;
   double* dst = Zp + (int64_t)mu * nj * n3 + (int64_t)j * n3;
-  for (int64_t m = threadIdx.x; m < n3; m += blockDim.x) dst[m] = src[m];
+  for (int64_t m = threadIdx.x; m < n3; m += blockDim.x) dst[m] = src[map ? map[m] : m];
 }
 
-void launch_perm_orbital_rows(int nbf, int64_t n3, int nj, const double* d_Z, double* d_Zp, cudaStream_t st) {
+void launch_perm_orbital_rows(int nbf, int64_t n3, int nj, const double* d_Z, int64_t ld, const int* d_map, double* d_Zp,
+                              cudaStream_t st) {
   count_launch();
-  k_perm_orbital_rows<<<(unsigned)((int64_t)nj * nbf), 256, 0, st>>>(nbf, n3, nj, d_Z, d_Zp);
+  k_perm_orbital_rows<<<(unsigned)((int64_t)nj * nbf), 256, 0, st>>>(nbf, n3, nj, d_Z, ld, d_map, d_Zp);
 }
 
 }  // namespace lrtei

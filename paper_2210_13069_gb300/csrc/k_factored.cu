@@ -277,6 +277,105 @@ __global__ void __launch_bounds__(512, 1) k_build_K_tiled(int n, int P, const do
   }
 }
 
+// The same sums of the matching parities only (one in eight: A(a, b) = 0 for odd a + b in every dimension),
+// placed by parity class.  Pair number e of a dimension: the even (a, b), then the odd ones.
+__device__ __forceinline__ void same_parity_pair(int e, int ce, int co, int& a, int& b) {
+  const int odd = e >= ce * ce, c = odd ? co : ce;
+  if (odd) e -= ce * ce;
+  a = 2 * (e / c) + odd;
+  b = 2 * (e % c) + odd;
+}
+
+__global__ void k_K_zpairs_parity(int n, int ce, int co, int P, const double* __restrict__ C, Pair32* __restrict__ zp) {
+  const int ne = ce * ce + co * co, nn = n * n;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ne * P; i += gridDim.x * blockDim.x) {
+    int a, b;
+    same_parity_pair(i % ne, ce, co, a, b);
+    zp[i] = to_pair(C[((size_t)2 * P + i / ne) * nn + a * n + b]);
+  }
+}
+
+// Block (g tile, (a1, b1)), thread t owning e = (a3, b3) in {t, t + blockDim} as in k_build_K_tiled, over the
+// pairs of equal parity: 3.4 -> 0.45 ms at n = 24, P = 32.
+__global__ void __launch_bounds__(512, 1) k_build_K_classes(int n, int P, ParityClasses pc, const int* __restrict__ blk,
+                                                           const double* __restrict__ C, const double* __restrict__ w,
+                                                           const Pair32* __restrict__ zp, double scale,
+                                                           double* __restrict__ K, int64_t ldK) {
+  __shared__ Pair32 r[2 * kKG * kMaxP];
+  const int nn = n * n, ce = pc.cnt[0], co = pc.cnt[1], ne = ce * ce + co * co;
+  const int g0 = blockIdx.x * 2 * kKG;
+  int a1, b1;
+  same_parity_pair(blockIdx.y, ce, co, a1, b1);
+  for (int i = threadIdx.x; i < 2 * kKG * P; i += blockDim.x) {
+    const int g = g0 + i / P, p = i % P;
+    double v = 0.0;
+    if (g < ne) {
+      int a2, b2;
+      same_parity_pair(g, ce, co, a2, b2);
+      v = scale * w[p] * C[(size_t)p * nn + a1 * n + b1] * C[((size_t)P + p) * nn + a2 * n + b2];
+    }
+    r[i] = to_pair(v);
+  }
+  __syncthreads();
+  for (int half = 0; half < 2; ++half) {
+    const Pair32* rh = r + half * kKG * P;
+    const int gb = g0 + half * kKG;
+    if (gb >= ne) break;
+    for (int eb = 0; eb < ne; eb += 2 * blockDim.x) {
+      const int e0 = eb + threadIdx.x, e1 = e0 + blockDim.x;
+      const bool l0 = e0 < ne, l1 = e1 < ne;
+      if (!l0) break;
+      float sum[2][kKG], err[2][kKG];
+#pragma unroll
+      for (int j = 0; j < kKG; ++j) sum[0][j] = err[0][j] = sum[1][j] = err[1][j] = 0.f;
+      for (int p = 0; p < P; ++p) {
+        const Pair32 z0 = zp[(size_t)p * ne + e0];
+        const Pair32 z1 = l1 ? zp[(size_t)p * ne + e1] : Pair32{0.f, 0.f};
+#pragma unroll
+        for (int j = 0; j < kKG; ++j) {
+          const Pair32 x = rh[j * P + p];
+          dot2_step(x, z0, sum[0][j], err[0][j]);
+          dot2_step(x, z1, sum[1][j], err[1][j]);
+        }
+      }
+      int a3[2], b3[2];
+      same_parity_pair(e0, ce, co, a3[0], b3[0]);
+      same_parity_pair(l1 ? e1 : e0, ce, co, a3[1], b3[1]);
+#pragma unroll
+      for (int j = 0; j < kKG; ++j) {
+        if (gb + j >= ne) break;
+        int a2, b2;
+        same_parity_pair(gb + j, ce, co, a2, b2);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if (h && !l1) break;
+          const int m = (b1 * n + b2) * n + b3[h];
+          const int t = blk[pc.cls(b1, b2, b3[h]) * (pc.units * 8) + m / 16];
+          K[pc.row(a1, a2, a3[h]) * ldK + t * 16 + m % 16] = (double)sum[h][j] + (double)err[h][j];
+        }
+      }
+    }
+  }
+}
+
+cudaError_t launch_build_K_classes(int n, int P, const ParityClasses& pc, const int* d_blk, const double* d_C,
+                                   const double* d_w, double scale, double* d_K, int64_t ldK, cudaStream_t st) {
+  const int ne = pc.cnt[0] * pc.cnt[0] + pc.cnt[1] * pc.cnt[1];
+  Pair32* zp = nullptr;
+  cudaError_t e = scratch_alloc((void**)&zp, sizeof(Pair32) * (size_t)ne * P, st);
+  if (e != cudaSuccess) return e;
+  count_launch();
+  k_K_zpairs_parity<<<(unsigned)std::min<int64_t>(((int64_t)ne * P + 255) / 256, 152 * 8), 256, 0, st>>>(
+      n, pc.cnt[0], pc.cnt[1], P, d_C, zp);
+  const int threads = std::min(512, ((ne + 1) / 2 + 31) / 32 * 32);
+  count_launch();
+  k_build_K_classes<<<dim3((unsigned)((ne + 2 * kKG - 1) / (2 * kKG)), (unsigned)ne), threads, 0, st>>>(
+      n, P, pc, d_blk, d_C, d_w, zp, scale, d_K, ldK);
+  e = cudaGetLastError();
+  cudaFreeAsync(zp, st);
+  return e;
+}
+
 cudaError_t launch_build_K(int n, int P, const double* d_C, const double* d_w, double scale, double* d_K,
                            cudaStream_t st) {
   const int nn = n * n;

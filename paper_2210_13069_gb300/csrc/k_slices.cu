@@ -38,69 +38,80 @@ __device__ __forceinline__ int row_exponent(uint64_t mxbits, uint64_t* red, bool
   return e;
 }
 
-// One block per row; rows of up to 1024 * EPT elements are read once and kept in registers.
-template <int EPT>
-__global__ void __launch_bounds__(1024) k_split_rows_reg(const double* __restrict__ src, int64_t rows, int64_t k, int64_t ld,
-                                                        int64_t kpad, uint16_t* __restrict__ s0, uint16_t* __restrict__ s1,
-                                                        uint16_t* __restrict__ s2, uint16_t* __restrict__ s1h,
-                                                        int* __restrict__ expo, int nslices) {
-  __shared__ uint64_t red[32];
-  const int64_t r = blockIdx.x;
-  const double* x = src + r * ld;
-  double v[EPT];
-  uint64_t mx = 0;
-#pragma unroll
-  for (int j = 0; j < EPT; ++j) {
-    const int64_t i = threadIdx.x + (int64_t)j * blockDim.x;
-    v[j] = i < k ? x[i] : 0.0;
-    const uint64_t a = (uint64_t)__double_as_longlong(v[j]) & 0x7FFFFFFFFFFFFFFFULL;
-    mx = a > mx ? a : mx;
-  }
-  bool nz;
-  const int e = row_exponent(mx, red, nz);
-  if (threadIdx.x == 0) expo[r] = e;
-#pragma unroll
-  for (int j = 0; j < EPT; ++j) {
-    const int64_t i = threadIdx.x + (int64_t)j * blockDim.x;
-    if (i < kpad) slice_store(v[j], e, i < k && nz, nslices, r * kpad + i, s0, s1, s2, s1h);
-  }
-  for (int64_t i = threadIdx.x + (int64_t)EPT * blockDim.x; i < kpad; i += blockDim.x)
-    slice_store(0.0, e, false, nslices, r * kpad + i, s0, s1, s2, s1h);
+// Where the eight consecutive columns j .. j + 7 (j a multiple of 8) of row i go: tiles of `tile` rows x 16
+// columns x `planes` planes, 32-byte rows whose two 16-byte pieces are swapped in every other group of
+// four rows (the 32-byte swizzle of shared memory, tc_gemm.h).  In units of 16-bit elements.
+__device__ __forceinline__ int64_t piece(int64_t i, int64_t j, int tile, int64_t kpad, int planes) {
+  const int rr = (int)(i % tile);
+  return ((i / tile) * (kpad / 16) + j / 16) * (int64_t)(planes * tile * 16) + rr * 16 +
+         ((int)((j >> 3) & 1) ^ ((rr >> 2) & 1)) * 8;
 }
 
-// Short rows (padded length at most 256): one warp per row, eight consecutive elements per lane
-// (16-byte loads where the rows allow them, one 16-byte store per plane); the exponent and the
-// slices are those of the one-block-per-row kernels.
+__device__ __forceinline__ uint4 pack8(const uint16_t (&h)[8]) {
+  return make_uint4(h[0] | (uint32_t)h[1] << 16, h[2] | (uint32_t)h[3] << 16, h[4] | (uint32_t)h[5] << 16,
+                    h[6] | (uint32_t)h[7] << 16);
+}
+
+// The three slice planes of eight elements (k: live columns of the row, nz: the row is not zero).
+__device__ __forceinline__ void store_slices(const double (&v)[8], int e, bool nz, int64_t i, int64_t j, int64_t k,
+                                             int tile, int64_t kpad, uint16_t* __restrict__ d) {
+  uint16_t h0[8], h1[8], h2[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const SliceBits q = slice_bits(v[u], e, j + u < k && nz);
+    h0[u] = q.s0;
+    h1[u] = q.s1;
+    h2[u] = q.s2;
+  }
+  uint16_t* o = d + piece(i, j, tile, kpad, 3);
+  *reinterpret_cast<uint4*>(o) = pack8(h0);
+  *reinterpret_cast<uint4*>(o + tile * 16) = pack8(h1);
+  *reinterpret_cast<uint4*>(o + 2 * tile * 16) = pack8(h2);
+}
+
+// Columns j .. j + 7 of a row: 16-byte loads where the row allows them, zeros beyond k; map (may be NULL):
+// the source column of each column.
+__device__ __forceinline__ void load8(const double* __restrict__ x, int64_t j, int64_t k, bool vec,
+                                      const int* __restrict__ map, double (&v)[8]) {
+  if (map) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = j + u < k ? x[map[j + u]] : 0.0;
+  } else if (vec && j + 7 < k) {
+#pragma unroll
+    for (int u = 0; u < 8; u += 2) {
+      const double2 a = *reinterpret_cast<const double2*>(x + j + u);
+      v[u] = a.x;
+      v[u + 1] = a.y;
+    }
+  } else {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = j + u < k ? x[j + u] : 0.0;
+  }
+}
+
+__device__ __forceinline__ uint64_t max_mag(const double (&v)[8], uint64_t mx) {
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const uint64_t a = (uint64_t)__double_as_longlong(v[u]) & 0x7FFFFFFFFFFFFFFFULL;
+    mx = a > mx ? a : mx;
+  }
+  return mx;
+}
+
+// Short rows (padded length at most 256): one warp per row, eight consecutive elements per lane.
 __global__ void __launch_bounds__(256) k_split_rows_warp(const double* __restrict__ src, int64_t rows, int64_t k,
-                                                         int64_t ld, int64_t kpad, uint16_t* __restrict__ s0,
-                                                         uint16_t* __restrict__ s1, uint16_t* __restrict__ s2,
-                                                         uint16_t* __restrict__ s1h, int* __restrict__ expo,
-                                                         int nslices) {
+                                                         int64_t ld, int64_t kpad, int tile,
+                                                         const int* __restrict__ map, uint16_t* __restrict__ d,
+                                                         int* __restrict__ expo) {
   const int lane = threadIdx.x & 31;
   const int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (r >= rows) return;  // the whole warp: r is the same on its lanes
   const double* x = src + r * ld;
   const bool vec = (ld & 1) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
-  constexpr uint64_t kMag = 0x7FFFFFFFFFFFFFFFULL;
   const int64_t i0 = 8 * (int64_t)lane;
   double v[8];
-  if (vec && i0 + 7 < k) {
-#pragma unroll
-    for (int j = 0; j < 8; j += 2) {
-      const double2 a = *reinterpret_cast<const double2*>(x + i0 + j);
-      v[j] = a.x;
-      v[j + 1] = a.y;
-    }
-  } else {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = i0 + j < k ? x[i0 + j] : 0.0;
-  }
-  uint64_t mx = 0;
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const uint64_t a = (uint64_t)__double_as_longlong(v[j]) & kMag;
-    mx = a > mx ? a : mx;
-  }
+  load8(x, i0, k, vec, map, v);
+  uint64_t mx = max_mag(v, 0);
   for (int o = 16; o > 0; o >>= 1) {
     const uint64_t other = __shfl_xor_sync(0xffffffffu, mx, o);
     mx = other > mx ? other : mx;
@@ -110,79 +121,47 @@ __global__ void __launch_bounds__(256) k_split_rows_warp(const double* __restric
   if (mxd > 0.0) frexp(mxd * (256.0 / 255.0), &e);
   const bool nz = mxd > 0.0 && e >= -1000;  // rows below ~1e-301 are treated as zero
   if (lane == 0) expo[r] = e;
-  if (i0 >= kpad) return;
-  SliceBits q[8];
-#pragma unroll
-  for (int j = 0; j < 8; ++j) q[j] = slice_bits(v[j], e, i0 + j < k && nz, nslices);
-  const int64_t o = r * kpad + i0;
-  *reinterpret_cast<uint4*>(s0 + o) =
-      make_uint4(q[0].s0 | (uint32_t)q[1].s0 << 16, q[2].s0 | (uint32_t)q[3].s0 << 16,
-                 q[4].s0 | (uint32_t)q[5].s0 << 16, q[6].s0 | (uint32_t)q[7].s0 << 16);
-  *reinterpret_cast<uint4*>(s1 + o) =
-      make_uint4(q[0].s1 | (uint32_t)q[1].s1 << 16, q[2].s1 | (uint32_t)q[3].s1 << 16,
-                 q[4].s1 | (uint32_t)q[5].s1 << 16, q[6].s1 | (uint32_t)q[7].s1 << 16);
-  *reinterpret_cast<uint4*>(s2 + o) =
-      make_uint4(q[0].s2 | (uint32_t)q[1].s2 << 16, q[2].s2 | (uint32_t)q[3].s2 << 16,
-                 q[4].s2 | (uint32_t)q[5].s2 << 16, q[6].s2 | (uint32_t)q[7].s2 << 16);
-  if (s1h)
-    *reinterpret_cast<uint4*>(s1h + o) =
-        make_uint4(q[0].s1h | (uint32_t)q[1].s1h << 16, q[2].s1h | (uint32_t)q[3].s1h << 16,
-                   q[4].s1h | (uint32_t)q[5].s1h << 16, q[6].s1h | (uint32_t)q[7].s1h << 16);
+  if (i0 < kpad) store_slices(v, e, nz, r, i0, k, tile, kpad, d);
 }
 
-// Long rows: two passes over the row (maximum, then slices), four consecutive elements per thread
-// and step: 16-byte loads where the rows allow them (even ld, 16-byte aligned source) and one
-// 8-byte store per plane (kpad is a multiple of 4).
-__global__ void __launch_bounds__(256) k_split_rows4(const double* __restrict__ src, int64_t rows, int64_t k,
-                                                     int64_t ld, int64_t kpad, uint16_t* __restrict__ s0,
-                                                     uint16_t* __restrict__ s1, uint16_t* __restrict__ s2,
-                                                     uint16_t* __restrict__ s1h, int* __restrict__ expo, int nslices) {
+// One block per row: rows of up to 2048 NREG columns are read once and kept in registers; longer ones
+// (NREG = 0) take two passes, the second from L2.
+template <int NREG>
+__global__ void __launch_bounds__(256) k_split_rows(const double* __restrict__ src, int64_t k, int64_t ld, int64_t kpad,
+                                                    int tile, const int* __restrict__ map, uint16_t* __restrict__ d,
+                                                    int* __restrict__ expo) {
   __shared__ uint64_t red[32];
   const int64_t r = blockIdx.x;
   const double* x = src + r * ld;
   const bool vec = (ld & 1) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
-  constexpr uint64_t kMag = 0x7FFFFFFFFFFFFFFFULL;
   uint64_t mx = 0;
-  for (int64_t i = 4 * (int64_t)threadIdx.x; i < k; i += 4 * (int64_t)blockDim.x) {
-    if (vec && i + 3 < k) {
-      const double2 a = *reinterpret_cast<const double2*>(x + i);
-      const double2 b = *reinterpret_cast<const double2*>(x + i + 2);
-      const uint64_t m0 = (uint64_t)__double_as_longlong(a.x) & kMag, m1 = (uint64_t)__double_as_longlong(a.y) & kMag;
-      const uint64_t m2 = (uint64_t)__double_as_longlong(b.x) & kMag, m3 = (uint64_t)__double_as_longlong(b.y) & kMag;
-      const uint64_t u = m0 > m1 ? m0 : m1, w = m2 > m3 ? m2 : m3;
-      const uint64_t t = u > w ? u : w;
-      mx = t > mx ? t : mx;
-    } else {
-      for (int j = 0; j < 4 && i + j < k; ++j) {
-        const uint64_t a = (uint64_t)__double_as_longlong(x[i + j]) & kMag;
-        mx = a > mx ? a : mx;
-      }
-    }
-  }
   bool nz;
-  const int e = row_exponent(mx, red, nz);
-  if (threadIdx.x == 0) expo[r] = e;
-  for (int64_t i = 4 * (int64_t)threadIdx.x; i < kpad; i += 4 * (int64_t)blockDim.x) {
-    double v[4];
-    if (vec && i + 3 < k) {
-      const double2 a = *reinterpret_cast<const double2*>(x + i);
-      const double2 b = *reinterpret_cast<const double2*>(x + i + 2);
-      v[0] = a.x;
-      v[1] = a.y;
-      v[2] = b.x;
-      v[3] = b.y;
-    } else {
+  if constexpr (NREG > 0) {
+    double v[NREG > 0 ? NREG : 1][8];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = i + j < k ? x[i + j] : 0.0;
+    for (int i = 0; i < NREG; ++i) {
+      load8(x, 8 * ((int64_t)threadIdx.x + 256 * i), k, vec, map, v[i]);
+      mx = max_mag(v[i], mx);
     }
-    SliceBits q[4];
+    const int e = row_exponent(mx, red, nz);
+    if (threadIdx.x == 0) expo[r] = e;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) q[j] = slice_bits(v[j], e, i + j < k && nz, nslices);
-    const int64_t o = r * kpad + i;
-    *reinterpret_cast<ushort4*>(s0 + o) = make_ushort4(q[0].s0, q[1].s0, q[2].s0, q[3].s0);
-    *reinterpret_cast<ushort4*>(s1 + o) = make_ushort4(q[0].s1, q[1].s1, q[2].s1, q[3].s1);
-    *reinterpret_cast<ushort4*>(s2 + o) = make_ushort4(q[0].s2, q[1].s2, q[2].s2, q[3].s2);
-    if (s1h) *reinterpret_cast<ushort4*>(s1h + o) = make_ushort4(q[0].s1h, q[1].s1h, q[2].s1h, q[3].s1h);
+    for (int i = 0; i < NREG; ++i) {
+      const int64_t j = 8 * ((int64_t)threadIdx.x + 256 * i);
+      if (j < kpad) store_slices(v[i], e, nz, r, j, k, tile, kpad, d);
+    }
+  } else {
+    double v[8];
+    for (int64_t j = 8 * (int64_t)threadIdx.x; j < k; j += 2048) {
+      load8(x, j, k, vec, map, v);
+      mx = max_mag(v, mx);
+    }
+    const int e = row_exponent(mx, red, nz);
+    if (threadIdx.x == 0) expo[r] = e;
+    for (int64_t j = 8 * (int64_t)threadIdx.x; j < kpad; j += 2048) {
+      load8(x, j, k, vec, map, v);
+      store_slices(v, e, nz, r, j, k, tile, kpad, d);
+    }
   }
 }
 
@@ -193,21 +172,22 @@ __global__ void __launch_bounds__(256) k_split_rows4(const double* __restrict__ 
 // those of the one-block-per-row kernels.
 constexpr int kSplitCluster = 8;
 __global__ void __cluster_dims__(kSplitCluster, 1, 1) __launch_bounds__(256)
-    k_split_rows_cluster(const double* __restrict__ src, int64_t k, int64_t ld, int64_t kpad,
-                         uint16_t* __restrict__ s0, uint16_t* __restrict__ s1, uint16_t* __restrict__ s2,
-                         uint16_t* __restrict__ s1h, int* __restrict__ expo, int nslices) {
+    k_split_rows_cluster(const double* __restrict__ src, int64_t k, int64_t ld, int64_t kpad, int tile,
+                         const int* __restrict__ map, uint16_t* __restrict__ d, int* __restrict__ expo) {
   __shared__ uint64_t red[8];
   __shared__ uint64_t share;
   cg::cluster_group cluster = cg::this_cluster();
   const unsigned rank = cluster.block_rank();
   const int64_t r = blockIdx.y;
   const double* x = src + r * ld;
-  const int64_t per = (kpad + kSplitCluster - 1) / kSplitCluster;
-  const int64_t c0 = (int64_t)rank * per, c1 = min(kpad, c0 + per), ck = min(c1, k);
+  const bool vec = (ld & 1) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
+  const int64_t per = (kpad / 8 + kSplitCluster - 1) / kSplitCluster * 8;
+  const int64_t c0 = (int64_t)rank * per, c1 = min(kpad, c0 + per);
   uint64_t mx = 0;
-  for (int64_t i = c0 + threadIdx.x; i < ck; i += blockDim.x) {
-    const uint64_t a = (uint64_t)__double_as_longlong(x[i]) & 0x7FFFFFFFFFFFFFFFULL;
-    mx = a > mx ? a : mx;
+  double v[8];
+  for (int64_t j = c0 + 8 * (int64_t)threadIdx.x; j < c1; j += 8 * (int64_t)blockDim.x) {
+    load8(x, j, k, vec, map, v);
+    mx = max_mag(v, mx);
   }
   for (int o = 16; o > 0; o >>= 1) {
     const uint64_t other = __shfl_xor_sync(0xffffffffu, mx, o);
@@ -216,36 +196,45 @@ __global__ void __cluster_dims__(kSplitCluster, 1, 1) __launch_bounds__(256)
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
   __syncthreads();
   if (threadIdx.x == 0) {
-    uint64_t v = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v = red[w] > v ? red[w] : v;
-    share = v;
+    uint64_t m = 0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = red[w] > m ? red[w] : m;
+    share = m;
   }
   cluster.sync();  // every CTA's share is written
-  uint64_t v = 0;
+  uint64_t all = 0;
   for (int q = 0; q < kSplitCluster; ++q) {
     const uint64_t o = *cluster.map_shared_rank(&share, q);
-    v = o > v ? o : v;
+    all = o > all ? o : all;
   }
   cluster.sync();  // every CTA has read the shares before any of them exits
-  const double mxd = __longlong_as_double((long long)v);
+  const double mxd = __longlong_as_double((long long)all);
   int e = 0;
   if (mxd > 0.0) frexp(mxd * (256.0 / 255.0), &e);
   const bool nz = mxd > 0.0 && e >= -1000;
   if (rank == 0 && threadIdx.x == 0) expo[r] = e;
-  for (int64_t i = c0 + threadIdx.x; i < c1; i += blockDim.x)
-    slice_store(i < k ? x[i] : 0.0, e, i < k && nz, nslices, r * kpad + i, s0, s1, s2, s1h);
+  for (int64_t j = c0 + 8 * (int64_t)threadIdx.x; j < c1; j += 8 * (int64_t)blockDim.x) {
+    load8(x, j, k, vec, map, v);
+    store_slices(v, e, nz, r, j, k, tile, kpad, d);
+  }
 }
 
 // Plain BF16 operands: one rounded copy per element, exponent 8 so that the epilogue scale
 // 2^(ea + eb - 16) is 1.
-__global__ void k_plain_rows(const double* __restrict__ src, int64_t rows, int64_t k, int64_t ld, int64_t kpad,
-                             uint16_t* __restrict__ s0, int* __restrict__ expo) {
+__global__ void k_plain_rows(const double* __restrict__ src, int64_t k, int64_t ld, int64_t kpad, int tile,
+                             const int* __restrict__ map, uint16_t* __restrict__ d, int* __restrict__ expo) {
   const int64_t r = blockIdx.x;
+  const double* x = src + r * ld;
   if (threadIdx.x == 0) expo[r] = 8;
-  for (int64_t i = threadIdx.x; i < kpad; i += blockDim.x) {
-    const float v = i < k ? (float)src[r * ld + i] : 0.f;
-    __nv_bfloat16 h = __float2bfloat16_rn(v);
-    s0[r * kpad + i] = *reinterpret_cast<uint16_t*>(&h);
+  for (int64_t j = 8 * (int64_t)threadIdx.x; j < kpad; j += 8 * (int64_t)blockDim.x) {
+    double v[8];
+    uint16_t h[8];
+    load8(x, j, k, false, map, v);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      __nv_bfloat16 b = __float2bfloat16_rn((float)v[u]);
+      h[u] = *reinterpret_cast<uint16_t*>(&b);
+    }
+    *reinterpret_cast<uint4*>(d + piece(r, j, tile, kpad, 1)) = pack8(h);
   }
 }
 
@@ -279,36 +268,32 @@ __global__ void k_reduce_splits(const double* __restrict__ part, int splits, int
 
 }  // namespace tc
 
-void launch_split_rows(const double* d_src, int64_t rows, int64_t k, int64_t ld, SplitMatrix& m, bool with_s1h,
-                       int nslices, cudaStream_t st) {
+void launch_split_rows(const double* d_src, int64_t rows, int64_t k, int64_t ld, const SplitMatrix& m, const int* d_map,
+                       cudaStream_t st) {
   if (rows <= 0) return;
   count_launch();
   if (m.plain) {
-    tc::k_plain_rows<<<(unsigned)rows, 256, 0, st>>>(d_src, rows, k, ld, m.kpad, m.s0, m.expo);
+    tc::k_plain_rows<<<(unsigned)rows, 256, 0, st>>>(d_src, k, ld, m.kpad, m.tile, d_map, m.d, m.expo);
     return;
   }
-  uint16_t* s1h = (with_s1h || m.eight) ? m.s1h : nullptr;
   if (m.kpad <= 256) {  // short rows (e.g. the N_b-long rows of the exchange's MT): a warp per row
-    tc::k_split_rows_warp<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(d_src, rows, k, ld, m.kpad, m.s0, m.s1, m.s2,
-                                                                      s1h, m.expo, nslices);
+    tc::k_split_rows_warp<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(d_src, rows, k, ld, m.kpad, m.tile, d_map, m.d,
+                                                                    m.expo);
     return;
   }
   // few long rows (fewer than four per SM, e.g. the R density rows of a J-build or the N_b rows of
   // the exchange's last product): eight CTAs per row
   if ((rows < 4 * 152 && k >= 8192) || (rows < 152 && k >= 2048)) {
-    tc::k_split_rows_cluster<<<dim3(tc::kSplitCluster, (unsigned)rows), 256, 0, st>>>(d_src, k, ld, m.kpad, m.s0, m.s1,
-                                                                                     m.s2, s1h, m.expo, nslices);
+    tc::k_split_rows_cluster<<<dim3(tc::kSplitCluster, (unsigned)rows), 256, 0, st>>>(d_src, k, ld, m.kpad, m.tile, d_map,
+                                                                                     m.d, m.expo);
     return;
   }
-  // Rows of up to 4096 elements stay in registers (one read); longer rows take two passes with
-  // 256 threads, more rows in flight per SM (the second pass reads the row from L2).  The padded
-  // length is a multiple of 256 here (kpad256).
-  if (k <= 4096)
-    tc::k_split_rows_reg<4><<<(unsigned)rows, 1024, 0, st>>>(d_src, rows, k, ld, m.kpad, m.s0, m.s1, m.s2, s1h,
-                                                            m.expo, nslices);
+  if (m.kpad <= 2048)
+    tc::k_split_rows<1><<<(unsigned)rows, 256, 0, st>>>(d_src, k, ld, m.kpad, m.tile, d_map, m.d, m.expo);
+  else if (m.kpad <= 4096)
+    tc::k_split_rows<2><<<(unsigned)rows, 256, 0, st>>>(d_src, k, ld, m.kpad, m.tile, d_map, m.d, m.expo);
   else
-    tc::k_split_rows4<<<(unsigned)rows, 256, 0, st>>>(d_src, rows, k, ld, m.kpad, m.s0, m.s1, m.s2, s1h, m.expo,
-                                                      nslices);
+    tc::k_split_rows<0><<<(unsigned)rows, 256, 0, st>>>(d_src, k, ld, m.kpad, m.tile, d_map, m.d, m.expo);
 }
 
 void launch_transpose(const double* in, int64_t rows, int64_t cols, int64_t ldi, double* out, int64_t ldo,

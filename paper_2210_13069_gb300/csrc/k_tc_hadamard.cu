@@ -401,8 +401,8 @@ __global__ void k_slice_short_rows(const double* __restrict__ src, int64_t rows,
   if (m > 0.0) frexp(m * (256.0 / 255.0), &e);
   const bool nz = m > 0.0 && e >= -1000;
   if (lane == 0) expo[row] = nz ? e : kZeroRowExpo;
-  if (lane < kpad) slice_store(x0, e, nz && lane < n, 3, row * kpad + lane, s0, s1, s2, s1h);
-  if (lane + 32 < kpad) slice_store(x1, e, nz && lane + 32 < n, 3, row * kpad + lane + 32, s0, s1, s2, s1h);
+  if (lane < kpad) slice_store(x0, e, nz && lane < n, row * kpad + lane, s0, s1, s2, s1h);
+  if (lane + 32 < kpad) slice_store(x1, e, nz && lane + 32 < n, row * kpad + lane + 32, s0, s1, s2, s1h);
 }
 
 // Per row j: Ea_p(j) = sum_d te[d][p][j], Ra(j) = max_p Ea_p(j), the node factors

@@ -1,101 +1,31 @@
-// k_tcgen05.cu -- tensor-core (tcgen05 + TMA + TMEM) GEMM of the factored form, sm_103a.
+// k_tcgen05.cu -- split-precision products of the factored form on the tensor cores (tc_gemm.h).
 //
-// C = scale * A B^T for FP64 matrices A (M x K) and B (N x K), both K-contiguous, through
-// integer slices held in FP16 (every slice is an integer or an integer times a power of two,
-// so the FP16 values are exact):
-//   x = 2^e (s0 2^-8 + t1 2^-20 + t2 2^-32),  e per row,  |s0| <= 255, |t1|, |t2| <= 2048.
-// Per 128-deep K chunk the tensor cores accumulate in TMEM (FP32):
-//   L0  = sum s0a s0b                      (products < 2^16, 128 of them: exact in FP32)
-//   L12 = sum s0a t1b + s0a t2'b + t1a s0b + t1a t1'b + t2'a s0b,   t' = t / 2^12
-// and the epilogue warps drain each chunk into registers: L0 into an int32 running sum
-// (exact for K <= 32768), L12 into an FP32 running sum.  The tile is written as
-//   C = scale 2^(ea+eb-16) (T0 + T12 / 2^12)  in FP64.
-// The leading term is exact whatever rounding the tensor core applies to its FP32 sums; the
-// rest carries 2^-12 of the weight.  The representation error is about 2^-33 of the row
-// maxima; the dropped products (t1 t2, t2 t1, t2 t2) are about 2^-29 of them.
-// The tensor core's FP32 accumulation truncates (measured against an emulation), so L12's
-// smaller terms are cut at the scale of its s0 t1 terms, and the truncation error of a chunk
-// grows with the chunk's depth: hence chunks of 128 rather than the 512 that L0's exactness
-// would allow.  The eight-product variant (P8) keeps t1 t2 and t2 t1 as well and splits L12 into
-// L1 = s0 t1 + t1 s0 and L2 (the rest, in its own accumulator): three accumulators per buffer,
-// 128 x 64 tiles, C from T0 + (T1 + T2) / 2^12.
+// C = scale * A B^T for FP64 matrices A (M x K) and B (N x K), both K-contiguous, through integer slices
+// held in FP16 (every slice is an integer times a power of two, so the FP16 values are exact):
+//   x = 2^e (s0 2^-8 + t1 2^-20 + t2 2^-32),  e per row,  |s0| <= 255, |t1|, |t2| <= 2048,
+// as planes a0 = s0, a1 = t1 / 2^12, a2 = t2 / 2^24 (subnormal FP16 below 2^-14, still exact), so that
+// a_i b_j carries its weight whichever operand it comes from.  Per 128-deep K chunk the tensor cores
+// accumulate in TMEM (FP32):
+//   L0  = sum a0 b0                      (products < 2^16, 128 of them: exact in FP32)
+//   L12 = sum a0 b1 + a0 b2 + a1 b0 + a1 b1 + a2 b0
+// and the epilogue warps drain each chunk into registers: L0 into an int32 running sum (exact for
+// K <= 32768), L12 into an FP32 running sum.  The tile is written as C = scale 2^(ea+eb-16) (T0 + T12) in
+// FP64.  The leading term is exact whatever rounding the tensor core applies to its FP32 sums; the rest
+// carries 2^-12 of the weight.  The representation error is about 2^-33 of the row maxima; the dropped
+// products (a1 b2, a2 b1, a2 b2) are about 2^-29 of them.
+// The tensor core's FP32 accumulation truncates (measured against an emulation), so L12's smaller terms are
+// cut at the scale of its s0 t1 terms, and the truncation error of a chunk grows with the chunk's depth:
+// hence chunks of 128 rather than the 512 that L0's exactness would allow.  The eight-product variant keeps
+// a1 b2 and a2 b1 as well and splits L12 into L1 = a0 b1 + a1 b0 and L2 (the rest, in its own accumulator):
+// three accumulators per buffer, 128 x 64 tiles, C from T0 + (T1 + T2).
 //
-// Kernel organisation (persistent: one CTA per SM walks 128 x BN output tiles, BN = 128 for
-// wide outputs, 18 warps):
-//   warp 0       TMA producer: 3 A slices + 4 B slices per 64- or 32-deep K step into a ring
-//                of shared-memory stages (128- or 64-byte swizzle), mbarrier transaction counts
-//   warp 1       TMEM allocation (512 columns) and the single MMA-issuing thread:
-//                6 tcgen05.mma (M=128, N=BN, K=16) per 16-deep k step into two accumulators,
-//                double-buffered across K chunks, grouped by A slice (collector reuse)
-//   warps 2..17  epilogue: tcgen05.ld of each finished chunk, running sums, the finished tile
-//                staged through the idle ring and stored coalesced
-// A 128 x 64 MMA is bound by its operand reads from shared memory (2/3 of the tensor rate
-// measured); from N = 128 on the pipe runs at its full rate.
-// Every mbarrier wait is bounded: on expiry the CTA raises the device status word, stops
-// issuing work, waits (bounded) for what it issued, frees TMEM and exits.
-#include <cuda.h>
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
-#include <cudaTypedefs.h>
-
-#include <stdlib.h>
-
-#include <algorithm>
-#include <map>
-#include <mutex>
-#include <tuple>
-
-#include "lrtei_internal.h"
-#include "tc_common.h"
+// Chunks lie at multiples of 128 of the natural K, also where a step table leaves steps of them out (the
+// zero blocks of K by parity, below): what is left out adds zeros, so every sum is the dense product's bit
+// for bit.
+#include "tc_gemm.h"
 
 namespace lrtei {
 namespace tc {
-
-constexpr int BM = 128;      // rows of A per tile (MMA M)
-constexpr int KCHUNK = 128;  // K per accumulation chunk drained by the epilogue
-// K per pipeline stage, BK: 64 (128-byte rows, 128-byte swizzle) or 32 (64-byte rows, 64-byte
-// swizzle, smaller stages so more of them fit in shared memory).
-constexpr int NA = 3;        // A slices: s0, t1, t2'
-constexpr int NB = 4;        // B slices: s0, t1, t1', t2'
-// Epilogue warps: 4 per TMEM lane quadrant, each draining BN/4 columns of its 32 lanes per
-// chunk (two running sums per element: 64 registers a thread at BN = 128; 96 available).
-template <int BN>
-__host__ __device__ constexpr int epi_warps() { return 16; }
-template <int BN>
-__host__ __device__ constexpr int block_threads() { return 64 + 32 * epi_warps<BN>(); }  // producer, MMA, epilogue
-
-constexpr int kGroupM = 16;    // tiles of M walked together (L2 reuse of both operands)
-constexpr int kGroupRows = 8;  // block rows walked together in the symmetric upper triangle
-
-struct Params {
-  int64_t M, N;
-  int64_t tiles_m, tiles_n;
-  int64_t ntiles;         // number of output tiles (upper triangle if symmetric)
-  int nchunks_total;      // kpad / KCHUNK
-  int chunks_per_split;
-  const int* ea;
-  const int* eb;
-  double scale;
-  double* C;
-  int64_t ldc;
-  int64_t split_stride;   // elements between split partials (splits > 1)
-  int transpose_out;
-  int symmetric;
-  int splits;
-  int* status;
-  int64_t a_row0;         // row of C that row 0 of A computes (a row band of a symmetric product)
-  int64_t blk0, blk1;     // symmetric product: the 128-row blocks [blk0, blk1) of the upper triangle
-  long long test_stall;   // > 0 (tests only): the MMA thread first waits this many cycles on a barrier
-                          // that nothing completes, so that the bounded-wait failure path runs
-};
-
-// Instruction descriptor: kind::f16, D FP32, both K-major, M = 128, N = BN; A/B FP16 (format 0)
-// for the integer slices, BF16 (format 1) for plain BF16 operands.
-template <int BN, bool PLAIN>
-__device__ __forceinline__ uint32_t instr_desc() {
-  constexpr uint32_t f = PLAIN ? 1u : 0u;
-  return (1u << 4) | (f << 7) | (f << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-}
 
 __device__ __forceinline__ double pow2(int k) {  // 2^k, exponent clamped to the normal range
   k = max(-1022, min(1023, k));
@@ -137,1100 +67,248 @@ __device__ __forceinline__ double combine_pow2(int t0, float t12, int k, float t
   return __longlong_as_double((long long)bits);
 }
 
-// Output element of a staged tile: scale 2^k (T0 + T12 / 2^12), or scale 2^k T12 for plain BF16.
-template <bool PLAIN, bool P8>
-__device__ __forceinline__ double tile_value(const int* st0, const float* st12, const float* st2, int i, int k,
-                                            double scale) {
-  if constexpr (PLAIN) return scale * pow2(k) * (double)st12[i];
-  const double v = combine_pow2(st0[i], st12[i], k, P8 ? st2[i] : 0.f);
-  return scale == 1.0 ? v : scale * v;
-}
+enum class Scheme { six, eight, plain };
 
-// One work item of the persistent grid: an output tile and a K range.
-struct Work {
-  int64_t m0, n0;
-  int c_begin, nchunks;
-  int split;
-  bool mirror;  // strictly above the diagonal block of a symmetric product: write C^T too
-};
+// KS_: 16-deep steps per stage; two halve the barrier rounds, one where a step table lists single blocks.
+template <int BN_, Scheme M, int KS_>
+struct Split {
+  static constexpr bool P8 = M == Scheme::eight, PLAIN = M == Scheme::plain;
+  static constexpr int BN = BN_, NP = PLAIN ? 1 : 3, PT = NP, NACC = PLAIN ? 1 : P8 ? 3 : 2, KS = KS_;
+  static constexpr int UNIT = 8, CHUNK = 8;  // 128 deep
+  static constexpr bool BF16 = PLAIN, ACCUM = false;
 
-// Item -> tile.  Items are split-major, so the ~152 items running at once belong to one split
-// and share operand slabs in L2: tiles are walked in groups of kGroupM M-tiles (M fastest inside
-// a group); the symmetric product walks the upper triangle of 128x128 blocks in groups of
-// kGroupRows block rows, column by column.
-template <int BN>
-__device__ __forceinline__ Work work_item(const Params& p, int64_t item) {
-  Work w;
-  const int64_t tile = item % p.ntiles;
-  w.split = (int)(item / p.ntiles);
-  int64_t ti, tj;
-  w.mirror = false;
-  if (p.symmetric) {
-    constexpr int SUB = BM / BN;
-    const int64_t nb = (p.tiles_n + SUB - 1) / SUB;  // 128x128 blocks per side
-    int64_t t = tile / SUB;
-    const int sub = (int)(tile % SUB);
-    int64_t r = 0, c = 0;
-    for (int64_t R0 = p.blk0; R0 < p.blk1; R0 += kGroupRows) {
-      const int64_t R1 = min(p.blk1, R0 + kGroupRows), g = R1 - R0;
-      const int64_t in_group = g * (g + 1) / 2 + (nb - R1) * g;
-      if (t >= in_group) { t -= in_group; continue; }
-      for (c = R0; c < nb; ++c) {
-        const int64_t rows_here = min(c, R1 - 1) - R0 + 1;
-        if (t < rows_here) { r = R0 + t; break; }
-        t -= rows_here;
+  static __device__ __forceinline__ void mma(uint32_t d0, uint64_t a0, uint64_t b0, uint32_t idesc, uint32_t first) {
+    if constexpr (PLAIN) {
+      mma_bf16(d0, a0, b0, idesc, first);
+    } else {
+      constexpr uint64_t AS = (128 * 32) >> 4, BS = (BN * 32) >> 4;  // from plane to plane
+      const uint32_t d1 = d0 + BN, d2 = P8 ? d0 + 2 * BN : d1;
+      const uint64_t a1 = a0 + AS, a2 = a0 + 2 * AS, b1 = b0 + BS, b2 = b0 + 2 * BS;
+      // grouped by A slice so that each is read from shared memory once per k step; with eight products the
+      // smaller terms go to their own accumulator d2, so that the tensor core's truncating FP32 accumulation
+      // cuts them at their own scale
+      mma_bf16_a<ACol::fill>(d0, a0, b0, idesc, first);
+      mma_bf16_a<ACol::use>(d1, a0, b1, idesc, first);
+      mma_bf16_a<ACol::lastuse>(d2, a0, b2, idesc, P8 ? first : 1u);
+      mma_bf16_a<ACol::fill>(d1, a1, b0, idesc, 1u);
+      mma_bf16_a<ACol::lastuse>(d2, a1, b1, idesc, 1u);
+      if constexpr (P8) {
+        mma_bf16_a<ACol::fill>(d2, a2, b0, idesc, 1u);
+        mma_bf16_a<ACol::lastuse>(d2, a2, b1, idesc, 1u);
+        mma_bf16(d2, a1, b2, idesc, 1u);
+      } else {
+        mma_bf16(d1, a2, b0, idesc, 1u);
       }
-      break;
     }
-    ti = r;
-    tj = c * SUB + sub;
-    w.mirror = c != r;
-  } else {
-    const int64_t per_group = (int64_t)kGroupM * p.tiles_n;
-    const int64_t first_m = (tile / per_group) * kGroupM;
-    const int64_t gsize = min((int64_t)kGroupM, p.tiles_m - first_m);
-    const int64_t in_g = tile % per_group;
-    ti = first_m + in_g % gsize;
-    tj = in_g / gsize;
   }
-  w.m0 = ti * BM;
-  w.n0 = tj * BN;
-  w.c_begin = w.split * p.chunks_per_split;
-  w.nchunks = max(0, min(p.nchunks_total, w.c_begin + p.chunks_per_split) - w.c_begin);
-  return w;
-}
 
-// ------------------------------------------------------------------ the kernel
-// Persistent: CTA b walks the items b, b + gridDim.x, ...  The producer, the MMA thread and the
-// epilogue warps keep running counters of k steps and chunks across items, so the ring stages
-// and the two accumulator buffers flow from one tile to the next.  A finished tile is staged
-// through the ring's shared memory (idle then: the producer waits for the epilogue's "staged
-// tile stored" barrier before it loads the next tile), then stored coalesced.
-// PLAIN: one BF16 operand plane each, one product per k step, FP32 sums (no exactness).
-// P8: eight products per k step (the next-order terms t1' t2' and t2' t1' kept, with a fourth A
-// slice t1' = t1 / 2^12) into three accumulators.
-template <int BN, int BK, int STAGES, bool PLAIN, bool P8>
-__global__ void __launch_bounds__(block_threads<BN>(), 1)
-    k_tc_gemm(const __grid_constant__ CUtensorMap ta0, const __grid_constant__ CUtensorMap ta1,
-              const __grid_constant__ CUtensorMap ta2, const __grid_constant__ CUtensorMap ta1h,
-              const __grid_constant__ CUtensorMap tb0, const __grid_constant__ CUtensorMap tb1,
-              const __grid_constant__ CUtensorMap tb1h, const __grid_constant__ CUtensorMap tb2, const Params p) {
-  constexpr uint32_t A_BYTES = BM * BK * 2;
-  constexpr uint32_t B_BYTES = BN * BK * 2;
-  constexpr int NA_ = PLAIN ? 1 : (P8 ? NA + 1 : NA), NB_ = PLAIN ? 1 : NB;
-  constexpr uint32_t STAGE_BYTES = NA_ * A_BYTES + NB_ * B_BYTES;
-  constexpr int KSTEPS = KCHUNK / BK;  // pipeline stages per chunk
-  constexpr int QC = BN / (epi_warps<BN>() / 4);  // columns per epilogue thread
-  constexpr int NACC = P8 ? 3 : 2;                 // accumulators per buffer: L0, L12 (L1, L2 if P8)
-  static_assert(2 * NACC * BN <= 512, "two buffers of the accumulators must fit in TMEM");
-  constexpr int NE = 32 * epi_warps<BN>();
-
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  constexpr uint32_t TILE_BYTES = BM * (BN + 1) * 4 * (P8 ? 3 : 2) + (BM + BN) * 4;
-  constexpr uint32_t RING_BYTES = (STAGES * STAGE_BYTES > TILE_BYTES) ? STAGES * STAGE_BYTES : TILE_BYTES;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + ((RING_BYTES + 7) & ~7u));
-  uint64_t* empty = full + STAGES;
-  uint64_t* accf = empty + STAGES;   // [2] accumulator buffer ready
-  uint64_t* acce = accf + 2;         // [2] accumulator buffer drained
-  uint64_t* done = acce + 2;         // all MMAs retired
-  uint64_t* tstored = done + 1;      // the staged tile was stored: the ring may be refilled
-  uint64_t* never = tstored + 1;     // completed by nobody (the test stall waits on it)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(never + 1);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t nitems = p.ntiles * (int64_t)p.splits;
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&accf[b], 1);
-      mbar_init(&acce[b], epi_warps<BN>());
-    }
-    mbar_init(done, 1);
-    mbar_init(tstored, epi_warps<BN>());
-    mbar_init(never, 1);
-    *abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(512)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
-
-  if (warp == 0) {
-    // ---------------------------------------------------------------- TMA producer
-    if (lane == 0) {
-      uint32_t it = 0, ntile = 0;  // k steps issued, items started by this CTA
-      bool stop = false;
-      for (int64_t item = blockIdx.x; item < nitems && !stop; item += gridDim.x, ++ntile) {
-        if (ntile > 0) {
-          // the previous tile is staged in the ring's memory until the epilogue has stored it
-          if (!mbar_wait(tstored, (ntile - 1) & 1u, abort_flag, p.status, 64)) break;
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        }
-        const Work w = work_item<BN>(p, item);
-        const int nk = w.nchunks * KSTEPS;
-        for (int kk = 0; kk < nk; ++kk, ++it) {
-          const int s = (int)(it % STAGES);
-          const uint32_t ph = (it / STAGES) & 1u;
-          if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag, p.status, 32)) { stop = true; break; }
-          mbar_arrive_expect_tx(&full[s], STAGE_BYTES);
-          uint8_t* st = smem + (size_t)s * STAGE_BYTES;
-          const int kx = (w.c_begin * KSTEPS + kk) * BK;
-          const int ay = (int)(w.m0 - p.a_row0);
-          uint8_t* sb = st + NA_ * A_BYTES;
-          tma_load_2d(&ta0, st + 0 * A_BYTES, &full[s], kx, ay);
-          tma_load_2d(&tb0, sb + 0 * B_BYTES, &full[s], kx, (int)w.n0);
-          if constexpr (!PLAIN) {
-            tma_load_2d(&ta1, st + 1 * A_BYTES, &full[s], kx, ay);
-            tma_load_2d(&ta2, st + 2 * A_BYTES, &full[s], kx, ay);
-            tma_load_2d(&tb1, sb + 1 * B_BYTES, &full[s], kx, (int)w.n0);
-            tma_load_2d(&tb1h, sb + 2 * B_BYTES, &full[s], kx, (int)w.n0);
-            tma_load_2d(&tb2, sb + 3 * B_BYTES, &full[s], kx, (int)w.n0);
-            if constexpr (P8) tma_load_2d(&ta1h, st + 3 * A_BYTES, &full[s], kx, ay);
-          }
-        }
-      }
-      // On abort, wait (bounded) for the loads still in flight before the CTA can exit.
-      if (*abort_flag) {
-        for (uint32_t j = (it > (uint32_t)STAGES ? it - STAGES : 0u); j < it; ++j) {
-          const int s = (int)(j % STAGES);
-          long long t0 = clock64();
-          while (!mbar_try_wait(&full[s], (j / STAGES) & 1u) && clock64() - t0 < kWaitCycles) {
-          }
-        }
-      }
-    }
-  } else if (warp == 1) {
-    // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      const uint32_t idesc = instr_desc<BN, PLAIN>();
-      uint32_t it = 0, cg = 0;  // k steps and chunks consumed, across items
-      bool ok = true;
-      // test hook: a wait that runs out (nothing arrives on `never`), then the abort path
-      if (p.test_stall > 0) ok = mbar_wait(never, 0u, abort_flag, p.status, 0, p.test_stall);
-      for (int64_t item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-        const Work w = work_item<BN>(p, item);
-        for (int c = 0; c < w.nchunks && ok; ++c, ++cg) {
-          const int buf = (int)(cg & 1u);
-          if (!mbar_wait(&acce[buf], ((cg >> 1) & 1u) ^ 1u, abort_flag, p.status)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t d0 = tmem_base + (uint32_t)(buf * NACC * BN);
-          const uint32_t d1 = d0 + BN;
-          const uint32_t d2 = P8 ? d0 + 2 * BN : d1;
-          for (int step = 0; step < KSTEPS; ++step, ++it) {
-            const int s = (int)(it % STAGES);
-            if (!mbar_wait(&full[s], (it / STAGES) & 1u, abort_flag, p.status)) { ok = false; break; }
-            tc_fence_after();
-            const uint32_t base = smem_u32(smem + (size_t)s * STAGE_BYTES);
-            const uint64_t a0 = smem_desc<BK>(base), a1 = smem_desc<BK>(base + A_BYTES),
-                           a2 = smem_desc<BK>(base + 2 * A_BYTES), a1h = smem_desc<BK>(base + 3 * A_BYTES);
-            const uint32_t bb = base + NA_ * A_BYTES;
-            const uint64_t b0 = smem_desc<BK>(bb), b1 = smem_desc<BK>(bb + B_BYTES),
-                           b1h = smem_desc<BK>(bb + 2 * B_BYTES), b2 = smem_desc<BK>(bb + 3 * B_BYTES);
-#pragma unroll
-            for (int k = 0; k < BK / 16; ++k) {
-              const uint64_t o = (uint64_t)((k * 32) >> 4);  // +32 bytes along K inside the swizzle atom
-              const uint32_t first = (step == 0 && k == 0) ? 0u : 1u;
-              if constexpr (PLAIN) {
-                mma_bf16(d0, a0 + o, b0 + o, idesc, first);
-              } else {
-                // grouped by A slice so that each is read from shared memory once per k step
-                // P8: L1 = s0 t1 + t1 s0 in d1, the smaller terms in their own accumulator d2, so
-                // that the tensor core's truncating FP32 accumulation cuts them at their own scale
-                mma_bf16_a<ACol::fill>(d0, a0 + o, b0 + o, idesc, first);
-                mma_bf16_a<ACol::use>(d1, a0 + o, b1 + o, idesc, first);
-                mma_bf16_a<ACol::lastuse>(d2, a0 + o, b2 + o, idesc, P8 ? first : 1u);
-                mma_bf16_a<ACol::fill>(d1, a1 + o, b0 + o, idesc, 1u);
-                mma_bf16_a<ACol::lastuse>(d2, a1 + o, b1h + o, idesc, 1u);
-                if constexpr (P8) {
-                  mma_bf16_a<ACol::fill>(d2, a2 + o, b0 + o, idesc, 1u);
-                  mma_bf16_a<ACol::lastuse>(d2, a2 + o, b1h + o, idesc, 1u);  // t2' t1'
-                  mma_bf16(d2, a1h + o, b2 + o, idesc, 1u);                  // t1' t2'
-                } else {
-                  mma_bf16(d1, a2 + o, b0 + o, idesc, 1u);
-                }
-              }
-            }
-            mma_commit(&empty[s]);  // stage s may be refilled once these MMAs retire
-          }
-          if (!ok) break;
-          mma_commit(&accf[buf]);
-        }
-      }
-      // retire every MMA this thread issued before TMEM is released
-      mma_commit(done);
-      long long t0 = clock64();
-      while (!mbar_try_wait(done, 0u) && clock64() - t0 < kWaitCycles) {
-      }
-    }
-  } else {
-    // ---------------------------------------------------------------- epilogue warps
-    const int ew = warp - 2;
-    const int quad = warp & 3;             // TMEM lane quadrant this warp may access
-    const int col0 = (ew >> 2) * QC;       // first column of this thread
-    const int row = quad * 32 + lane;      // row inside the tile
-    const int et = threadIdx.x - 64;       // 0..NE-1 over the epilogue warps
-    constexpr int LDS = BN + 1;            // padded row stride (words) against bank conflicts
-    int* st0 = reinterpret_cast<int*>(smem);
-    float* st12 = reinterpret_cast<float*>(st0 + BM * LDS);
-    float* st2 = st12 + BM * LDS;  // P8 only
-    int* sea = reinterpret_cast<int*>(st2 + (P8 ? BM * LDS : 0));
-    int* seb = sea + BM;
-    uint32_t cg = 0;                       // chunks drained, across items
-    bool ok = true;
-    for (int64_t item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-      const Work w = work_item<BN>(p, item);
-      int T0[QC];
-      float T12[QC];
-      float T2[P8 ? QC : 1];
+  template <int QC>
+  struct Sums {
+    int T0[PLAIN ? 1 : QC];
+    float T1[QC], T2[P8 ? QC : 1];
+    __device__ __forceinline__ void clear() {
 #pragma unroll
       for (int j = 0; j < QC; ++j) {
-        T0[j] = 0;
-        T12[j] = 0.f;
+        if constexpr (!PLAIN) T0[j] = 0;
+        T1[j] = 0.f;
         if constexpr (P8) T2[j] = 0.f;
       }
-      for (int c = 0; c < w.nchunks; ++c, ++cg) {
-        const int buf = (int)(cg & 1u);
-        // one lane waits, the warp reconverges before the .sync.aligned TMEM loads
-        int got = 1;
-        if (lane == 0) got = mbar_wait(&accf[buf], (cg >> 1) & 1u, abort_flag, p.status, 128) ? 1 : 0;
-        got = __shfl_sync(0xffffffffu, got, 0);
-        if (!got) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t tbase = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * NACC * BN + col0);
-        // both accumulators' loads of an 8-column group are in flight together (one wait per group)
-#pragma unroll
-        for (int j0 = 0; j0 < QC; j0 += 8) {
-          uint32_t r[8], q[8];
-          tmem_ld8(tbase + j0, r);
-          if constexpr (!PLAIN) tmem_ld8(tbase + BN + j0, q);
-          tmem_wait_ld();
-          if constexpr (PLAIN) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) T12[j0 + j] += __uint_as_float(r[j]);
-          } else {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              T0[j0 + j] += __float2int_rn(__uint_as_float(r[j]));
-              T12[j0 + j] += __uint_as_float(q[j]);
-            }
-            if constexpr (P8) {
-              tmem_ld8(tbase + 2 * BN + j0, q);
-              tmem_wait_ld();
-#pragma unroll
-              for (int j = 0; j < 8; ++j) T2[j0 + j] += __uint_as_float(q[j]);
-            }
-          }
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&acce[buf]);
-      }
-      if (!ok || *abort_flag) break;
-      // Every MMA of this tile has retired (its last accumulator buffer was signalled) and the
-      // producer loads nothing until this tile is stored: stage it through the ring's memory.
-      // The running sums are staged as 32-bit words and combined by the store loop.
-#pragma unroll
-      for (int j = 0; j < QC; ++j) {
-        st0[row * LDS + col0 + j] = T0[j];
-        st12[row * LDS + col0 + j] = T12[j];
-        if constexpr (P8) st2[row * LDS + col0 + j] = T2[j];
-      }
-      if (et < BM) sea[et] = (w.m0 + et < p.M) ? p.ea[w.m0 - p.a_row0 + et] : 0;
-      if (et < BN) seb[et] = (w.n0 + et < p.N) ? p.eb[w.n0 + et] : 0;
-      asm volatile("bar.sync 1, %0;" ::"r"(NE) : "memory");
-      double* Cs = p.C + (int64_t)w.split * p.split_stride;
-      // On a diagonal block of a symmetric product only the upper triangle (gm <= gn) is
-      // kept and mirrored, so that C comes out exactly symmetric.
-      const bool diag = p.symmetric && !w.mirror;
-      if (!p.transpose_out) {  // row-major: consecutive threads along a row
-        for (int idx = et; idx < BM * BN; idx += NE) {
-          const int r = idx / BN, c = idx % BN;
-          const int64_t gm = w.m0 + r, gn = w.n0 + c;
-          if (gm < p.M && gn < p.N && (!diag || gm <= gn))
-            Cs[gm * p.ldc + gn] = tile_value<PLAIN, P8>(st0, st12, st2, r * LDS + c, sea[r] + seb[c] - 16, p.scale);
-        }
-      }
-      if (p.transpose_out || p.symmetric) {  // C^T: consecutive threads along a column of C
-        for (int idx = et; idx < BM * BN; idx += NE) {
-          const int c = idx / BM, r = idx % BM;
-          const int64_t gm = w.m0 + r, gn = w.n0 + c;
-          if (gm < p.M && gn < p.N && (!diag || gm < gn))
-            Cs[gn * p.ldc + gm] = tile_value<PLAIN, P8>(st0, st12, st2, r * LDS + c, sea[r] + seb[c] - 16, p.scale);
-        }
-      }
-      // every epilogue thread has read the staged tile: the ring may be refilled
-      asm volatile("bar.sync 1, %0;" ::"r"(NE) : "memory");
-      if (lane == 0) mbar_arrive(tstored);
     }
-  }
-  __syncthreads();
-  if (warp == 1) {
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
-  }
-}
-
-// ------------------------------------------------------------------ host side
-template <int BN, int BK, int STAGES, bool PLAIN, bool P8>
-static lrtei_status launch_tc(const SplitMatrix& A, const SplitMatrix& B, const Params& p, int splits,
-                              cudaStream_t st) {
-  CUtensorMap m[8];  // A: s0, s1, s2, s1h (eight-product scheme); B: s0, s1, s1h, s2
-  bool ok;
-  if (PLAIN) {
-    ok = encode_plane(&m[0], A.s0, A.rows, A.kpad, BM, true, BK) && encode_plane(&m[4], B.s0, B.rows, B.kpad, BN, true, BK);
-    m[1] = m[2] = m[3] = m[0];
-    m[5] = m[6] = m[7] = m[4];
-  } else {
-    ok = encode_plane(&m[0], A.s0, A.rows, A.kpad, BM, false, BK) &&
-         encode_plane(&m[1], A.s1, A.rows, A.kpad, BM, false, BK) &&
-         encode_plane(&m[2], A.s2, A.rows, A.kpad, BM, false, BK) &&
-         encode_plane(&m[4], B.s0, B.rows, B.kpad, BN, false, BK) &&
-         encode_plane(&m[5], B.s1, B.rows, B.kpad, BN, false, BK) &&
-         encode_plane(&m[6], B.s1h, B.rows, B.kpad, BN, false, BK) &&
-         encode_plane(&m[7], B.s2, B.rows, B.kpad, BN, false, BK);
-    if (ok && P8) ok = encode_plane(&m[3], A.s1h, A.rows, A.kpad, BM, false, BK);
-    if (!P8) m[3] = m[0];
-  }
-  if (!ok) {
-    set_error("cuTensorMapEncodeTiled failed (driver entry point unavailable or bad operand layout)");
-    return LRTEI_ERR_CUDA;
-  }
-  constexpr size_t stage =
-      (size_t)(PLAIN ? 1 : (P8 ? NA + 1 : NA)) * BM * BK * 2 + (size_t)(PLAIN ? 1 : NB) * BN * BK * 2;
-  const size_t tile_bytes = (size_t)BM * (BN + 1) * 4 * (P8 ? 3 : 2) + (BM + BN) * 4;
-  const size_t smem = std::max(STAGES * stage, tile_bytes) + 1024 + 256;
-  static bool attr_set = false;  // once per instantiation (also keeps it out of stream capture)
-  cudaError_t e = cudaSuccess;
-  if (!attr_set) {
-    e = cudaFuncSetAttribute(k_tc_gemm<BN, BK, STAGES, PLAIN, P8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-    if (e != cudaSuccess) return cuda_fail(e, "tc_gemm smem attribute");
-    attr_set = true;
-  }
-  static int nsm = 0;  // persistent grid: one CTA per SM (shared memory and TMEM allow one)
-  if (nsm <= 0) {
-    int dev = 0;
-    LRTEI_CUDA(cudaGetDevice(&dev));
-    LRTEI_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  }
-  const int64_t nitems = p.ntiles * (int64_t)splits;
-  dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(nitems, nsm)));
-  count_launch();
-  k_tc_gemm<BN, BK, STAGES, PLAIN, P8>
-      <<<grid, block_threads<BN>(), smem, st>>>(m[0], m[1], m[2], m[3], m[4], m[5], m[6], m[7], p);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_fail(e, "tc_gemm launch");
-  return LRTEI_OK;
-}
-
-
-// ------------------------------------------------------------------ the 2-SM variant
-// cta_group::2: a cluster of two CTAs (on the two SMs of a TPC) computes a 256 x 128 tile of C.
-// Each CTA loads its own 128 rows of A and half of B (64 rows) into its shared memory; the
-// leader CTA (rank 0) issues M = 256, N = 128 MMAs that read A from both CTAs and both halves of
-// B, and write each CTA's 128 rows of the two accumulators into that CTA's TMEM.  Per 64-deep
-// stage an SM receives 80 KB (three 128-row A planes, four 64-row B planes) instead of 112 KB for
-// the same MMA work per SM.  Both CTAs' TMA loads complete on the leader's "full" barrier; the
-// leader's MMA commits arrive on both CTAs' "empty" and "accumulator ready" barriers (multicast);
-// both CTAs' epilogue warps arrive on the leader's "accumulator drained" barrier.  Six products,
-// 128 x 128 tiles per CTA, two 64-deep or five 32-deep stages; the symmetric product walks pairs
-// of block rows.  The tuner times it beside the one-SM configurations (run_tuned).  Every wait is
-// bounded as in k_tc_gemm.
-namespace pair2 {
-constexpr int BN = 128;      // columns of the pair's tile (N of the MMA)
-constexpr int HB = BN / 2;   // B rows each CTA loads
-constexpr int kGroupM2 = 8;  // 256-row tiles walked together
-constexpr uint32_t TILE_BYTES = BM * (BN + 1) * 4 * 2 + (BM + BN) * 4;
-constexpr int EPI = 16;  // epilogue warps
-constexpr int THREADS = 64 + 32 * EPI;
-// stage depth BK and count: 64-deep (128-byte swizzle) x 2 or 32-deep (64-byte swizzle) x 5
-template <int BK>
-__host__ __device__ constexpr uint32_t a_bytes() { return BM * BK * 2; }  // one A plane (128 rows)
-template <int BK>
-__host__ __device__ constexpr uint32_t b_bytes() { return HB * BK * 2; }  // one B plane half (64 rows)
-template <int BK>
-__host__ __device__ constexpr uint32_t stage_bytes() { return NA * a_bytes<BK>() + NB * b_bytes<BK>(); }
-template <int BK, int STAGES>
-__host__ __device__ constexpr uint32_t ring_bytes() {
-  return (STAGES * stage_bytes<BK>() > TILE_BYTES) ? STAGES * stage_bytes<BK>() : TILE_BYTES;
-}
-}  // namespace pair2
-
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ uint32_t cluster_idx() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ uint32_t cluster_count() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%nclusterid.x;" : "=r"(r));
-  return r;
-}
-// shared::cluster address of the same shared-memory offset in CTA `rank` of the cluster
-__device__ __forceinline__ uint32_t map_rank(uint32_t saddr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-// TMA load into this CTA's shared memory, completing on an mbarrier of either CTA of the pair
-__device__ __forceinline__ void tma_load_2d_pair(const CUtensorMap* map, void* dst, uint32_t bar_cluster_addr, int x,
-                                                 int y) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
-      "[%4];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar_cluster_addr)
-      : "memory");
-}
-template <ACol C>
-__device__ __forceinline__ void mma2_a(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                       uint32_t accumulate) {
-  if constexpr (C == ACol::fill)
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16.collector::a::fill [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-  else if constexpr (C == ACol::use)
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16.collector::a::use [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-  else
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16.collector::a::lastuse [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-__device__ __forceinline__ void mma2(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                     uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(
-          d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// arrive on the same barrier offset in both CTAs of the pair once the MMAs issued so far retire
-__device__ __forceinline__ void mma2_commit_both(uint64_t* bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-          smem_u32(bar)),
-      "h"((uint16_t)3)
-      : "memory");
-}
-
-struct Work2 {
-  int64_t m0, n0;
-  int c_begin, nchunks;
-  int split;
-  int64_t cblk;  // symmetric product: the 128-column block of the tile
-};
-
-// Item -> tile.  Non-symmetric: groups of kGroupM2 256-row tiles, M fastest.  Symmetric (the upper
-// triangle of 128 x 128 blocks, block rows [blk0, blk1), blk0 even): pairs of block rows
-// (2i, 2i + 1) and the column blocks c >= 2i, in groups of kGroupM2 pairs, column by column; the
-// lower CTA's block (2i + 1, 2i) lies below the diagonal and is not stored.
-__device__ __forceinline__ Work2 work_item2(const Params& p, int64_t item) {
-  Work2 w;
-  const int64_t tile = item % p.ntiles;
-  w.split = (int)(item / p.ntiles);
-  if (p.symmetric) {
-    const int64_t nb = (p.N + BM - 1) / BM;
-    const int64_t P0 = p.blk0 / 2, P1 = (p.blk1 + 1) / 2;
-    int64_t t = tile, pi = P0, c = 2 * P0;
-    for (int64_t G0 = P0; G0 < P1; G0 += pair2::kGroupM2) {
-      const int64_t G1 = min(P1, G0 + (int64_t)pair2::kGroupM2);
-      int64_t in_group = 0;
-      for (int64_t cc = 2 * G0; cc < nb; ++cc) in_group += max((int64_t)0, min(G1, cc / 2 + 1) - G0);
-      if (t >= in_group) { t -= in_group; continue; }
-      for (c = 2 * G0; c < nb; ++c) {
-        const int64_t rows_here = max((int64_t)0, min(G1, c / 2 + 1) - G0);
-        if (t < rows_here) { pi = G0 + t; break; }
-        t -= rows_here;
-      }
-      break;
-    }
-    w.m0 = pi * (2 * BM);
-    w.n0 = c * pair2::BN;
-    w.cblk = c;
-    w.c_begin = 0;
-    w.nchunks = p.nchunks_total;
-    return w;
-  }
-  w.cblk = 0;
-  const int64_t per_group = (int64_t)pair2::kGroupM2 * p.tiles_n;
-  const int64_t first_m = (tile / per_group) * pair2::kGroupM2;
-  const int64_t gsize = min((int64_t)pair2::kGroupM2, p.tiles_m - first_m);
-  const int64_t in_g = tile % per_group;
-  w.m0 = (first_m + in_g % gsize) * (2 * BM);
-  w.n0 = (in_g / gsize) * pair2::BN;
-  w.c_begin = w.split * p.chunks_per_split;
-  w.nchunks = max(0, min(p.nchunks_total, w.c_begin + p.chunks_per_split) - w.c_begin);
-  return w;
-}
-
-template <int BK, int STAGES>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair2::THREADS, 1)
-    k_tc_gemm_2sm(const __grid_constant__ CUtensorMap ta0, const __grid_constant__ CUtensorMap ta1,
-                  const __grid_constant__ CUtensorMap ta2, const __grid_constant__ CUtensorMap tb0,
-                  const __grid_constant__ CUtensorMap tb1, const __grid_constant__ CUtensorMap tb1h,
-                  const __grid_constant__ CUtensorMap tb2, const Params p) {
-  using namespace pair2;
-  constexpr uint32_t A_BYTES = a_bytes<BK>(), B_BYTES = b_bytes<BK>(), STAGE_BYTES = stage_bytes<BK>();
-  constexpr uint32_t RING_BYTES = ring_bytes<BK, STAGES>();
-  constexpr int KSTEPS = KCHUNK / BK;
-  constexpr int QC = BN / (EPI / 4);  // columns per epilogue thread
-  constexpr int NE = 32 * EPI;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + ((RING_BYTES + 7) & ~7u));
-  uint64_t* empty = full + STAGES;
-  uint64_t* accf = empty + STAGES;   // [2] accumulator buffer ready (both CTAs)
-  uint64_t* acce = accf + 2;         // [2] accumulator buffer drained (leader: both CTAs' epilogues)
-  uint64_t* done = acce + 2;         // all MMAs retired (both CTAs)
-  uint64_t* tstored = done + 1;      // this CTA's staged tile was stored
-  uint64_t* never = tstored + 1;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(never + 1);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_ctarank();
-  const bool leader = rank == 0;
-  const int64_t nitems = p.ntiles * (int64_t)p.splits;
-  const int64_t cid = cluster_idx(), ncl = cluster_count();
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&accf[b], 1);
-      mbar_init(&acce[b], 2 * EPI);
-    }
-    mbar_init(done, 1);
-    mbar_init(tstored, EPI);
-    mbar_init(never, 1);
-    *abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(512)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-  }
-  __syncthreads();
-  cluster_sync_all();  // both CTAs' barriers are initialised before any remote arrival
-  tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
-  const uint32_t full_l0 = map_rank(smem_u32(&full[0]), 0);  // the leader's full barriers
-  const uint32_t acce_l0 = map_rank(smem_u32(&acce[0]), 0);  // the leader's drained barriers
-
-  if (warp == 0) {
-    // ---------------------------------------------------------------- TMA producer (both CTAs)
-    if (lane == 0) {
-      uint32_t it = 0, ntile = 0;
-      bool stop = false;
-      for (int64_t item = cid; item < nitems && !stop; item += ncl, ++ntile) {
-        if (ntile > 0) {
-          if (!mbar_wait(tstored, (ntile - 1) & 1u, abort_flag, p.status, 64)) break;
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        }
-        const Work2 w = work_item2(p, item);
-        const int nk = w.nchunks * KSTEPS;
-        for (int kk = 0; kk < nk; ++kk, ++it) {
-          const int s = (int)(it % STAGES);
-          const uint32_t ph = (it / STAGES) & 1u;
-          if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag, p.status, 32)) { stop = true; break; }
-          if (leader) mbar_arrive_expect_tx(&full[s], 2 * STAGE_BYTES);  // both CTAs' bytes
-          uint8_t* st = smem + (size_t)s * STAGE_BYTES;
-          uint8_t* sb = st + NA * A_BYTES;
-          const uint32_t fb = full_l0 + (uint32_t)(s * sizeof(uint64_t));
-          const int kx = (w.c_begin * KSTEPS + kk) * BK;
-          const int ay = (int)(w.m0 + rank * BM - p.a_row0);
-          const int by = (int)(w.n0 + rank * HB);
-          tma_load_2d_pair(&ta0, st + 0 * A_BYTES, fb, kx, ay);
-          tma_load_2d_pair(&ta1, st + 1 * A_BYTES, fb, kx, ay);
-          tma_load_2d_pair(&ta2, st + 2 * A_BYTES, fb, kx, ay);
-          tma_load_2d_pair(&tb0, sb + 0 * B_BYTES, fb, kx, by);
-          tma_load_2d_pair(&tb1, sb + 1 * B_BYTES, fb, kx, by);
-          tma_load_2d_pair(&tb1h, sb + 2 * B_BYTES, fb, kx, by);
-          tma_load_2d_pair(&tb2, sb + 3 * B_BYTES, fb, kx, by);
-        }
-      }
-      // On abort the leader waits (bounded) for the stages in flight: they complete only when both
-      // CTAs' loads have landed.
-      if (*abort_flag && leader) {
-        for (uint32_t j = (it > (uint32_t)STAGES ? it - STAGES : 0u); j < it; ++j) {
-          const int s = (int)(j % STAGES);
-          long long t0 = clock64();
-          while (!mbar_try_wait(&full[s], (j / STAGES) & 1u) && clock64() - t0 < kWaitCycles) {
-          }
-        }
-      }
-    }
-  } else if (warp == 1) {
-    // ---------------------------------------------------------------- MMA issuer (leader only)
-    if (lane == 0 && leader) {
-      // M = 256 (two CTAs), N = 128, FP16 operands, FP32 accumulators, both K-major
-      const uint32_t idesc = (1u << 4) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)((2 * BM) >> 4) << 24);
-      uint32_t it = 0, cg = 0;
-      bool ok = true;
-      if (p.test_stall > 0) ok = mbar_wait(never, 0u, abort_flag, p.status, 0, p.test_stall);
-      for (int64_t item = cid; item < nitems && ok; item += ncl) {
-        const Work2 w = work_item2(p, item);
-        for (int c = 0; c < w.nchunks && ok; ++c, ++cg) {
-          const int buf = (int)(cg & 1u);
-          if (!mbar_wait(&acce[buf], ((cg >> 1) & 1u) ^ 1u, abort_flag, p.status)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t d0 = tmem_base + (uint32_t)(buf * 2 * BN);
-          const uint32_t d1 = d0 + BN;
-          for (int step = 0; step < KSTEPS; ++step, ++it) {
-            const int s = (int)(it % STAGES);
-            if (!mbar_wait(&full[s], (it / STAGES) & 1u, abort_flag, p.status)) { ok = false; break; }
-            tc_fence_after();
-            const uint32_t base = smem_u32(smem + (size_t)s * STAGE_BYTES);
-            const uint64_t a0 = smem_desc<BK>(base), a1 = smem_desc<BK>(base + A_BYTES),
-                           a2 = smem_desc<BK>(base + 2 * A_BYTES);
-            const uint32_t bb = base + NA * A_BYTES;
-            const uint64_t b0 = smem_desc<BK>(bb), b1 = smem_desc<BK>(bb + B_BYTES),
-                           b1h = smem_desc<BK>(bb + 2 * B_BYTES), b2 = smem_desc<BK>(bb + 3 * B_BYTES);
+    __device__ __forceinline__ void drain(uint32_t t) {
 #pragma unroll
-            for (int k = 0; k < BK / 16; ++k) {
-              const uint64_t o = (uint64_t)((k * 32) >> 4);
-              const uint32_t first = (step == 0 && k == 0) ? 0u : 1u;
-              mma2_a<ACol::fill>(d0, a0 + o, b0 + o, idesc, first);
-              mma2_a<ACol::use>(d1, a0 + o, b1 + o, idesc, first);
-              mma2_a<ACol::lastuse>(d1, a0 + o, b2 + o, idesc, 1u);
-              mma2_a<ACol::fill>(d1, a1 + o, b0 + o, idesc, 1u);
-              mma2_a<ACol::lastuse>(d1, a1 + o, b1h + o, idesc, 1u);
-              mma2(d1, a2 + o, b0 + o, idesc, 1u);
-            }
-            mma2_commit_both(&empty[s]);
-          }
-          if (!ok) break;
-          mma2_commit_both(&accf[buf]);
+      for (int j0 = 0; j0 < QC; j0 += 8) {  // the loads of an 8-column group are in flight together
+        uint32_t r[8], q[8];
+        if constexpr (!PLAIN) tmem_ld8(t + j0, r);
+        tmem_ld8(t + (PLAIN ? 0 : BN) + j0, q);
+        tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          if constexpr (!PLAIN) T0[j0 + j] += __float2int_rn(__uint_as_float(r[j]));
+          T1[j0 + j] += __uint_as_float(q[j]);
         }
-      }
-      mma2_commit_both(done);
-      long long t0 = clock64();
-      while (!mbar_try_wait(done, 0u) && clock64() - t0 < kWaitCycles) {
-      }
-    }
-  } else {
-    // ---------------------------------------------------------------- epilogue warps (both CTAs)
-    const int ew = warp - 2;
-    const int quad = warp & 3;
-    const int col0 = (ew >> 2) * QC;
-    const int row = quad * 32 + lane;
-    const int et = threadIdx.x - 64;
-    constexpr int LDS = BN + 1;
-    int* st0 = reinterpret_cast<int*>(smem);
-    float* st12 = reinterpret_cast<float*>(st0 + BM * LDS);
-    int* sea = reinterpret_cast<int*>(st12 + BM * LDS);
-    int* seb = sea + BM;
-    uint32_t cg = 0;
-    bool ok = true;
-    for (int64_t item = cid; item < nitems && ok; item += ncl) {
-      const Work2 w = work_item2(p, item);
-      const int64_t m0 = w.m0 + rank * BM;  // this CTA's 128 rows
-      int T0[QC];
-      float T12[QC];
-#pragma unroll
-      for (int j = 0; j < QC; ++j) {
-        T0[j] = 0;
-        T12[j] = 0.f;
-      }
-      for (int c = 0; c < w.nchunks; ++c, ++cg) {
-        const int buf = (int)(cg & 1u);
-        int got = 1;
-        if (lane == 0) got = mbar_wait(&accf[buf], (cg >> 1) & 1u, abort_flag, p.status, 128) ? 1 : 0;
-        got = __shfl_sync(0xffffffffu, got, 0);
-        if (!got) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t tbase = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * 2 * BN + col0);
-#pragma unroll
-        for (int j0 = 0; j0 < QC; j0 += 8) {
-          uint32_t r[8], q[8];
-          tmem_ld8(tbase + j0, r);
-          tmem_ld8(tbase + BN + j0, q);
+        if constexpr (P8) {
+          tmem_ld8(t + 2 * BN + j0, q);
           tmem_wait_ld();
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            T0[j0 + j] += __float2int_rn(__uint_as_float(r[j]));
-            T12[j0 + j] += __uint_as_float(q[j]);
-          }
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) {
-          if (leader) mbar_arrive(&acce[buf]);
-          else mbar_arrive_remote(acce_l0 + (uint32_t)(buf * sizeof(uint64_t)));
+          for (int j = 0; j < 8; ++j) T2[j0 + j] += __uint_as_float(q[j]);
         }
       }
-      if (!ok || *abort_flag) break;
+    }
+    template <int C>
+    __device__ __forceinline__ void hold(int j0) {
+      if constexpr (!PLAIN) {
 #pragma unroll
-      for (int j = 0; j < QC; ++j) {
-        st0[row * LDS + col0 + j] = T0[j];
-        st12[row * LDS + col0 + j] = T12[j];
-      }
-      if (et < BM) sea[et] = (m0 + et < p.M) ? p.ea[m0 - p.a_row0 + et] : 0;
-      if (et < BN) seb[et] = (w.n0 + et < p.N) ? p.eb[w.n0 + et] : 0;
-      asm volatile("bar.sync 1, %0;" ::"r"(NE) : "memory");
-      double* Cs = p.C + (int64_t)w.split * p.split_stride;
-      if (p.symmetric) {
-        // this CTA's block (br, c): below the diagonal nothing is stored; on it the upper triangle
-        // is kept and mirrored, so that C comes out exactly symmetric; above it, block and mirror
-        const int64_t br = m0 / BM;
-        if (w.cblk >= br) {
-          const bool diag = w.cblk == br;
-          for (int idx = et; idx < BM * BN; idx += NE) {
-            const int r = idx / BN, c = idx % BN;
-            const int64_t gm = m0 + r, gn = w.n0 + c;
-            if (gm < p.M && gn < p.N && (!diag || gm <= gn))
-              Cs[gm * p.ldc + gn] = tile_value<false, false>(st0, st12, st12, r * LDS + c, sea[r] + seb[c] - 16, p.scale);
-          }
-          for (int idx = et; idx < BM * BN; idx += NE) {
-            const int c = idx / BM, r = idx % BM;
-            const int64_t gm = m0 + r, gn = w.n0 + c;
-            if (gm < p.M && gn < p.N && (!diag || gm < gn))
-              Cs[gn * p.ldc + gm] = tile_value<false, false>(st0, st12, st12, r * LDS + c, sea[r] + seb[c] - 16, p.scale);
-          }
-        }
-      } else if (!p.transpose_out) {
-        for (int idx = et; idx < BM * BN; idx += NE) {
-          const int r = idx / BN, c = idx % BN;
-          const int64_t gm = m0 + r, gn = w.n0 + c;
-          if (gm < p.M && gn < p.N)
-            Cs[gm * p.ldc + gn] = tile_value<false, false>(st0, st12, st12, r * LDS + c, sea[r] + seb[c] - 16, p.scale);
-        }
-      } else {
-        for (int idx = et; idx < BM * BN; idx += NE) {
-          const int c = idx / BM, r = idx % BM;
-          const int64_t gm = m0 + r, gn = w.n0 + c;
-          if (gm < p.M && gn < p.N)
-            Cs[gn * p.ldc + gm] = tile_value<false, false>(st0, st12, st12, r * LDS + c, sea[r] + seb[c] - 16, p.scale);
+        for (int j = 0; j < C; ++j) {
+          asm volatile("" : "+r"(T0[j0 + j]), "+f"(T1[j0 + j]) : : "memory");
+          if constexpr (P8) asm volatile("" : "+f"(T2[j0 + j]) : : "memory");
         }
       }
-      asm volatile("bar.sync 1, %0;" ::"r"(NE) : "memory");
-      if (lane == 0) mbar_arrive(tstored);
     }
-  }
-  __syncthreads();
-  // the leader's MMAs write this CTA's TMEM: wait (bounded) until they have all retired
-  if (!leader && threadIdx.x == 0) {
-    long long t0 = clock64();
-    while (!mbar_try_wait(done, 0u) && clock64() - t0 < kWaitCycles) {
+    // The planes' weights make T1 and T2 those of the sums of s0 t1 over 2^12.
+    __device__ __forceinline__ double value(int j, int k, double scale) const {
+      if constexpr (PLAIN) return scale * pow2(k - 16) * (double)T1[j];
+      const double v = combine_pow2(T0[PLAIN ? 0 : j], T1[j] * 4096.f, k - 16, P8 ? T2[P8 ? j : 0] * 4096.f : 0.f);
+      return scale == 1.0 ? v : scale * v;
     }
-  }
-  __syncthreads();
-  cluster_sync_all();
-  if (warp == 1) {
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
-  }
-}
-
-template <int BK, int STAGES>
-static lrtei_status launch_tc_2sm(const SplitMatrix& A, const SplitMatrix& B, const Params& p0, cudaStream_t st) {
-  using namespace pair2;
-  CUtensorMap m[7];
-  const bool ok = encode_plane(&m[0], A.s0, A.rows, A.kpad, BM, false, BK) &&
-                  encode_plane(&m[1], A.s1, A.rows, A.kpad, BM, false, BK) &&
-                  encode_plane(&m[2], A.s2, A.rows, A.kpad, BM, false, BK) &&
-                  encode_plane(&m[3], B.s0, B.rows, B.kpad, HB, false, BK) &&
-                  encode_plane(&m[4], B.s1, B.rows, B.kpad, HB, false, BK) &&
-                  encode_plane(&m[5], B.s1h, B.rows, B.kpad, HB, false, BK) &&
-                  encode_plane(&m[6], B.s2, B.rows, B.kpad, HB, false, BK);
-  if (!ok) {
-    set_error("cuTensorMapEncodeTiled failed (2-SM GEMM operands)");
-    return LRTEI_ERR_CUDA;
-  }
-  Params p = p0;
-  p.tiles_m = (p.M + 2 * BM - 1) / (2 * BM);
-  p.tiles_n = (p.N + BN - 1) / BN;
-  p.ntiles = p.tiles_m * p.tiles_n;
-  if (p.symmetric) {  // pairs of block rows [blk0 / 2, ceil(blk1 / 2)), column blocks c >= 2i
-    const int64_t nb = (p.N + BM - 1) / BM;
-    p.ntiles = 0;
-    for (int64_t i = p.blk0 / 2; i < (p.blk1 + 1) / 2; ++i) p.ntiles += std::max<int64_t>(0, nb - 2 * i);
-  }
-  const size_t smem = (size_t)ring_bytes<BK, STAGES>() + 1024 + 256;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_tc_gemm_2sm<BK, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cuda_fail(e, "2-SM tc_gemm smem attribute");
-    attr_set = true;
-  }
-  static int nsm = 0;
-  if (nsm <= 0) {
-    int dev = 0;
-    LRTEI_CUDA(cudaGetDevice(&dev));
-    LRTEI_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  }
-  const int64_t nitems = p.ntiles * (int64_t)p.splits;
-  const int64_t nclusters = std::max<int64_t>(1, std::min<int64_t>(nitems, nsm / 2));
-  count_launch();
-  k_tc_gemm_2sm<BK, STAGES><<<(unsigned)(2 * nclusters), THREADS, smem, st>>>(m[0], m[1], m[2], m[3], m[4], m[5], m[6],
-                                                                              p);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_fail(e, "2-SM tc_gemm launch");
-  return LRTEI_OK;
-}
-
-}  // namespace tc
-
-namespace tc {
-// Kernel configurations (BN, BK, stages) the tuner chooses from.
-struct Config {
-  int bn, bk, stages;
-};
-static const Config kSplitCfg128[] = {{128, 64, 2}, {128, 32, 4}};
-// eight products, three accumulators (at most 64-column tiles: 2 x 3 x 64 TMEM columns), a
-// fourth A plane
-static const Config kSplit8Cfg64[] = {{64, 64, 2}, {64, 32, 4}};
-static const Config kSplit8Cfg32[] = {{32, 64, 2}, {32, 32, 5}};
-static const Config kSplitCfg64[] = {{64, 64, 2}, {64, 32, 5}};
-static const Config kSplitCfg32[] = {{32, 64, 3}, {32, 32, 6}};
-static const Config kPlainCfg64[] = {{64, 64, 6}, {64, 32, 8}};
-static const Config kPlainCfg32[] = {{32, 64, 6}, {32, 32, 8}};
-
-static lrtei_status launch_cfg(const SplitMatrix& A, const SplitMatrix& B, const Params& p, int splits, bool plain,
-                               const Config& c, cudaStream_t st) {
-  if (A.eight) {
-    if (c.bn == 64) return c.bk == 64 ? launch_tc<64, 64, 2, false, true>(A, B, p, splits, st)
-                                      : launch_tc<64, 32, 4, false, true>(A, B, p, splits, st);
-    return c.bk == 64 ? launch_tc<32, 64, 2, false, true>(A, B, p, splits, st)
-                      : launch_tc<32, 32, 5, false, true>(A, B, p, splits, st);
-  }
-  if (plain) {
-    if (c.bn == 64) return c.bk == 64 ? launch_tc<64, 64, 6, true, false>(A, B, p, splits, st)
-                                      : launch_tc<64, 32, 8, true, false>(A, B, p, splits, st);
-    return c.bk == 64 ? launch_tc<32, 64, 6, true, false>(A, B, p, splits, st) : launch_tc<32, 32, 8, true, false>(A, B, p, splits, st);
-  }
-  if (c.bn == 128) return c.bk == 64 ? launch_tc<128, 64, 2, false, false>(A, B, p, splits, st)
-                                     : launch_tc<128, 32, 4, false, false>(A, B, p, splits, st);
-  if (c.bn == 64) return c.bk == 64 ? launch_tc<64, 64, 2, false, false>(A, B, p, splits, st)
-                                    : launch_tc<64, 32, 5, false, false>(A, B, p, splits, st);
-  return c.bk == 64 ? launch_tc<32, 64, 3, false, false>(A, B, p, splits, st) : launch_tc<32, 32, 6, false, false>(A, B, p, splits, st);
-}
-
-// Tuning cache: one entry per GEMM shape class; filled the first time a shape is seen outside
-// stream capture by timing every candidate once (each candidate writes the full, correct C).
-static std::mutex g_tune_mu;
-static std::map<std::tuple<int64_t, int64_t, int64_t, int, int, int, int>, int> g_tune;
-
-static lrtei_status run_tuned(const SplitMatrix& A, const SplitMatrix& B, const Params& p, int splits, int BN,
-                              bool plain, cudaStream_t st) {
-  const Config* cands = plain    ? (BN == 64 ? kPlainCfg64 : kPlainCfg32)
-                        : A.eight ? (BN == 64 ? kSplit8Cfg64 : kSplit8Cfg32)
-                                  : (BN == 128 ? kSplitCfg128 : BN == 64 ? kSplitCfg64 : kSplitCfg32);
-  // A third candidate for the non-symmetric six-product products with 128-column tiles: the CTA
-  // pair (cta_group::2, 256 x 128 tiles, each SM loading half of B), bit-identical results.
-  const bool pair_ok = !plain && !A.eight && BN == 128 && B.s1h && !p.symmetric && splits == 1 &&
-                       p.M < (1LL << 31);
-  const int ncand = pair_ok ? 3 : 2;
-  auto launch_cand = [&](int i) {
-    return i == 2 ? launch_tc_2sm<64, 2>(A, B, p, st) : launch_cfg(A, B, p, splits, plain, cands[i], st);
   };
-  const char* force = getenv("LRTEI_TC_CONFIG");
-  if (force && *force) {
-    const int i = atoi(force);
-    ProfScope ps("tc_gemm", st);
-    return launch_cand((i < 0 || i >= ncand) ? 0 : i);
-  }
-  const auto key = std::make_tuple(p.M, p.N, A.kpad, splits, (int)plain + 2 * (int)A.eight,
-                                   p.symmetric ? (int)(1 + p.blk0) : 0, p.transpose_out);
-  int choice = -1;
-  {
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    auto it = g_tune.find(key);
-    if (it != g_tune.end()) choice = it->second;
-  }
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (choice < 0 && cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
-    float best = 1e30f;
-    cudaEvent_t e0, e1;
-    if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return cuda_fail(cudaGetLastError(), "tune events");
-    // two rounds, best of each candidate: the first launch of a kernel carries one-time costs
-    for (int round = 0; round < 2; ++round)
-      for (int i = 0; i < ncand; ++i) {
-        cudaEventRecord(e0, st);
-        lrtei_status s = launch_cand(i);
-        if (s != LRTEI_OK) { cudaEventDestroy(e0); cudaEventDestroy(e1); return s; }
-        cudaEventRecord(e1, st);
-        cudaError_t e = cudaEventSynchronize(e1);
-        if (e != cudaSuccess) { cudaEventDestroy(e0); cudaEventDestroy(e1); return cuda_fail(e, "tune sync"); }
-        float ms = 0.f;
-        cudaEventElapsedTime(&ms, e0, e1);
-        if (ms < best) { best = ms; choice = i; }
-      }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    g_tune[key] = choice;
-    return LRTEI_OK;  // C holds the last candidate's (correct) result
-  }
-  if (choice < 0) choice = 0;
-  ProfScope ps("tc_gemm", st);
-  return launch_cand(choice);
-}
-}  // namespace tc
+};
 
-// C = scale * A B^T.  A: M rows (slices s0,s1,s2), B: N rows (slices s0,s1,s1h,s2), same kpad
-// (multiple of 256, <= 32768 per split).  d_C: FP64, ldc; transpose_out writes C^T.
-// When splits > 1, d_part (splits * M * N doubles) receives the partials, which are reduced into d_C.
-static lrtei_status tc_gemm_impl(const SplitMatrix& A, const SplitMatrix& B, int64_t M, int64_t N, double scale,
-                                 double* d_C, int64_t ldc, bool transpose_out, bool symmetric_upper, int splits,
-                                 double* d_part, int* d_status, cudaStream_t st, int64_t row0) {
-  if (A.kpad != B.kpad || A.kpad % tc::KCHUNK != 0) {
-    set_error("tc_gemm: operands must share a K padded to a multiple of %d", tc::KCHUNK);
+// Tile width: 128 columns for wide six-product outputs (a 128 x 64 MMA is bound by its operand reads from
+// shared memory); the eight-product scheme has TMEM for 64 (2 x 3 accumulators), plain BF16 takes 64.
+static int tile_n(int64_t N, bool plain, bool eight) { return N <= 32 ? 32 : (N <= 64 || plain || eight) ? 64 : 128; }
+
+template <int KS>
+static lrtei_status run_ks(const tcg::Params& p, int BN, bool plain, bool eight, cudaStream_t st) {
+  if (plain) return BN == 64 ? tcg::launch<Split<64, Scheme::plain, KS>>(p, st) : tcg::launch<Split<32, Scheme::plain, KS>>(p, st);
+  if (eight) return BN == 64 ? tcg::launch<Split<64, Scheme::eight, KS>>(p, st) : tcg::launch<Split<32, Scheme::eight, KS>>(p, st);
+  if (BN == 128) return tcg::launch<Split<128, Scheme::six, KS>>(p, st);
+  return BN == 64 ? tcg::launch<Split<64, Scheme::six, KS>>(p, st) : tcg::launch<Split<32, Scheme::six, KS>>(p, st);
+}
+static lrtei_status run(const tcg::Params& p, int BN, bool plain, bool eight, cudaStream_t st) {
+  ProfScope ps("tc_gemm", st);
+  return p.seg[0].tab ? run_ks<1>(p, BN, plain, eight, st) : run_ks<2>(p, BN, plain, eight, st);
+}
+
+// What the products share: operands, output (or split partials) and checks.  units: 128-deep chunks of K.
+static lrtei_status fill(tcg::Params& p, const SplitMatrix& A, const SplitMatrix& B, int BN, int64_t units, double scale,
+                         double* d_C, int64_t ldc, bool transpose_out, int& splits, int64_t c_rows, int64_t c_cols,
+                         double* d_part, int* d_status) {
+  if (A.plain != B.plain || A.eight != B.eight) {
+    set_error("tc_gemm: operands must share one precision scheme");
     return LRTEI_ERR_ARG;
   }
-  const int nchunks = (int)(A.kpad / tc::KCHUNK);
-  splits = std::max(1, std::min(splits, nchunks));
-  int cps = (nchunks + splits - 1) / splits;
-  if ((int64_t)cps * tc::KCHUNK > 32768) {
+  if (A.tile != 128 || B.tile % BN != 0) {
+    set_error("tc_gemm: operand tiles of %d and %d rows for %d columns", A.tile, B.tile, BN);
+    return LRTEI_ERR_ARG;
+  }
+  splits = (int)std::max<int64_t>(1, std::min<int64_t>(splits, units));
+  const int64_t per = (units + splits - 1) / splits;
+  if (per * 128 > 32768) {
     set_error("tc_gemm: more than 32768 K per split (use more splits)");
     return LRTEI_ERR_UNSUPPORTED;
   }
-  splits = (nchunks + cps - 1) / cps;
-  if (symmetric_upper && (splits != 1 || M > N || transpose_out || row0 % tc::BM != 0 || row0 >= M ||
-                          A.rows < M - row0)) {
-    set_error("tc_gemm: symmetric mode needs one split and a square output (or a 128-aligned row band)");
+  splits = (int)((units + per - 1) / per);
+  if (splits > 1 && !d_part) {
+    set_error("tc_gemm: split-K needs a partial buffer");
     return LRTEI_ERR_ARG;
   }
-  tc::Params p{};
-  p.M = M;
-  p.N = N;
-  p.nchunks_total = nchunks;
-  p.chunks_per_split = cps;
+  p.splits = splits;
+  p.a = reinterpret_cast<const uint8_t*>(A.d);
+  p.b = reinterpret_cast<const uint8_t*>(B.d);
+  p.a_steps = A.kpad / tcg::KB;
+  p.b_steps = B.kpad / tcg::KB;
+  p.b_tile = B.tile;
   p.ea = A.expo;
   p.eb = B.expo;
   p.scale = scale;
   p.transpose_out = transpose_out ? 1 : 0;
-  p.symmetric = symmetric_upper ? 1 : 0;
+  p.C = splits > 1 ? d_part : d_C;
+  p.ldc = splits > 1 ? c_cols : ldc;
+  p.split_stride = splits > 1 ? c_rows * c_cols : 0;
   p.status = d_status;
-  p.splits = splits;
-  p.a_row0 = row0;
-  {
-    // LRTEI_TEST_STALL_CYCLES (tests only): every CTA's MMA thread first waits that many cycles on
-    // a barrier nothing completes, gives up, raises LRTEI_ERR_TIMEOUT and leaves the kernel
-    // through the bounded drain path.
-    const char* v = getenv("LRTEI_TEST_STALL_CYCLES");
-    p.test_stall = (v && *v) ? std::max(0LL, atoll(v)) : 0;
-  }
-  // Tile width: the tensor pipe runs at full rate from N = 128 on (a 128 x 64 MMA is bound by
-  // its operand reads from shared memory); narrow outputs take narrower tiles.  Plain BF16 keeps
-  // 64-column tiles.
-  const bool plain_ops = A.plain;
-  const int BN = (N <= 32) ? 32 : (N <= 64 || plain_ops || A.eight) ? 64 : 128;
-  const int64_t tiles_m = (M + tc::BM - 1) / tc::BM, tiles_n = (N + BN - 1) / BN;
-  p.tiles_m = tiles_m;
-  p.tiles_n = tiles_n;
-  if (symmetric_upper) {
-    // upper-triangular enumeration in units of 128 x 128 blocks, each done as 128 / BN tiles;
-    // block rows [row0 / 128, ceil(M / 128)) of the nb x nb block triangle
-    const int64_t nb = (N + tc::BM - 1) / tc::BM;
-    p.blk0 = row0 / tc::BM;
-    p.blk1 = tiles_m;
-    p.ntiles = ((nb - p.blk0) * (nb - p.blk0 + 1) / 2 - (nb - p.blk1) * (nb - p.blk1 + 1) / 2) * (tc::BM / BN);
-  } else {
-    p.ntiles = tiles_m * tiles_n;
-  }
-  if (splits > 1) {
-    if (!d_part) {
-      set_error("tc_gemm: split-K needs a partial buffer");
-      return LRTEI_ERR_ARG;
-    }
-    p.C = d_part;
-    p.ldc = transpose_out ? M : N;
-    p.split_stride = M * N;
-  } else {
-    p.C = d_C;
-    p.ldc = ldc;
-    p.split_stride = 0;
-  }
-  const bool plain = A.plain;
-  if (plain != B.plain || A.eight != B.eight) {
-    set_error("tc_gemm: operands must share one precision scheme");
-    return LRTEI_ERR_ARG;
-  }
-  if (A.eight && !A.s1h) {
-    set_error("tc_gemm: the eight-product scheme needs the A operand's t1 / 2^12 plane");
-    return LRTEI_ERR_ARG;
-  }
-  lrtei_status s;
-  // LRTEI_TC_2SM=1: the 2-SM variant for the non-symmetric products; =2: for the symmetric ones
-  // too (block bands starting on an even 128-row block)
-  const char* two = getenv("LRTEI_TC_2SM");
-  const bool two_ok = two && (two[0] == '1' || two[0] == '2') && !plain && !A.eight && BN == 128 && B.s1h &&
-                      (!symmetric_upper || (two[0] == '2' && p.blk0 % 2 == 0)) && p.M < (1LL << 31);
-  if (two_ok) {
-    ProfScope ps("tc_gemm", st);
-    // stage shape: LRTEI_TC_2SM_BK=32 selects five 32-deep stages, else two 64-deep ones
-    const char* bk = getenv("LRTEI_TC_2SM_BK");
-    s = (bk && atoi(bk) == 32) ? tc::launch_tc_2sm<32, 5>(A, B, p, st) : tc::launch_tc_2sm<64, 2>(A, B, p, st);
-  } else {
-    s = tc::run_tuned(A, B, p, splits, BN, plain, st);
-  }
-  if (s != LRTEI_OK) return s;
-  if (splits > 1) {
-    if (transpose_out)
-      launch_reduce_splits(d_part, splits, M * N, N, M, M, d_C, ldc, st);
-    else
-      launch_reduce_splits(d_part, splits, M * N, M, N, N, d_C, ldc, st);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "reduce_splits");
-  }
+  p.align = tcg::store_align(p.C, p.ldc);
+  p.test_stall = tcg::test_stall_cycles();
   return LRTEI_OK;
 }
 
-lrtei_status tc_gemm(const SplitMatrix& A, const SplitMatrix& B, int64_t M, int64_t N, double scale, double* d_C,
-                     int64_t ldc, bool transpose_out, bool symmetric_upper, int splits, double* d_part,
+static lrtei_status reduce(const double* part, int splits, int64_t rows, int64_t cols, double* C, int64_t ldc,
+                           cudaStream_t st) {
+  launch_reduce_splits(part, splits, rows * cols, rows, cols, cols, C, ldc, st);
+  cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? LRTEI_OK : cuda_fail(e, "reduce_splits");
+}
+
+}  // namespace tc
+
+lrtei_status tc_gemm(const SplitMatrix& A, int64_t a_row0, const SplitMatrix& B, int64_t M, int64_t N, double scale,
+                     double* d_C, int64_t ldc, bool transpose_out, bool symmetric_upper, int splits, double* d_part,
                      int* d_status, cudaStream_t st) {
-  if (symmetric_upper && M != N) {
+  if (A.kpad != B.kpad || A.kpad % 128 != 0) {
+    set_error("tc_gemm: operands must share a K padded to a multiple of 128");
+    return LRTEI_ERR_ARG;
+  }
+  if (symmetric_upper && (M != N || a_row0 != 0)) {
     set_error("tc_gemm: symmetric mode needs a square output");
     return LRTEI_ERR_ARG;
   }
-  return tc_gemm_impl(A, B, M, N, scale, d_C, ldc, transpose_out, symmetric_upper, splits, d_part, d_status, st, 0);
+  if (symmetric_upper) return tc_gemm_sym_band(A, B, 0, N, N, d_C, ldc, d_status, st);
+  const int BN = tc::tile_n(N, A.plain, A.eight), m_lo = (int)(a_row0 % 128), units = (int)(A.kpad / 128);
+  tcg::Params p{};
+  const int64_t c_rows = transpose_out ? N : M, c_cols = transpose_out ? M : N;
+  lrtei_status s = tc::fill(p, A, B, BN, units, scale, d_C, ldc, transpose_out, splits, c_rows, c_cols, d_part, d_status);
+  if (s != LRTEI_OK) return s;
+  p.nseg = 1;
+  p.seg[0] = {a_row0 - m_lo, 0, M + m_lo, N, transpose_out ? -m_lo : -m_lo * p.ldc, 0, 0, 0, units,
+              (int)((M + m_lo + 127) / 128), (int)((N + BN - 1) / BN), m_lo, nullptr};
+  p.nitems = (int64_t)p.seg[0].tiles_m * p.seg[0].tiles_n;
+  s = tc::run(p, BN, A.plain, A.eight, st);
+  if (s != LRTEI_OK || splits == 1) return s;
+  return tc::reduce(d_part, splits, c_rows, c_cols, d_C, ldc, st);
 }
 
 lrtei_status tc_gemm_sym_band(const SplitMatrix& A, const SplitMatrix& B, int64_t row0, int64_t row1, int64_t N,
                               double* d_C, int64_t ldc, int* d_status, cudaStream_t st) {
-  if (row0 == 0 && row1 == N) return tc_gemm_impl(A, B, N, N, 1.0, d_C, ldc, false, true, 1, nullptr, d_status, st, 0);
-  if (row0 % tc::BM != 0 || row0 >= row1 || row1 > N || (row1 < N && row1 % tc::BM != 0)) {
+  if (row0 % 128 != 0 || row0 >= row1 || row1 > N || (row1 < N && row1 % 128 != 0) || A.rows < row1 - row0 ||
+      A.kpad != B.kpad || A.kpad % 128 != 0) {
     set_error("tc_gemm_sym_band: rows [%lld, %lld) are not a 128-aligned band of %lld", (long long)row0,
               (long long)row1, (long long)N);
     return LRTEI_ERR_ARG;
   }
-  return tc_gemm_impl(A, B, row1, N, 1.0, d_C, ldc, false, true, 1, nullptr, d_status, st, row0);
+  const int BN = tc::tile_n(std::max<int64_t>(N, 65), A.plain, A.eight), units = (int)(A.kpad / 128);
+  tcg::Params p{};
+  int splits = 1;
+  lrtei_status s = tc::fill(p, A, B, BN, units, 1.0, d_C, ldc, false, splits, N, N, nullptr, d_status);
+  if (s != LRTEI_OK) return s;
+  // upper-triangular enumeration in 128 x 128 blocks (128 / BN tiles each); A holds rows [row0, row1) only
+  const int64_t nb = (N + 127) / 128, b0 = row0 / 128, b1 = (row1 + 127) / 128;
+  p.symmetric = p.mirror = 1;
+  p.nseg = 1;
+  p.blk0 = b0;
+  p.blk1 = b1;
+  p.nb = nb;
+  p.seg[0] = {-row0, 0, row1, N, 0, 0, 0, 0, units, (int)(b1 - b0), (int)nb, 0, nullptr};
+  p.nitems = ((nb - b0) * (nb - b0 + 1) / 2 - (nb - b1) * (nb - b1 + 1) / 2) * (128 / BN);
+  return tc::run(p, BN, A.plain, A.eight, st);
+}
+
+// Products with K by parity classes: of the dense K (columns m in the natural order) only the K blocks that
+// hold a class's columns are stored and multiplied, with chunks and sums as in the dense product.
+// Order n = 24: 288 of 864 blocks per row, a third of the MMAs of G = F_u K and of the bytes of K in a
+// J-build (all zeros left out would be an eighth, but a 16-deep block mixes degrees: bit-equal sums want
+// whole blocks).
+lrtei_status tc_gemm_K(const SplitMatrix& X, int64_t x_row0, const SplitMatrix& K, const ParityClasses& pc, int64_t rows,
+                       bool k_is_a, double* d_C, int splits, double* d_part, int* d_status, cudaStream_t st) {
+  const SplitMatrix &A = k_is_a ? K : X, &B = k_is_a ? X : K;
+  int64_t nmax = rows;
+  if (!k_is_a) {
+    nmax = 0;
+    for (int c = 0; c < pc.nclass; ++c) nmax = std::max<int64_t>(nmax, pc.size[c]);
+  }
+  const int BN = tc::tile_n(nmax, A.plain, A.eight), m_lo = k_is_a ? 0 : (int)(x_row0 % 128);
+  if ((k_is_a && x_row0 != 0) || X.kpad / 128 != pc.units) {
+    set_error("tc_gemm_K: operand does not match the plan's K");
+    return LRTEI_ERR_ARG;
+  }
+  tcg::Params p{};
+  lrtei_status s = tc::fill(p, A, B, BN, pc.units, 1.0, d_C, pc.cols, k_is_a, splits, rows, pc.cols, d_part, d_status);
+  if (s != LRTEI_OK) return s;
+  p.list_is_a = k_is_a ? 0 : 1;
+  for (int c = 0; c < pc.nclass; ++c) {
+    const int64_t w = (pc.size[c] + 63) / 64 * 64;  // the padding columns come out as zeros
+    if (w == 0) continue;
+    tcg::Seg& o = p.seg[p.nseg++];
+    const int* tab = pc.tab ? pc.tab + pc.tab_off[c] : nullptr;
+    if (k_is_a)
+      o = {pc.row0[c], 0, w, rows, pc.off[c], p.nitems, 0, 0, pc.units, (int)((w + 127) / 128), (int)((rows + BN - 1) / BN),
+           0, tab};
+    else
+      o = {x_row0 - m_lo, pc.row0[c], rows + m_lo, w, pc.off[c] - m_lo * p.ldc, p.nitems, 0, 0, pc.units,
+           (int)((rows + m_lo + 127) / 128), (int)((w + BN - 1) / BN), m_lo, tab};
+    p.nitems += (int64_t)o.tiles_m * o.tiles_n;
+  }
+  s = tc::run(p, BN, A.plain, A.eight, st);
+  if (s != LRTEI_OK || splits == 1) return s;
+  return tc::reduce(d_part, splits, rows, pc.cols, d_C, pc.cols, st);
 }
 
 }  // namespace lrtei

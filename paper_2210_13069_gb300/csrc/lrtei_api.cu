@@ -121,6 +121,9 @@ struct lrtei_plan {
   // FP64 plans on the tensor cores: digit planes of F_u, F_u^T and K in parity-class order
   ParityClasses pc;
   int* d_perm = nullptr;  // [pc.cols] natural column of each permuted one (-1: padding)
+  int* d_pos = nullptr;   // [n^3] permuted column of each natural one
+  std::vector<size_t> class_ints;  // lengths of d_pos, d_blk, pc.tab and d_perm
+  int* d_blk = nullptr;   // [8][units 8] place of each 16-deep K block in its class's list (with parity)
   OzMatrix ozF, ozFT, ozK;
   std::vector<void*> allocs;
   size_t bytes = 0;
@@ -656,25 +659,113 @@ lrtei_status ensure_F32(lrtei_plan* pl, cudaStream_t st) {
   return finish_launch("build_F32");
 }
 
+// Parity classes of the plan's columns: the permutation, its inverse and the step tables on the device.
+lrtei_status ensure_classes(lrtei_plan* pl, cudaStream_t st) {
+  if (pl->d_perm) return LRTEI_OK;
+  ParityClasses pc;
+  const int n = pl->n;
+  const int64_t n3 = (int64_t)n * n * n;
+  pc.n = n;
+  pc.par = has_parity(pl) ? 1 : 0;
+  pc.cnt[0] = (n + 1) / 2;
+  pc.cnt[1] = n / 2;
+  pc.nclass = pc.par ? 8 : 1;
+  for (int c = 0; c < pc.nclass; ++c) {
+    pc.size[c] = pc.par ? pc.cnt[(c >> 2) & 1] * pc.cnt[(c >> 1) & 1] * pc.cnt[c & 1] : n * n * n;
+    pc.off[c] = pc.cols;
+    pc.row0[c] = pc.rows;
+    const int k = (pc.size[c] + 63) / 64 * 64;
+    pc.cols += k;
+    pc.rows += (pc.size[c] + 127) / 128 * 128;
+    pc.kmax = std::max(pc.kmax, k);
+  }
+  pc.units = (int)(kpad256(n3) / 128);
+  const int nblk = pc.units * 8;
+  std::vector<int> perm((size_t)pc.cols, -1), pos((size_t)n3), blk, tab;
+  std::vector<uint8_t> holds((size_t)8 * nblk, 0);  // [class][16-deep block] holds a column of the class
+  for (int m1 = 0, m = 0; m1 < n; ++m1)
+    for (int m2 = 0; m2 < n; ++m2)
+      for (int m3 = 0; m3 < n; ++m3, ++m) {
+        const int c = pc.cls(m1, m2, m3);
+        pos[m] = pc.off[c] + pc.index(m1, m2, m3);
+        perm[pos[m]] = m;
+        holds[(size_t)c * nblk + m / 16] = 1;
+      }
+  pc.blocks = nblk;
+  if (pc.par) {
+    pc.blocks = 0;
+    blk.assign((size_t)8 * nblk, 0);
+    for (int c = 0; c < 8; ++c) {
+      pc.tab_off[c] = (int)tab.size();
+      std::vector<int> first, chunks, list;
+      int nonempty = 0;
+      for (int u = 0; u < pc.units; ++u) {
+        first.push_back((int)list.size());
+        chunks.push_back(nonempty);
+        const size_t before = list.size();
+        for (int b = 8 * u; b < 8 * u + 8; ++b)
+          if (holds[(size_t)c * nblk + b]) {
+            blk[(size_t)c * nblk + b] = (int)list.size();
+            list.push_back(b);
+          }
+        if (list.size() > before) {
+          list.back() |= 1 << 30;  // the chunk's last step
+          ++nonempty;
+        }
+      }
+      first.push_back((int)list.size());
+      chunks.push_back(nonempty);
+      pc.blocks = std::max(pc.blocks, (int)list.size());
+      for (const auto* v : {&first, &chunks, &list}) tab.insert(tab.end(), v->begin(), v->end());
+    }
+  }
+  int *d = nullptr, *d_pos = nullptr, *d_blk = nullptr, *d_tab = nullptr;
+  LRTEI_TRY(pl->alloc(&d_pos, pos.size()));
+  LRTEI_CUDA(cudaMemcpyAsync(d_pos, pos.data(), sizeof(int) * pos.size(), cudaMemcpyHostToDevice, st));
+  if (pc.par) {
+    LRTEI_TRY(pl->alloc(&d_blk, blk.size()));
+    LRTEI_TRY(pl->alloc(&d_tab, tab.size()));
+    LRTEI_CUDA(cudaMemcpyAsync(d_blk, blk.data(), sizeof(int) * blk.size(), cudaMemcpyHostToDevice, st));
+    LRTEI_CUDA(cudaMemcpyAsync(d_tab, tab.data(), sizeof(int) * tab.size(), cudaMemcpyHostToDevice, st));
+  }
+  LRTEI_TRY(pl->alloc(&d, perm.size()));
+  LRTEI_CUDA(cudaMemcpyAsync(d, perm.data(), sizeof(int) * perm.size(), cudaMemcpyHostToDevice, st));
+  pc.tab = d_tab;
+  pl->pc = pc;
+  pl->d_pos = d_pos;
+  pl->d_blk = d_blk;
+  pl->class_ints = {pos.size(), blk.size(), tab.size(), perm.size()};
+  pl->d_perm = d;
+  return LRTEI_OK;
+}
+void release_classes(lrtei_plan* pl) {
+  if (!pl->d_perm) return;
+  void* ptr[4] = {pl->d_pos, pl->d_blk, const_cast<int*>(pl->pc.tab), pl->d_perm};
+  for (int i = 0; i < 4; ++i) pl->release(ptr[i], sizeof(int) * pl->class_ints[i]);
+  pl->d_pos = pl->d_blk = pl->d_perm = nullptr;
+  pl->pc = ParityClasses();
+}
+
 bool is_split(const lrtei_plan* pl) {
   return pl->prec == LRTEI_SPLIT_F16 || pl->prec == LRTEI_SPLIT_F16_8 || pl->prec == LRTEI_BF16;
 }
 bool eight_products(const lrtei_plan* pl) { return pl->prec == LRTEI_SPLIT_F16_8; }
-int nslices(const lrtei_plan* pl) { return pl->prec == LRTEI_BF16 ? 1 : 3; }
 
-lrtei_status alloc_split(lrtei_plan* pl, SplitMatrix& m, int64_t rows, int64_t k, bool with_s1h) {
+SplitMatrix split_shape(const lrtei_plan* pl, int64_t rows, int64_t kpad, int tile) {
+  SplitMatrix m;
   m.rows = rows;
-  m.kpad = kpad256(k);
+  m.kpad = kpad;
+  m.tile = tile;
   m.plain = pl->prec == LRTEI_BF16;
   m.eight = eight_products(pl);
-  const size_t cnt = (size_t)rows * m.kpad;
-  LRTEI_TRY(pl->alloc(&m.s0, cnt));
-  if (!m.plain) {
-    LRTEI_TRY(pl->alloc(&m.s1, cnt));
-    LRTEI_TRY(pl->alloc(&m.s2, cnt));
-    if (with_s1h || m.eight) LRTEI_TRY(pl->alloc(&m.s1h, cnt));
-  }
-  LRTEI_TRY(pl->alloc(&m.expo, rows));
+  return m;
+}
+
+lrtei_status alloc_split(lrtei_plan* pl, SplitMatrix& m, int64_t rows, int64_t kpad) {
+  SplitMatrix q = split_shape(pl, rows, kpad, 128);
+  LRTEI_TRY(pl->alloc(&q.d, (size_t)q.count()));
+  LRTEI_TRY(pl->alloc(&q.expo, rows));
+  m = q;
   return LRTEI_OK;
 }
 
@@ -683,29 +774,20 @@ lrtei_status alloc_split(lrtei_plan* pl, SplitMatrix& m, int64_t rows, int64_t k
 // through its freed address by the next replay).
 void release_split(lrtei_plan* pl, SplitMatrix& m) {
   forget_plan_graphs(pl);
-  const size_t b = (size_t)m.rows * m.kpad * sizeof(uint16_t);
-  pl->release(m.s0, b);
-  pl->release(m.s1, b);
-  pl->release(m.s2, b);
-  pl->release(m.s1h, b);
+  pl->release(m.d, sizeof(uint16_t) * (size_t)m.count());
   pl->release(m.expo, (size_t)m.rows * sizeof(int));
   m = SplitMatrix();
 }
 
-// F_u slices.  The fourth plane (t1 / 2^12) is only needed when F_u is the B operand (the
-// assembly B_u = G F_u^T); J-builds use F_u as the A operand only.
-lrtei_status ensure_Fsp(lrtei_plan* pl, cudaStream_t st, bool need_s1h) {
-  if (pl->have_Fsp && (!need_s1h || pl->Fsp.plain || pl->Fsp.s1h)) return LRTEI_OK;
-  if (pl->have_Fsp) {
-    release_split(pl, pl->Fsp);
-    pl->have_Fsp = false;
-  }
+// F_u slices, the left operand of J-builds and of G, the right one of B_u = G F_u^T.
+lrtei_status ensure_Fsp(lrtei_plan* pl, cudaStream_t st) {
+  if (pl->have_Fsp) return LRTEI_OK;
   const int64_t n3 = (int64_t)pl->n * pl->n * pl->n;
   LRTEI_TRY(ensure_F64(pl, st));
-  LRTEI_TRY(alloc_split(pl, pl->Fsp, pl->t.npair, n3, need_s1h));
+  LRTEI_TRY(alloc_split(pl, pl->Fsp, pl->t.npair, kpad256(n3)));
   {
     ProfScope ps("split", st);
-    launch_split_rows(pl->d_F, pl->t.npair, n3, n3, pl->Fsp, need_s1h, nslices(pl), st);
+    launch_split_rows(pl->d_F, pl->t.npair, n3, n3, pl->Fsp, nullptr, st);
   }
   pl->have_Fsp = true;
   return finish_launch("split F");
@@ -744,29 +826,40 @@ struct Scratch {
   }
 };
 
-// Dense K = (omega / sqrt(pi)) sum_p w_p A_x^p (x) A_y^p (x) A_z^p as slices: the prefactor of
-// eq. approx33 is carried by K, so that every tensor-core GEMM runs with scale 1 and its
-// epilogue needs no FP64 multiply.  The fourth plane only when K is the B operand (G = F_u K);
-// the J-build uses K as the A operand.
-lrtei_status ensure_Ksp(lrtei_plan* pl, cudaStream_t st, bool need_s1h) {
-  if (pl->have_Ksp && (!need_s1h || pl->Ksp.plain || pl->Ksp.s1h)) return LRTEI_OK;
-  if (pl->have_Ksp) {
-    release_split(pl, pl->Ksp);
-    pl->have_Ksp = false;
-  }
-  const int64_t n3 = (int64_t)pl->n * pl->n * pl->n;
-  Scratch sc(st);
-  double* K;
-  LRTEI_TRY(sc.get(&K, (size_t)n3 * n3));
+// K = (omega / sqrt(pi)) sum_p w_p A_x^p (x) A_y^p (x) A_z^p from the coefficients d_C into slices: the
+// prefactor of eq. approx33 is carried by K, so that every tensor-core GEMM runs with scale 1 and its
+// epilogue needs no FP64 multiply.  Rows and K blocks by parity class (tc_gemm_K).
+int64_t K_kpad(const ParityClasses& pc) { return (int64_t)pc.blocks * 16; }
+int64_t K_cols(const lrtei_plan* pl) {  // of the FP64 K that is sliced
+  return pl->pc.par ? K_kpad(pl->pc) : (int64_t)pl->n * pl->n * pl->n;
+}
+// clear: K holds no K of the same plan yet (its zeros lie in the same places for every d_C).
+lrtei_status slice_K(lrtei_plan* pl, const double* d_C, bool clear, double* K, const SplitMatrix& m, cudaStream_t st) {
+  const ParityClasses& pc = pl->pc;
+  const int64_t ld = K_cols(pl);
   {
     ProfScope ps("build_K", st);
-    LRTEI_CUDA(launch_build_K(pl->n, pl->P, pl->d_C, pl->d_w, pl->omega / sqrt(kPi), K, st));
+    if (pc.par) {
+      if (clear) LRTEI_CUDA(cudaMemsetAsync(K, 0, sizeof(double) * (size_t)pc.rows * ld, st));
+      LRTEI_CUDA(launch_build_K_classes(pl->n, pl->P, pc, pl->d_blk, d_C, pl->d_w, pl->omega / sqrt(kPi), K, ld, st));
+    } else {
+      LRTEI_CUDA(cudaMemsetAsync(K + ld * ld, 0, sizeof(double) * (size_t)(pc.rows - ld) * ld, st));
+      LRTEI_CUDA(launch_build_K(pl->n, pl->P, d_C, pl->d_w, pl->omega / sqrt(kPi), K, st));
+    }
   }
-  LRTEI_TRY(alloc_split(pl, pl->Ksp, n3, n3, need_s1h));
-  {
-    ProfScope ps("split", st);
-    launch_split_rows(K, n3, n3, n3, pl->Ksp, need_s1h, nslices(pl), st);
-  }
+  ProfScope ps("split", st);
+  launch_split_rows(K, pc.rows, ld, ld, m, nullptr, st);
+  return LRTEI_OK;
+}
+
+lrtei_status ensure_Ksp(lrtei_plan* pl, cudaStream_t st) {
+  if (pl->have_Ksp) return LRTEI_OK;
+  LRTEI_TRY(ensure_classes(pl, st));
+  Scratch sc(st);
+  double* K;
+  LRTEI_TRY(sc.get(&K, (size_t)pl->pc.rows * K_cols(pl)));
+  LRTEI_TRY(alloc_split(pl, pl->Ksp, pl->pc.rows, K_kpad(pl->pc)));
+  LRTEI_TRY(slice_K(pl, pl->d_C, true, K, pl->Ksp, st));
   pl->have_Ksp = true;
   return finish_launch("split K");
 }
@@ -779,10 +872,10 @@ lrtei_status ensure_FTsp(lrtei_plan* pl, cudaStream_t st) {
   double* FT;
   LRTEI_TRY(sc.get(&FT, (size_t)n3 * npair));
   launch_transpose(pl->d_F, npair, n3, n3, FT, npair, st);
-  LRTEI_TRY(alloc_split(pl, pl->FTsp, n3, npair, false));
+  LRTEI_TRY(alloc_split(pl, pl->FTsp, n3, kpad256(npair)));
   {
     ProfScope ps("split", st);
-    launch_split_rows(FT, n3, npair, npair, pl->FTsp, false, nslices(pl), st);
+    launch_split_rows(FT, n3, npair, npair, pl->FTsp, nullptr, st);
   }
   pl->have_FTsp = true;
   return finish_launch("split F^T");
@@ -791,27 +884,18 @@ lrtei_status ensure_FTsp(lrtei_plan* pl, cudaStream_t st) {
 // Operands of the tensor-core J-build: F_u^T and F_u (A operands) and K (A operand).
 lrtei_status ensure_jbuild_operands(lrtei_plan* pl, cudaStream_t st) {
   LRTEI_TRY(ensure_FTsp(pl, st));
-  LRTEI_TRY(ensure_Fsp(pl, st, false));
-  LRTEI_TRY(ensure_Ksp(pl, st, false));
+  LRTEI_TRY(ensure_Fsp(pl, st));
+  LRTEI_TRY(ensure_Ksp(pl, st));
   drop_F64_if_sliced(pl, st);
   return LRTEI_OK;
 }
 
-// A scratch split operand (planes owned by the call).
-lrtei_status scratch_split(Scratch& sc, SplitMatrix& m, int64_t rows, int64_t k, bool with_s1h, const lrtei_plan* pl) {
-  m.rows = rows;
-  m.kpad = kpad256(k);
-  m.plain = pl->prec == LRTEI_BF16;
-  m.eight = eight_products(pl);
-  const size_t cnt = (size_t)rows * m.kpad;
-  LRTEI_TRY(sc.get(&m.s0, cnt));
-  if (!m.plain) {
-    LRTEI_TRY(sc.get(&m.s1, cnt));
-    LRTEI_TRY(sc.get(&m.s2, cnt));
-    if (with_s1h || m.eight) LRTEI_TRY(sc.get(&m.s1h, cnt));
-  }
-  LRTEI_TRY(sc.get(&m.expo, rows));
-  return LRTEI_OK;
+// A scratch split operand (planes owned by the call).  tile: 128, or split_tile(R) for the R-row right
+// operand of a skinny product.
+lrtei_status scratch_split(Scratch& sc, SplitMatrix& m, int64_t rows, int64_t k, int tile, const lrtei_plan* pl) {
+  m = split_shape(pl, rows, kpad256(k), tile);
+  LRTEI_TRY(sc.get(&m.d, (size_t)m.count()));
+  return sc.get(&m.expo, rows);
 }
 
 // Positive integer from the environment (0 when unset): the host-output pipeline's band count
@@ -834,27 +918,21 @@ int splits_for(int64_t M, int64_t K) {
 // Rows [r0, r1) of B_u through the tensor-core GEMMs (split precision); the prefactor is in K.
 lrtei_status bu_rows_tc(lrtei_plan* pl, int64_t r0, int64_t r1, double* out, int64_t ld, cudaStream_t st) {
   const int64_t n3 = (int64_t)pl->n * pl->n * pl->n, npair = pl->t.npair, nr = r1 - r0;
-  LRTEI_TRY(ensure_Fsp(pl, st, true));
-  LRTEI_TRY(ensure_Ksp(pl, st, true));
+  LRTEI_TRY(ensure_Fsp(pl, st));
+  LRTEI_TRY(ensure_Ksp(pl, st));
+  const ParityClasses& pc = pl->pc;
   Scratch sc(st);
   double* G;
-  LRTEI_TRY(sc.get(&G, (size_t)nr * n3));
-  SplitMatrix Fr = pl->Fsp;  // row view [r0, r1)
-  Fr.rows = nr;
-  Fr.s0 += r0 * Fr.kpad;
-  if (Fr.s1h) Fr.s1h += r0 * Fr.kpad;
-  if (Fr.s1) Fr.s1 += r0 * Fr.kpad;
-  if (Fr.s2) Fr.s2 += r0 * Fr.kpad;
-  Fr.expo += r0;
-  LRTEI_TRY(tc_gemm(Fr, pl->Ksp, nr, n3, 1.0, G, n3, false, false, 1, nullptr, pl->d_status, st));
+  LRTEI_TRY(sc.get(&G, (size_t)nr * pc.cols));
+  LRTEI_TRY(tc_gemm_K(pl->Fsp, r0, pl->Ksp, pc, nr, false, G, 1, nullptr, pl->d_status, st));
   SplitMatrix Gs;
-  LRTEI_TRY(scratch_split(sc, Gs, nr, n3, false, pl));
+  LRTEI_TRY(scratch_split(sc, Gs, nr, n3, 128, pl));
   {
     ProfScope ps("split", st);
-    launch_split_rows(G, nr, n3, n3, Gs, false, nslices(pl), st);
+    launch_split_rows(G, nr, n3, pc.cols, Gs, pl->d_pos, st);  // back to the natural column order
   }
-  const bool sym = (r0 == 0 && r1 == npair && ld == npair);
-  return tc_gemm(Gs, pl->Fsp, nr, npair, 1.0, out, ld, false, sym, 1, nullptr, pl->d_status, st);
+  const bool sym = r0 == 0 && r1 == npair;
+  return tc_gemm(Gs, 0, pl->Fsp, nr, npair, 1.0, out, ld, false, sym, 1, nullptr, pl->d_status, st);
 }
 
 // B into page-locked host memory through the tensor-core path.  B_u is computed in bands of
@@ -867,8 +945,9 @@ lrtei_status bu_rows_tc(lrtei_plan* pl, int64_t r0, int64_t r1, double* out, int
 static lrtei_status assemble_B_host_banded(lrtei_plan* pl, double* hB, int64_t ld, cudaStream_t st) {
   const int nbf = pl->basis.nbf;
   const int64_t nb2 = (int64_t)nbf * nbf, npair = pl->t.npair, n3 = (int64_t)pl->n * pl->n * pl->n;
-  LRTEI_TRY(ensure_Fsp(pl, st, true));
-  LRTEI_TRY(ensure_Ksp(pl, st, true));
+  LRTEI_TRY(ensure_Fsp(pl, st));
+  LRTEI_TRY(ensure_Ksp(pl, st));
+  const ParityClasses& pc = pl->pc;
   const int64_t nblk = (npair + 127) / 128;
   int64_t nbands = env_count("LRTEI_HOST_BANDS");
   if (nbands <= 0) nbands = 16;
@@ -892,11 +971,11 @@ static lrtei_status assemble_B_host_banded(lrtei_plan* pl, double* hB, int64_t l
   Scratch sc(st);
   double *Bu, *G, *stage[2];
   LRTEI_TRY(sc.get(&Bu, (size_t)npair * npair));
-  LRTEI_TRY(sc.get(&G, (size_t)maxrows * n3));
+  LRTEI_TRY(sc.get(&G, (size_t)maxrows * pc.cols));
   LRTEI_TRY(sc.get(&stage[0], (size_t)chunk * nb2));
   LRTEI_TRY(sc.get(&stage[1], (size_t)chunk * nb2));
   SplitMatrix Gs;
-  LRTEI_TRY(scratch_split(sc, Gs, maxrows, n3, false, pl));
+  LRTEI_TRY(scratch_split(sc, Gs, maxrows, n3, 128, pl));
   cudaStream_t cs = nullptr;
   cudaEvent_t ready[2] = {nullptr, nullptr}, copied[2] = {nullptr, nullptr}, fin = nullptr;
   lrtei_status status = LRTEI_OK;
@@ -911,18 +990,11 @@ static lrtei_status assemble_B_host_banded(lrtei_plan* pl, double* hB, int64_t l
   int64_t a_done = 0, nchunk = 0;
   for (size_t k = 0; k + 1 < edge.size() && status == LRTEI_OK; ++k) {
     const int64_t r0 = 128 * edge[k], r1 = std::min(npair, 128 * edge[k + 1]), nr = r1 - r0;
-    SplitMatrix Fr = pl->Fsp;  // row view [r0, r1)
-    Fr.rows = nr;
-    Fr.s0 += r0 * Fr.kpad;
-    if (Fr.s1h) Fr.s1h += r0 * Fr.kpad;
-    if (Fr.s1) Fr.s1 += r0 * Fr.kpad;
-    if (Fr.s2) Fr.s2 += r0 * Fr.kpad;
-    Fr.expo += r0;
-    if ((status = tc_gemm(Fr, pl->Ksp, nr, n3, 1.0, G, n3, false, false, 1, nullptr, pl->d_status, st)) != LRTEI_OK) break;
+    if ((status = tc_gemm_K(pl->Fsp, r0, pl->Ksp, pc, nr, false, G, 1, nullptr, pl->d_status, st)) != LRTEI_OK) break;
     Gs.rows = nr;
     {
       ProfScope ps("split", st);
-      launch_split_rows(G, nr, n3, n3, Gs, false, nslices(pl), st);
+      launch_split_rows(G, nr, n3, pc.cols, Gs, pl->d_pos, st);
     }
     if ((status = tc_gemm_sym_band(Gs, pl->Fsp, r0, r1, npair, Bu, npair, pl->d_status, st)) != LRTEI_OK) break;
     // basis functions a whose pairs (a, b >= a) all lie below r1: rows [a_done N_b, a_end N_b) of B
@@ -1006,51 +1078,44 @@ lrtei_status bu_adaptive(lrtei_plan* pl, double* Bu, cudaStream_t st) {
   int64_t maxr = 0;
   for (int s = 0; s < np; ++s) maxr = std::max(maxr, ar.off[s + 1] - ar.off[s]);
   double *G, *blk;
-  LRTEI_TRY(sc.get(&G, (size_t)maxr * n3));
+  if (is_split(pl)) LRTEI_TRY(ensure_classes(pl, st));
+  LRTEI_TRY(sc.get(&G, (size_t)maxr * std::max<int64_t>(n3, pl->pc.cols)));
   LRTEI_TRY(sc.get(&blk, (size_t)maxr * maxr));
   if (is_split(pl)) {
+    const ParityClasses& pc = pl->pc;
     SplitMatrix Fsp, Ksp, Gsp;
-    LRTEI_TRY(scratch_split(sc, Fsp, npair, n3, true, pl));
-    LRTEI_TRY(scratch_split(sc, Ksp, n3, n3, true, pl));
-    LRTEI_TRY(scratch_split(sc, Gsp, maxr, n3, false, pl));
+    std::vector<int64_t> tile0{0};  // first row of each partition in the sliced F: a multiple of 128
+    for (int s = 0; s < np; ++s) tile0.push_back(tile0.back() + (ar.off[s + 1] - ar.off[s] + 127) / 128 * 128);
+    LRTEI_TRY(scratch_split(sc, Fsp, tile0.back(), n3, 128, pl));
+    Ksp = split_shape(pl, pc.rows, K_kpad(pc), 128);
+    LRTEI_TRY(sc.get(&Ksp.d, (size_t)Ksp.count()));
+    LRTEI_TRY(sc.get(&Ksp.expo, (size_t)pc.rows));
+    LRTEI_TRY(scratch_split(sc, Gsp, maxr, n3, 128, pl));
     double* K;
-    LRTEI_TRY(sc.get(&K, (size_t)n3 * n3));
+    LRTEI_TRY(sc.get(&K, (size_t)pc.rows * K_cols(pl)));
+    auto rows_of = [&](int s) { return Fsp.from_row(tile0[s], ar.off[s + 1] - ar.off[s]); };
     {
       ProfScope ps("split", st);
-      launch_split_rows(ar.Fp, npair, n3, n3, Fsp, true, nslices(pl), st);
+      for (int s = 0; s < np; ++s)
+        launch_split_rows(ar.Fp + ar.off[s] * n3, ar.off[s + 1] - ar.off[s], n3, n3, rows_of(s), nullptr, st);
     }
-    auto rows_of = [&](int s) {  // row view of partition s
-      SplitMatrix v = Fsp;
-      const int64_t r0 = ar.off[s];
-      v.rows = ar.off[s + 1] - r0;
-      v.s0 += r0 * v.kpad;
-      if (v.s1) v.s1 += r0 * v.kpad;
-      if (v.s2) v.s2 += r0 * v.kpad;
-      if (v.s1h) v.s1h += r0 * v.kpad;
-      v.expo += r0;
-      return v;
-    };
+    bool first = true;
     for (int t = 0; t < np; ++t) {
       const int64_t nt = ar.off[t + 1] - ar.off[t];
       for (int s = 0; s <= t; ++s) {
         const int64_t ns = ar.off[s + 1] - ar.off[s];
         if (ns == 0 || nt == 0) continue;
-        {  // K_{ts} = (w/sqrt(pi)) sum_p w_p (x)_d A^(p)_{ts,d}, so that G = F_s K_{ts}^T = F_s K_{st}
-          ProfScope ps("build_K", st);
-          LRTEI_CUDA(launch_build_K(n, P, pl->d_C + (size_t)(t * np + s) * cblk, pl->d_w, pref, K, st));
-        }
-        {
-          ProfScope ps("split", st);
-          launch_split_rows(K, n3, n3, n3, Ksp, true, nslices(pl), st);
-        }
-        SplitMatrix Fs = rows_of(s), Ft = rows_of(t);
-        LRTEI_TRY(tc_gemm(Fs, Ksp, ns, n3, 1.0, G, n3, false, false, 1, nullptr, pl->d_status, st));
+        // K_{ts} = (w/sqrt(pi)) sum_p w_p (x)_d A^(p)_{ts,d}, so that G = F_s K_{ts}^T = F_s K_{st}
+        LRTEI_TRY(slice_K(pl, pl->d_C + (size_t)(t * np + s) * cblk, first, K, Ksp, st));
+        first = false;
+        const SplitMatrix Fs = rows_of(s), Ft = rows_of(t);
+        LRTEI_TRY(tc_gemm_K(Fs, 0, Ksp, pc, ns, false, G, 1, nullptr, pl->d_status, st));
         Gsp.rows = ns;
         {
           ProfScope ps("split", st);
-          launch_split_rows(G, ns, n3, n3, Gsp, false, nslices(pl), st);
+          launch_split_rows(G, ns, n3, pc.cols, Gsp, pl->d_pos, st);
         }
-        LRTEI_TRY(tc_gemm(Gsp, Ft, ns, nt, 1.0, blk, nt, false, false, 1, nullptr, pl->d_status, st));
+        LRTEI_TRY(tc_gemm(Gsp, 0, Ft, ns, nt, 1.0, blk, nt, false, false, 1, nullptr, pl->d_status, st));
         launch_scatter_block(blk, nt, ar.d_idx + ar.off[s], ns, ar.d_idx + ar.off[t], nt, Bu, npair, s != t, st);
       }
     }
@@ -1122,37 +1187,6 @@ lrtei_status jbuild_adaptive(lrtei_plan* pl, const double* d_D, int R, double* d
 }
 
 // ---- FP64 plans on the tensor cores (k_ozaki.cu) ---------------------------------------------
-// Parity classes of the plan's columns and the permutation on the device.
-lrtei_status ensure_classes(lrtei_plan* pl, cudaStream_t st) {
-  if (pl->d_perm) return LRTEI_OK;
-  ParityClasses& pc = pl->pc;
-  const int n = pl->n;
-  pc = ParityClasses();
-  pc.n = n;
-  pc.par = has_parity(pl) ? 1 : 0;
-  pc.cnt[0] = (n + 1) / 2;
-  pc.cnt[1] = n / 2;
-  pc.nclass = pc.par ? 8 : 1;
-  for (int c = 0; c < pc.nclass; ++c) {
-    pc.size[c] = pc.par ? pc.cnt[(c >> 2) & 1] * pc.cnt[(c >> 1) & 1] * pc.cnt[c & 1] : n * n * n;
-    pc.off[c] = pc.cols;
-    pc.row0[c] = pc.rows;
-    const int k = (pc.size[c] + 63) / 64 * 64;
-    pc.cols += k;
-    pc.rows += (pc.size[c] + 127) / 128 * 128;
-    pc.kmax = std::max(pc.kmax, k);
-  }
-  std::vector<int> perm((size_t)pc.cols, -1);
-  for (int m1 = 0, m = 0; m1 < n; ++m1)
-    for (int m2 = 0; m2 < n; ++m2)
-      for (int m3 = 0; m3 < n; ++m3, ++m) perm[pc.off[pc.cls(m1, m2, m3)] + pc.index(m1, m2, m3)] = m;
-  int* d = nullptr;
-  LRTEI_TRY(pl->alloc(&d, perm.size()));
-  LRTEI_CUDA(cudaMemcpyAsync(d, perm.data(), sizeof(int) * perm.size(), cudaMemcpyHostToDevice, st));
-  pl->d_perm = d;
-  return LRTEI_OK;
-}
-
 lrtei_status alloc_oz(lrtei_plan* pl, OzMatrix& m, int64_t rows, int64_t kpad) {
   OzMatrix q;
   q.rows = rows;
@@ -1708,19 +1742,20 @@ lrtei_status lrtei_exchange(lrtei_plan* plan, const double* d_Q, int norb, doubl
   double *MT, *X, *Y, *Xp, *Yp, *Kb;
   LRTEI_TRY(sc.get(&MT, (size_t)rowlen * nbf));
   LRTEI_TRY(sc.get(&X, (size_t)ob * rowlen));
-  LRTEI_TRY(sc.get(&Y, (size_t)ob * rowlen));
+  if (tc) LRTEI_TRY(ensure_Ksp(plan, st));  // K as the right operand of Y = X K^T (K symmetric)
+  const int64_t ycols = tc ? plan->pc.cols : n3;
+  LRTEI_TRY(sc.get(&Y, (size_t)ob * nbf * ycols));
   LRTEI_TRY(sc.get(&Xp, (size_t)ob * rowlen));
   LRTEI_TRY(sc.get(&Yp, (size_t)ob * rowlen));
   LRTEI_TRY(sc.get(&Kb, (size_t)nblk * nbf * nbf));
   launch_gather_MT(nbf, n3, plan->d_F, n3, MT, st);
   if (tc) {
-    LRTEI_TRY(ensure_Ksp(plan, st, true));  // K as the B operand of Y = X K^T (K symmetric)
     SplitMatrix Qsp, MTsp, Xsp, Ypsp, Xpsp;
-    LRTEI_TRY(scratch_split(sc, Qsp, norb, nbf, false, plan));
-    LRTEI_TRY(scratch_split(sc, MTsp, rowlen, nbf, true, plan));
-    LRTEI_TRY(scratch_split(sc, Xsp, (int64_t)ob * nbf, n3, false, plan));
-    LRTEI_TRY(scratch_split(sc, Ypsp, nbf, (int64_t)ob * n3, false, plan));
-    LRTEI_TRY(scratch_split(sc, Xpsp, nbf, (int64_t)ob * n3, true, plan));
+    LRTEI_TRY(scratch_split(sc, Qsp, norb, nbf, 128, plan));
+    LRTEI_TRY(scratch_split(sc, MTsp, rowlen, nbf, split_tile(rowlen), plan));
+    LRTEI_TRY(scratch_split(sc, Xsp, (int64_t)ob * nbf, n3, 128, plan));
+    LRTEI_TRY(scratch_split(sc, Ypsp, nbf, (int64_t)ob * n3, 128, plan));
+    LRTEI_TRY(scratch_split(sc, Xpsp, nbf, (int64_t)ob * n3, split_tile(nbf), plan));
     // split-K partials of the last product: the largest split count of any block (a shorter last
     // block can take more splits than a full one)
     const int nlast = norb - (nblk - 1) * ob;
@@ -1729,38 +1764,31 @@ lrtei_status lrtei_exchange(lrtei_plan* plan, const double* d_Q, int norb, doubl
     LRTEI_TRY(sc.get(&part, (size_t)sK * nbf * nbf));
     {
       ProfScope ps("split", st);
-      launch_split_rows(d_Q, norb, nbf, nbf, Qsp, false, nslices(plan), st);
-      launch_split_rows(MT, rowlen, nbf, nbf, MTsp, true, nslices(plan), st);
+      launch_split_rows(d_Q, norb, nbf, nbf, Qsp, nullptr, st);
+      launch_split_rows(MT, rowlen, nbf, nbf, MTsp, nullptr, st);
     }
     for (int b = 0; b < nblk; ++b) {
       const int j0 = b * ob, nj = std::min(ob, norb - j0);
-      SplitMatrix Qb = Qsp;  // rows [j0, j0 + nj)
-      Qb.rows = nj;
-      Qb.s0 += (int64_t)j0 * Qb.kpad;
-      if (Qb.s1) Qb.s1 += (int64_t)j0 * Qb.kpad;
-      if (Qb.s2) Qb.s2 += (int64_t)j0 * Qb.kpad;
-      if (Qb.s1h) Qb.s1h += (int64_t)j0 * Qb.kpad;
-      Qb.expo += j0;
-      LRTEI_TRY(tc_gemm(Qb, MTsp, nj, rowlen, 1.0, X, rowlen, false, false, 1, nullptr, plan->d_status, st));
+      LRTEI_TRY(tc_gemm(Qsp, j0, MTsp, nj, rowlen, 1.0, X, rowlen, false, false, 1, nullptr, plan->d_status, st));
       SplitMatrix Xb = Xsp;
       Xb.rows = (int64_t)nj * nbf;
       {
         ProfScope ps("split", st);
-        launch_split_rows(X, Xb.rows, n3, n3, Xb, false, nslices(plan), st);
+        launch_split_rows(X, Xb.rows, n3, n3, Xb, nullptr, st);
       }
-      LRTEI_TRY(tc_gemm(Xb, plan->Ksp, Xb.rows, n3, 1.0, Y, n3, false, false, 1, nullptr, plan->d_status, st));
-      launch_perm_orbital_rows(nbf, n3, nj, X, Xp, st);
-      launch_perm_orbital_rows(nbf, n3, nj, Y, Yp, st);
+      LRTEI_TRY(tc_gemm_K(Xb, 0, plan->Ksp, plan->pc, Xb.rows, false, Y, 1, nullptr, plan->d_status, st));
+      launch_perm_orbital_rows(nbf, n3, nj, X, n3, nullptr, Xp, st);
+      launch_perm_orbital_rows(nbf, n3, nj, Y, ycols, plan->d_pos, Yp, st);
       SplitMatrix Ya = Ypsp, Xa = Xpsp;
       Ya.kpad = Xa.kpad = kpad256((int64_t)nj * n3);
       {
         ProfScope ps("split", st);
-        launch_split_rows(Yp, nbf, (int64_t)nj * n3, (int64_t)nj * n3, Ya, false, nslices(plan), st);
-        launch_split_rows(Xp, nbf, (int64_t)nj * n3, (int64_t)nj * n3, Xa, true, nslices(plan), st);
+        launch_split_rows(Yp, nbf, (int64_t)nj * n3, (int64_t)nj * n3, Ya, nullptr, st);
+        launch_split_rows(Xp, nbf, (int64_t)nj * n3, (int64_t)nj * n3, Xa, nullptr, st);
       }
       const int sb = splits_for(nbf, (int64_t)nj * n3);
       if (sb > sK) { set_error("exchange: split count %d beyond the partial buffer's %d", sb, sK); return LRTEI_ERR_CUDA; }
-      LRTEI_TRY(tc_gemm(Ya, Xa, nbf, nbf, 2.0, Kb + (size_t)b * nbf * nbf, nbf, false, false, sb, part,
+      LRTEI_TRY(tc_gemm(Ya, 0, Xa, nbf, nbf, 2.0, Kb + (size_t)b * nbf * nbf, nbf, false, false, sb, part,
                         plan->d_status, st));
     }
   } else {
@@ -1778,8 +1806,8 @@ lrtei_status lrtei_exchange(lrtei_plan* plan, const double* d_Q, int norb, doubl
         ProfScope ps("kron", st);
         LRTEI_CUDA(launch_kron_apply(n, P, plan->d_C, plan->d_w, X, 1, 0, Y, (int64_t)nj * nbf, has_parity(plan), st));
       }
-      launch_perm_orbital_rows(nbf, n3, nj, X, Xp, st);
-      launch_perm_orbital_rows(nbf, n3, nj, Y, Yp, st);
+      launch_perm_orbital_rows(nbf, n3, nj, X, n3, nullptr, Xp, st);
+      launch_perm_orbital_rows(nbf, n3, nj, Y, n3, nullptr, Yp, st);
       const int64_t K = (int64_t)nj * n3, nc = (K + kc - 1) / kc;
       for (int64_t q = 0; q < nc; ++q) {
         const int64_t k0 = q * kc, kk = std::min(kc, K - k0);
@@ -1868,8 +1896,7 @@ lrtei_status lrtei_plan_compress(lrtei_plan* plan, double eps, int max_rank, dou
   release_oz(plan, plan->ozF);
   release_oz(plan, plan->ozFT);
   release_oz(plan, plan->ozK);
-  plan->release(plan->d_perm, sizeof(int) * (size_t)plan->pc.cols);
-  plan->d_perm = nullptr;
+  release_classes(plan);
   plan->release(plan->d_S, sizeof(double) * 3 * (size_t)nrows * n);
   plan->release(plan->d_C, sizeof(double) * 3 * (size_t)P * n * n);
   plan->release(V, sizeof(double) * 3 * (size_t)n * n);
@@ -1890,35 +1917,36 @@ static lrtei_status jbuild_tc(lrtei_plan* plan, const double* d_D, int R, double
   LRTEI_TRY(sc.get(&Du, (size_t)npair * R));
   LRTEI_TRY(sc.get(&DuT, (size_t)npair * R));
   LRTEI_TRY(sc.get(&XT, (size_t)R * n3));
-  LRTEI_TRY(sc.get(&YT, (size_t)R * n3));
+  const ParityClasses& pc = plan->pc;
+  LRTEI_TRY(sc.get(&YT, (size_t)R * pc.cols));
   LRTEI_TRY(sc.get(&Ju, (size_t)npair * R));
   const int s1 = splits_for(n3, npair), s2 = splits_for(n3, n3), s3 = splits_for(npair, n3);
   const int smax = std::max(s1, std::max(s2, s3));
-  LRTEI_TRY(sc.get(&part, (size_t)smax * std::max(n3, npair) * R));
+  LRTEI_TRY(sc.get(&part, (size_t)smax * std::max<int64_t>(pc.cols, npair) * R));
   SplitMatrix Dsp, Xsp, Ysp;
-  LRTEI_TRY(scratch_split(sc, Dsp, R, npair, true, plan));
-  LRTEI_TRY(scratch_split(sc, Xsp, R, n3, true, plan));
-  LRTEI_TRY(scratch_split(sc, Ysp, R, n3, true, plan));
+  LRTEI_TRY(scratch_split(sc, Dsp, R, npair, split_tile(R), plan));
+  LRTEI_TRY(scratch_split(sc, Xsp, R, n3, split_tile(R), plan));
+  LRTEI_TRY(scratch_split(sc, Ysp, R, n3, split_tile(R), plan));
   launch_pack_density(nbf, R, d_D, Du, st);
   launch_transpose(Du, npair, R, R, DuT, npair, st);
   {
     ProfScope ps("split", st);
-    launch_split_rows(DuT, R, npair, npair, Dsp, true, nslices(plan), st);
+    launch_split_rows(DuT, R, npair, npair, Dsp, nullptr, st);
   }
   // X^T = (F^T D_u)^T : R x n^3
-  LRTEI_TRY(tc_gemm(plan->FTsp, Dsp, n3, R, 1.0, XT, n3, true, false, s1, part, plan->d_status, st));
+  LRTEI_TRY(tc_gemm(plan->FTsp, 0, Dsp, n3, R, 1.0, XT, n3, true, false, s1, part, plan->d_status, st));
   {
     ProfScope ps("split", st);
-    launch_split_rows(XT, R, n3, n3, Xsp, true, nslices(plan), st);
+    launch_split_rows(XT, R, n3, n3, Xsp, nullptr, st);
   }
-  // Y^T = (K X)^T : R x n^3  (K symmetric)
-  LRTEI_TRY(tc_gemm(plan->Ksp, Xsp, n3, R, 1.0, YT, n3, true, false, s2, part, plan->d_status, st));
+  // Y^T = (K X)^T (K symmetric), its columns in class order
+  LRTEI_TRY(tc_gemm_K(Xsp, 0, plan->Ksp, pc, R, true, YT, s2, part, plan->d_status, st));
   {
     ProfScope ps("split", st);
-    launch_split_rows(YT, R, n3, n3, Ysp, true, nslices(plan), st);
+    launch_split_rows(YT, R, n3, pc.cols, Ysp, plan->d_pos, st);
   }
   // J_u = F Y : npair x R
-  LRTEI_TRY(tc_gemm(plan->Fsp, Ysp, npair, R, 1.0, Ju, R, false, false, s3, part, plan->d_status, st));
+  LRTEI_TRY(tc_gemm(plan->Fsp, 0, Ysp, npair, R, 1.0, Ju, R, false, false, s3, part, plan->d_status, st));
   launch_unpack_J(nbf, R, Ju, 1.0, d_J, plan->d_status, st);
   return finish_launch("jbuild (tensor cores)");
 }
@@ -1975,10 +2003,10 @@ static lrtei_status jbuild_streamed(lrtei_plan* plan, const double* d_D, int R, 
                                    (int64_t)splits_for(rb, n3) * rb, (int64_t)splits_for(nlast, n3) * nlast});
   LRTEI_TRY(sc.get(&part, (size_t)part_n * R));
   SplitMatrix FbTsp, Dbsp, Fbsp, Ysp;
-  LRTEI_TRY(scratch_split(sc, FbTsp, n3, rb, false, plan));
-  LRTEI_TRY(scratch_split(sc, Dbsp, R, rb, true, plan));
-  LRTEI_TRY(scratch_split(sc, Fbsp, rb, n3, false, plan));
-  LRTEI_TRY(scratch_split(sc, Ysp, R, n3, true, plan));
+  LRTEI_TRY(scratch_split(sc, FbTsp, n3, rb, 128, plan));
+  LRTEI_TRY(scratch_split(sc, Dbsp, R, rb, split_tile(R), plan));
+  LRTEI_TRY(scratch_split(sc, Fbsp, rb, n3, 128, plan));
+  LRTEI_TRY(scratch_split(sc, Ysp, R, n3, split_tile(R), plan));
   for (int64_t b = 0; b < nblk; ++b) {
     const int64_t r0 = b * rb, nr = std::min(npair, r0 + rb) - r0;
     launch_build_F<double>(plan->t, n, plan->d_S, r0, r0 + nr, Fb, n3, st);
@@ -1988,11 +2016,11 @@ static lrtei_status jbuild_streamed(lrtei_plan* plan, const double* d_D, int R, 
     A.kpad = Bm.kpad = kpad256(nr);
     {
       ProfScope ps("split", st);
-      launch_split_rows(FbT, n3, nr, nr, A, false, nslices(plan), st);
-      launch_split_rows(DbT, R, nr, nr, Bm, true, nslices(plan), st);
+      launch_split_rows(FbT, n3, nr, nr, A, nullptr, st);
+      launch_split_rows(DbT, R, nr, nr, Bm, nullptr, st);
     }
     const int sb = splits_for(n3, nr);
-    LRTEI_TRY(tc_gemm(A, Bm, n3, R, 1.0, Xparts + b * R * n3, n3, true, false, sb, part, plan->d_status, st));
+    LRTEI_TRY(tc_gemm(A, 0, Bm, n3, R, 1.0, Xparts + b * R * n3, n3, true, false, sb, part, plan->d_status, st));
   }
   launch_reduce_splits(Xparts, (int)nblk, R * n3, R, n3, n3, Xt, n3, st);
   {
@@ -2001,7 +2029,7 @@ static lrtei_status jbuild_streamed(lrtei_plan* plan, const double* d_D, int R, 
   }
   {
     ProfScope ps("split", st);
-    launch_split_rows(Yt, R, n3, n3, Ysp, true, nslices(plan), st);
+    launch_split_rows(Yt, R, n3, n3, Ysp, nullptr, st);
   }
   for (int64_t b = 0; b < nblk; ++b) {
     const int64_t r0 = b * rb, nr = std::min(npair, r0 + rb) - r0;
@@ -2010,9 +2038,9 @@ static lrtei_status jbuild_streamed(lrtei_plan* plan, const double* d_D, int R, 
     A.rows = nr;
     {
       ProfScope ps("split", st);
-      launch_split_rows(Fb, nr, n3, n3, A, false, nslices(plan), st);
+      launch_split_rows(Fb, nr, n3, n3, A, nullptr, st);
     }
-    LRTEI_TRY(tc_gemm(A, Ysp, nr, R, 1.0, Ju + r0 * R, R, false, false, splits_for(nr, n3), part, plan->d_status, st));
+    LRTEI_TRY(tc_gemm(A, 0, Ysp, nr, R, 1.0, Ju + r0 * R, R, false, false, splits_for(nr, n3), part, plan->d_status, st));
   }
   launch_unpack_J(nbf, R, Ju, pref, d_J, plan->d_status, st);
   return finish_launch("jbuild (streamed, tensor cores)");
@@ -2061,16 +2089,16 @@ lrtei_status lrtei_jbuild_partial_x(lrtei_plan* plan, const double* d_D, int R, 
   const int sb = splits_for(n3, nr);
   LRTEI_TRY(sc.get(&part, (size_t)sb * n3 * R));
   SplitMatrix A, Bm;
-  LRTEI_TRY(scratch_split(sc, A, n3, nr, false, plan));
-  LRTEI_TRY(scratch_split(sc, Bm, R, nr, true, plan));
+  LRTEI_TRY(scratch_split(sc, A, n3, nr, 128, plan));
+  LRTEI_TRY(scratch_split(sc, Bm, R, nr, split_tile(R), plan));
   launch_transpose(Fb, nr, n3, n3, FbT, nr, st);
   launch_transpose(Du + pair_begin * R, nr, R, R, DbT, nr, st);
   {
     ProfScope ps("split", st);
-    launch_split_rows(FbT, n3, nr, nr, A, false, nslices(plan), st);
-    launch_split_rows(DbT, R, nr, nr, Bm, true, nslices(plan), st);
+    launch_split_rows(FbT, n3, nr, nr, A, nullptr, st);
+    launch_split_rows(DbT, R, nr, nr, Bm, nullptr, st);
   }
-  LRTEI_TRY(tc_gemm(A, Bm, n3, R, 1.0, d_X, n3, true, false, sb, part, plan->d_status, st));
+  LRTEI_TRY(tc_gemm(A, 0, Bm, n3, R, 1.0, d_X, n3, true, false, sb, part, plan->d_status, st));
   return finish_launch("partial X (tensor cores)");
 }
 
@@ -2103,14 +2131,14 @@ lrtei_status lrtei_jbuild_apply_x(lrtei_plan* plan, const double* d_X, int R, in
     const int s3 = splits_for(nr, n3);
     LRTEI_TRY(sc.get(&part, (size_t)s3 * nr * R));
     SplitMatrix A, Ysp;
-    LRTEI_TRY(scratch_split(sc, A, nr, n3, false, plan));
-    LRTEI_TRY(scratch_split(sc, Ysp, R, n3, true, plan));
+    LRTEI_TRY(scratch_split(sc, A, nr, n3, 128, plan));
+    LRTEI_TRY(scratch_split(sc, Ysp, R, n3, split_tile(R), plan));
     {
       ProfScope ps("split", st);
-      launch_split_rows(Fb, nr, n3, n3, A, false, nslices(plan), st);
-      launch_split_rows(Y, R, n3, n3, Ysp, true, nslices(plan), st);
+      launch_split_rows(Fb, nr, n3, n3, A, nullptr, st);
+      launch_split_rows(Y, R, n3, n3, Ysp, nullptr, st);
     }
-    LRTEI_TRY(tc_gemm(A, Ysp, nr, R, 1.0, Ju, R, false, false, s3, part, plan->d_status, st));
+    LRTEI_TRY(tc_gemm(A, 0, Ysp, nr, R, 1.0, Ju, R, false, false, s3, part, plan->d_status, st));
   }
   launch_unpack_J_range(plan->t, nbf, R, pair_begin, pair_end, Ju, pref, d_J, plan->d_status, st);
   return finish_launch("apply X");

@@ -167,6 +167,36 @@ void launch_hadamard_rows(const PairTable& t, int n, int P, const double* d_S, c
 void launch_idx4_to_pairs(int nbf, const int32_t* d_idx4, int64_t count, int64_t* d_r, int64_t* d_c, int* d_status,
                           cudaStream_t st);
 
+// ---------------------------------------------------------------- parity classes
+// The columns (m1, m2, m3) of F_u and the rows and columns of K in classes of the degrees' parities: K
+// couples equal parities only (A_d^(p)(a, b) = 0 for odd a + b), so it is block diagonal in them.
+// Without that symmetry (compressed plans) there is one class in the natural order.
+struct ParityClasses {
+  int n = 0, nclass = 0, par = 0;
+  int cnt[2] = {0, 0};     // even and odd degrees below n
+  int size[8] = {};        // columns of each class
+  int off[8] = {};         // first column of each class in the permuted order, a multiple of 64
+  int64_t row0[8] = {};    // first row of each class in K, a multiple of 128
+  int cols = 0;            // permuted columns, padding included
+  int64_t rows = 0;        // rows of K, padding included
+  int kmax = 0;            // columns of K (the largest class, a multiple of 64)
+  // Step tables of the split-precision products, whose K runs in the natural order (device; NULL without
+  // parity): per class, at tab + tab_off[c], [units + 1] the first list entry of each 128-deep chunk,
+  // [units + 1] the number of chunks with entries before it, and the list of the 16-deep K blocks that
+  // hold columns of the class, the last one of each chunk flagged with 2^30.
+  const int* tab = nullptr;
+  int tab_off[8] = {};
+  int units = 0;           // chunks of the padded n^3
+  int blocks = 0;          // listed blocks of the largest class (of all n^3 columns without parity)
+  __host__ __device__ int cls(int m1, int m2, int m3) const {
+    return par ? (m1 & 1) * 4 + (m2 & 1) * 2 + (m3 & 1) : 0;
+  }
+  __host__ __device__ int index(int m1, int m2, int m3) const {  // inside the class
+    return par ? ((m1 >> 1) * cnt[m2 & 1] + (m2 >> 1)) * cnt[m3 & 1] + (m3 >> 1) : (m1 * n + m2) * n + m3;
+  }
+  __host__ __device__ int64_t row(int m1, int m2, int m3) const { return row0[cls(m1, m2, m3)] + index(m1, m2, m3); }
+};
+
 // ---------------------------------------------------------------- factored form
 // F_u[r][m] = sum_{j in r} c_j S_x(j,m1) S_y(j,m2) S_z(j,m3), m = (m1 n + m2) n + m3, for r in [r0, r1).
 template <typename T>
@@ -176,6 +206,11 @@ void launch_build_F(const PairTable& t, int n, const double* d_S, int64_t r0, in
 // tensor-core precisions, whose F_u only feeds 30-bit slices.
 void launch_build_F_pairs(const PairTable& t, int n, const double* d_S, int64_t r0, int64_t r1, double* d_F,
                           int64_t ldF, cudaStream_t st);
+// The same sums by parity class for the split-precision products: row pc.row(a1, a2, a3), column 16 t + m % 16
+// for the listed block t of column m = (b1 n + b2) n + b3 (d_pos[16 c..]: see ensure_classes); the caller
+// zero-fills K (pc.rows x ldK).
+cudaError_t launch_build_K_classes(int n, int P, const ParityClasses& pc, const int* d_blk, const double* d_C,
+                                   const double* d_w, double scale, double* d_K, int64_t ldK, cudaStream_t st);
 // Dense K = sum_p w_p C_x^p (x) C_y^p (x) C_z^p  (n^3 x n^3), FP64.
 cudaError_t launch_build_K(int n, int P, const double* d_C, const double* d_w, double scale, double* d_K,
                            cudaStream_t st);
@@ -238,8 +273,9 @@ void launch_adaptive_entries(const PairTable& t, int n, int P, int npart, const 
 // ---------------------------------------------------------------- long-range exchange
 // MT[(mu n3 + m) nbf + la] = F[pair(mu, la) ldF + m]  (nbf n3 rows of nbf).
 void launch_gather_MT(int nbf, int64_t n3, const double* d_F, int64_t ldF, double* d_MT, cudaStream_t st);
-// Zp[mu][j n3 + m] = Z[(j nbf + mu) n3 + m] for j < nj.
-void launch_perm_orbital_rows(int nbf, int64_t n3, int nj, const double* d_Z, double* d_Zp, cudaStream_t st);
+// Zp[mu][j n3 + m] = Z[(j nbf + mu) ld + map[m]] for j < nj (map NULL: m).
+void launch_perm_orbital_rows(int nbf, int64_t n3, int nj, const double* d_Z, int64_t ld, const int* d_map, double* d_Zp,
+                              cudaStream_t st);
 
 // ---------------------------------------------------------------- CUDA-core GEMM
 // C[M x N] = alpha * op(A) op(B) + beta * C, row-major; transA: A is K x M; transB: B is N x K.
@@ -250,26 +286,6 @@ void convert_f64_to_f32(const double* in, float* out, int64_t count, cudaStream_
 void convert_f32_to_f64(const float* in, double* out, int64_t count, cudaStream_t st);
 
 // ---------------------------------------------------------------- FP64 on the tensor cores (k_ozaki.cu)
-// The columns (m1, m2, m3) of F_u and the rows and columns of K in classes of the degrees' parities: K
-// couples equal parities only (A_d^(p)(a, b) = 0 for odd a + b), so it is block diagonal in them.
-// Without that symmetry (compressed plans) there is one class in the natural order.
-struct ParityClasses {
-  int n = 0, nclass = 0, par = 0;
-  int cnt[2] = {0, 0};     // even and odd degrees below n
-  int size[8] = {};        // columns of each class
-  int off[8] = {};         // first column of each class in the permuted order, a multiple of 64
-  int64_t row0[8] = {};    // first row of each class in K, a multiple of 128
-  int cols = 0;            // permuted columns, padding included
-  int64_t rows = 0;        // rows of K, padding included
-  int kmax = 0;            // columns of K (the largest class, a multiple of 64)
-  __host__ __device__ int cls(int m1, int m2, int m3) const {
-    return par ? (m1 & 1) * 4 + (m2 & 1) * 2 + (m3 & 1) : 0;
-  }
-  __host__ __device__ int index(int m1, int m2, int m3) const {  // inside the class
-    return par ? ((m1 >> 1) * cnt[m2 & 1] + (m2 >> 1)) * cnt[m3 & 1] + (m3 >> 1) : (m1 * n + m2) * n + m3;
-  }
-  __host__ __device__ int64_t row(int m1, int m2, int m3) const { return row0[cls(m1, m2, m3)] + index(m1, m2, m3); }
-};
 constexpr int kOzSlices = 6;      // base-512 digits of an FP64 element
 constexpr int kOzBad = 1 << 20;   // exponent of a row that holds a NaN or an infinity
 struct OzMatrix {                 // rows x kpad (a multiple of 64), kOzSlices digit planes, in tiles of
@@ -295,28 +311,43 @@ lrtei_status oz_gemm(const OzMatrix& A, const OzMatrix& B, const std::vector<OzS
                      bool transpose_out, bool symmetric, int64_t c_rows, int64_t c_cols, int* d_status, cudaStream_t st);
 
 // ---------------------------------------------------------------- tensor cores (tcgen05)
-struct SplitMatrix {  // row-major rows x kpad, three FP16 integer slices + per-row scale exponent
+struct SplitMatrix {  // rows x kpad (a multiple of 256), three FP16 slice planes + per-row scale exponent, in
+                      // tiles of `tile` rows x 16 columns (tc_gemm.h)
   int64_t rows = 0, kpad = 0;
-  uint16_t* s0 = nullptr;
-  uint16_t* s1 = nullptr;
-  uint16_t* s2 = nullptr;  // third slice t2, pre-scaled by 2^-11 (FP16 bits)
-  uint16_t* s1h = nullptr; // second slice t1 pre-scaled by 2^-11 (B operand only)
+  int tile = 128;          // 128; 32 or 64 for the right operand of a product that narrow
+  uint16_t* d = nullptr;
   int* expo = nullptr;     // [rows]
-  bool plain = false;      // plain BF16 operands in s0 only (no slices)
-  bool eight = false;      // eight-product scheme: every operand carries s1h (A: t1 t2 products)
+  bool plain = false;      // one plane of plain BF16 operands (no slices)
+  bool eight = false;      // eight-product scheme
+  int planes() const { return plain ? 1 : 3; }
+  int64_t count() const { return (rows + tile - 1) / tile * tile * kpad * planes(); }
+  SplitMatrix from_row(int64_t r0, int64_t nr) const {  // rows [r0, r0 + nr), r0 a multiple of the tile
+    SplitMatrix v = *this;
+    v.rows = nr;
+    v.d += r0 * kpad * planes();
+    v.expo += r0;
+    return v;
+  }
 };
-// Slice an FP64 row-major matrix (rows x k, ld) into a SplitMatrix (zero padded to kpad).
-void launch_split_rows(const double* d_src, int64_t rows, int64_t k, int64_t ld, SplitMatrix& m, bool with_s1h,
-                       int nslices, cudaStream_t st);
-// nslices == 1 keeps only the leading slice (s1 = s2 = 0): plain BF16 operands.
-// C = scale * A B^T through tcgen05 (see k_tcgen05.cu).  A: M rows with slices s0, s1, s2;
-// B: N rows with s0, s1, s1h, s2; shared kpad (multiple of 256).  transpose_out writes C^T;
-// symmetric_upper computes the upper-triangular 128x128 blocks of a square C and mirrors them.
+// Right-operand tile rows for N columns of C.
+inline int split_tile(int64_t N) { return N <= 32 ? 32 : N <= 64 ? 64 : 128; }
+// Slice an FP64 row-major matrix (rows x k, ld) into a SplitMatrix (zero padded to kpad); column j is
+// source column d_map[j] (NULL: j).
+void launch_split_rows(const double* d_src, int64_t rows, int64_t k, int64_t ld, const SplitMatrix& m, const int* d_map,
+                       cudaStream_t st);
+// C = scale * A B^T through tcgen05 (see k_tcgen05.cu).  A: rows [a_row0, a_row0 + M) of its operand; B: N rows;
+// shared kpad (multiple of 256).  transpose_out writes C^T; symmetric_upper computes the
+// upper-triangular 128x128 blocks of a square C and mirrors them.
 // splits > 1 splits K (at most 32768 per split) into d_part (splits * M * N doubles), reduced
 // into C afterwards.
-lrtei_status tc_gemm(const SplitMatrix& A, const SplitMatrix& B, int64_t M, int64_t N, double scale, double* d_C,
-                     int64_t ldc, bool transpose_out, bool symmetric_upper, int splits, double* d_part,
+lrtei_status tc_gemm(const SplitMatrix& A, int64_t a_row0, const SplitMatrix& B, int64_t M, int64_t N, double scale,
+                     double* d_C, int64_t ldc, bool transpose_out, bool symmetric_upper, int splits, double* d_part,
                      int* d_status, cudaStream_t st);
+// Products with the node sum K by parity classes, in class order (pc.cols columns, padding zero):
+// k_is_a false: C[rows][pc.cols] = X K^T from rows [x_row0, x_row0 + rows) of X; k_is_a: C[r][:] = K X_r for
+// the rows r of X.  X in the natural column order.
+lrtei_status tc_gemm_K(const SplitMatrix& X, int64_t x_row0, const SplitMatrix& K, const ParityClasses& pc, int64_t rows,
+                       bool k_is_a, double* d_C, int splits, double* d_part, int* d_status, cudaStream_t st);
 // Block rows [row0, row1) of the symmetric product C = A B^T (N x N): the upper-triangular
 // 128 x 128 blocks of those rows, computed and mirrored.  A holds rows [row0, row1) only; row0 is a
 // multiple of 128, as is row1 unless it is N.  Rows of C at or above row0 are complete once every

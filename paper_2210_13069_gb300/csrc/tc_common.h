@@ -33,14 +33,27 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t by
                : "memory");
 }
 
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_try_wait_at(uint32_t addr, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
       : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
+      : "r"(addr), "r"(parity)
       : "memory");
   return ok != 0;
+}
+// The same without suspending the thread.
+__device__ __forceinline__ bool mbar_test_wait_at(uint32_t addr, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(addr), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
+  return mbar_try_wait_at(smem_u32(bar), parity);
 }
 
 // Bounded wait: false if the CTA is aborting or the wait gave up (which raises the abort).
@@ -181,33 +194,40 @@ __device__ __forceinline__ int64_t fixed32(double x, int e) {
 
 // Slices of one element: q = round(x 2^(32-e)), s0 = round(q / 2^24), r = q - s0 2^24,
 // t1 = round(r / 2^12), t2 = r - t1 2^12; x ~ 2^e (s0 2^-8 + t1 2^-20 + t2 2^-32), |s0| <= 255,
-// |t1|, |t2| <= 2048.  As FP16 bit patterns: s0, t1, t2 / 2^12 and t1 / 2^12 -- all exact
-// (integers up to 2^11 in magnitude, and those times 2^-12).
-struct SliceBits {
-  uint16_t s0, s1, s2, s1h;
-};
-__device__ __forceinline__ SliceBits slice_bits(double x, int e, bool live, int nslices) {
-  float a = 0.f, b = 0.f, c = 0.f;
+// |t1|, |t2| <= 2048: integers that FP16 holds exactly, also over 2^12 and 2^24.
+__device__ __forceinline__ void slice_ints(double x, int e, bool live, float& s0, float& t1, float& t2) {
+  s0 = t1 = t2 = 0.f;
   if (live) {
     const int64_t q = fixed32(x, e);
     const int64_t q0 = (q + (1LL << 23)) >> 24;
     const int64_t r = q - (q0 << 24);
     const int64_t q1 = (r + (1LL << 11)) >> 12;
     const int64_t q2 = r - (q1 << 12);
-    a = (float)q0;
-    b = nslices > 1 ? (float)q1 : 0.f;
-    c = nslices > 2 ? (float)q2 : 0.f;
+    s0 = (float)q0;
+    t1 = (float)q1;
+    t2 = (float)q2;
   }
-  return {f16_bits(a), f16_bits(b), f16_bits(c * (1.0f / 4096.0f)), f16_bits(b * (1.0f / 4096.0f))};
 }
 
-__device__ __forceinline__ void slice_store(double x, int e, bool live, int nslices, int64_t o, uint16_t* s0,
-                                            uint16_t* s1, uint16_t* s2, uint16_t* s1h) {
-  const SliceBits q = slice_bits(x, e, live, nslices);
-  s0[o] = q.s0;
-  s1[o] = q.s1;
-  s2[o] = q.s2;
-  if (s1h) s1h[o] = q.s1h;
+// The planes of the GEMM operands as FP16 bit patterns: s0, t1 / 2^12, t2 / 2^24.
+struct SliceBits {
+  uint16_t s0, s1, s2;
+};
+__device__ __forceinline__ SliceBits slice_bits(double x, int e, bool live) {
+  float a, b, c;
+  slice_ints(x, e, live, a, b, c);
+  return {f16_bits(a), f16_bits(b * 0x1p-12f), f16_bits(c * 0x1p-24f)};
+}
+
+// The planes of the Hadamard form's operands: s0, t1, t2 / 2^12 and, where s1h is given, t1 / 2^12.
+__device__ __forceinline__ void slice_store(double x, int e, bool live, int64_t o, uint16_t* s0, uint16_t* s1,
+                                            uint16_t* s2, uint16_t* s1h) {
+  float a, b, c;
+  slice_ints(x, e, live, a, b, c);
+  s0[o] = f16_bits(a);
+  s1[o] = f16_bits(b);
+  s2[o] = f16_bits(c * 0x1p-12f);
+  if (s1h) s1h[o] = f16_bits(b * 0x1p-12f);
 }
 
 // ------------------------------------------------------------------ FP32 pairs to FP64
