@@ -321,7 +321,7 @@ lrtei_status oz_gemm(const OzMatrix& A, const OzMatrix& B, const std::vector<OzS
   p.split_stride = part ? c_rows * c_cols : 0;
   for (int i = 0; i < p.nseg; ++i) p.seg[i].c_off -= transpose_out ? p.seg[i].m_lo : p.seg[i].m_lo * p.ldc;
   p.status = d_status;
-  p.align = tcg::store_align(p.C, p.ldc);
+  p.align = tc::store_align(p.C, p.ldc);
   p.test_stall = tcg::test_stall_cycles();
   lrtei_status s;
   {

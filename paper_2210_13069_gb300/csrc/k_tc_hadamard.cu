@@ -72,6 +72,7 @@ struct Params {
   const int* eb;      // [nrows]
   double* out;
   int64_t ld;
+  int align;          // doubles per access that every row of out allows
   int* status;
   long long test_stall;  // > 0 (tests only): the MMA thread first waits this many cycles on a barrier
                          // that nothing completes, so that the bounded-wait failure path runs
@@ -95,25 +96,66 @@ __device__ __forceinline__ void tile_of(const Params& p, int64_t item, int64_t& 
   }
 }
 
+// Two FP32 numbers in a register pair, each operation rounded as the scalar one; one instruction for both
+// (25 operations per element and node as scalars: the epilogue is the longer side of this kernel; 7.8 -> 6.4 ms
+// at 180 functions with every warp waiting for itself, 6.1 with four-column stores).
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float x, float y) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ f32x2 pack2(uint32_t x, uint32_t y) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(x), "r"(y));
+  return r;
+}
+__device__ __forceinline__ float half_of(f32x2 v, int odd) {
+  float x, y;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+  return (odd & 1) ? y : x;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 neg2(f32x2 a) { return a ^ 0x8000000080000000ULL; }
+
 // (ah + al)(bh + bl) as an unevaluated FP32 pair; every partial product kept (|al|, |bl| may be
-// 2^-9 of |ah|, |bh| here), the leading one split exactly with fmaf.
-__device__ __forceinline__ void pmul(float ah, float al, float bh, float bl, float& ph, float& pl) {
-  const float p = ah * bh;
-  float e = fmaf(ah, bh, -p);
-  e = fmaf(ah, bl, e);
-  e = fmaf(al, bh, e);
-  e = fmaf(al, bl, e);
+// 2^-9 of |ah|, |bh| here), the leading one split exactly by the FMA.
+__device__ __forceinline__ void pmul(f32x2 ah, f32x2 al, f32x2 bh, f32x2 bl, f32x2& ph, f32x2& pl) {
+  const f32x2 p = mul2(ah, bh);
+  f32x2 e = fma2(ah, bh, neg2(p));
+  e = fma2(ah, bl, e);
+  e = fma2(al, bh, e);
+  e = fma2(al, bl, e);
   ph = p;
   pl = e;
 }
 
 // (ah, al) += (bh, bl): two-sum of the leading parts, the rest summed into the trailing part.
-__device__ __forceinline__ void padd(float& ah, float& al, float bh, float bl) {
-  const float s = ah + bh;
-  const float v = s - ah;
-  const float err = (ah - (s - v)) + (bh - v);
+__device__ __forceinline__ void padd(f32x2& ah, f32x2& al, f32x2 bh, f32x2 bl) {
+  const f32x2 s = add2(ah, bh);
+  const f32x2 v = sub2(s, ah);
+  const f32x2 err = add2(sub2(ah, sub2(s, v)), sub2(bh, v));
   ah = s;
-  al = al + (bl + err);
+  al = add2(al, add2(bl, err));
 }
 
 // ------------------------------------------------------------------ the kernel
@@ -139,9 +181,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   uint64_t* never = done + 1;        // completed by nobody (the test stall waits on it)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(never + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  volatile int* epi_flag = abort_flag + 1;  // [2] the poller's result for the epilogue warps
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int steps_per_tile = p.P * 3;  // (p, d) products per tile
 
   if (threadIdx.x == 0) {
@@ -220,34 +261,40 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
+      // One elected thread runs the loop, the next T stage's barrier tested before the MMAs issue.  Behind
+      // `if (lane == 0)` the ~12 MMAs of a (p, d) step took ~2 000 clocks to issue (they execute in ~500),
+      // and the kernel 10.9 ms at 180 functions.
       // kind::f16, FP32 accumulators, FP16 operands, both K-major, M = 128, N = 64
       const uint32_t idesc = (1u << 4) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-      uint32_t it = 0, cg = 0, tl = 0;
-      bool ok = true;
+      const uint64_t a_desc = smem_desc<BK>(smem_u32(sA)), b_desc = smem_desc<BK>(smem_u32(sB));
+      const uint32_t full0 = smem_u32(full);
+      uint32_t s = 0, ph = 0, buf = 0, bph = 1, tl = 0;  // T stage and its phase, accumulator buffer and its phase
+      bool ok = true, ready = false;
       // test hook: a wait that runs out (nothing arrives on `never`), then the abort path
       if (p.test_stall > 0) ok = mbar_wait(never, 0u, abort_flag, p.status, 0, p.test_stall);
       for (int64_t item = blockIdx.x; item < p.ntiles && ok; item += gridDim.x, ++tl) {
         if (!mbar_wait(bfull, tl & 1u, abort_flag, p.status)) break;
         tc_fence_after();
-        for (int q = 0; q < steps_per_tile && ok; ++q, ++cg) {
-          const int d = q % 3;
-          const int buf = (int)(cg % NBUF);
-          // the epilogue is the slower side: poll its drained buffers at a relaxed pace
-          if (!mbar_wait(&acce[buf], ((cg / NBUF) & 1u) ^ 1u, abort_flag, p.status, 128)) { ok = false; break; }
+        uint32_t d = 0;
+        for (int q = 0; q < steps_per_tile; ++q) {
+          if (!mbar_wait(&acce[buf], bph, abort_flag, p.status, 32)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t d0 = tmem_base + (uint32_t)(buf * 2 * BN);
+          const uint32_t d0 = tmem_base + buf * (uint32_t)(2 * BN);
           const uint32_t d1 = d0 + BN;
-          for (int ks = 0; ks < KS; ++ks, ++it) {
-            const int s = (int)(it % STAGES);
-            if (!mbar_wait(&full[s], (it / STAGES) & 1u, abort_flag, p.status)) { ok = false; break; }
+#pragma unroll
+          for (int ks = 0; ks < KS; ++ks) {
+            if (!ready && !mbar_wait(&full[s], ph, abort_flag, p.status)) { ok = false; break; }
             tc_fence_after();
-            const uint32_t abase = smem_u32(sA + (size_t)s * A_STAGE);
-            const uint32_t bbase = smem_u32(sB + (size_t)((d * KS + ks) * 4) * B_PLANE);
-            const uint64_t a0 = smem_desc<BK>(abase), a1 = smem_desc<BK>(abase + A_PLANE),
-                           a2 = smem_desc<BK>(abase + 2 * A_PLANE);
-            const uint64_t b0 = smem_desc<BK>(bbase), b1 = smem_desc<BK>(bbase + B_PLANE),
-                           b1h = smem_desc<BK>(bbase + 2 * B_PLANE), b2 = smem_desc<BK>(bbase + 3 * B_PLANE);
+            const uint32_t cur = s;
+            if (++s == STAGES) {
+              s = 0;
+              ph ^= 1u;
+            }
+            ready = mbar_test_wait_at(full0 + s * 8, ph);
+            constexpr uint64_t AP = A_PLANE >> 4, BP = B_PLANE >> 4;
+            const uint64_t a0 = a_desc + (uint64_t)(cur * (A_STAGE >> 4)), a1 = a0 + AP, a2 = a0 + 2 * AP;
+            const uint64_t b0 = b_desc + (uint64_t)((d * KS + ks) * 4) * BP, b1 = b0 + BP, b1h = b0 + 2 * BP, b2 = b0 + 3 * BP;
 #pragma unroll
             for (int k = 0; k < BK / 16; ++k) {
               const uint64_t o = (uint64_t)((k * 32) >> 4);  // +32 bytes along K inside the swizzle atom
@@ -259,10 +306,15 @@ __global__ void __launch_bounds__(THREADS, 1)
               mma_bf16_a<ACol::lastuse>(d1, a1 + o, b1h + o, idesc, 1u);
               mma_bf16(d1, a2 + o, b0 + o, idesc, 1u);
             }
-            mma_commit(&empty[s]);  // the T stage may be refilled once these MMAs retire
+            mma_commit(&empty[cur]);  // the T stage may be refilled once these MMAs retire
           }
           if (!ok) break;
           mma_commit(&accf[buf]);
+          if (++buf == NBUF) {
+            buf = 0;
+            bph ^= 1u;
+          }
+          if (++d == 3) d = 0;
         }
         if (!ok) break;
         mma_commit(bempty);  // the S block may be replaced once the tile's MMAs retire
@@ -272,6 +324,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       while (!mbar_try_wait(done, 0u) && clock64() - t0 < kWaitCycles) {
       }
     }
+    __syncwarp();
   } else {
     // ---------------------------------------------------------------- epilogue warps
     const int ew = warp - 2;
@@ -285,22 +338,22 @@ __global__ void __launch_bounds__(THREADS, 1)
       const int64_t r = I * BM + quad * 32 + lane;  // this thread's row of B_u
       const bool rlive = r < p.nrows;
       // node sum as an FP32 pair (as, al): two-sum of the leading parts, the rest in the trailing one
-      float as[QC], al[QC];
+      f32x2 as[QC / 2], al[QC / 2];
 #pragma unroll
-      for (int j = 0; j < QC; ++j) as[j] = al[j] = 0.f;
+      for (int j = 0; j < QC / 2; ++j) as[j] = al[j] = 0;
       float2 fnext = rlive ? p.f[r * p.P] : make_float2(0.f, 0.f);
+      const f32x2 scale = pack2(1.0f / 4096.0f, 1.0f / 4096.0f);
       for (int pp = 0; pp < p.P && ok; ++pp) {
-        const float2 f = fnext;  // this node's factor; the next one is fetched while it is used
-        if (pp + 1 < p.P && rlive) fnext = p.f[r * p.P + pp + 1];
-        float ph[QC], pl[QC];
+        const f32x2 fx = pack2(fnext.x, fnext.x), fy = pack2(fnext.y, fnext.y);  // this node's factor; the
+        if (pp + 1 < p.P && rlive) fnext = p.f[r * p.P + pp + 1];                 // next one is fetched meanwhile
+        f32x2 ph[QC / 2], pl[QC / 2];
 #pragma unroll
         for (int d = 0; d < 3; ++d, ++cg) {
           const int buf = (int)(cg % NBUF);
-          // one thread polls the buffer's barrier; the epilogue warps meet on a named barrier
-          if (ew == 0 && lane == 0)
-            epi_flag[cg & 1u] = mbar_wait(&accf[buf], (cg / NBUF) & 1u, abort_flag, p.status) ? 1 : 0;
-          asm volatile("bar.sync 1, %0;" ::"r"(32 * EPI) : "memory");
-          if (!epi_flag[cg & 1u]) { ok = false; break; }
+          // every warp waits for itself (the wait parks it), so that the warps' TMEM reads and arithmetic overlap
+          if (!mbar_wait(&accf[buf], (cg / NBUF) & 1u, abort_flag, p.status)) ok = false;
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
           tc_fence_after();
           const uint32_t tb = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * 2 * BN + col0);
 #pragma unroll
@@ -310,19 +363,20 @@ __global__ void __launch_bounds__(THREADS, 1)
             tmem_ld8(tb + BN + j0, l12);
             tmem_wait_ld();
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const float gh = __uint_as_float(l0[j]);                      // exact integer sum
-              const float gl = __uint_as_float(l12[j]) * (1.0f / 4096.0f);  // exact scaling
+            for (int j = 0; j < 8; j += 2) {
+              const int q = (j0 + j) / 2;
+              const f32x2 gh = pack2(l0[j], l0[j + 1]);                  // exact integer sums
+              const f32x2 gl = mul2(pack2(l12[j], l12[j + 1]), scale);  // exact scaling
               if (d == 0) {
                 // f g: f is a normalised pair, so its trailing part times gl (below 2^-33) is dropped
-                const float t = f.x * gh;
-                float e = fmaf(f.x, gh, -t);
-                e = fmaf(f.x, gl, e);
-                e = fmaf(f.y, gh, e);
-                ph[j0 + j] = t;
-                pl[j0 + j] = e;
+                const f32x2 t = mul2(fx, gh);
+                f32x2 e = fma2(fx, gh, neg2(t));
+                e = fma2(fx, gl, e);
+                e = fma2(fy, gh, e);
+                ph[q] = t;
+                pl[q] = e;
               } else {
-                pmul(ph[j0 + j], pl[j0 + j], gh, gl, ph[j0 + j], pl[j0 + j]);
+                pmul(ph[q], pl[q], gh, gl, ph[q], pl[q]);
               }
             }
           }
@@ -332,29 +386,29 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
         if (!ok) break;
 #pragma unroll
-        for (int j = 0; j < QC; ++j) padd(as[j], al[j], ph[j], pl[j]);
+        for (int j = 0; j < QC / 2; ++j) padd(as[j], al[j], ph[j], pl[j]);
       }
-      // every epilogue warp takes the same exits (the poller's flag), as the named barrier needs
       if (!ok) break;
-      // store: B_u(r, c) = 2^(Ra(r) + Eb(c) - 48) (as + al); the mirror B_u(c, r) too
+      // store: B_u(r, c) = 2^(Ra(r) + Eb(c) - 48) (as + al), four columns of the row at a time; the mirror
+      // B_u(c, r) too, consecutive lanes along a row of it
       if (rlive && r >= p.r0 && r < p.r1) {
         const int rk = p.ra[r] - 48;
         const int64_t c0 = J * BN + col0;
-        if (p.symmetric) {
+        double* orow = p.out + (r - (p.symmetric ? 0 : p.r0)) * p.ld;
 #pragma unroll
-          for (int j = 0; j < QC; ++j) {
-            const int64_t c = c0 + j;
-            if (c >= p.nrows || c < r) continue;
-            const double v = fpair_ldexp(as[j], al[j], rk + p.eb[c]);
-            p.out[r * p.ld + c] = v;
-            if (c != r) p.out[c * p.ld + r] = v;
-          }
-        } else {
-          double* orow = p.out + (r - p.r0) * p.ld;
+        for (int j0 = 0; j0 < QC; j0 += 4) {
+          const int64_t c = c0 + j0;
+          const int lo = p.symmetric ? (int)max((int64_t)0, min((int64_t)4, r - c)) : 0;
+          const int live = (int)max((int64_t)0, min((int64_t)4, p.nrows - c));
+          double v[4];
 #pragma unroll
-          for (int j = 0; j < QC; ++j) {
-            const int64_t c = c0 + j;
-            if (c < p.nrows) orow[c] = fpair_ldexp(as[j], al[j], rk + p.eb[c]);
+          for (int j = 0; j < 4; ++j)
+            v[j] = j < live ? fpair_ldexp(half_of(as[(j0 + j) / 2], j), half_of(al[(j0 + j) / 2], j), rk + p.eb[c + j]) : 0.0;
+          store4(orow + c, p.align, lo, live, v);
+          if (p.symmetric) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              if (j < live && c + j > r) p.out[(c + j) * p.ld + r] = v[j];
           }
         }
       }
@@ -522,6 +576,7 @@ lrtei_status had_tc_rows(const HadOperands& h, int64_t r0, int64_t r1, double* d
   p.eb = h.eb;
   p.out = d_out;
   p.ld = ld;
+  p.align = tc::store_align(d_out, ld);
   p.status = d_status;
   {
     // LRTEI_TEST_STALL_CYCLES (tests only), as for the GEMM: every CTA's MMA thread first waits that

@@ -206,7 +206,7 @@ static lrtei_status fill(tcg::Params& p, const SplitMatrix& A, const SplitMatrix
   p.ldc = splits > 1 ? c_cols : ldc;
   p.split_stride = splits > 1 ? c_rows * c_cols : 0;
   p.status = d_status;
-  p.align = tcg::store_align(p.C, p.ldc);
+  p.align = tc::store_align(p.C, p.ldc);
   p.test_stall = tcg::test_stall_cycles();
   return LRTEI_OK;
 }

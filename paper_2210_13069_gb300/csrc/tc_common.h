@@ -92,6 +92,14 @@ __device__ __forceinline__ void tma_load_2d(const CUtensorMap* map, void* dst, u
       : "memory");
 }
 
+// A contiguous copy into shared memory (16-byte aligned, a multiple of 16 bytes), completing on `bar`.
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_u32(dst)),
+               "l"(src), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
+}
+
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
@@ -294,6 +302,41 @@ __device__ __forceinline__ double fpair_ldexp(float hi, float lo, int k) {
   if (E > 2046) E = 2046;
   const uint64_t bits = ((uint64_t)(X < 0) << 63) | ((uint64_t)E << 52) | (mant & ((1ULL << 52) - 1));
   return __longlong_as_double((long long)bits);
+}
+
+// ------------------------------------------------------------------ stores
+// Four consecutive columns of one row of C: 32-byte accesses where ldc and C allow them.
+__device__ __forceinline__ void load4(const double* c, int al, int live, double (&v)[4]) {
+  if (al == 4 && live == 4) {
+    const double4_32a x = *reinterpret_cast<const double4_32a*>(c);
+    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+  } else if (al >= 2 && live == 4) {
+    const double2 x = *reinterpret_cast<const double2*>(c), y = *reinterpret_cast<const double2*>(c + 2);
+    v[0] = x.x; v[1] = x.y; v[2] = y.x; v[3] = y.y;
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = j < live ? c[j] : 0.0;
+  }
+}
+__device__ __forceinline__ void store4(double* c, int al, int lo, int live, const double (&v)[4]) {
+  if (al == 4 && live == 4 && lo <= 0) {
+    double4_32a x;
+    x.x = v[0]; x.y = v[1]; x.z = v[2]; x.w = v[3];
+    *reinterpret_cast<double4_32a*>(c) = x;
+  } else if (al >= 2 && live == 4 && lo <= 0) {
+    *reinterpret_cast<double2*>(c) = make_double2(v[0], v[1]);
+    *reinterpret_cast<double2*>(c + 2) = make_double2(v[2], v[3]);
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (j >= lo && j < live) c[j] = v[j];
+  }
+}
+
+// Doubles per access that every row of C allows (tiles and segments start at multiples of four columns).
+inline int store_align(const double* C, int64_t ldc) {
+  const uintptr_t a = reinterpret_cast<uintptr_t>(C);
+  return (ldc % 4 == 0 && (a & 31) == 0) ? 4 : (ldc % 2 == 0 && (a & 15) == 0) ? 2 : 1;
 }
 
 // ------------------------------------------------------------------ host: tensor maps

@@ -81,46 +81,10 @@ __device__ __forceinline__ double int_ldexp(long long X, int k) {
                                           ((unsigned long long)min(E, 2047) << 52) | m));
 }
 
-// A contiguous copy into shared memory (16-byte aligned, a multiple of 16 bytes), completing on `bar`.
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(dst)),
-               "l"(src), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
-}
-
 // K-major operand block of 32-byte rows in the 32-byte swizzle: 8-row atoms of 256 bytes.
 __device__ __forceinline__ uint64_t block_desc(uint32_t addr) {
   return (uint64_t)((addr & 0x3FFFFu) >> 4) | (uint64_t)1 << 16 | (uint64_t)(256 >> 4) << 32 | (uint64_t)1 << 46 |
          (uint64_t)6 << 61;
-}
-
-// Four consecutive columns of one row of C: 32-byte accesses where ldc and C allow them.
-__device__ __forceinline__ void load4(const double* c, int al, int live, double (&v)[4]) {
-  if (al == 4 && live == 4) {
-    const double4_32a x = *reinterpret_cast<const double4_32a*>(c);
-    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
-  } else if (al >= 2 && live == 4) {
-    const double2 x = *reinterpret_cast<const double2*>(c), y = *reinterpret_cast<const double2*>(c + 2);
-    v[0] = x.x; v[1] = x.y; v[2] = y.x; v[3] = y.y;
-  } else {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] = j < live ? c[j] : 0.0;
-  }
-}
-__device__ __forceinline__ void store4(double* c, int al, int lo, int live, const double (&v)[4]) {
-  if (al == 4 && live == 4 && lo <= 0) {
-    double4_32a x;
-    x.x = v[0]; x.y = v[1]; x.z = v[2]; x.w = v[3];
-    *reinterpret_cast<double4_32a*>(c) = x;
-  } else if (al >= 2 && live == 4 && lo <= 0) {
-    *reinterpret_cast<double2*>(c) = make_double2(v[0], v[1]);
-    *reinterpret_cast<double2*>(c + 2) = make_double2(v[2], v[3]);
-  } else {
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      if (j >= lo && j < live) c[j] = v[j];
-  }
 }
 
 // A work item: a tile (m0, n0: its first row and column inside the segment) and the K steps [t0, t1).
@@ -426,11 +390,5 @@ inline long long test_stall_cycles() {
   const char* v = getenv("LRTEI_TEST_STALL_CYCLES");
   return (v && *v) ? std::max(0LL, atoll(v)) : 0;
 }
-// Doubles per access that every row of C allows (tiles and segments start at multiples of four columns).
-inline int store_align(const double* C, int64_t ldc) {
-  const uintptr_t a = reinterpret_cast<uintptr_t>(C);
-  return (ldc % 4 == 0 && (a & 31) == 0) ? 4 : (ldc % 2 == 0 && (a & 15) == 0) ? 2 : 1;
-}
-
 }  // namespace tcg
 }  // namespace lrtei
