@@ -421,20 +421,18 @@ __device__ __forceinline__ bool nonfinite_bits(double v) {
   return ((__double_as_longlong(v) >> 52) & 0x7FF) == 0x7FF;
 }
 
-__global__ void k_expand_B(int nbf, const double* __restrict__ Bu, int64_t ldu, double scale, double* __restrict__ B,
-                           int64_t ldB, const int* __restrict__ pair_mu, const int* __restrict__ pair_nu, int* status) {
+__global__ void k_expand_B(int nbf, const double* __restrict__ Bu, int64_t ldu, double* __restrict__ B, int64_t ldB,
+                           const int* __restrict__ pair_mu, const int* __restrict__ pair_nu, int* status) {
   const int64_t r = blockIdx.x;
   const int mu = pair_mu[r], nu = pair_nu[r];
   const double* src = Bu + (size_t)r * ldu;
   double* row1 = B + ((size_t)mu * nbf + nu) * ldB;
   double* row2 = B + ((size_t)nu * nbf + mu) * ldB;
   const int nc = nbf * nbf;
-  const bool scaled = scale != 1.0;
   bool bad = false;
   ColWalk w(nbf, threadIdx.x, blockDim.x);
   for (int col = threadIdx.x; col < nc; col += blockDim.x, w.next()) {
-    double v = src[pair_idx(nbf, w.ka, w.la)];
-    if (scaled) v *= scale;
+    const double v = src[pair_idx(nbf, w.ka, w.la)];
     bad |= nonfinite_bits(v);
     row1[col] = v;
     if (mu != nu) row2[col] = v;
@@ -442,10 +440,90 @@ __global__ void k_expand_B(int nbf, const double* __restrict__ Bu, int64_t ldu, 
   latch_nonfinite_warp(status, bad);
 }
 
-void launch_expand_B(const PairTable& t, int nbf, const double* d_Bu, int64_t ldu, double scale, double* d_B,
+// The same from shared memory: the row of B_u (130 KB at N_b = 180, rows of up to kExpandPairs pairs) arrives by
+// one bulk copy, its gathers (half of a row's are one element per 32-byte sector) hit shared memory, and
+// every thread stores V consecutive columns of both rows.  N_b a multiple of V keeps them in one block of
+// equal ka; V doubles per store need ldB and B aligned to them.  HBM-bound: 10.5 GB at N_b = 180.
+constexpr int64_t kExpandPairs = 28000;  // N_b <= 236
+template <int V>
+__global__ void __launch_bounds__(1024) k_expand_B_row(int nbf, int64_t npair, const double* __restrict__ Bu,
+                                                       int64_t ldu, int bulk, double* __restrict__ B, int64_t ldB,
+                                                       const int* __restrict__ pair_mu, const int* __restrict__ pair_nu,
+                                                       int* status) {
+  extern __shared__ __align__(16) double row[];
+  __shared__ uint64_t bar;
+  const int64_t r = blockIdx.x;
+  const double* src = Bu + (size_t)r * ldu;
+  const int np = (int)npair;
+  if (bulk) {
+    if (threadIdx.x == 0) {
+      tc::mbar_init(&bar, 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      const uint32_t bytes = (uint32_t)((np + 1) / 2 * 16);  // the padding of a row holds the odd element
+      tc::mbar_arrive_expect_tx(&bar, bytes);
+      tc::bulk_load(row, src, bytes, &bar);
+    }
+  } else {
+#pragma unroll 4
+    for (int i = threadIdx.x; i < np; i += blockDim.x) row[i] = src[i];
+  }
+  const int mu = pair_mu[r], nu = pair_nu[r];
+  double* row1 = B + ((size_t)mu * nbf + nu) * ldB;
+  double* row2 = B + ((size_t)nu * nbf + mu) * ldB;
+  const int nc = nbf * nbf / V;
+  ColWalk w(nbf, V * (int)threadIdx.x, V * (int)blockDim.x);
+  __syncthreads();
+  if (bulk) {
+    for (long long t0 = clock64(); !tc::mbar_try_wait(&bar, 0u);)
+      if (clock64() - t0 > tc::kWaitCycles) {
+        latch_status(status, (int)kDevTimeout);
+        break;
+      }
+  }
+  bool bad = false;
+  for (int c = threadIdx.x; c < nc; c += blockDim.x, w.next()) {
+    double v[V];
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+      v[j] = row[(int)pair_idx(nbf, w.ka, w.la + j)];
+      bad |= nonfinite_bits(v[j]);
+    }
+    if constexpr (V == 4) {
+      double4_32a x;
+      x.x = v[0]; x.y = v[1]; x.z = v[2]; x.w = v[3];
+      *reinterpret_cast<double4_32a*>(row1 + 4 * c) = x;
+      if (mu != nu) *reinterpret_cast<double4_32a*>(row2 + 4 * c) = x;
+    } else {
+      row1[c] = v[0];
+      if (mu != nu) row2[c] = v[0];
+    }
+  }
+  latch_nonfinite_warp(status, bad);
+}
+
+void launch_expand_B(const PairTable& t, int nbf, int64_t npair, const double* d_Bu, int64_t ldu, double* d_B,
                      int64_t ldB, int* d_status, cudaStream_t st) {
   count_launch();
-  k_expand_B<<<(unsigned)t.npair, 256, 0, st>>>(nbf, d_Bu, ldu, scale, d_B, ldB, t.pair_mu, t.pair_nu, d_status);
+  if (npair > kExpandPairs) {
+    k_expand_B<<<(unsigned)t.npair, 256, 0, st>>>(nbf, d_Bu, ldu, d_B, ldB, t.pair_mu, t.pair_nu, d_status);
+    return;
+  }
+  const size_t smem = sizeof(double) * (size_t)(npair + 2);
+  static bool attr_set = false;
+  if (!attr_set) {
+    const int most = (int)(sizeof(double) * (kExpandPairs + 2));
+    attr_set = cudaFuncSetAttribute(k_expand_B_row<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess &&
+               cudaFuncSetAttribute(k_expand_B_row<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess;
+  }
+  // a row alone on its SM takes all its threads; several short ones share it
+  const int threads = npair >= 8192 ? 1024 : npair >= 2048 ? 512 : 256;
+  const int bulk = (ldu % 2 == 0 && ldu >= (npair + 1) / 2 * 2 && (reinterpret_cast<uintptr_t>(d_Bu) & 15) == 0) ? 1 : 0;
+  if (nbf % 4 == 0 && ldB % 4 == 0 && (reinterpret_cast<uintptr_t>(d_B) & 31) == 0)
+    k_expand_B_row<4><<<(unsigned)t.npair, threads, smem, st>>>(nbf, npair, d_Bu, ldu, bulk, d_B, ldB, t.pair_mu, t.pair_nu,
+                                                              d_status);
+  else
+    k_expand_B_row<1><<<(unsigned)t.npair, threads, smem, st>>>(nbf, npair, d_Bu, ldu, bulk, d_B, ldB, t.pair_mu, t.pair_nu,
+                                                              d_status);
 }
 
 // One block per row R = a N_b + b of B: out row R - R0 = B_u row pair(a, b) over the columns (ka, la).

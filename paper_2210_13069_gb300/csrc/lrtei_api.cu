@@ -1636,7 +1636,7 @@ lrtei_status lrtei_assemble_B(lrtei_plan* plan, lrtei_form form, double* d_B, in
     LRTEI_TRY(bu_adaptive(plan, Bu, st));
     {
       ProfScope ps("expand_B", st);
-      launch_expand_B(plan->t, nbf, Bu, npair, 1.0, d_B, ld, plan->d_status, st);
+      launch_expand_B(plan->t, nbf, npair, Bu, npair, d_B, ld, plan->d_status, st);
     }
     return finish_launch("expand_B");
   }
@@ -1655,17 +1655,18 @@ lrtei_status lrtei_assemble_B(lrtei_plan* plan, lrtei_form form, double* d_B, in
   }
   Scratch sc(st);
   double* blk;
-  LRTEI_TRY(sc.get(&blk, (size_t)rb * npair));
+  const int64_t ldu = (npair + 3) / 4 * 4;  // rows on 32-byte boundaries: the products store four columns at once
+  LRTEI_TRY(sc.get(&blk, (size_t)rb * ldu));
   for (int64_t r0 = 0; r0 < npair; r0 += rb) {
     const int64_t r1 = std::min(npair, r0 + rb);
-    LRTEI_TRY(bu_rows(plan, f, r0, r1, blk, npair, st));
+    LRTEI_TRY(bu_rows(plan, f, r0, r1, blk, ldu, st));
     PairTable sub = plan->t;
     sub.pair_mu += r0;
     sub.pair_nu += r0;
     sub.npair = r1 - r0;
     {
       ProfScope ps("expand_B", st);
-      launch_expand_B(sub, nbf, blk, npair, 1.0, d_B, ld, plan->d_status, st);
+      launch_expand_B(sub, nbf, npair, blk, ldu, d_B, ld, plan->d_status, st);
     }
     LRTEI_TRY(finish_launch("expand_B"));
   }

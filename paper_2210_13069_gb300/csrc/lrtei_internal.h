@@ -226,10 +226,10 @@ int launch_jx(const PairTable& t, int nbf, int64_t n3, int R, int nsplit, const 
               double* d_part, cudaStream_t st);
 void launch_jy(const PairTable& t, int nbf, int64_t n3, int R, const double* d_F, const double* d_Y, double scale,
                double* d_J, int* d_status, cudaStream_t st);
-// Expand the unique-pair square B_u (npair x npair, ld) into full B (N_b^2 x N_b^2, ldB), times scale.
+// Expand rows of the unique-pair square B_u (t.npair rows of npair, ld) into full B (N_b^2 x N_b^2, ldB).
 // The expansion and unpacking kernels latch kDevNonFinite into *d_status if they store a NaN or an
 // infinity (a warp vote per store loop; no extra memory traffic).
-void launch_expand_B(const PairTable& t, int nbf, const double* d_Bu, int64_t ldu, double scale, double* d_B,
+void launch_expand_B(const PairTable& t, int nbf, int64_t npair, const double* d_Bu, int64_t ldu, double* d_B,
                      int64_t ldB, int* d_status, cudaStream_t st);
 // Rows [R0, R1) of full B (R = a N_b + b) from complete rows of B_u: out row R - R0 (ldo) is
 // row pair(min(a, b), max(a, b)) of B_u gathered over the columns (ka, la).
