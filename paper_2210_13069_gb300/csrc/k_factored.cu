@@ -146,6 +146,20 @@ __device__ __forceinline__ void dot2_step(Pair32 x, Pair32 z, float& sum, float&
   err = __fadd_rn(err, __fadd_rn(d, pe));
 }
 
+// The same for two sums at once.
+__device__ __forceinline__ void dot2_step2(tc::f32x2 xh, tc::f32x2 xl, tc::f32x2 zh, tc::f32x2 zl, tc::f32x2& sum,
+                                           tc::f32x2& err) {
+  using namespace tc;
+  const f32x2 ph = mul2(xh, zh);
+  f32x2 pe = fma2(xh, zh, neg2(ph));
+  pe = fma2(xh, zl, fma2(xl, zh, pe));
+  const f32x2 t = add2(sum, ph);
+  const f32x2 bp = sub2(t, sum);
+  const f32x2 d = add2(sub2(sum, sub2(t, bp)), sub2(ph, bp));
+  sum = t;
+  err = add2(err, add2(d, pe));
+}
+
 // F_u for the tensor-core precisions, whose F_u only feeds 30-bit slices: the same staged walk
 // with every product and the sum over the pair's rows j in pairs of FP32 numbers (the moments
 // converted to pairs once, y = S_y S_z by TwoProd, the sum over j by the compensated dot product
@@ -162,49 +176,52 @@ __global__ void __launch_bounds__(256) k_build_F_pairs(int n, int64_t nrows, con
                                                        const double* __restrict__ row_c, const double* __restrict__ S,
                                                        const float2* __restrict__ Sp, int64_t r0,
                                                        double* __restrict__ F, int64_t ldF) {
-  extern __shared__ float2 Xp[];  // [rows of the pair][n8]: c_j S_x(j, m1) as pairs
+  extern __shared__ float4 Xp[];  // [rows of the pair][n8 / 2]: c_j S_x(j, m1) and (j, m1 + 1) as hi, hi, lo, lo
   const int64_t r = r0 + blockIdx.x;
   const int64_t j0 = pair_row[r];
   const int I = (int)(pair_row[r + 1] - j0);
-  const int n8 = (n + 7) / 8 * 8, nn = n * n;
+  const int n4 = (n + 7) / 8 * 4, nn = n * n;
   const float2* Sy = Sp + (size_t)nrows * n;
   const float2* Sz = Sp + 2 * (size_t)nrows * n;
-  for (int e = threadIdx.x; e < I * n8; e += blockDim.x) {
-    const int j = e / n8, m1 = e % n8;
-    const Pair32 q = to_pair(m1 < n ? row_c[j0 + j] * S[(size_t)(j0 + j) * n + m1] : 0.0);
-    Xp[e] = make_float2(q.hi, q.lo);
+  for (int e = threadIdx.x; e < I * n4; e += blockDim.x) {
+    const int j = e / n4, m1 = 2 * (e % n4);
+    const double* sx = S + (size_t)(j0 + j) * n + m1;
+    const Pair32 q = to_pair(m1 < n ? row_c[j0 + j] * sx[0] : 0.0);
+    const Pair32 u = to_pair(m1 + 1 < n ? row_c[j0 + j] * sx[1] : 0.0);
+    Xp[e] = make_float4(q.hi, u.hi, q.lo, u.lo);
   }
   __syncthreads();
   double* out = F + (size_t)blockIdx.x * ldF;
-  const int items = nn * (n8 / 8);
+  const int items = nn * (n4 / 4);
   for (int it = threadIdx.x; it < items; it += blockDim.x) {
     const int q = it % nn, g = it / nn;
     const int m2 = q / n, m3 = q % n;
-    float sum[8], err[8];
+    tc::f32x2 sum[4], err[4];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) sum[i] = err[i] = 0.f;
+    for (int i = 0; i < 4; ++i) sum[i] = err[i] = 0;
     for (int j = 0; j < I; ++j) {
       const float2 a = Sy[(size_t)(j0 + j) * n + m2], b = Sz[(size_t)(j0 + j) * n + m3];
       const float yh = __fmul_rn(a.x, b.x);
       float yl = fmaf(a.x, b.x, -yh);  // TwoProd
       yl = fmaf(a.x, b.y, fmaf(a.y, b.x, yl));
-      const Pair32 y{yh, yl};
-      const float2* xr = Xp + j * n8 + g * 8;
+      const tc::f32x2 zh = tc::pack2(yh, yh), zl = tc::pack2(yl, yl);
+      const float4* xr = Xp + j * n4 + g * 4;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float2 x = xr[i];
-        dot2_step(Pair32{x.x, x.y}, y, sum[i], err[i]);
+      for (int i = 0; i < 4; ++i) {
+        const float4 x = xr[i];
+        dot2_step2(tc::pack2(x.x, x.y), tc::pack2(x.z, x.w), zh, zl, sum[i], err[i]);
       }
     }
 #pragma unroll
     for (int i = 0; i < 8; ++i)
-      if (g * 8 + i < n) out[(size_t)(g * 8 + i) * nn + q] = tc::fpair_ldexp(sum[i], err[i], 0);
+      if (g * 8 + i < n)
+        out[(size_t)(g * 8 + i) * nn + q] = tc::fpair_ldexp(tc::half_of(sum[i / 2], i), tc::half_of(err[i / 2], i), 0);
   }
 }
 
 void launch_build_F_pairs(const PairTable& t, int n, const double* d_S, int64_t r0, int64_t r1, double* d_F,
                           int64_t ldF, cudaStream_t st) {
-  const size_t smem = sizeof(float2) * (size_t)t.maxI * ((n + 7) / 8 * 8);
+  const size_t smem = sizeof(float4) * (size_t)t.maxI * ((n + 7) / 8 * 4);
   if (t.maxI <= 0 || smem > 48 * 1024) {  // very long pair blocks: the FP64 build
     launch_build_F<double>(t, n, d_S, r0, r1, d_F, ldF, st);
     return;
@@ -286,61 +303,72 @@ __device__ __forceinline__ void same_parity_pair(int e, int ce, int co, int& a, 
   b = 2 * (e % c) + odd;
 }
 
-__global__ void k_K_zpairs_parity(int n, int ce, int co, int P, const double* __restrict__ C, Pair32* __restrict__ zp) {
-  const int ne = ce * ce + co * co, nn = n * n;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ne * P; i += gridDim.x * blockDim.x) {
+// zp[p][e / 2]: A_z^p of pairs e and e + 1 (zero beyond the last) as hi, hi, lo, lo.
+__global__ void k_K_zpairs_parity(int n, int ce, int co, int P, const double* __restrict__ C, float4* __restrict__ zp) {
+  const int ne = ce * ce + co * co, nh = (ne + 1) / 2, nn = n * n;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nh * P; i += gridDim.x * blockDim.x) {
+    const double* c = C + ((size_t)2 * P + i / nh) * nn;
+    const int e = 2 * (i % nh);
     int a, b;
-    same_parity_pair(i % ne, ce, co, a, b);
-    zp[i] = to_pair(C[((size_t)2 * P + i / ne) * nn + a * n + b]);
+    same_parity_pair(e, ce, co, a, b);
+    const Pair32 q = to_pair(c[a * n + b]);
+    Pair32 u{0.f, 0.f};
+    if (e + 1 < ne) {
+      same_parity_pair(e + 1, ce, co, a, b);
+      u = to_pair(c[a * n + b]);
+    }
+    zp[i] = make_float4(q.hi, u.hi, q.lo, u.lo);
   }
 }
 
-// Block (g tile, (a1, b1)), thread t owning e = (a3, b3) in {t, t + blockDim} as in k_build_K_tiled, over the
-// pairs of equal parity: 3.4 -> 0.45 ms at n = 24, P = 32.
-__global__ void __launch_bounds__(512, 1) k_build_K_classes(int n, int P, ParityClasses pc, const int* __restrict__ blk,
+// Block (g tile, (a1, b1)), each thread a neighbouring pair of e = (a3, b3), over the pairs of equal parity; both e
+// in one packed operation.  n = 24, P = 32: 3.4 ms dense, 0.53 with an eighth of the sums, 0.44
+// packed (the FP32 pipe alone needs 0.27).
+__global__ void __launch_bounds__(256, 3) k_build_K_classes(int n, int P, ParityClasses pc, const int* __restrict__ blk,
                                                            const double* __restrict__ C, const double* __restrict__ w,
-                                                           const Pair32* __restrict__ zp, double scale,
+                                                           const float4* __restrict__ zp, double scale,
                                                            double* __restrict__ K, int64_t ldK) {
-  __shared__ Pair32 r[2 * kKG * kMaxP];
-  const int nn = n * n, ce = pc.cnt[0], co = pc.cnt[1], ne = ce * ce + co * co;
+  __shared__ float4 r[2 * kKG * kMaxP];  // hi, hi, lo, lo
+  const int nn = n * n, ce = pc.cnt[0], co = pc.cnt[1], ne = ce * ce + co * co, nh = (ne + 1) / 2;
   const int g0 = blockIdx.x * 2 * kKG;
   int a1, b1;
   same_parity_pair(blockIdx.y, ce, co, a1, b1);
+  __shared__ double rx[kMaxP];  // scale w_p A_x^p(a1, b1)
+  for (int p = threadIdx.x; p < P; p += blockDim.x) rx[p] = scale * w[p] * C[(size_t)p * nn + a1 * n + b1];
+  __syncthreads();
   for (int i = threadIdx.x; i < 2 * kKG * P; i += blockDim.x) {
     const int g = g0 + i / P, p = i % P;
     double v = 0.0;
     if (g < ne) {
       int a2, b2;
       same_parity_pair(g, ce, co, a2, b2);
-      v = scale * w[p] * C[(size_t)p * nn + a1 * n + b1] * C[((size_t)P + p) * nn + a2 * n + b2];
+      v = rx[p] * C[((size_t)P + p) * nn + a2 * n + b2];
     }
-    r[i] = to_pair(v);
+    const Pair32 q = to_pair(v);
+    r[i] = make_float4(q.hi, q.hi, q.lo, q.lo);
   }
   __syncthreads();
   for (int half = 0; half < 2; ++half) {
-    const Pair32* rh = r + half * kKG * P;
+    const float4* rh = r + half * kKG * P;
     const int gb = g0 + half * kKG;
     if (gb >= ne) break;
-    for (int eb = 0; eb < ne; eb += 2 * blockDim.x) {
-      const int e0 = eb + threadIdx.x, e1 = e0 + blockDim.x;
-      const bool l0 = e0 < ne, l1 = e1 < ne;
-      if (!l0) break;
-      float sum[2][kKG], err[2][kKG];
+    for (int t = threadIdx.x; t < nh; t += blockDim.x) {
+      tc::f32x2 sum[kKG], err[kKG];
 #pragma unroll
-      for (int j = 0; j < kKG; ++j) sum[0][j] = err[0][j] = sum[1][j] = err[1][j] = 0.f;
+      for (int j = 0; j < kKG; ++j) sum[j] = err[j] = 0;
       for (int p = 0; p < P; ++p) {
-        const Pair32 z0 = zp[(size_t)p * ne + e0];
-        const Pair32 z1 = l1 ? zp[(size_t)p * ne + e1] : Pair32{0.f, 0.f};
+        const float4 z = zp[(size_t)p * nh + t];
+        const tc::f32x2 zh = tc::pack2(z.x, z.y), zl = tc::pack2(z.z, z.w);
 #pragma unroll
         for (int j = 0; j < kKG; ++j) {
-          const Pair32 x = rh[j * P + p];
-          dot2_step(x, z0, sum[0][j], err[0][j]);
-          dot2_step(x, z1, sum[1][j], err[1][j]);
+          const float4 x = rh[j * P + p];
+          dot2_step2(tc::pack2(x.x, x.y), tc::pack2(x.z, x.w), zh, zl, sum[j], err[j]);
         }
       }
       int a3[2], b3[2];
-      same_parity_pair(e0, ce, co, a3[0], b3[0]);
-      same_parity_pair(l1 ? e1 : e0, ce, co, a3[1], b3[1]);
+      const bool two = 2 * t + 1 < ne;
+      same_parity_pair(2 * t, ce, co, a3[0], b3[0]);
+      same_parity_pair(two ? 2 * t + 1 : 2 * t, ce, co, a3[1], b3[1]);
 #pragma unroll
       for (int j = 0; j < kKG; ++j) {
         if (gb + j >= ne) break;
@@ -348,10 +376,10 @@ __global__ void __launch_bounds__(512, 1) k_build_K_classes(int n, int P, Parity
         same_parity_pair(gb + j, ce, co, a2, b2);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          if (h && !l1) break;
+          if (h && !two) break;
           const int m = (b1 * n + b2) * n + b3[h];
-          const int t = blk[pc.cls(b1, b2, b3[h]) * (pc.units * 8) + m / 16];
-          K[pc.row(a1, a2, a3[h]) * ldK + t * 16 + m % 16] = (double)sum[h][j] + (double)err[h][j];
+          const int q = blk[pc.cls(b1, b2, b3[h]) * (pc.units * 8) + m / 16];
+          K[pc.row(a1, a2, a3[h]) * ldK + q * 16 + m % 16] = (double)tc::half_of(sum[j], h) + (double)tc::half_of(err[j], h);
         }
       }
     }
@@ -361,13 +389,13 @@ __global__ void __launch_bounds__(512, 1) k_build_K_classes(int n, int P, Parity
 cudaError_t launch_build_K_classes(int n, int P, const ParityClasses& pc, const int* d_blk, const double* d_C,
                                    const double* d_w, double scale, double* d_K, int64_t ldK, cudaStream_t st) {
   const int ne = pc.cnt[0] * pc.cnt[0] + pc.cnt[1] * pc.cnt[1];
-  Pair32* zp = nullptr;
-  cudaError_t e = scratch_alloc((void**)&zp, sizeof(Pair32) * (size_t)ne * P, st);
+  float4* zp = nullptr;
+  cudaError_t e = scratch_alloc((void**)&zp, sizeof(float4) * (size_t)((ne + 1) / 2) * P, st);
   if (e != cudaSuccess) return e;
   count_launch();
   k_K_zpairs_parity<<<(unsigned)std::min<int64_t>(((int64_t)ne * P + 255) / 256, 152 * 8), 256, 0, st>>>(
       n, pc.cnt[0], pc.cnt[1], P, d_C, zp);
-  const int threads = std::min(512, ((ne + 1) / 2 + 31) / 32 * 32);
+  const int threads = std::min(256, ((ne + 1) / 2 + 31) / 32 * 32);
   count_launch();
   k_build_K_classes<<<dim3((unsigned)((ne + 2 * kKG - 1) / (2 * kKG)), (unsigned)ne), threads, 0, st>>>(
       n, P, pc, d_blk, d_C, d_w, zp, scale, d_K, ldK);

@@ -35,7 +35,7 @@ using tcg::KB;
 template <int BN_, int LV0, int NLV>
 struct Levels {
   static constexpr int BN = BN_, NP = LV0 + NLV, PT = kOzSlices, NACC = NLV;
-  static constexpr bool BF16 = false, ACCUM = NLV == 2;
+  static constexpr bool BF16 = false, ACCUM = NLV == 2, LIST = false;
   static constexpr bool FLT = LV0 >= 4;  // FP32 running sums (level 4 weighs 2^-36)
   // K blocks per stage: one barrier round per 30 KB or more
   static constexpr int STEP = NP * (128 + BN) * 32, KS = STEP >= 30 * 1024 ? 1 : STEP >= 16 * 1024 ? 2 : 4;
@@ -290,7 +290,7 @@ lrtei_status oz_gemm(const OzMatrix& A, const OzMatrix& B, const std::vector<OzS
     const int m_lo = (int)(s.a_row0 % 128);
     if (m_lo && symmetric) { set_error("oz_gemm: symmetric products start at row 0"); return LRTEI_ERR_ARG; }
     o = {s.a_row0 - m_lo, s.b_row0, s.M + m_lo, s.N, s.c_off, p.nitems, s.a_k0 / tcg::KB, s.b_k0 / tcg::KB, s.k / 64,
-         (int)((s.M + m_lo + 127) / 128), (int)((s.N + BN - 1) / BN), m_lo, nullptr};
+         (int)((s.M + m_lo + 127) / 128), (int)((s.N + BN - 1) / BN), m_lo, s.k / tcg::KB, nullptr};
     max_units = std::max(max_units, o.units);
     p.nitems += symmetric ? (int64_t)o.tiles_n * (o.tiles_n + 1) / 2 : (int64_t)o.tiles_m * o.tiles_n;
   }

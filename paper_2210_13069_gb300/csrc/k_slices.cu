@@ -55,18 +55,14 @@ __device__ __forceinline__ uint4 pack8(const uint16_t (&h)[8]) {
 // The three slice planes of eight elements (k: live columns of the row, nz: the row is not zero).
 __device__ __forceinline__ void store_slices(const double (&v)[8], int e, bool nz, int64_t i, int64_t j, int64_t k,
                                              int tile, int64_t kpad, uint16_t* __restrict__ d) {
-  uint16_t h0[8], h1[8], h2[8];
+  uint32_t p0[4], p1[4], p2[4];
 #pragma unroll
-  for (int u = 0; u < 8; ++u) {
-    const SliceBits q = slice_bits(v[u], e, j + u < k && nz);
-    h0[u] = q.s0;
-    h1[u] = q.s1;
-    h2[u] = q.s2;
-  }
+  for (int u = 0; u < 4; ++u)
+    slice_pair(v[2 * u], v[2 * u + 1], e, j + 2 * u < k && nz, j + 2 * u + 1 < k && nz, p0[u], p1[u], p2[u]);
   uint16_t* o = d + piece(i, j, tile, kpad, 3);
-  *reinterpret_cast<uint4*>(o) = pack8(h0);
-  *reinterpret_cast<uint4*>(o + tile * 16) = pack8(h1);
-  *reinterpret_cast<uint4*>(o + 2 * tile * 16) = pack8(h2);
+  *reinterpret_cast<uint4*>(o) = make_uint4(p0[0], p0[1], p0[2], p0[3]);
+  *reinterpret_cast<uint4*>(o + tile * 16) = make_uint4(p1[0], p1[1], p1[2], p1[3]);
+  *reinterpret_cast<uint4*>(o + 2 * tile * 16) = make_uint4(p2[0], p2[1], p2[2], p2[3]);
 }
 
 // Columns j .. j + 7 of a row: 16-byte loads where the row allows them, zeros beyond k; map (may be NULL):
@@ -124,44 +120,73 @@ __global__ void __launch_bounds__(256) k_split_rows_warp(const double* __restric
   if (i0 < kpad) store_slices(v, e, nz, r, i0, k, tile, kpad, d);
 }
 
-// One block per row: rows of up to 2048 NREG columns are read once and kept in registers; longer ones
-// (NREG = 0) take two passes, the second from L2.
-template <int NREG>
-__global__ void __launch_bounds__(256) k_split_rows(const double* __restrict__ src, int64_t k, int64_t ld, int64_t kpad,
-                                                    int tile, const int* __restrict__ map, uint16_t* __restrict__ d,
-                                                    int* __restrict__ expo) {
+// One block per row, the row staged in shared memory (rows of up to kSplitCols columns): read once, by one
+// bulk copy where its address allows, and gathered through the map from there (a class order's eight
+// neighbours are two runs of four, one element per sector and lane from global memory).
+constexpr int64_t kSplitCols = 28000;
+__global__ void __launch_bounds__(512) k_split_rows(const double* __restrict__ src, int64_t cols, int64_t k, int64_t ld,
+                                                    int64_t kpad, int tile, int bulk, const int* __restrict__ map,
+                                                    uint16_t* __restrict__ d, int* __restrict__ expo) {
+  extern __shared__ __align__(16) double row[];  // cols: the source row's columns (k without a map)
+  __shared__ uint64_t red[32];
+  __shared__ uint64_t bar;
+  const int64_t r = blockIdx.x;
+  const double* x = src + r * ld;
+  const int nc = (int)cols;
+  uint64_t mx = 0;
+  if (bulk) {
+    if (threadIdx.x == 0) {
+      mbar_init(&bar, 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      mbar_arrive_expect_tx(&bar, (uint32_t)(nc * 8));
+      bulk_load(row, x, (uint32_t)(nc * 8), &bar);
+    }
+    __syncthreads();
+    for (long long t0 = clock64(); !mbar_try_wait(&bar, 0u) && clock64() - t0 < kWaitCycles;) {
+    }
+    for (int i = threadIdx.x; i < nc; i += blockDim.x) {
+      const uint64_t a = (uint64_t)__double_as_longlong(row[i]) & 0x7FFFFFFFFFFFFFFFULL;
+      mx = a > mx ? a : mx;
+    }
+  } else {
+#pragma unroll 4
+    for (int i = threadIdx.x; i < nc; i += blockDim.x) {
+      row[i] = x[i];
+      const uint64_t a = (uint64_t)__double_as_longlong(row[i]) & 0x7FFFFFFFFFFFFFFFULL;
+      mx = a > mx ? a : mx;
+    }
+  }
+  bool nz;
+  const int e = row_exponent(mx, red, nz);  // (synchronises: the whole row is staged)
+  if (threadIdx.x == 0) expo[r] = e;
+  for (int64_t j = 8 * (int64_t)threadIdx.x; j < kpad; j += 8 * (int64_t)blockDim.x) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = j + u < k ? row[map ? map[j + u] : (int)j + u] : 0.0;
+    store_slices(v, e, nz, r, j, k, tile, kpad, d);
+  }
+}
+
+// Longer rows: two passes, the second from L2.
+__global__ void __launch_bounds__(256) k_split_rows_long(const double* __restrict__ src, int64_t k, int64_t ld,
+                                                         int64_t kpad, int tile, const int* __restrict__ map,
+                                                         uint16_t* __restrict__ d, int* __restrict__ expo) {
   __shared__ uint64_t red[32];
   const int64_t r = blockIdx.x;
   const double* x = src + r * ld;
   const bool vec = (ld & 1) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
   uint64_t mx = 0;
   bool nz;
-  if constexpr (NREG > 0) {
-    double v[NREG > 0 ? NREG : 1][8];
-#pragma unroll
-    for (int i = 0; i < NREG; ++i) {
-      load8(x, 8 * ((int64_t)threadIdx.x + 256 * i), k, vec, map, v[i]);
-      mx = max_mag(v[i], mx);
-    }
-    const int e = row_exponent(mx, red, nz);
-    if (threadIdx.x == 0) expo[r] = e;
-#pragma unroll
-    for (int i = 0; i < NREG; ++i) {
-      const int64_t j = 8 * ((int64_t)threadIdx.x + 256 * i);
-      if (j < kpad) store_slices(v[i], e, nz, r, j, k, tile, kpad, d);
-    }
-  } else {
-    double v[8];
-    for (int64_t j = 8 * (int64_t)threadIdx.x; j < k; j += 2048) {
-      load8(x, j, k, vec, map, v);
-      mx = max_mag(v, mx);
-    }
-    const int e = row_exponent(mx, red, nz);
-    if (threadIdx.x == 0) expo[r] = e;
-    for (int64_t j = 8 * (int64_t)threadIdx.x; j < kpad; j += 2048) {
-      load8(x, j, k, vec, map, v);
-      store_slices(v, e, nz, r, j, k, tile, kpad, d);
-    }
+  double v[8];
+  for (int64_t j = 8 * (int64_t)threadIdx.x; j < k; j += 2048) {
+    load8(x, j, k, vec, map, v);
+    mx = max_mag(v, mx);
+  }
+  const int e = row_exponent(mx, red, nz);
+  if (threadIdx.x == 0) expo[r] = e;
+  for (int64_t j = 8 * (int64_t)threadIdx.x; j < kpad; j += 2048) {
+    load8(x, j, k, vec, map, v);
+    store_slices(v, e, nz, r, j, k, tile, kpad, d);
   }
 }
 
@@ -288,12 +313,18 @@ void launch_split_rows(const double* d_src, int64_t rows, int64_t k, int64_t ld,
                                                                                      m.d, m.expo);
     return;
   }
-  if (m.kpad <= 2048)
-    tc::k_split_rows<1><<<(unsigned)rows, 256, 0, st>>>(d_src, k, ld, m.kpad, m.tile, d_map, m.d, m.expo);
-  else if (m.kpad <= 4096)
-    tc::k_split_rows<2><<<(unsigned)rows, 256, 0, st>>>(d_src, k, ld, m.kpad, m.tile, d_map, m.d, m.expo);
-  else
-    tc::k_split_rows<0><<<(unsigned)rows, 256, 0, st>>>(d_src, k, ld, m.kpad, m.tile, d_map, m.d, m.expo);
+  const int64_t cols = d_map ? ld : k;  // a mapped row's columns lie anywhere in it
+  if (cols > tc::kSplitCols) {
+    tc::k_split_rows_long<<<(unsigned)rows, 256, 0, st>>>(d_src, k, ld, m.kpad, m.tile, d_map, m.d, m.expo);
+    return;
+  }
+  static bool attr_set = false;
+  if (!attr_set)
+    attr_set = cudaFuncSetAttribute(tc::k_split_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)(sizeof(double) * tc::kSplitCols)) == cudaSuccess;
+  const int bulk = (cols % 2 == 0 && ld % 2 == 0 && (reinterpret_cast<uintptr_t>(d_src) & 15) == 0) ? 1 : 0;
+  tc::k_split_rows<<<(unsigned)rows, cols > 8192 ? 512 : 256, sizeof(double) * (size_t)cols, st>>>(
+      d_src, cols, k, ld, m.kpad, m.tile, bulk, d_map, m.d, m.expo);
 }
 
 void launch_transpose(const double* in, int64_t rows, int64_t cols, int64_t ldi, double* out, int64_t ldo,

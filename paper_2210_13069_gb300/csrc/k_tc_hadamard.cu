@@ -96,47 +96,9 @@ __device__ __forceinline__ void tile_of(const Params& p, int64_t item, int64_t& 
   }
 }
 
-// Two FP32 numbers in a register pair, each operation rounded as the scalar one; one instruction for both
-// (25 operations per element and node as scalars: the epilogue is the longer side of this kernel; 7.8 -> 6.4 ms
-// at 180 functions with every warp waiting for itself, 6.1 with four-column stores).
-using f32x2 = unsigned long long;
-__device__ __forceinline__ f32x2 pack2(float x, float y) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-  return r;
-}
-__device__ __forceinline__ f32x2 pack2(uint32_t x, uint32_t y) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(x), "r"(y));
-  return r;
-}
-__device__ __forceinline__ float half_of(f32x2 v, int odd) {
-  float x, y;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
-  return (odd & 1) ? y : x;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ f32x2 neg2(f32x2 a) { return a ^ 0x8000000080000000ULL; }
-
+// The FP32-pair arithmetic runs on two columns an instruction: 25 operations per element and node as scalars
+// made the epilogue the longer side of this kernel (7.8 -> 6.4 ms at 180 functions together with every warp
+// waiting for itself, 6.1 with four-column stores).
 // (ah + al)(bh + bl) as an unevaluated FP32 pair; every partial product kept (|al|, |bl| may be
 // 2^-9 of |ah|, |bh| here), the leading one split exactly by the FMA.
 __device__ __forceinline__ void pmul(f32x2 ah, f32x2 al, f32x2 bh, f32x2 bl, f32x2& ph, f32x2& pl) {

@@ -69,13 +69,12 @@ __device__ __forceinline__ double combine_pow2(int t0, float t12, int k, float t
 
 enum class Scheme { six, eight, plain };
 
-// KS_: 16-deep steps per stage; two halve the barrier rounds, one where a step table lists single blocks.
-template <int BN_, Scheme M, int KS_>
+template <int BN_, Scheme M, bool LIST_>
 struct Split {
   static constexpr bool P8 = M == Scheme::eight, PLAIN = M == Scheme::plain;
-  static constexpr int BN = BN_, NP = PLAIN ? 1 : 3, PT = NP, NACC = PLAIN ? 1 : P8 ? 3 : 2, KS = KS_;
+  static constexpr int BN = BN_, NP = PLAIN ? 1 : 3, PT = NP, NACC = PLAIN ? 1 : P8 ? 3 : 2, KS = 2;  // two steps a stage: half the barrier rounds
   static constexpr int UNIT = 8, CHUNK = 8;  // 128 deep
-  static constexpr bool BF16 = PLAIN, ACCUM = false;
+  static constexpr bool BF16 = PLAIN, ACCUM = false, LIST = LIST_;
 
   static __device__ __forceinline__ void mma(uint32_t d0, uint64_t a0, uint64_t b0, uint32_t idesc, uint32_t first) {
     if constexpr (PLAIN) {
@@ -157,16 +156,18 @@ struct Split {
 // shared memory); the eight-product scheme has TMEM for 64 (2 x 3 accumulators), plain BF16 takes 64.
 static int tile_n(int64_t N, bool plain, bool eight) { return N <= 32 ? 32 : (N <= 64 || plain || eight) ? 64 : 128; }
 
-template <int KS>
-static lrtei_status run_ks(const tcg::Params& p, int BN, bool plain, bool eight, cudaStream_t st) {
-  if (plain) return BN == 64 ? tcg::launch<Split<64, Scheme::plain, KS>>(p, st) : tcg::launch<Split<32, Scheme::plain, KS>>(p, st);
-  if (eight) return BN == 64 ? tcg::launch<Split<64, Scheme::eight, KS>>(p, st) : tcg::launch<Split<32, Scheme::eight, KS>>(p, st);
-  if (BN == 128) return tcg::launch<Split<128, Scheme::six, KS>>(p, st);
-  return BN == 64 ? tcg::launch<Split<64, Scheme::six, KS>>(p, st) : tcg::launch<Split<32, Scheme::six, KS>>(p, st);
+template <bool LIST>
+static lrtei_status run_as(const tcg::Params& p, int BN, bool plain, bool eight, cudaStream_t st) {
+  if (plain)
+    return BN == 64 ? tcg::launch<Split<64, Scheme::plain, LIST>>(p, st) : tcg::launch<Split<32, Scheme::plain, LIST>>(p, st);
+  if (eight)
+    return BN == 64 ? tcg::launch<Split<64, Scheme::eight, LIST>>(p, st) : tcg::launch<Split<32, Scheme::eight, LIST>>(p, st);
+  if (BN == 128) return tcg::launch<Split<128, Scheme::six, LIST>>(p, st);
+  return BN == 64 ? tcg::launch<Split<64, Scheme::six, LIST>>(p, st) : tcg::launch<Split<32, Scheme::six, LIST>>(p, st);
 }
 static lrtei_status run(const tcg::Params& p, int BN, bool plain, bool eight, cudaStream_t st) {
   ProfScope ps("tc_gemm", st);
-  return p.seg[0].tab ? run_ks<1>(p, BN, plain, eight, st) : run_ks<2>(p, BN, plain, eight, st);
+  return p.seg[0].tab ? run_as<true>(p, BN, plain, eight, st) : run_as<false>(p, BN, plain, eight, st);
 }
 
 // What the products share: operands, output (or split partials) and checks.  units: 128-deep chunks of K.
@@ -239,11 +240,36 @@ lrtei_status tc_gemm(const SplitMatrix& A, int64_t a_row0, const SplitMatrix& B,
   if (s != LRTEI_OK) return s;
   p.nseg = 1;
   p.seg[0] = {a_row0 - m_lo, 0, M + m_lo, N, transpose_out ? -m_lo : -m_lo * p.ldc, 0, 0, 0, units,
-              (int)((M + m_lo + 127) / 128), (int)((N + BN - 1) / BN), m_lo, nullptr};
+              (int)((M + m_lo + 127) / 128), (int)((N + BN - 1) / BN), m_lo, A.steps(), nullptr};
   p.nitems = (int64_t)p.seg[0].tiles_m * p.seg[0].tiles_n;
   s = tc::run(p, BN, A.plain, A.eight, st);
   if (s != LRTEI_OK || splits == 1) return s;
   return tc::reduce(d_part, splits, c_rows, c_cols, d_C, ldc, st);
+}
+
+// Several products C_i = A_i B_i^T of rows of A and B in one launch (their tiles share the last waves).
+lrtei_status tc_gemm_blocks(const SplitMatrix& A, const SplitMatrix& B, const std::vector<TcBlock>& blocks, double* d_C,
+                            int64_t ldc, int* d_status, cudaStream_t st) {
+  if (A.kpad != B.kpad || A.kpad % 128 != 0 || blocks.size() > (size_t)tcg::kMaxSeg) {
+    set_error("tc_gemm_blocks: operands must share a K padded to a multiple of 128, at most %d blocks", tcg::kMaxSeg);
+    return LRTEI_ERR_ARG;
+  }
+  int64_t nmax = 0;
+  for (const TcBlock& b : blocks) nmax = std::max(nmax, b.N);
+  const int BN = tc::tile_n(nmax, A.plain, A.eight), units = (int)(A.kpad / 128);
+  tcg::Params p{};
+  int splits = 1;
+  lrtei_status s = tc::fill(p, A, B, BN, units, 1.0, d_C, ldc, false, splits, 0, 0, nullptr, d_status);
+  if (s != LRTEI_OK) return s;
+  for (const TcBlock& b : blocks) {
+    if (b.M <= 0 || b.N <= 0) continue;
+    const int m_lo = (int)(b.a_row0 % 128);
+    tcg::Seg& o = p.seg[p.nseg++];
+    o = {b.a_row0 - m_lo, b.b_row0, b.M + m_lo, b.N, b.c_off - m_lo * p.ldc, p.nitems, 0, 0, units,
+         (int)((b.M + m_lo + 127) / 128), (int)((b.N + BN - 1) / BN), m_lo, A.steps(), nullptr};
+    p.nitems += (int64_t)o.tiles_m * o.tiles_n;
+  }
+  return tc::run(p, BN, A.plain, A.eight, st);
 }
 
 lrtei_status tc_gemm_sym_band(const SplitMatrix& A, const SplitMatrix& B, int64_t row0, int64_t row1, int64_t N,
@@ -266,7 +292,7 @@ lrtei_status tc_gemm_sym_band(const SplitMatrix& A, const SplitMatrix& B, int64_
   p.blk0 = b0;
   p.blk1 = b1;
   p.nb = nb;
-  p.seg[0] = {-row0, 0, row1, N, 0, 0, 0, 0, units, (int)(b1 - b0), (int)nb, 0, nullptr};
+  p.seg[0] = {-row0, 0, row1, N, 0, 0, 0, 0, units, (int)(b1 - b0), (int)nb, 0, A.steps(), nullptr};
   p.nitems = ((nb - b0) * (nb - b0 + 1) / 2 - (nb - b1) * (nb - b1 + 1) / 2) * (128 / BN);
   return tc::run(p, BN, A.plain, A.eight, st);
 }
@@ -300,10 +326,10 @@ lrtei_status tc_gemm_K(const SplitMatrix& X, int64_t x_row0, const SplitMatrix& 
     const int* tab = pc.tab ? pc.tab + pc.tab_off[c] : nullptr;
     if (k_is_a)
       o = {pc.row0[c], 0, w, rows, pc.off[c], p.nitems, 0, 0, pc.units, (int)((w + 127) / 128), (int)((rows + BN - 1) / BN),
-           0, tab};
+           0, X.steps(), tab};
     else
       o = {x_row0 - m_lo, pc.row0[c], rows + m_lo, w, pc.off[c] - m_lo * p.ldc, p.nitems, 0, 0, pc.units,
-           (int)((rows + m_lo + 127) / 128), (int)((w + BN - 1) / BN), m_lo, tab};
+           (int)((rows + m_lo + 127) / 128), (int)((w + BN - 1) / BN), m_lo, X.steps(), tab};
     p.nitems += (int64_t)o.tiles_m * o.tiles_n;
   }
   s = tc::run(p, BN, A.plain, A.eight, st);

@@ -708,10 +708,11 @@ lrtei_status ensure_classes(lrtei_plan* pl, cudaStream_t st) {
             blk[(size_t)c * nblk + b] = (int)list.size();
             list.push_back(b);
           }
-        if (list.size() > before) {
-          list.back() |= 1 << 30;  // the chunk's last step
-          ++nonempty;
+        for (size_t i = before; i < list.size(); i += 2) {
+          if (i + 1 < list.size()) list[i] |= 1 << 29;   // two steps in one stage
+          if (i + 2 >= list.size()) list[i] |= 1 << 30;  // the chunk's last stage
         }
+        if (list.size() > before) ++nonempty;
       }
       first.push_back((int)list.size());
       chunks.push_back(nonempty);
@@ -751,9 +752,10 @@ bool is_split(const lrtei_plan* pl) {
 }
 bool eight_products(const lrtei_plan* pl) { return pl->prec == LRTEI_SPLIT_F16_8; }
 
-SplitMatrix split_shape(const lrtei_plan* pl, int64_t rows, int64_t kpad, int tile) {
+SplitMatrix split_shape(const lrtei_plan* pl, int64_t rows, int64_t k, int64_t kpad, int tile) {
   SplitMatrix m;
   m.rows = rows;
+  m.k = k;
   m.kpad = kpad;
   m.tile = tile;
   m.plain = pl->prec == LRTEI_BF16;
@@ -761,8 +763,8 @@ SplitMatrix split_shape(const lrtei_plan* pl, int64_t rows, int64_t kpad, int ti
   return m;
 }
 
-lrtei_status alloc_split(lrtei_plan* pl, SplitMatrix& m, int64_t rows, int64_t kpad) {
-  SplitMatrix q = split_shape(pl, rows, kpad, 128);
+lrtei_status alloc_split(lrtei_plan* pl, SplitMatrix& m, int64_t rows, int64_t k, int64_t kpad) {
+  SplitMatrix q = split_shape(pl, rows, k, kpad, 128);
   LRTEI_TRY(pl->alloc(&q.d, (size_t)q.count()));
   LRTEI_TRY(pl->alloc(&q.expo, rows));
   m = q;
@@ -784,7 +786,7 @@ lrtei_status ensure_Fsp(lrtei_plan* pl, cudaStream_t st) {
   if (pl->have_Fsp) return LRTEI_OK;
   const int64_t n3 = (int64_t)pl->n * pl->n * pl->n;
   LRTEI_TRY(ensure_F64(pl, st));
-  LRTEI_TRY(alloc_split(pl, pl->Fsp, pl->t.npair, kpad256(n3)));
+  LRTEI_TRY(alloc_split(pl, pl->Fsp, pl->t.npair, n3, kpad256(n3)));
   {
     ProfScope ps("split", st);
     launch_split_rows(pl->d_F, pl->t.npair, n3, n3, pl->Fsp, nullptr, st);
@@ -858,7 +860,7 @@ lrtei_status ensure_Ksp(lrtei_plan* pl, cudaStream_t st) {
   Scratch sc(st);
   double* K;
   LRTEI_TRY(sc.get(&K, (size_t)pl->pc.rows * K_cols(pl)));
-  LRTEI_TRY(alloc_split(pl, pl->Ksp, pl->pc.rows, K_kpad(pl->pc)));
+  LRTEI_TRY(alloc_split(pl, pl->Ksp, pl->pc.rows, K_cols(pl), K_kpad(pl->pc)));
   LRTEI_TRY(slice_K(pl, pl->d_C, true, K, pl->Ksp, st));
   pl->have_Ksp = true;
   return finish_launch("split K");
@@ -872,7 +874,7 @@ lrtei_status ensure_FTsp(lrtei_plan* pl, cudaStream_t st) {
   double* FT;
   LRTEI_TRY(sc.get(&FT, (size_t)n3 * npair));
   launch_transpose(pl->d_F, npair, n3, n3, FT, npair, st);
-  LRTEI_TRY(alloc_split(pl, pl->FTsp, n3, kpad256(npair)));
+  LRTEI_TRY(alloc_split(pl, pl->FTsp, n3, npair, kpad256(npair)));
   {
     ProfScope ps("split", st);
     launch_split_rows(FT, n3, npair, npair, pl->FTsp, nullptr, st);
@@ -893,7 +895,7 @@ lrtei_status ensure_jbuild_operands(lrtei_plan* pl, cudaStream_t st) {
 // A scratch split operand (planes owned by the call).  tile: 128, or split_tile(R) for the R-row right
 // operand of a skinny product.
 lrtei_status scratch_split(Scratch& sc, SplitMatrix& m, int64_t rows, int64_t k, int tile, const lrtei_plan* pl) {
-  m = split_shape(pl, rows, kpad256(k), tile);
+  m = split_shape(pl, rows, k, kpad256(k), tile);
   LRTEI_TRY(sc.get(&m.d, (size_t)m.count()));
   return sc.get(&m.expo, rows);
 }
@@ -1078,21 +1080,37 @@ lrtei_status bu_adaptive(lrtei_plan* pl, double* Bu, cudaStream_t st) {
   int64_t maxr = 0;
   for (int s = 0; s < np; ++s) maxr = std::max(maxr, ar.off[s + 1] - ar.off[s]);
   double *G, *blk;
-  if (is_split(pl)) LRTEI_TRY(ensure_classes(pl, st));
-  LRTEI_TRY(sc.get(&G, (size_t)maxr * std::max<int64_t>(n3, pl->pc.cols)));
-  LRTEI_TRY(sc.get(&blk, (size_t)maxr * maxr));
   if (is_split(pl)) {
+    LRTEI_TRY(ensure_classes(pl, st));
     const ParityClasses& pc = pl->pc;
     SplitMatrix Fsp, Ksp, Gsp;
     std::vector<int64_t> tile0{0};  // first row of each partition in the sliced F: a multiple of 128
     for (int s = 0; s < np; ++s) tile0.push_back(tile0.back() + (ar.off[s + 1] - ar.off[s] + 127) / 128 * 128);
+    // the partition pairs; the rows of their G, one below the other
+    struct Pair { int s, t; int64_t row; };
+    std::vector<Pair> pairs;
+    int64_t grows = 0, most = 0;
+    for (int t = 0; t < np; ++t)
+      for (int s = 0; s <= t; ++s) {
+        const int64_t ns = ar.off[s + 1] - ar.off[s], nt = ar.off[t + 1] - ar.off[t];
+        if (ns == 0 || nt == 0) continue;
+        pairs.push_back({s, t, grows});
+        grows += ns;
+        most = std::max(most, ns);
+      }
+    // Small blocks B_st (fewer tiles than SMs) are formed in one launch for all pairs once every G is there: at
+    // 60 functions a block's 16 tiles took as long as all 160.  Large ones pair by pair, with one G.
+    const bool together = (most + 127) / 128 * ((maxr + 127) / 128) < 152;
+    if (!together) grows = most;
     LRTEI_TRY(scratch_split(sc, Fsp, tile0.back(), n3, 128, pl));
-    Ksp = split_shape(pl, pc.rows, K_kpad(pc), 128);
+    Ksp = split_shape(pl, pc.rows, K_cols(pl), K_kpad(pc), 128);
     LRTEI_TRY(sc.get(&Ksp.d, (size_t)Ksp.count()));
     LRTEI_TRY(sc.get(&Ksp.expo, (size_t)pc.rows));
-    LRTEI_TRY(scratch_split(sc, Gsp, maxr, n3, 128, pl));
+    LRTEI_TRY(scratch_split(sc, Gsp, grows, n3, 128, pl));
     double* K;
     LRTEI_TRY(sc.get(&K, (size_t)pc.rows * K_cols(pl)));
+    LRTEI_TRY(sc.get(&G, (size_t)grows * pc.cols));
+    LRTEI_TRY(sc.get(&blk, (size_t)grows * maxr));
     auto rows_of = [&](int s) { return Fsp.from_row(tile0[s], ar.off[s + 1] - ar.off[s]); };
     {
       ProfScope ps("split", st);
@@ -1100,27 +1118,39 @@ lrtei_status bu_adaptive(lrtei_plan* pl, double* Bu, cudaStream_t st) {
         launch_split_rows(ar.Fp + ar.off[s] * n3, ar.off[s + 1] - ar.off[s], n3, n3, rows_of(s), nullptr, st);
     }
     bool first = true;
-    for (int t = 0; t < np; ++t) {
-      const int64_t nt = ar.off[t + 1] - ar.off[t];
-      for (int s = 0; s <= t; ++s) {
-        const int64_t ns = ar.off[s + 1] - ar.off[s];
-        if (ns == 0 || nt == 0) continue;
-        // K_{ts} = (w/sqrt(pi)) sum_p w_p (x)_d A^(p)_{ts,d}, so that G = F_s K_{ts}^T = F_s K_{st}
-        LRTEI_TRY(slice_K(pl, pl->d_C + (size_t)(t * np + s) * cblk, first, K, Ksp, st));
-        first = false;
-        const SplitMatrix Fs = rows_of(s), Ft = rows_of(t);
-        LRTEI_TRY(tc_gemm_K(Fs, 0, Ksp, pc, ns, false, G, 1, nullptr, pl->d_status, st));
-        Gsp.rows = ns;
-        {
-          ProfScope ps("split", st);
-          launch_split_rows(G, ns, n3, pc.cols, Gsp, pl->d_pos, st);
-        }
-        LRTEI_TRY(tc_gemm(Gsp, 0, Ft, ns, nt, 1.0, blk, nt, false, false, 1, nullptr, pl->d_status, st));
-        launch_scatter_block(blk, nt, ar.d_idx + ar.off[s], ns, ar.d_idx + ar.off[t], nt, Bu, npair, s != t, st);
+    for (const Pair& q : pairs) {
+      const int64_t ns = ar.off[q.s + 1] - ar.off[q.s], nt = ar.off[q.t + 1] - ar.off[q.t];
+      // K_{ts} = (w/sqrt(pi)) sum_p w_p (x)_d A^(p)_{ts,d}, so that G = F_s K_{ts}^T = F_s K_{st}
+      LRTEI_TRY(slice_K(pl, pl->d_C + (size_t)(q.t * np + q.s) * cblk, first, K, Ksp, st));
+      first = false;
+      LRTEI_TRY(tc_gemm_K(rows_of(q.s), 0, Ksp, pc, ns, false, G + (together ? q.row * pc.cols : 0), 1, nullptr,
+                          pl->d_status, st));
+      if (together) continue;
+      Gsp.rows = ns;
+      {
+        ProfScope ps("split", st);
+        launch_split_rows(G, ns, n3, pc.cols, Gsp, pl->d_pos, st);
       }
+      LRTEI_TRY(tc_gemm(Gsp, 0, rows_of(q.t), ns, nt, 1.0, blk, nt, false, false, 1, nullptr, pl->d_status, st));
+      launch_scatter_block(blk, nt, ar.d_idx + ar.off[q.s], ns, ar.d_idx + ar.off[q.t], nt, Bu, npair, q.s != q.t, st);
+    }
+    if (together) {
+      {
+        ProfScope ps("split", st);
+        launch_split_rows(G, grows, n3, pc.cols, Gsp, pl->d_pos, st);
+      }
+      std::vector<TcBlock> blocks;
+      for (const Pair& q : pairs)
+        blocks.push_back({q.row, tile0[q.t], ar.off[q.s + 1] - ar.off[q.s], ar.off[q.t + 1] - ar.off[q.t], q.row * maxr});
+      LRTEI_TRY(tc_gemm_blocks(Gsp, Fsp, blocks, blk, maxr, pl->d_status, st));
+      for (const Pair& q : pairs)
+        launch_scatter_block(blk + q.row * maxr, maxr, ar.d_idx + ar.off[q.s], ar.off[q.s + 1] - ar.off[q.s],
+                             ar.d_idx + ar.off[q.t], ar.off[q.t + 1] - ar.off[q.t], Bu, npair, q.s != q.t, st);
     }
     return finish_launch("adaptive B (tensor cores)");
   }
+  LRTEI_TRY(sc.get(&G, (size_t)maxr * n3));
+  LRTEI_TRY(sc.get(&blk, (size_t)maxr * maxr));
   for (int t = 0; t < np; ++t) {
     const int64_t nt = ar.off[t + 1] - ar.off[t];
     for (int s = 0; s <= t; ++s) {
@@ -1781,7 +1811,8 @@ lrtei_status lrtei_exchange(lrtei_plan* plan, const double* d_Q, int norb, doubl
       launch_perm_orbital_rows(nbf, n3, nj, X, n3, nullptr, Xp, st);
       launch_perm_orbital_rows(nbf, n3, nj, Y, ycols, plan->d_pos, Yp, st);
       SplitMatrix Ya = Ypsp, Xa = Xpsp;
-      Ya.kpad = Xa.kpad = kpad256((int64_t)nj * n3);
+      Ya.set_k((int64_t)nj * n3);
+      Xa.set_k((int64_t)nj * n3);
       {
         ProfScope ps("split", st);
         launch_split_rows(Yp, nbf, (int64_t)nj * n3, (int64_t)nj * n3, Ya, nullptr, st);
@@ -2014,7 +2045,8 @@ static lrtei_status jbuild_streamed(lrtei_plan* plan, const double* d_D, int R, 
     launch_transpose(Fb, nr, n3, n3, FbT, nr, st);
     launch_transpose(Du + r0 * R, nr, R, R, DbT, nr, st);
     SplitMatrix A = FbTsp, Bm = Dbsp;  // K = nr for this block
-    A.kpad = Bm.kpad = kpad256(nr);
+    A.set_k(nr);
+    Bm.set_k(nr);
     {
       ProfScope ps("split", st);
       launch_split_rows(FbT, n3, nr, nr, A, nullptr, st);

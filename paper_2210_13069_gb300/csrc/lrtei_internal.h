@@ -183,7 +183,8 @@ struct ParityClasses {
   // Step tables of the split-precision products, whose K runs in the natural order (device; NULL without
   // parity): per class, at tab + tab_off[c], [units + 1] the first list entry of each 128-deep chunk,
   // [units + 1] the number of chunks with entries before it, and the list of the 16-deep K blocks that
-  // hold columns of the class, the last one of each chunk flagged with 2^30.
+  // hold columns of the class, two to a stage where a chunk allows (2^29 on the first), the stage that
+  // ends a chunk flagged with 2^30.
   const int* tab = nullptr;
   int tab_off[8] = {};
   int units = 0;           // chunks of the padded n^3
@@ -314,12 +315,18 @@ lrtei_status oz_gemm(const OzMatrix& A, const OzMatrix& B, const std::vector<OzS
 struct SplitMatrix {  // rows x kpad (a multiple of 256), three FP16 slice planes + per-row scale exponent, in
                       // tiles of `tile` rows x 16 columns (tc_gemm.h)
   int64_t rows = 0, kpad = 0;
+  int64_t k = 0;           // columns that are not padding
   int tile = 128;          // 128; 32 or 64 for the right operand of a product that narrow
   uint16_t* d = nullptr;
   int* expo = nullptr;     // [rows]
   bool plain = false;      // one plane of plain BF16 operands (no slices)
   bool eight = false;      // eight-product scheme
   int planes() const { return plain ? 1 : 3; }
+  int steps() const { return (int)((k + 15) / 16); }  // 16-deep blocks that hold columns
+  void set_k(int64_t cols) {
+    k = cols;
+    kpad = (cols + 255) / 256 * 256;
+  }
   int64_t count() const { return (rows + tile - 1) / tile * tile * kpad * planes(); }
   SplitMatrix from_row(int64_t r0, int64_t nr) const {  // rows [r0, r0 + nr), r0 a multiple of the tile
     SplitMatrix v = *this;
@@ -343,6 +350,12 @@ void launch_split_rows(const double* d_src, int64_t rows, int64_t k, int64_t ld,
 lrtei_status tc_gemm(const SplitMatrix& A, int64_t a_row0, const SplitMatrix& B, int64_t M, int64_t N, double scale,
                      double* d_C, int64_t ldc, bool transpose_out, bool symmetric_upper, int splits, double* d_part,
                      int* d_status, cudaStream_t st);
+// Products of rows [a_row0, + M) of A with rows [b_row0, + N) of B (b_row0 a multiple of 128), each at C + c_off.
+struct TcBlock {
+  int64_t a_row0, b_row0, M, N, c_off;
+};
+lrtei_status tc_gemm_blocks(const SplitMatrix& A, const SplitMatrix& B, const std::vector<TcBlock>& blocks, double* d_C,
+                            int64_t ldc, int* d_status, cudaStream_t st);
 // Products with the node sum K by parity classes, in class order (pc.cols columns, padding zero):
 // k_is_a false: C[rows][pc.cols] = X K^T from rows [x_row0, x_row0 + rows) of X; k_is_a: C[r][:] = K X_r for
 // the rows r of X.  X in the natural column order.

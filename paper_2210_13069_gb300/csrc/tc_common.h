@@ -203,40 +203,85 @@ __device__ __forceinline__ int64_t fixed32(double x, int e) {
 // Slices of one element: q = round(x 2^(32-e)), s0 = round(q / 2^24), r = q - s0 2^24,
 // t1 = round(r / 2^12), t2 = r - t1 2^12; x ~ 2^e (s0 2^-8 + t1 2^-20 + t2 2^-32), |s0| <= 255,
 // |t1|, |t2| <= 2048: integers that FP16 holds exactly, also over 2^12 and 2^24.
-__device__ __forceinline__ void slice_ints(double x, int e, bool live, float& s0, float& t1, float& t2) {
-  s0 = t1 = t2 = 0.f;
-  if (live) {
-    const int64_t q = fixed32(x, e);
-    const int64_t q0 = (q + (1LL << 23)) >> 24;
-    const int64_t r = q - (q0 << 24);
-    const int64_t q1 = (r + (1LL << 11)) >> 12;
-    const int64_t q2 = r - (q1 << 12);
-    s0 = (float)q0;
-    t1 = (float)q1;
-    t2 = (float)q2;
-  }
+__device__ __forceinline__ void slice_ints(double x, int e, bool live, int& s0, int& t1, int& t2) {
+  const int64_t q = live ? fixed32(x, e) : 0;  // |q| < 255 2^24
+  s0 = (int)((q + (1LL << 23)) >> 24);
+  const int r = (int)((uint32_t)q - ((uint32_t)s0 << 24));  // |r| <= 2^23
+  t1 = (r + (1 << 11)) >> 12;
+  t2 = r - (t1 << 12);
 }
 
-// The planes of the GEMM operands as FP16 bit patterns: s0, t1 / 2^12, t2 / 2^24.
-struct SliceBits {
-  uint16_t s0, s1, s2;
-};
-__device__ __forceinline__ SliceBits slice_bits(double x, int e, bool live) {
-  float a, b, c;
-  slice_ints(x, e, live, a, b, c);
-  return {f16_bits(a), f16_bits(b * 0x1p-12f), f16_bits(c * 0x1p-24f)};
+// Integers of magnitude up to 2^22 as FP32 by the exponent trick, times a power of two: no pass through the
+// conversion unit (16 a clock and SM; slicing took three of them and three more to FP16 per element).
+__device__ __forceinline__ float small_float(int i, float scale) {
+  return __fmaf_rn(__int_as_float(0x4B400000 + i), scale, -12582912.f * scale);
+}
+__device__ __forceinline__ uint32_t f16x2_bits(float lo, float hi) {
+  const __half2 h = __floats2half2_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// The planes of the GEMM operands, s0, t1 / 2^12 and t2 / 2^24, of two neighbouring elements as FP16 pairs.
+__device__ __forceinline__ void slice_pair(double x, double y, int e, bool lx, bool ly, uint32_t& p0, uint32_t& p1,
+                                           uint32_t& p2) {
+  int a0, a1, a2, b0, b1, b2;
+  slice_ints(x, e, lx, a0, a1, a2);
+  slice_ints(y, e, ly, b0, b1, b2);
+  p0 = f16x2_bits(small_float(a0, 1.f), small_float(b0, 1.f));
+  p1 = f16x2_bits(small_float(a1, 0x1p-12f), small_float(b1, 0x1p-12f));
+  p2 = f16x2_bits(small_float(a2, 0x1p-24f), small_float(b2, 0x1p-24f));
 }
 
 // The planes of the Hadamard form's operands: s0, t1, t2 / 2^12 and, where s1h is given, t1 / 2^12.
 __device__ __forceinline__ void slice_store(double x, int e, bool live, int64_t o, uint16_t* s0, uint16_t* s1,
                                             uint16_t* s2, uint16_t* s1h) {
-  float a, b, c;
+  int a, b, c;
   slice_ints(x, e, live, a, b, c);
-  s0[o] = f16_bits(a);
-  s1[o] = f16_bits(b);
-  s2[o] = f16_bits(c * 0x1p-12f);
-  if (s1h) s1h[o] = f16_bits(b * 0x1p-12f);
+  s0[o] = f16_bits((float)a);
+  s1[o] = f16_bits((float)b);
+  s2[o] = f16_bits((float)c * 0x1p-12f);
+  if (s1h) s1h[o] = f16_bits((float)b * 0x1p-12f);
 }
+
+// ------------------------------------------------------------------ packed FP32
+// Two FP32 numbers in a register pair, each operation rounded as the scalar one, one instruction for both.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float x, float y) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ f32x2 pack2(uint32_t x, uint32_t y) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(x), "r"(y));
+  return r;
+}
+__device__ __forceinline__ float half_of(f32x2 v, int odd) {
+  float x, y;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+  return (odd & 1) ? y : x;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 neg2(f32x2 a) { return a ^ 0x8000000080000000ULL; }
 
 // ------------------------------------------------------------------ FP32 pairs to FP64
 // An FP32 number as m 2^e, |m| < 2^24.

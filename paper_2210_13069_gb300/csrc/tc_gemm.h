@@ -36,20 +36,24 @@ constexpr int EPI = 16;      // epilogue warps: four per TMEM lane quadrant
 constexpr int THREADS = 64 + 32 * EPI;
 constexpr int kGroupM = 16;  // M tiles walked together (operand slabs shared in L2)
 constexpr int kGroupRows = 8;
-constexpr int kLast = 1 << 30;  // flag of a step table's entry: the last step of its chunk
+// Flags of a step table's entries (K block numbers): the entry opens a stage that ends its chunk; the entry and
+// the next one share a stage.
+constexpr int kLast = 1 << 30, kTwo = 1 << 29;
 
 // One block of the product: rows a_row0 + [0, M) of A, b_row0 + [0, N) of B, `units` split units of K from
 // block a_blk and b_blk, written at C + c_off.  Rows below m_lo belong to the first tile only (a_row0 is a
 // multiple of 128) and are not stored.
-// tab: NULL, or the product's step table (see StepTables): the K blocks of the operand that holds them all;
+// tab: the step table (ParityClasses) of a scheme with LIST: the K blocks of the operand that holds them all;
 // the other operand holds only the listed ones, one after the other.
+constexpr int kMaxSeg = 36;  // the pairs of eight partitions (adaptive boxes)
 struct Seg {
   int64_t a_row0, b_row0, M, N, c_off, item0;
   int a_blk, b_blk, units, tiles_m, tiles_n, m_lo;
+  int steps;       // K blocks that hold columns (the rest of the last unit is zeros); without a table
   const int* tab;
 };
 struct Params {
-  Seg seg[8];
+  Seg seg[kMaxSeg];
   int nseg, splits, symmetric, transpose_out, accumulate, mirror, align;
   int list_is_a;    // step tables list blocks of A (B is the compact operand), else of B
   int64_t nitems;   // per split
@@ -135,13 +139,13 @@ __device__ __forceinline__ Work work_item(const Params& p, int64_t item) {
   }
   const int per = (s.units + p.splits - 1) / p.splits;
   const int u0 = min(s.units, w.split * per), u1 = min(s.units, u0 + per);
-  if (s.tab) {  // [units + 1] first list entry of each unit, [units + 1] chunks with entries before it, the list
+  if constexpr (S::LIST) {  // [units + 1] first list entry of each unit, [units + 1] chunks with entries before it, the list
     w.t0 = s.tab[u0];
     w.t1 = s.tab[u1];
     w.nch = s.tab[s.units + 1 + u1] - s.tab[s.units + 1 + u0];
   } else {
-    w.t0 = u0 * S::UNIT;
-    w.t1 = u1 * S::UNIT;
+    w.t1 = min((s.steps + S::KS - 1) / S::KS * S::KS, u1 * S::UNIT);  // whole stages (the padding is zeros)
+    w.t0 = min(w.t1, u0 * S::UNIT);
     w.nch = (w.t1 - w.t0 + S::CHUNK - 1) / S::CHUNK;
   }
   return w;
@@ -205,19 +209,22 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
       for (int64_t item = blockIdx.x; item < nitems && !stop; item += gridDim.x) {
         const Work w = work_item<S>(p, item);
         const Seg& sg = p.seg[w.seg];
-        const int* list = sg.tab ? sg.tab + 2 * (sg.units + 1) : nullptr;
+        const int* list = S::LIST ? sg.tab + 2 * (sg.units + 1) : nullptr;
         const uint8_t* a = p.a + (((sg.a_row0 + w.m0) / BM) * p.a_steps + sg.a_blk) * (S::PT * G::A_BYTES);
         const int64_t br = sg.b_row0 + w.n0, b_blk = (int64_t)S::PT * p.b_tile * KB * 2;
         const uint8_t* b = p.b + ((br / p.b_tile) * p.b_steps + sg.b_blk) * b_blk + (br % p.b_tile) * (KB * 2);
-        for (int t = w.t0; t < w.t1; t += KS, ++it) {
+        for (int t = w.t0; t < w.t1; ++it) {
           const int s = (int)(it % STAGES);
+          const int e = S::LIST ? list[t] : 0;
+          const int cnt = S::LIST ? ((e & kTwo) ? 2 : 1) : KS;  // steps of this stage
           if (!mbar_wait(&empty[s], ((it / STAGES) & 1u) ^ 1u, abort_flag, p.status, 32)) { stop = true; break; }
-          mbar_arrive_expect_tx(&full[s], G::STAGE);
+          mbar_arrive_expect_tx(&full[s], (uint32_t)cnt * G::STEP);
           uint8_t* st = smem + (size_t)s * G::STAGE;
 #pragma unroll
           for (int q = 0; q < KS; ++q) {
-            const int pos = t + q, nat = list ? list[pos] & (kLast - 1) : pos;
-            const int ka = list && p.list_is_a ? nat : pos, kb = list && !p.list_is_a ? nat : pos;
+            if (q >= cnt) break;
+            const int pos = t + q, nat = S::LIST ? (q == 0 ? e : list[pos]) & (kTwo - 1) : pos;
+            const int ka = S::LIST && p.list_is_a ? nat : pos, kb = S::LIST && !p.list_is_a ? nat : pos;
             bulk_load(st + q * G::STEP, a + (int64_t)ka * (S::PT * G::A_BYTES), NP * G::A_BYTES, &full[s]);
             uint8_t* sb = st + q * G::STEP + NP * G::A_BYTES;
             const uint8_t* bs = b + kb * b_blk;
@@ -229,6 +236,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
                 bulk_load(sb + i * G::B_BYTES, bs + (int64_t)i * p.b_tile * KB * 2, G::B_BYTES, &full[s]);
             }
           }
+          t += cnt;
         }
       }
       if (*abort_flag) {  // bounded wait for the loads in flight before the CTA can exit
@@ -257,13 +265,15 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
       for (int64_t item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
         const Work w = work_item<S>(p, item);
         const Seg& sg = p.seg[w.seg];
-        const int* list = sg.tab ? sg.tab + 2 * (sg.units + 1) : nullptr;
+        const int* list = S::LIST ? sg.tab + 2 * (sg.units + 1) : nullptr;
         int in_chunk = 0;  // steps of the current chunk so far
-        int next = list && w.t0 < w.t1 ? list[w.t0] : 0;
-        for (int t = w.t0; t < w.t1; t += KS) {
-          // the chunk ends with a flagged step, after CHUNK steps, or with the item
-          const bool last = (list ? (next & kLast) != 0 : in_chunk + KS >= S::CHUNK) || t + KS >= w.t1;
-          if (list) next = list[min(t + 1, w.t1 - 1)];
+        int next = S::LIST && w.t0 < w.t1 ? list[w.t0] : 0;
+        for (int t = w.t0; t < w.t1;) {
+          const int e = next, cnt = S::LIST ? ((e & kTwo) ? 2 : 1) : KS;
+          t += cnt;
+          // the chunk ends with a flagged stage, after CHUNK steps, or with the item
+          const bool last = (S::LIST ? (e & kLast) != 0 : in_chunk + cnt >= S::CHUNK) || t >= w.t1;
+          if (S::LIST) next = list[min(t, w.t1 - 1)];
           if (in_chunk == 0 && !mbar_wait(&acce[cg & 1u], ((cg >> 1) & 1u) ^ 1u, abort_flag, p.status)) { ok = false; break; }
           if (!ready && !mbar_wait(&full[s], ph, abort_flag, p.status)) { ok = false; break; }
           tc_fence_after();
@@ -277,11 +287,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
           const uint64_t so = (uint64_t)(cur * (G::STAGE >> 4));
 #pragma unroll
           for (int k = 0; k < KS; ++k)
-            S::mma(d0, a_desc + so + (uint64_t)((k * G::STEP) >> 4), b_desc + so + (uint64_t)((k * G::STEP) >> 4), idesc,
-                   (in_chunk == 0 && k == 0) ? 0u : 1u);
+            if (k < cnt)
+              S::mma(d0, a_desc + so + (uint64_t)((k * G::STEP) >> 4), b_desc + so + (uint64_t)((k * G::STEP) >> 4), idesc,
+                     (in_chunk == 0 && k == 0) ? 0u : 1u);
           mma_commit(&empty[cur]);
           if (last) mma_commit(&accf[cg & 1u]);
-          in_chunk = last ? 0 : in_chunk + KS;
+          in_chunk = last ? 0 : in_chunk + cnt;
           cg += last ? 1u : 0u;
         }
       }
