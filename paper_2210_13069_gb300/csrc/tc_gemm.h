@@ -314,10 +314,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
       T.clear();
       for (int c = 0; c < w.nch; ++c, ++cg) {
         const int buf = (int)(cg & 1u);
-        int got = 1;
-        if (lane == 0) got = mbar_wait(&accf[buf], (cg >> 1) & 1u, abort_flag, p.status, 32) ? 1 : 0;
-        got = __shfl_sync(0xffffffffu, got, 0);
-        if (!got) { ok = false; break; }
+        ok = __all_sync(0xffffffffu, mbar_wait(&accf[buf], (cg >> 1) & 1u, abort_flag, p.status));
+        if (!ok) break;
         tc_fence_after();
         T.drain(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * S::NACC * BN + col0));
         tc_fence_before();
