@@ -243,6 +243,120 @@ __global__ void __cluster_dims__(kSplitCluster, 1, 1) __launch_bounds__(256)
   }
 }
 
+// ---- operands of the long-range exchange, sliced where they lie (no transposed or permuted FP64 copies)
+// Rows (mu, m) of MT, columns la: F_u(pair(mu, la), m), N_b <= 256 columns.  One CTA per mu and 32 columns m of
+// F_u: the rows of F_u are read along m into shared memory, the row maxima are taken, then the slices stored.  Blocks beyond the last column but one are not read by the products and stay
+// unwritten.  Gather and slicing of 2.5 M rows of 180 took 1.66 + 1.65 ms through a 3.6 GB copy.
+__global__ void __launch_bounds__(256) k_split_MT(int nbf, int64_t n3, const double* __restrict__ F, int64_t ldF,
+                                                  int64_t kpad, int kuse, int tile, uint16_t* __restrict__ d,
+                                                  int* __restrict__ expo) {
+  extern __shared__ double t[];  // [nbf][33]
+  const int mu = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t m0 = (int64_t)blockIdx.x * 32;
+  for (int l0 = warp; l0 < nbf; l0 += 64) {  // eight rows' loads in flight per warp
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int la = l0 + 8 * u, lo = mu < la ? mu : la, hi = mu < la ? la : mu;
+      const int64_t r = (int64_t)lo * nbf - (int64_t)lo * (lo - 1) / 2 + (hi - lo);
+      v[u] = la < nbf && m0 + lane < n3 ? F[r * ldF + m0 + lane] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (l0 + 8 * u < nbf) t[(l0 + 8 * u) * 33 + lane] = v[u];
+  }
+  __syncthreads();
+  __shared__ int re[32];  // row exponents; kZeroRow: nothing to slice
+  constexpr int kZeroRow = 1 << 20;
+  for (int q = warp; q < 32; q += 8) {
+    uint64_t mx = 0;
+    for (int la = lane; la < nbf; la += 32) {
+      const uint64_t a = (uint64_t)__double_as_longlong(t[la * 33 + q]) & 0x7FFFFFFFFFFFFFFFULL;
+      mx = a > mx ? a : mx;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      const uint64_t other = __shfl_xor_sync(0xffffffffu, mx, o);
+      mx = other > mx ? other : mx;
+    }
+    if (lane == 0) {
+      const double mxd = __longlong_as_double((long long)mx);
+      int e = 0;
+      if (mxd > 0.0) frexp(mxd * (256.0 / 255.0), &e);
+      re[q] = mxd > 0.0 && e >= -1000 ? e : kZeroRow;
+      if (m0 + q < n3) expo[(int64_t)mu * n3 + m0 + q] = e;
+    }
+  }
+  __syncthreads();
+  // a warp takes 16 rows of one 16-column block, a lane half a row of it: 512 contiguous bytes per plane and store
+  const int nitem = kuse / 16 * 2;
+  for (int it = warp; it < nitem; it += 8) {
+    const int q = (it & 1) * 16 + (lane >> 1), c0 = (it >> 1) * 16 + (lane & 1) * 8;
+    if (m0 + q >= n3) continue;
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = c0 + u < nbf ? t[(c0 + u) * 33 + q] : 0.0;
+    const int e = re[q];
+    store_slices(v, e, e != kZeroRow, (int64_t)mu * n3 + m0 + q, c0, nbf, tile, kpad, d);
+  }
+}
+
+// Largest magnitude (bits) over the rows (j, mu), j < nj, of Z for each mu: the row maxima of Zp[mu][(j, m)].
+__global__ void __launch_bounds__(256) k_orbital_max(int nbf, int64_t cols, int64_t ld, const double* __restrict__ Z,
+                                                     unsigned long long* __restrict__ mx) {
+  const int64_t row = blockIdx.x;  // j nbf + mu
+  const double* x = Z + row * ld;
+  unsigned long long v = 0;
+#pragma unroll 4
+  for (int64_t m = threadIdx.x; m < cols; m += 256) {
+    const unsigned long long a = (unsigned long long)__double_as_longlong(x[m]) & 0x7FFFFFFFFFFFFFFFULL;
+    v = a > v ? a : v;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long other = __shfl_xor_sync(0xffffffffu, v, o);
+    v = other > v ? other : v;
+  }
+  if ((threadIdx.x & 31) == 0) atomicMax(mx + row % nbf, v);
+}
+
+// Zp[mu][(j, m)] = Z[(j, mu)][map[m]] into slices (n3 a multiple of 8): one CTA per row (j, mu), staged by one
+// bulk copy, with the exponent of row mu.
+__global__ void __launch_bounds__(512) k_split_orbital_rows(int nbf, int64_t n3, int64_t cols, int64_t ld,
+                                                            const double* __restrict__ Z, const int* __restrict__ map,
+                                                            const unsigned long long* __restrict__ mx, int64_t k,
+                                                            int64_t kpad, int tile, uint16_t* __restrict__ d,
+                                                            int* __restrict__ expo) {
+  extern __shared__ __align__(16) double row[];
+  __shared__ uint64_t bar;
+  const int64_t i = blockIdx.x;
+  const int j = (int)(i / nbf), mu = (int)(i % nbf);
+  if (threadIdx.x == 0) {
+    mbar_init(&bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    mbar_arrive_expect_tx(&bar, (uint32_t)(cols * 8));
+    bulk_load(row, Z + i * ld, (uint32_t)(cols * 8), &bar);
+  }
+  const double mxd = __longlong_as_double((long long)mx[mu]);
+  int e = 0;
+  if (mxd > 0.0) frexp(mxd * (256.0 / 255.0), &e);
+  const bool nz = mxd > 0.0 && e >= -1000;
+  if (j == 0 && threadIdx.x == 0) expo[mu] = e;
+  __syncthreads();
+  for (long long t0 = clock64(); !mbar_try_wait(&bar, 0u) && clock64() - t0 < kWaitCycles;) {
+  }
+  const int64_t c0 = (int64_t)j * n3;
+  for (int64_t m = 8 * (int64_t)threadIdx.x; m < n3; m += 8 * (int64_t)blockDim.x) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = row[map ? map[m + u] : (int)m + u];
+    store_slices(v, e, nz, mu, c0 + m, k, tile, kpad, d);
+  }
+  if ((int64_t)(j + 1) * n3 == k) {  // the padding after the last orbital
+    double z[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int64_t c = k + 8 * (int64_t)threadIdx.x; c < kpad; c += 8 * (int64_t)blockDim.x)
+      store_slices(z, e, nz, mu, c, k, tile, kpad, d);
+  }
+}
+
 // Plain BF16 operands: one rounded copy per element, exponent 8 so that the epilogue scale
 // 2^(ea + eb - 16) is 1.
 __global__ void k_plain_rows(const double* __restrict__ src, int64_t k, int64_t ld, int64_t kpad, int tile,
@@ -325,6 +439,34 @@ void launch_split_rows(const double* d_src, int64_t rows, int64_t k, int64_t ld,
   const int bulk = (cols % 2 == 0 && ld % 2 == 0 && (reinterpret_cast<uintptr_t>(d_src) & 15) == 0) ? 1 : 0;
   tc::k_split_rows<<<(unsigned)rows, cols > 8192 ? 512 : 256, sizeof(double) * (size_t)cols, st>>>(
       d_src, cols, k, ld, m.kpad, m.tile, bulk, d_map, m.d, m.expo);
+}
+
+bool launch_split_MT(int nbf, int64_t n3, const double* d_F, int64_t ldF, const SplitMatrix& m, cudaStream_t st) {
+  const size_t smem = sizeof(double) * 33 * (size_t)nbf;
+  if (m.plain || nbf > 256 || m.kpad > 256) return false;
+  static bool attr_set = false;
+  if (!attr_set)
+    attr_set = cudaFuncSetAttribute(tc::k_split_MT, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)(sizeof(double) * 33 * 256)) == cudaSuccess;
+  count_launch();
+  tc::k_split_MT<<<dim3((unsigned)((n3 + 31) / 32), (unsigned)nbf), 256, smem, st>>>(
+      nbf, n3, d_F, ldF, m.kpad, (m.steps() + 1) / 2 * 32, m.tile, m.d, m.expo);
+  return true;
+}
+
+bool launch_split_orbitals(int nbf, int64_t n3, int nj, const double* d_Z, int64_t cols, const int* d_map,
+                           unsigned long long* d_max, const SplitMatrix& m, cudaStream_t st) {
+  if (m.plain || n3 % 8 != 0 || cols % 2 != 0 || cols > tc::kSplitCols || (reinterpret_cast<uintptr_t>(d_Z) & 15)) return false;
+  static bool attr_set = false;
+  if (!attr_set)
+    attr_set = cudaFuncSetAttribute(tc::k_split_orbital_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)(sizeof(double) * tc::kSplitCols)) == cudaSuccess;
+  cudaMemsetAsync(d_max, 0, sizeof(unsigned long long) * (size_t)nbf, st);
+  count_launches(2);
+  tc::k_orbital_max<<<(unsigned)((int64_t)nj * nbf), 256, 0, st>>>(nbf, cols, cols, d_Z, d_max);
+  tc::k_split_orbital_rows<<<(unsigned)((int64_t)nj * nbf), cols > 8192 ? 512 : 256, sizeof(double) * (size_t)cols, st>>>(
+      nbf, n3, cols, cols, d_Z, d_map, d_max, m.k, m.kpad, m.tile, m.d, m.expo);
+  return true;
 }
 
 void launch_transpose(const double* in, int64_t rows, int64_t cols, int64_t ldi, double* out, int64_t ldo,

@@ -1829,17 +1829,17 @@ lrtei_status lrtei_exchange(lrtei_plan* plan, const double* d_Q, int norb, doubl
   if (env_count("LRTEI_EXCHANGE_BLOCK") > 0) ob = (int)std::min<int64_t>(norb, env_count("LRTEI_EXCHANGE_BLOCK"));
   const int nblk = (norb + ob - 1) / ob;
   Scratch sc(st);
-  double *MT, *X, *Y, *Xp, *Yp, *Kb;
-  LRTEI_TRY(sc.get(&MT, (size_t)rowlen * nbf));
+  double *MT = nullptr, *X, *Y, *Xp = nullptr, *Yp = nullptr, *Kb;
+  // FP64 copies of the transposed and permuted operands, where they are needed
+  auto need_copy = [&](double** p, size_t count) { return *p ? LRTEI_OK : sc.get(p, count); };
   LRTEI_TRY(sc.get(&X, (size_t)ob * rowlen));
   if (tc) LRTEI_TRY(ensure_Ksp(plan, st));  // K as the right operand of Y = X K^T (K symmetric)
   const int64_t ycols = tc ? plan->pc.cols : n3;
   LRTEI_TRY(sc.get(&Y, (size_t)ob * nbf * ycols));
-  LRTEI_TRY(sc.get(&Xp, (size_t)ob * rowlen));
-  LRTEI_TRY(sc.get(&Yp, (size_t)ob * rowlen));
   LRTEI_TRY(sc.get(&Kb, (size_t)nblk * nbf * nbf));
-  launch_gather_MT(nbf, n3, plan->d_F, n3, MT, st);
   if (tc) {
+    unsigned long long* dmax;
+    LRTEI_TRY(sc.get(&dmax, (size_t)nbf));
     SplitMatrix Qsp, MTsp, Xsp, Ypsp, Xpsp;
     LRTEI_TRY(scratch_split(sc, Qsp, norb, nbf, 128, plan));
     LRTEI_TRY(scratch_split(sc, MTsp, rowlen, nbf, split_tile(rowlen), plan));
@@ -1855,7 +1855,11 @@ lrtei_status lrtei_exchange(lrtei_plan* plan, const double* d_Q, int norb, doubl
     {
       ProfScope ps("split", st);
       launch_split_rows(d_Q, norb, nbf, nbf, Qsp, nullptr, st);
-      launch_split_rows(MT, rowlen, nbf, nbf, MTsp, nullptr, st);
+      if (!launch_split_MT(nbf, n3, plan->d_F, n3, MTsp, st)) {
+        LRTEI_TRY(need_copy(&MT, (size_t)rowlen * nbf));
+        launch_gather_MT(nbf, n3, plan->d_F, n3, MT, st);
+        launch_split_rows(MT, rowlen, nbf, nbf, MTsp, nullptr, st);
+      }
     }
     for (int b = 0; b < nblk; ++b) {
       const int j0 = b * ob, nj = std::min(ob, norb - j0);
@@ -1867,15 +1871,21 @@ lrtei_status lrtei_exchange(lrtei_plan* plan, const double* d_Q, int norb, doubl
         launch_split_rows(X, Xb.rows, n3, n3, Xb, nullptr, st);
       }
       LRTEI_TRY(tc_gemm_K(Xb, 0, plan->Ksp, plan->pc, Xb.rows, false, Y, 1, nullptr, plan->d_status, st));
-      launch_perm_orbital_rows(nbf, n3, nj, X, n3, nullptr, Xp, st);
-      launch_perm_orbital_rows(nbf, n3, nj, Y, ycols, plan->d_pos, Yp, st);
       SplitMatrix Ya = Ypsp, Xa = Xpsp;
       Ya.set_k((int64_t)nj * n3);
       Xa.set_k((int64_t)nj * n3);
       {
         ProfScope ps("split", st);
-        launch_split_rows(Yp, nbf, (int64_t)nj * n3, (int64_t)nj * n3, Ya, nullptr, st);
-        launch_split_rows(Xp, nbf, (int64_t)nj * n3, (int64_t)nj * n3, Xa, nullptr, st);
+        if (!launch_split_orbitals(nbf, n3, nj, Y, ycols, plan->d_pos, dmax, Ya, st)) {
+          LRTEI_TRY(need_copy(&Yp, (size_t)ob * rowlen));
+          launch_perm_orbital_rows(nbf, n3, nj, Y, ycols, plan->d_pos, Yp, st);
+          launch_split_rows(Yp, nbf, (int64_t)nj * n3, (int64_t)nj * n3, Ya, nullptr, st);
+        }
+        if (!launch_split_orbitals(nbf, n3, nj, X, n3, nullptr, dmax, Xa, st)) {
+          LRTEI_TRY(need_copy(&Xp, (size_t)ob * rowlen));
+          launch_perm_orbital_rows(nbf, n3, nj, X, n3, nullptr, Xp, st);
+          launch_split_rows(Xp, nbf, (int64_t)nj * n3, (int64_t)nj * n3, Xa, nullptr, st);
+        }
       }
       const int sb = splits_for(nbf, (int64_t)nj * n3);
       if (sb > sK) { set_error("exchange: split count %d beyond the partial buffer's %d", sb, sK); return LRTEI_ERR_CUDA; }
@@ -1883,6 +1893,10 @@ lrtei_status lrtei_exchange(lrtei_plan* plan, const double* d_Q, int norb, doubl
                         plan->d_status, st));
     }
   } else {
+    LRTEI_TRY(need_copy(&MT, (size_t)rowlen * nbf));
+    LRTEI_TRY(need_copy(&Xp, (size_t)ob * rowlen));
+    LRTEI_TRY(need_copy(&Yp, (size_t)ob * rowlen));
+    launch_gather_MT(nbf, n3, plan->d_F, n3, MT, st);
     const int64_t kc = 32768;  // split-K chunk of the last product (an N_b x N_b output)
     const int64_t maxk = (int64_t)ob * n3, nchunk = (maxk + kc - 1) / kc;
     double* part;

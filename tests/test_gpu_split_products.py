@@ -63,3 +63,19 @@ def test_jbuild_density_tiles(lib, prec, R):
     pl.status()
     assert rel_fro(J, oracle.Oracle.from_molecule(m).jbuild_factored(D)) <= TOL[prec]
     pl.close()
+
+
+# n^3 a multiple of eight (orbital rows sliced in place) and not (through the permuted copy); one orbital and several.
+@pytest.mark.parametrize("prec", ["split_f16", "split_f16_8"])
+@pytest.mark.parametrize("n,orbs", [(9, 3), (10, 1), (12, 5)])
+def test_exchange_operand_layouts(lib, prec, n, orbs):
+    import torch
+    m = molecule(n, 5)
+    Q = np.random.Generator(np.random.Philox(11)).normal(0.0, 1.0 / np.sqrt(m.nbf), size=(orbs, m.nbf))
+    B = oracle.Oracle.from_molecule(m).assemble_B().reshape(m.nbf, m.nbf, m.nbf, m.nbf)
+    ref = 2.0 * np.einsum("jl,jk,mlkn->mn", Q, Q, B, optimize=True)
+    pl = lib.Plan(m, prec)
+    K = pl.exchange(torch.as_tensor(Q, device="cuda")).cpu().numpy()
+    pl.status()
+    assert rel_fro(K, ref) <= TOL[prec]
+    pl.close()
