@@ -16,8 +16,12 @@
 // The tensor core's FP32 accumulation truncates (measured against an emulation), so L12's smaller terms are
 // cut at the scale of its s0 t1 terms, and the truncation error of a chunk grows with the chunk's depth:
 // hence chunks of 128 rather than the 512 that L0's exactness would allow.  The eight-product variant keeps
-// a1 b2 and a2 b1 as well and splits L12 into L1 = a0 b1 + a1 b0 and L2 (the rest, in its own accumulator):
-// three accumulators per buffer, 128 x 64 tiles, C from T0 + (T1 + T2).
+// a1 b2 and a2 b1 as well and splits L12 into L1 = a0 b1 + a1 b0 and L2 (the rest, in its own accumulator),
+// C from T0 + (T1 + T2): wide outputs in two launches, (T0, T1) and then T2 added to C (both exact multiples of
+// one power of two with a sum below 53 bits, so C is that of one launch bit for bit), as TMEM double-buffers
+// three accumulators for 64 columns only, and an MMA of 64 columns issues no faster than one of 128: the two
+// products of 180 functions compressed at 1e-8 took 16.2 ms in one launch each of
+// 64 columns and take 12.6 ms in four of 128.
 //
 // Chunks lie at multiples of 128 of the natural K, also where a step table leaves steps of them out (the
 // zero blocks of K by parity, below): what is left out adds zeros, so every sum is the dense product's bit
@@ -67,14 +71,17 @@ __device__ __forceinline__ double combine_pow2(int t0, float t12, int k, float t
   return __longlong_as_double((long long)bits);
 }
 
-enum class Scheme { six, eight, plain };
+// eight_hi and eight_lo: the two launches of eight products on 128 columns.
+enum class Scheme { six, eight, eight_hi, eight_lo, plain };
 
 template <int BN_, Scheme M, bool LIST_>
 struct Split {
-  static constexpr bool P8 = M == Scheme::eight, PLAIN = M == Scheme::plain;
-  static constexpr int BN = BN_, NP = PLAIN ? 1 : 3, PT = NP, NACC = PLAIN ? 1 : P8 ? 3 : 2, KS = 2;  // two steps a stage: half the barrier rounds
+  static constexpr bool P8 = M == Scheme::eight, PLAIN = M == Scheme::plain, HI = M == Scheme::eight_hi,
+                        LO = M == Scheme::eight_lo, ONE = PLAIN || LO;  // ONE: a single FP32 accumulator
+  static constexpr int BN = BN_, NP = PLAIN ? 1 : HI ? 2 : 3, PT = PLAIN ? 1 : 3, NACC = ONE ? 1 : P8 ? 3 : 2, KS = 2;
+  // KS: two steps a stage, half the barrier rounds
   static constexpr int UNIT = 8, CHUNK = 8;  // 128 deep
-  static constexpr bool BF16 = PLAIN, ACCUM = false, LIST = LIST_;
+  static constexpr bool BF16 = PLAIN, ACCUM = LO, LIST = LIST_;
 
   static __device__ __forceinline__ void mma(uint32_t d0, uint64_t a0, uint64_t b0, uint32_t idesc, uint32_t first) {
     if constexpr (PLAIN) {
@@ -86,6 +93,20 @@ struct Split {
       // grouped by A slice so that each is read from shared memory once per k step; with eight products the
       // smaller terms go to their own accumulator d2, so that the tensor core's truncating FP32 accumulation
       // cuts them at their own scale
+      if constexpr (HI) {
+        mma_bf16_a<ACol::fill>(d0, a0, b0, idesc, first);
+        mma_bf16_a<ACol::lastuse>(d1, a0, b1, idesc, first);
+        mma_bf16(d1, a1, b0, idesc, 1u);
+        return;
+      }
+      if constexpr (LO) {
+        mma_bf16(d0, a0, b2, idesc, first);
+        mma_bf16(d0, a1, b1, idesc, 1u);
+        mma_bf16_a<ACol::fill>(d0, a2, b0, idesc, 1u);
+        mma_bf16_a<ACol::lastuse>(d0, a2, b1, idesc, 1u);
+        mma_bf16(d0, a1, b2, idesc, 1u);
+        return;
+      }
       mma_bf16_a<ACol::fill>(d0, a0, b0, idesc, first);
       mma_bf16_a<ACol::use>(d1, a0, b1, idesc, first);
       mma_bf16_a<ACol::lastuse>(d2, a0, b2, idesc, P8 ? first : 1u);
@@ -103,12 +124,12 @@ struct Split {
 
   template <int QC>
   struct Sums {
-    int T0[PLAIN ? 1 : QC];
+    int T0[ONE ? 1 : QC];
     float T1[QC], T2[P8 ? QC : 1];
     __device__ __forceinline__ void clear() {
 #pragma unroll
       for (int j = 0; j < QC; ++j) {
-        if constexpr (!PLAIN) T0[j] = 0;
+        if constexpr (!ONE) T0[j] = 0;
         T1[j] = 0.f;
         if constexpr (P8) T2[j] = 0.f;
       }
@@ -117,12 +138,12 @@ struct Split {
 #pragma unroll
       for (int j0 = 0; j0 < QC; j0 += 8) {  // the loads of an 8-column group are in flight together
         uint32_t r[8], q[8];
-        if constexpr (!PLAIN) tmem_ld8(t + j0, r);
-        tmem_ld8(t + (PLAIN ? 0 : BN) + j0, q);
+        if constexpr (!ONE) tmem_ld8(t + j0, r);
+        tmem_ld8(t + (ONE ? 0 : BN) + j0, q);
         tmem_wait_ld();
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          if constexpr (!PLAIN) T0[j0 + j] += __float2int_rn(__uint_as_float(r[j]));
+          if constexpr (!ONE) T0[j0 + j] += __float2int_rn(__uint_as_float(r[j]));
           T1[j0 + j] += __uint_as_float(q[j]);
         }
         if constexpr (P8) {
@@ -135,7 +156,7 @@ struct Split {
     }
     template <int C>
     __device__ __forceinline__ void hold(int j0) {
-      if constexpr (!PLAIN) {
+      if constexpr (!ONE) {
 #pragma unroll
         for (int j = 0; j < C; ++j) {
           asm volatile("" : "+r"(T0[j0 + j]), "+f"(T1[j0 + j]) : : "memory");
@@ -146,20 +167,29 @@ struct Split {
     // The planes' weights make T1 and T2 those of the sums of s0 t1 over 2^12.
     __device__ __forceinline__ double value(int j, int k, double scale) const {
       if constexpr (PLAIN) return scale * pow2(k - 16) * (double)T1[j];
-      const double v = combine_pow2(T0[PLAIN ? 0 : j], T1[j] * 4096.f, k - 16, P8 ? T2[P8 ? j : 0] * 4096.f : 0.f);
+      const double v = combine_pow2(LO ? 0 : T0[ONE ? 0 : j], T1[j] * 4096.f, k - 16, P8 ? T2[P8 ? j : 0] * 4096.f : 0.f);
       return scale == 1.0 ? v : scale * v;
     }
   };
 };
 
-// Tile width: 128 columns for wide six-product outputs (a 128 x 64 MMA is bound by its operand reads from
-// shared memory); the eight-product scheme has TMEM for 64 (2 x 3 accumulators), plain BF16 takes 64.
-static int tile_n(int64_t N, bool plain, bool eight) { return N <= 32 ? 32 : (N <= 64 || plain || eight) ? 64 : 128; }
+// Tile width: 128 columns for wide outputs (a 128 x 64 MMA is bound by its operand reads from shared memory and
+// by its issue); plain BF16 takes 64.
+static int tile_n(int64_t N, bool plain) { return N <= 32 ? 32 : (N <= 64 || plain) ? 64 : 128; }
 
 template <bool LIST>
 static lrtei_status run_as(const tcg::Params& p, int BN, bool plain, bool eight, cudaStream_t st) {
   if (plain)
     return BN == 64 ? tcg::launch<Split<64, Scheme::plain, LIST>>(p, st) : tcg::launch<Split<32, Scheme::plain, LIST>>(p, st);
+  if (eight && BN == 128) {
+    tcg::Params q = p;
+    q.mirror = 0;
+    const lrtei_status s = tcg::launch<Split<128, Scheme::eight_hi, LIST>>(q, st);
+    if (s != LRTEI_OK) return s;
+    q.mirror = p.mirror;
+    q.accumulate = 1;
+    return tcg::launch<Split<128, Scheme::eight_lo, LIST>>(q, st);
+  }
   if (eight)
     return BN == 64 ? tcg::launch<Split<64, Scheme::eight, LIST>>(p, st) : tcg::launch<Split<32, Scheme::eight, LIST>>(p, st);
   if (BN == 128) return tcg::launch<Split<128, Scheme::six, LIST>>(p, st);
@@ -233,7 +263,7 @@ lrtei_status tc_gemm(const SplitMatrix& A, int64_t a_row0, const SplitMatrix& B,
     return LRTEI_ERR_ARG;
   }
   if (symmetric_upper) return tc_gemm_sym_band(A, B, 0, N, N, d_C, ldc, d_status, st);
-  const int BN = tc::tile_n(N, A.plain, A.eight), m_lo = (int)(a_row0 % 128), units = (int)(A.kpad / 128);
+  const int BN = tc::tile_n(N, A.plain), m_lo = (int)(a_row0 % 128), units = (int)(A.kpad / 128);
   tcg::Params p{};
   const int64_t c_rows = transpose_out ? N : M, c_cols = transpose_out ? M : N;
   lrtei_status s = tc::fill(p, A, B, BN, units, scale, d_C, ldc, transpose_out, splits, c_rows, c_cols, d_part, d_status);
@@ -256,7 +286,7 @@ lrtei_status tc_gemm_blocks(const SplitMatrix& A, const SplitMatrix& B, const st
   }
   int64_t nmax = 0;
   for (const TcBlock& b : blocks) nmax = std::max(nmax, b.N);
-  const int BN = tc::tile_n(nmax, A.plain, A.eight), units = (int)(A.kpad / 128);
+  const int BN = tc::tile_n(nmax, A.plain), units = (int)(A.kpad / 128);
   tcg::Params p{};
   int splits = 1;
   lrtei_status s = tc::fill(p, A, B, BN, units, 1.0, d_C, ldc, false, splits, 0, 0, nullptr, d_status);
@@ -280,7 +310,7 @@ lrtei_status tc_gemm_sym_band(const SplitMatrix& A, const SplitMatrix& B, int64_
               (long long)row1, (long long)N);
     return LRTEI_ERR_ARG;
   }
-  const int BN = tc::tile_n(std::max<int64_t>(N, 65), A.plain, A.eight), units = (int)(A.kpad / 128);
+  const int BN = tc::tile_n(std::max<int64_t>(N, 65), A.plain), units = (int)(A.kpad / 128);
   tcg::Params p{};
   int splits = 1;
   lrtei_status s = tc::fill(p, A, B, BN, units, 1.0, d_C, ldc, false, splits, N, N, nullptr, d_status);
@@ -310,7 +340,7 @@ lrtei_status tc_gemm_K(const SplitMatrix& X, int64_t x_row0, const SplitMatrix& 
     nmax = 0;
     for (int c = 0; c < pc.nclass; ++c) nmax = std::max<int64_t>(nmax, pc.size[c]);
   }
-  const int BN = tc::tile_n(nmax, A.plain, A.eight), m_lo = k_is_a ? 0 : (int)(x_row0 % 128);
+  const int BN = tc::tile_n(nmax, A.plain), m_lo = k_is_a ? 0 : (int)(x_row0 % 128);
   if ((k_is_a && x_row0 != 0) || X.kpad / 128 != pc.units) {
     set_error("tc_gemm_K: operand does not match the plan's K");
     return LRTEI_ERR_ARG;
