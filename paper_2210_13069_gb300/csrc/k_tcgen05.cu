@@ -176,6 +176,14 @@ struct Split {
 // Tile width: 128 columns for wide outputs (a 128 x 64 MMA is bound by its operand reads from shared memory and
 // by its issue); plain BF16 takes 64.
 static int tile_n(int64_t N, bool plain) { return N <= 32 ? 32 : (N <= 64 || plain) ? 64 : 128; }
+// Of 128 and 64 columns the ones whose waves take less.  A 64-column tile takes ~0.72 of a 128-column one (its
+// MMAs half, the reads of A and the latencies the same): 64 where they fill SMs that 128 leave idle.  1035 pairs,
+// 2197 deep: B_u (45 tiles of 128) 48 -> 42 us; G (180) stays at two waves of 128, 63 us.
+static int tile_of_waves(int BN, int64_t tiles128, int64_t tiles64) {
+  if (BN != 128) return BN;
+  const int64_t sms = 152, w128 = (tiles128 + sms - 1) / sms, w64 = (tiles64 + sms - 1) / sms;
+  return 72 * w64 < 100 * w128 ? 64 : 128;
+}
 
 template <bool LIST>
 static lrtei_status run_as(const tcg::Params& p, int BN, bool plain, bool eight, cudaStream_t st) {
@@ -310,20 +318,22 @@ lrtei_status tc_gemm_sym_band(const SplitMatrix& A, const SplitMatrix& B, int64_
               (long long)row1, (long long)N);
     return LRTEI_ERR_ARG;
   }
-  const int BN = tc::tile_n(std::max<int64_t>(N, 65), A.plain), units = (int)(A.kpad / 128);
+  // upper-triangular enumeration in 128 x 128 blocks (128 / BN tiles each); A holds rows [row0, row1) only
+  const int64_t nb = (N + 127) / 128, b0 = row0 / 128, b1 = (row1 + 127) / 128;
+  const int64_t blocks = (nb - b0) * (nb - b0 + 1) / 2 - (nb - b1) * (nb - b1 + 1) / 2;
+  const int BN = tc::tile_of_waves(tc::tile_n(std::max<int64_t>(N, 65), A.plain), blocks, 2 * blocks);
+  const int units = (int)(A.kpad / 128);
   tcg::Params p{};
   int splits = 1;
   lrtei_status s = tc::fill(p, A, B, BN, units, 1.0, d_C, ldc, false, splits, N, N, nullptr, d_status);
   if (s != LRTEI_OK) return s;
-  // upper-triangular enumeration in 128 x 128 blocks (128 / BN tiles each); A holds rows [row0, row1) only
-  const int64_t nb = (N + 127) / 128, b0 = row0 / 128, b1 = (row1 + 127) / 128;
   p.symmetric = p.mirror = 1;
   p.nseg = 1;
   p.blk0 = b0;
   p.blk1 = b1;
   p.nb = nb;
   p.seg[0] = {-row0, 0, row1, N, 0, 0, 0, 0, units, (int)(b1 - b0), (int)nb, 0, A.steps(), nullptr};
-  p.nitems = ((nb - b0) * (nb - b0 + 1) / 2 - (nb - b1) * (nb - b1 + 1) / 2) * (128 / BN);
+  p.nitems = blocks * (128 / BN);
   return tc::run(p, BN, A.plain, A.eight, st);
 }
 
@@ -335,12 +345,18 @@ lrtei_status tc_gemm_sym_band(const SplitMatrix& A, const SplitMatrix& B, int64_
 lrtei_status tc_gemm_K(const SplitMatrix& X, int64_t x_row0, const SplitMatrix& K, const ParityClasses& pc, int64_t rows,
                        bool k_is_a, double* d_C, int splits, double* d_part, int* d_status, cudaStream_t st) {
   const SplitMatrix &A = k_is_a ? K : X, &B = k_is_a ? X : K;
-  int64_t nmax = rows;
+  const int m_lo = k_is_a ? 0 : (int)(x_row0 % 128);
+  int BN = tc::tile_n(rows, A.plain);
   if (!k_is_a) {
-    nmax = 0;
-    for (int c = 0; c < pc.nclass; ++c) nmax = std::max<int64_t>(nmax, pc.size[c]);
+    int64_t nmax = 0, t128 = 0, t64 = 0;
+    for (int c = 0; c < pc.nclass; ++c) {
+      nmax = std::max<int64_t>(nmax, pc.size[c]);
+      t128 += (pc.size[c] + 127) / 128;
+      t64 += (pc.size[c] + 63) / 64;
+    }
+    const int64_t tiles_m = (rows + m_lo + 127) / 128;
+    BN = tc::tile_of_waves(tc::tile_n(nmax, A.plain), tiles_m * t128, tiles_m * t64);
   }
-  const int BN = tc::tile_n(nmax, A.plain), m_lo = k_is_a ? 0 : (int)(x_row0 % 128);
   if ((k_is_a && x_row0 != 0) || X.kpad / 128 != pc.units) {
     set_error("tc_gemm_K: operand does not match the plan's K");
     return LRTEI_ERR_ARG;
