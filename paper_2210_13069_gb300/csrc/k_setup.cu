@@ -190,43 +190,49 @@ __device__ __forceinline__ double dfact_d(int k) {
   return r;
 }
 
-// One thread per basis function: primitive normalisation (2a/pi)^{3/4} (4a)^{L/2} / sqrt(prod
+// One block per basis function: primitive normalisation (2a/pi)^{3/4} (4a)^{L/2} / sqrt(prod
 // (2l_d - 1)!!) and contraction normalisation so that the contracted component has unit norm:
 // the overlap of two normalised primitives of one component is (2 sqrt(ab)/(a+b))^{L + 3/2}.
-__global__ void k_normalise(int nbf, const int* bf_shell, const int* bf_pow, const int* shell_nprim,
-                            const int* shell_poff, const double* exps, const double* coefs, const int* bf_coff,
-                            double* ncoef) {
-  int mu = blockIdx.x * blockDim.x + threadIdx.x;
-  if (mu >= nbf) return;
+// A thread per pow() (K + K^2 of them; one after the other on one thread they took 62 us for K = 3, 14 us now);
+// thread 0 adds the overlaps in order.
+constexpr int kMaxPrim = 16;  // a row holds each primitive's number in four bits
+__global__ void __launch_bounds__(64) k_normalise(const int* bf_shell, const int* bf_pow, const int* shell_nprim,
+                                                  const int* shell_poff, const double* exps, const double* coefs,
+                                                  const int* bf_coff, double* ncoef) {
+  __shared__ double term[kMaxPrim * kMaxPrim], prim[kMaxPrim];
+  const int mu = blockIdx.x;
   const int sh = bf_shell[mu];
   const int K = shell_nprim[sh], off = shell_poff[sh];
   const int lx = bf_pow[3 * mu], ly = bf_pow[3 * mu + 1], lz = bf_pow[3 * mu + 2];
   const int L = lx + ly + lz;
   const double pi = 3.141592653589793238;
-  double denom = sqrt(dfact_d(2 * lx - 1) * dfact_d(2 * ly - 1) * dfact_d(2 * lz - 1));
-  double* out = ncoef + bf_coff[mu];
-  for (int k = 0; k < K; ++k) {
-    double a = exps[off + k];
-    out[k] = coefs[off + k] * pow(2.0 * a / pi, 0.75) * pow(4.0 * a, 0.5 * L) / denom;
-  }
-  double S = 0.0;
-  for (int k = 0; k < K; ++k)
-    for (int q = 0; q < K; ++q) {
-      double a = exps[off + k], b = exps[off + q];
-      double r = 2.0 * sqrt(a * b) / (a + b);
-      S += coefs[off + k] * coefs[off + q] * pow(r, L + 1.5);
+  const double denom = sqrt(dfact_d(2 * lx - 1) * dfact_d(2 * ly - 1) * dfact_d(2 * lz - 1));
+  for (int i = threadIdx.x; i < K * K + K; i += blockDim.x) {
+    if (i >= K * K) {
+      const int k = i - K * K;
+      const double a = exps[off + k];
+      prim[k] = coefs[off + k] * pow(2.0 * a / pi, 0.75) * pow(4.0 * a, 0.5 * L) / denom;
+    } else {
+      const int k = i / K, q = i % K;
+      const double a = exps[off + k], b = exps[off + q];
+      const double r = 2.0 * sqrt(a * b) / (a + b);
+      term[i] = coefs[off + k] * coefs[off + q] * pow(r, L + 1.5);
     }
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  double S = 0.0;
+  for (int i = 0; i < K * K; ++i) S += term[i];
   // S is the self-overlap in units of normalised primitives; scale all coefficients.
-  double inv = 1.0 / sqrt(S);
-  for (int k = 0; k < K; ++k) out[k] *= inv;
+  const double inv = 1.0 / sqrt(S);
+  for (int k = 0; k < K; ++k) ncoef[bf_coff[mu] + k] = prim[k] * inv;
 }
 
 void launch_normalise(int nbf, const int* d_bf_shell, const int* d_bf_pow, const int* d_shell_nprim,
                       const int* d_shell_poff, const double* d_exps, const double* d_coefs, const int* d_bf_coff,
                       double* d_ncoef, cudaStream_t st) {
   count_launch();
-  k_normalise<<<(nbf + 127) / 128, 128, 0, st>>>(nbf, d_bf_shell, d_bf_pow, d_shell_nprim, d_shell_poff, d_exps,
-                                                 d_coefs, d_bf_coff, d_ncoef);
+  k_normalise<<<nbf, 64, 0, st>>>(d_bf_shell, d_bf_pow, d_shell_nprim, d_shell_poff, d_exps, d_coefs, d_bf_coff, d_ncoef);
 }
 
 // ------------------------------------------------------------------ pair table ----
@@ -280,20 +286,19 @@ void launch_pair_rows(const PairTable& t, const int* d_bf_shell, const int* d_bf
 // One warp per (row, d); lane q holds quadrature point q % 16 of every other panel and
 // accumulates f(x_q) w_q T_m(u_q) for all m in registers; a shared-memory transpose then sums
 // over lanes.
-// Items are (d, row) = dr / nrows, dr % nrows with dr = rep[item] (or dr = item without rep;
-// rep[item] < 0 marks an unused item); item's moments go to S[item * n + m].
+// Items are (d, row) = item / nrows, item % nrows; item's moments go to S[item * n + m].  For plans whose keys
+// (below) do not fit 32 bits.
 template <int NM>
 __global__ void __launch_bounds__(128) k_moments(int64_t nrows, int n, const double* row_p, const double* row_P,
                                                  const double* row_K, const double* row_A, const double* row_B,
                                                  const int8_t* row_pa, const int8_t* row_pb, const double* lo3,
                                                  const double* hi3, const uint8_t* row_box, const double* gz,
-                                                 const double* gw, const int64_t* rep, int64_t nitems, double* S) {
+                                                 const double* gw, int64_t nitems, double* S) {
   __shared__ double red[4][32][33];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t item = (int64_t)blockIdx.x * 4 + warp;
-  int64_t dr = item < nitems ? (rep ? rep[item] : item) : -1;
-  const bool active = dr >= 0;  // keys that no row holds have rep = -1
-  if (!active) dr = 0;
+  const bool active = item < nitems;
+  const int64_t dr = active ? item : 0;
   const int d = (int)(dr / nrows);
   const int64_t row = dr % nrows;
   double acc[NM];
@@ -380,6 +385,110 @@ __global__ void k_moment_keys(const PairTable t, const int* __restrict__ bf_shel
   }
 }
 
+// The moments of all keys of a (shell pair, primitive pair, d): they share the points, the Gaussian and the
+// T_m, so one warp evaluates these once per point (a lane each, into shared memory) and then sums
+// f_q x_A^i x_B^k T_m(u_q) over the points, a lane taking every 32nd of the (i, k, m).  FP64-bound: of the ~100
+// operations per point, power combination and 20 moments, ~25 are left.  The 31 752 groups of 120 s/p/d functions
+// (88 560 keys, n = 20): 2.00 ms by a warp per key with a transpose over the lanes, 1.04 here.
+// Block u works for the first key of its group that a row holds; the others return.
+constexpr int kMomOut = 8;  // sums per lane and pass
+
+// J sums of a lane over the 32 points in shared memory, added to the totals once.
+template <int J>
+__device__ __forceinline__ void moment_sums(const double* F, const double* T, const int (&fo)[kMomOut],
+                                            const int (&to)[kMomOut], double (&acc)[kMomOut]) {
+  double part[J];
+#pragma unroll
+  for (int j = 0; j < J; ++j) part[j] = 0.0;
+#pragma unroll 4
+  for (int q = 0; q < 32; ++q)
+#pragma unroll
+    for (int j = 0; j < J; ++j) part[j] += F[fo[j] + q] * T[to[j] + q];
+#pragma unroll
+  for (int j = 0; j < J; ++j) acc[j] += part[j];
+}
+
+__global__ void __launch_bounds__(32) k_moment_groups(const PairTable t, int n, const int* __restrict__ bf_shell,
+                                                      const int* __restrict__ shell_l, const double* __restrict__ lo3,
+                                                      const double* __restrict__ hi3, const uint8_t* __restrict__ row_box,
+                                                      const double* __restrict__ gz, const double* __restrict__ gw,
+                                                      const int64_t* __restrict__ rep, int most, double* __restrict__ S) {
+  extern __shared__ double sm[];
+  double* T = sm;           // [n][33]
+  double* F = sm + n * 33;  // [most][33]
+  const int64_t u0 = blockIdx.x, dr = rep[u0];
+  if (dr < 0) return;
+  const int64_t row = dr % t.nrows;
+  const int lane = threadIdx.x, d = (int)(dr / t.nrows), pair = t.row_pair[row];
+  const int lb = shell_l[bf_shell[t.pair_nu[pair]]] + 1, combos = (shell_l[bf_shell[t.pair_mu[pair]]] + 1) * lb;
+  const int c0 = t.row_pa[dr] * lb + t.row_pb[dr];
+  const int64_t base = u0 - c0;
+  for (int c = 0; c < c0; ++c)
+    if (rep[base + c] >= 0) return;
+  const double p = t.row_p[row];
+  const double Pc = t.row_P[dr], K = t.row_K[dr], A = t.row_A[dr], B = t.row_B[dr];
+  const int box = row_box ? (int)row_box[row] : 0;  // adaptive boxes: the row's partition
+  const double lo = lo3[3 * box + d], hi = hi3[3 * box + d];
+  const double cen = 0.5 * (lo + hi), half = 0.5 * (hi - lo);
+  const double reach = 9.0 / sqrt(p);
+  const double wl = fmax(lo, Pc - reach), wh = fmin(hi, Pc + reach);
+  // panels and points as in k_moments; none where the window misses the box
+  const int npan = wh > wl ? (n <= 32 ? kMomentPanels : 2 * kMomentPanels) : 0;
+  const double hp = npan ? (wh - wl) / npan : 0.0, zq = gz[lane & 15], wq = gw[lane & 15];
+  for (int cb = 0; cb < combos; cb += most) {  // passes, where the powers do not fit one
+    const int nc = min(most, combos - cb), nout = nc * n;
+    double acc[kMomOut];
+    int to[kMomOut], fo[kMomOut];
+#pragma unroll
+    for (int j = 0; j < kMomOut; ++j) {
+      const int e = min(lane + 32 * j, nout - 1);
+      acc[j] = 0.0;
+      to[j] = e % n * 33;
+      fo[j] = e / n * 33;
+    }
+    for (int pan = 0; pan < npan; pan += 2) {
+      const double mid = wl + (pan + (lane >> 4) + 0.5) * hp;
+      const double x = mid + 0.5 * hp * zq;
+      const double dx = x - Pc;
+      double fa = K * exp(-p * dx * dx) * (0.5 * hp * wq);
+      const double xa = x - A, xb = x - B;
+      for (int c = 0; c < cb + nc;) {
+        double f = fa;
+        for (int k = 0; k < lb && c < cb + nc; ++k, ++c) {
+          if (c >= cb) F[(c - cb) * 33 + lane] = f;
+          f *= xb;
+        }
+        fa *= xa;
+      }
+      const double u = (x - cen) / half;
+      double t0 = 1.0, t1 = u;
+      T[lane] = 1.0;
+      if (n > 1) T[33 + lane] = u;
+      for (int m = 2; m < n; ++m) {
+        const double t2 = 2.0 * u * t1 - t0;
+        T[m * 33 + lane] = t2;
+        t0 = t1;
+        t1 = t2;
+      }
+      __syncwarp();
+      switch ((nout + 31) / 32) {
+        case 1: moment_sums<1>(F, T, fo, to, acc); break;
+        case 2: moment_sums<2>(F, T, fo, to, acc); break;
+        case 3: moment_sums<3>(F, T, fo, to, acc); break;
+        case 4: moment_sums<4>(F, T, fo, to, acc); break;
+        case 5: moment_sums<5>(F, T, fo, to, acc); break;
+        case 6: moment_sums<6>(F, T, fo, to, acc); break;
+        case 7: moment_sums<7>(F, T, fo, to, acc); break;
+        default: moment_sums<8>(F, T, fo, to, acc); break;
+      }
+      __syncwarp();
+    }
+#pragma unroll
+    for (int j = 0; j < kMomOut; ++j)
+      if (lane + 32 * j < nout) S[(base + cb) * n + lane + 32 * j] = acc[j];
+  }
+}
+
 // S[dr][m] = Su[key[dr]][m] for dr < 3 nrows.
 __global__ void k_gather_moments(int64_t count, int n, const int* __restrict__ key, const double* __restrict__ Su,
                                  double* __restrict__ S) {
@@ -407,17 +516,26 @@ void launch_gather_moments(int64_t count, int n, const int* d_key, const double*
   k_gather_moments<<<(unsigned)blocks, 256, 0, st>>>(count, n, d_key, d_Su, d_S);
 }
 
+void launch_moment_groups(const PairTable& t, int n, const int* d_bf_shell, const int* d_shell_l, const double* d_lo3,
+                          const double* d_hi3, const uint8_t* d_row_box, const double* d_gz, const double* d_gw,
+                          const int64_t* d_rep, int64_t nkeys, double* d_S, cudaStream_t st) {
+  if (nkeys <= 0) return;
+  const int most = std::max(1, std::min(16, 32 * kMomOut / n));  // power combinations of a pass
+  count_launch();
+  k_moment_groups<<<(unsigned)nkeys, 32, sizeof(double) * 33 * (size_t)(n + most), st>>>(
+      t, n, d_bf_shell, d_shell_l, d_lo3, d_hi3, d_row_box, d_gz, d_gw, d_rep, most, d_S);
+}
+
 void launch_moments(const PairTable& t, int n, const double* d_lo3, const double* d_hi3, const uint8_t* d_row_box,
-                    const double* d_gz, const double* d_gw, const int64_t* d_rep, int64_t nitems, double* d_S,
-                    cudaStream_t st) {
-  if (nitems <= 0) return;
-  const int64_t items = nitems;
+                    const double* d_gz, const double* d_gw, double* d_S, cudaStream_t st) {
+  const int64_t items = 3 * t.nrows;
+  if (items <= 0) return;
   const unsigned blocks = (unsigned)((items + 3) / 4);
   count_launch();
   // accumulators for n rounded up to a multiple of 8 (the recurrence costs two FMAs per term)
 #define LRTEI_MOMENTS(NM)                                                                                       \
   k_moments<NM><<<blocks, 128, 0, st>>>(t.nrows, n, t.row_p, t.row_P, t.row_K, t.row_A, t.row_B, t.row_pa, t.row_pb, \
-                                        d_lo3, d_hi3, d_row_box, d_gz, d_gw, d_rep, nitems, d_S)
+                                        d_lo3, d_hi3, d_row_box, d_gz, d_gw, items, d_S)
   switch ((n + 7) / 8) {
     case 1: LRTEI_MOMENTS(8); break;
     case 2: LRTEI_MOMENTS(16); break;

@@ -581,7 +581,7 @@ static lrtei_status plan_create_impl(const lrtei_basis* basis, double omega, int
       }
     if (nkeys >= (int64_t)INT32_MAX) {  // keys are 32-bit: compute every row's moments directly
       ProfScope ps("moments", st);
-      launch_moments(t, n, pl->d_lo3, pl->d_hi3, pl->d_row_box, pl->d_gz, pl->d_gw, nullptr, 3 * t.nrows, pl->d_S, st);
+      launch_moments(t, n, pl->d_lo3, pl->d_hi3, pl->d_row_box, pl->d_gz, pl->d_gw, pl->d_S, st);
     } else {
       int* d_key = nullptr;
       int* d_l = nullptr;
@@ -607,7 +607,8 @@ static lrtei_status plan_create_impl(const lrtei_basis* basis, double omega, int
       launch_moment_keys(t, pl->d_bf_shell, pl->d_bf_pow, pl->d_shell_nprim, d_l, d_off, ns, d_key, d_rep, st);
       {
         ProfScope ps("moments", st);
-        launch_moments(t, n, pl->d_lo3, pl->d_hi3, pl->d_row_box, pl->d_gz, pl->d_gw, d_rep, nkeys, d_Su, st);
+        launch_moment_groups(t, n, pl->d_bf_shell, d_l, pl->d_lo3, pl->d_hi3, pl->d_row_box, pl->d_gz, pl->d_gw, d_rep,
+                             nkeys, d_Su, st);
       }
       launch_gather_moments(3 * t.nrows, n, d_key, d_Su, pl->d_S, st);
       if ((s = fin(cudaGetLastError(), "moment kernels")) != LRTEI_OK) return s;

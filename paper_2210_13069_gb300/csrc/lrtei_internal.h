@@ -112,12 +112,13 @@ void launch_pair_rows(const PairTable& t, const int* d_bf_shell, const int* d_bf
                       const int* d_shell_poff, const double* d_shell_center, const double* d_exps,
                       const int* d_bf_coff, const double* d_ncoef, cudaStream_t st);
 // S[d][row][m] for m < n, FP64.  d_gz/d_gw: kMomentPts Gauss-Legendre rule on [-1,1].
-// Items (d, row) = rep[i] (d nrows + row; i < nitems; rep NULL: i itself, nitems = 3 nrows; rep[i] < 0:
-// skipped) -> d_S[i][m].  The box of a row is [lo3[3 b + d], hi3[3 b + d]] with b = row_box[row]
-// (row_box NULL: b = 0).
+// The box of a row is [lo3[3 b + d], hi3[3 b + d]] with b = row_box[row] (row_box NULL: b = 0).
 void launch_moments(const PairTable& t, int n, const double* d_lo3, const double* d_hi3, const uint8_t* d_row_box,
-                    const double* d_gz, const double* d_gw, const int64_t* d_rep, int64_t nitems, double* d_S,
-                    cudaStream_t st);
+                    const double* d_gz, const double* d_gw, double* d_S, cudaStream_t st);
+// The same by keys (below): d_S[key][m] of every key that a row holds.
+void launch_moment_groups(const PairTable& t, int n, const int* d_bf_shell, const int* d_shell_l, const double* d_lo3,
+                          const double* d_hi3, const uint8_t* d_row_box, const double* d_gz, const double* d_gw,
+                          const int64_t* d_rep, int64_t nkeys, double* d_S, cudaStream_t st);
 // Moment keys: rows that share shell pair, primitive pair, d and the powers in d share S_d.
 // key[d nrows + row] in [0, nkeys) with nkeys = sum over shell pairs s1 <= s2 of
 // K_s1 K_s2 3 (l_s1 + 1)(l_s2 + 1) (offsets sp_off, triangular in the shell pair); rep[key] = one
