@@ -190,28 +190,55 @@ __global__ void __launch_bounds__(256) k_split_rows_long(const double* __restric
   }
 }
 
+// Columns j .. j + 7 of row r: of FP64 rows, or of packed densities D_r(mu, nu) (mu == nu ? 1 : 2).
+struct RowSource {
+  const double* src;
+  int64_t ld;
+  const int* map;
+  __device__ __forceinline__ void load(int64_t r, int64_t j, int64_t k, double (&v)[8]) const {
+    const bool vec = (ld & 1) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
+    load8(src + r * ld, j, k, vec, map, v);
+  }
+};
+struct DensitySource {
+  const double* D;
+  int nbf;
+  const int *mu, *nu;
+  __device__ __forceinline__ void load(int64_t r, int64_t j, int64_t k, double (&v)[8]) const {
+    const double* x = D + r * nbf * nbf;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      v[u] = 0.0;
+      if (j + u < k) {
+        const int a = mu[j + u], b = nu[j + u];
+        v[u] = x[a * nbf + b] * (a == b ? 1.0 : 2.0);
+      }
+    }
+  }
+};
+
 // Few long rows (fewer rows than SMs, e.g. the R density rows of a J-build): a cluster of
 // kSplitCluster CTAs per row, each taking an eighth of the padded row.  Every CTA reduces the
 // magnitude bits over its share, the cluster combines the eight maxima through distributed shared
 // memory, and each CTA slices its share with the row's exponent: the exponent and the slices are
-// those of the one-block-per-row kernels.
+// those of the one-block-per-row kernels.  A share of one step stays in registers between the two.
+// 32 densities of 180 functions: 15.5 us packed, transposed and sliced by three kernels, 8.8 from the densities.
 constexpr int kSplitCluster = 8;
+template <class Source>
 __global__ void __cluster_dims__(kSplitCluster, 1, 1) __launch_bounds__(256)
-    k_split_rows_cluster(const double* __restrict__ src, int64_t k, int64_t ld, int64_t kpad, int tile,
-                         const int* __restrict__ map, uint16_t* __restrict__ d, int* __restrict__ expo) {
+    k_split_rows_cluster(Source src, int64_t k, int64_t kpad, int tile, uint16_t* __restrict__ d,
+                         int* __restrict__ expo) {
   __shared__ uint64_t red[8];
   __shared__ uint64_t share;
   cg::cluster_group cluster = cg::this_cluster();
   const unsigned rank = cluster.block_rank();
   const int64_t r = blockIdx.y;
-  const double* x = src + r * ld;
-  const bool vec = (ld & 1) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
   const int64_t per = (kpad / 8 + kSplitCluster - 1) / kSplitCluster * 8;
   const int64_t c0 = (int64_t)rank * per, c1 = min(kpad, c0 + per);
   uint64_t mx = 0;
   double v[8];
   for (int64_t j = c0 + 8 * (int64_t)threadIdx.x; j < c1; j += 8 * (int64_t)blockDim.x) {
-    load8(x, j, k, vec, map, v);
+    src.load(r, j, k, v);
     mx = max_mag(v, mx);
   }
   for (int o = 16; o > 0; o >>= 1) {
@@ -237,8 +264,9 @@ __global__ void __cluster_dims__(kSplitCluster, 1, 1) __launch_bounds__(256)
   if (mxd > 0.0) frexp(mxd * (256.0 / 255.0), &e);
   const bool nz = mxd > 0.0 && e >= -1000;
   if (rank == 0 && threadIdx.x == 0) expo[r] = e;
+  const bool once = per <= 8 * (int64_t)blockDim.x;
   for (int64_t j = c0 + 8 * (int64_t)threadIdx.x; j < c1; j += 8 * (int64_t)blockDim.x) {
-    load8(x, j, k, vec, map, v);
+    if (!once) src.load(r, j, k, v);
     store_slices(v, e, nz, r, j, k, tile, kpad, d);
   }
 }
@@ -405,7 +433,39 @@ __global__ void k_reduce_splits(const double* __restrict__ part, int splits, int
   }
 }
 
+// Few outputs of many parts (the exchange's N_b x N_b): a block per 32 outputs, eight threads to each.  75 x 75
+// outputs of 128 parts: 30 us by a thread each, 5.3 here.
+__global__ void __launch_bounds__(256) k_reduce_many(const double* __restrict__ part, int splits, int64_t stride,
+                                                     int64_t rows, int64_t cols, int64_t ld, double* __restrict__ out,
+                                                     int64_t ldo) {
+  __shared__ double sum[8][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t t = blockIdx.x * (int64_t)32 + lane, i = t / cols, j = t % cols;
+  double s = 0.0;
+  if (i < rows) {
+    const double* x = part + i * ld + j;
+#pragma unroll 8
+    for (int q = w; q < splits; q += 8) s += x[q * stride];
+  }
+  sum[w][lane] = s;
+  __syncthreads();
+  if (w == 0 && i < rows) {
+#pragma unroll
+    for (int q = 1; q < 8; ++q) s += sum[q][lane];
+    out[i * ldo + j] = s;
+  }
+}
+
 }  // namespace tc
+
+bool launch_split_density(const PairTable& t, int nbf, int64_t R, const double* d_D, const SplitMatrix& m,
+                          cudaStream_t st) {
+  if (R <= 0 || R >= 4 * 152 || m.plain) return false;
+  count_launch();
+  tc::k_split_rows_cluster<<<dim3(tc::kSplitCluster, (unsigned)R), 256, 0, st>>>(
+      tc::DensitySource{d_D, nbf, t.pair_mu, t.pair_nu}, t.npair, m.kpad, m.tile, m.d, m.expo);
+  return true;
+}
 
 void launch_split_rows(const double* d_src, int64_t rows, int64_t k, int64_t ld, const SplitMatrix& m, const int* d_map,
                        cudaStream_t st) {
@@ -423,8 +483,8 @@ void launch_split_rows(const double* d_src, int64_t rows, int64_t k, int64_t ld,
   // few long rows (fewer than four per SM, e.g. the R density rows of a J-build or the N_b rows of
   // the exchange's last product): eight CTAs per row
   if ((rows < 4 * 152 && k >= 8192) || (rows < 152 && k >= 2048)) {
-    tc::k_split_rows_cluster<<<dim3(tc::kSplitCluster, (unsigned)rows), 256, 0, st>>>(d_src, k, ld, m.kpad, m.tile, d_map,
-                                                                                     m.d, m.expo);
+    tc::k_split_rows_cluster<<<dim3(tc::kSplitCluster, (unsigned)rows), 256, 0, st>>>(
+        tc::RowSource{d_src, ld, d_map}, k, m.kpad, m.tile, m.d, m.expo);
     return;
   }
   const int64_t cols = d_map ? ld : k;  // a mapped row's columns lie anywhere in it
@@ -484,6 +544,10 @@ void launch_reduce_splits(const double* part, int splits, int64_t stride, int64_
   int64_t b = (total + 255) / 256;
   if (b > 152 * 32) b = 152 * 32;
   count_launch();
+  if (splits > 32 && total <= 152 * 256) {  // one output per thread would leave SMs without work
+    tc::k_reduce_many<<<(unsigned)((total + 31) / 32), 256, 0, st>>>(part, splits, stride, rows, cols, ld, out, ldo);
+    return;
+  }
   tc::k_reduce_splits<<<(unsigned)b, 256, 0, st>>>(part, splits, stride, rows, cols, ld, out, ldo);
 }
 

@@ -2019,9 +2019,7 @@ static lrtei_status jbuild_tc(lrtei_plan* plan, const double* d_D, int R, double
   const int64_t npair = plan->t.npair, n3 = (int64_t)n * n * n;
   LRTEI_TRY(ensure_jbuild_operands(plan, st));  // K carries the prefactor omega / sqrt(pi)
   Scratch sc(st);
-  double *Du, *DuT, *XT, *YT, *Ju, *part;
-  LRTEI_TRY(sc.get(&Du, (size_t)npair * R));
-  LRTEI_TRY(sc.get(&DuT, (size_t)npair * R));
+  double *XT, *YT, *Ju, *part;
   LRTEI_TRY(sc.get(&XT, (size_t)R * n3));
   const ParityClasses& pc = plan->pc;
   LRTEI_TRY(sc.get(&YT, (size_t)R * pc.cols));
@@ -2033,9 +2031,17 @@ static lrtei_status jbuild_tc(lrtei_plan* plan, const double* d_D, int R, double
   LRTEI_TRY(scratch_split(sc, Dsp, R, npair, split_tile(R), plan));
   LRTEI_TRY(scratch_split(sc, Xsp, R, n3, split_tile(R), plan));
   LRTEI_TRY(scratch_split(sc, Ysp, R, n3, split_tile(R), plan));
-  launch_pack_density(nbf, R, d_D, Du, st);
-  launch_transpose(Du, npair, R, R, DuT, npair, st);
+  bool sliced;
   {
+    ProfScope ps("split", st);
+    sliced = launch_split_density(plan->t, nbf, R, d_D, Dsp, st);
+  }
+  if (!sliced) {
+    double *Du, *DuT;
+    LRTEI_TRY(sc.get(&Du, (size_t)npair * R));
+    LRTEI_TRY(sc.get(&DuT, (size_t)npair * R));
+    launch_pack_density(nbf, R, d_D, Du, st);
+    launch_transpose(Du, npair, R, R, DuT, npair, st);
     ProfScope ps("split", st);
     launch_split_rows(DuT, R, npair, npair, Dsp, nullptr, st);
   }

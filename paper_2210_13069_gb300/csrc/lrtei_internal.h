@@ -343,6 +343,10 @@ inline int split_tile(int64_t N) { return N <= 32 ? 32 : N <= 64 ? 64 : 128; }
 // source column d_map[j] (NULL: j).
 void launch_split_rows(const double* d_src, int64_t rows, int64_t k, int64_t ld, const SplitMatrix& m, const int* d_map,
                        cudaStream_t st);
+// R densities D as rows over the unique pairs (the off-diagonal ones doubled) into slices; false, and nothing
+// launched, where a plain operand or too many rows want the packed copy.
+bool launch_split_density(const PairTable& t, int nbf, int64_t R, const double* d_D, const SplitMatrix& m,
+                          cudaStream_t st);
 // C = scale * A B^T through tcgen05 (see k_tcgen05.cu).  A: rows [a_row0, a_row0 + M) of its operand; B: N rows;
 // shared kpad (multiple of 256).  transpose_out writes C^T; symmetric_upper computes the
 // upper-triangular 128x128 blocks of a square C and mirrors them.
