@@ -13,29 +13,13 @@ namespace cg = cooperative_groups;
 namespace lrtei {
 namespace tc {
 
-// Largest |x| of the row from the bit patterns (finite inputs order like their magnitudes),
-// then e with max|x| * 256/255 < 2^e (0 for an all-zero row).
-__device__ __forceinline__ int row_exponent(uint64_t mxbits, uint64_t* red, bool& nonzero) {
-  for (int o = 16; o > 0; o >>= 1) {
-    const uint64_t other = __shfl_xor_sync(0xffffffffu, mxbits, o);
-    mxbits = other > mxbits ? other : mxbits;
-  }
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mxbits;
+// The block's largest magnitude, on all its threads (red: a word per warp).
+__device__ __forceinline__ uint32_t block_max(uint32_t mx, uint32_t* red) {
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  const unsigned lane = threadIdx.x & 31;
+  if (lane == 0) red[threadIdx.x >> 5] = mx;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    uint64_t v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0ULL;
-    for (int o = 16; o > 0; o >>= 1) {
-      const uint64_t other = __shfl_xor_sync(0xffffffffu, v, o);
-      v = other > v ? other : v;
-    }
-    if (threadIdx.x == 0) red[0] = v;
-  }
-  __syncthreads();
-  const double mx = __longlong_as_double((long long)red[0]);
-  int e = 0;
-  if (mx > 0.0) frexp(mx * (256.0 / 255.0), &e);
-  nonzero = mx > 0.0 && e >= -1000;  // rows below ~1e-301 are treated as zero
-  return e;
+  return __reduce_max_sync(0xffffffffu, lane < (blockDim.x >> 5) ? red[lane] : 0u);
 }
 
 // Where the eight consecutive columns j .. j + 7 (j a multiple of 8) of row i go: tiles of `tile` rows x 16
@@ -85,13 +69,43 @@ __device__ __forceinline__ void load8(const double* __restrict__ x, int64_t j, i
   }
 }
 
-__device__ __forceinline__ uint64_t max_mag(const double (&v)[8], uint64_t mx) {
+__device__ __forceinline__ uint32_t max_mag(const double (&v)[8], uint32_t mx) {
 #pragma unroll
-  for (int u = 0; u < 8; ++u) {
-    const uint64_t a = (uint64_t)__double_as_longlong(v[u]) & 0x7FFFFFFFFFFFFFFFULL;
-    mx = a > mx ? a : mx;
-  }
+  for (int u = 0; u < 8; ++u) mx = max(mx, magnitude(v[u]));
   return mx;
+}
+
+// A row staged in shared memory (16-byte aligned) into columns j0 .. j0 + n of operand row i, j0 a multiple of 8 and n
+// of 2; zeros from its column k on.  A thread takes two neighbouring columns: the reads have no bank conflicts
+// (eight columns of one thread are 16-way ones) and a warp's stores fill whole sectors.  16290 rows of 13824 (3.15 GB):
+// 0.84 ms by eight columns, 0.61 by two; 1035 rows of 2197 12.8 us, 9.3.
+__device__ __forceinline__ void store_row(const double* __restrict__ row, const int* __restrict__ map, int64_t k, int e,
+                                          int64_t i, int64_t j0, int64_t n, int tile, int64_t kpad,
+                                          uint16_t* __restrict__ d) {
+  const bool nz = e != kZeroRowExpo;
+  const int rr = (int)(i % tile), sw = (rr >> 2) & 1;
+  uint16_t* base = d + (i / tile) * (kpad / 16) * (int64_t)(3 * tile * 16) + rr * 16;
+  for (int j = 2 * (int)threadIdx.x; j < n; j += 2 * (int)blockDim.x) {
+    const bool l0 = nz && j < k, l1 = nz && j + 1 < k;
+    double x = 0.0, y = 0.0;
+    if (map) {
+      if (l0) x = row[map[j]];
+      if (l1) y = row[map[j + 1]];
+    } else if (l1) {
+      const double2 t = *reinterpret_cast<const double2*>(row + j);
+      x = t.x;
+      y = t.y;
+    } else if (l0) {
+      x = row[j];
+    }
+    uint32_t p0, p1, p2;
+    slice_pair(x, y, e, l0, l1, p0, p1, p2);
+    const int64_t c = j0 + j;
+    uint16_t* o = base + (c >> 4) * (int64_t)(3 * tile * 16) + ((int)((c >> 3) & 1) ^ sw) * 8 + (int)(c & 7);
+    *reinterpret_cast<uint32_t*>(o) = p0;
+    *reinterpret_cast<uint32_t*>(o + tile * 16) = p1;
+    *reinterpret_cast<uint32_t*>(o + 2 * tile * 16) = p2;
+  }
 }
 
 // Short rows (padded length at most 256): one warp per row, eight consecutive elements per lane.
@@ -107,17 +121,9 @@ __global__ void __launch_bounds__(256) k_split_rows_warp(const double* __restric
   const int64_t i0 = 8 * (int64_t)lane;
   double v[8];
   load8(x, i0, k, vec, map, v);
-  uint64_t mx = max_mag(v, 0);
-  for (int o = 16; o > 0; o >>= 1) {
-    const uint64_t other = __shfl_xor_sync(0xffffffffu, mx, o);
-    mx = other > mx ? other : mx;
-  }
-  const double mxd = __longlong_as_double((long long)mx);
-  int e = 0;
-  if (mxd > 0.0) frexp(mxd * (256.0 / 255.0), &e);
-  const bool nz = mxd > 0.0 && e >= -1000;  // rows below ~1e-301 are treated as zero
+  const int e = slice_exponent(__reduce_max_sync(0xffffffffu, max_mag(v, 0)));
   if (lane == 0) expo[r] = e;
-  if (i0 < kpad) store_slices(v, e, nz, r, i0, k, tile, kpad, d);
+  if (i0 < kpad) store_slices(v, e, e != kZeroRowExpo, r, i0, k, tile, kpad, d);
 }
 
 // One block per row, the row staged in shared memory (rows of up to kSplitCols columns): read once, by one
@@ -128,12 +134,12 @@ __global__ void __launch_bounds__(512) k_split_rows(const double* __restrict__ s
                                                     int64_t kpad, int tile, int bulk, const int* __restrict__ map,
                                                     uint16_t* __restrict__ d, int* __restrict__ expo) {
   extern __shared__ __align__(16) double row[];  // cols: the source row's columns (k without a map)
-  __shared__ uint64_t red[32];
+  __shared__ uint32_t red[32];
   __shared__ uint64_t bar;
   const int64_t r = blockIdx.x;
   const double* x = src + r * ld;
   const int nc = (int)cols;
-  uint64_t mx = 0;
+  uint32_t mx = 0;
   if (bulk) {
     if (threadIdx.x == 0) {
       mbar_init(&bar, 1);
@@ -144,45 +150,37 @@ __global__ void __launch_bounds__(512) k_split_rows(const double* __restrict__ s
     __syncthreads();
     for (long long t0 = clock64(); !mbar_try_wait(&bar, 0u) && clock64() - t0 < kWaitCycles;) {
     }
-    for (int i = threadIdx.x; i < nc; i += blockDim.x) {
-      const uint64_t a = (uint64_t)__double_as_longlong(row[i]) & 0x7FFFFFFFFFFFFFFFULL;
-      mx = a > mx ? a : mx;
-    }
+#pragma unroll 4
+    for (int i = threadIdx.x; i < nc; i += blockDim.x) mx = max(mx, magnitude(row[i]));
   } else {
 #pragma unroll 4
     for (int i = threadIdx.x; i < nc; i += blockDim.x) {
-      row[i] = x[i];
-      const uint64_t a = (uint64_t)__double_as_longlong(row[i]) & 0x7FFFFFFFFFFFFFFFULL;
-      mx = a > mx ? a : mx;
+      const double v = x[i];
+      row[i] = v;
+      mx = max(mx, magnitude(v));
     }
   }
-  bool nz;
-  const int e = row_exponent(mx, red, nz);  // (synchronises: the whole row is staged)
+  const int e = slice_exponent(block_max(mx, red));  // (synchronises: the whole row is staged)
   if (threadIdx.x == 0) expo[r] = e;
-  for (int64_t j = 8 * (int64_t)threadIdx.x; j < kpad; j += 8 * (int64_t)blockDim.x) {
-    double v[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = j + u < k ? row[map ? map[j + u] : (int)j + u] : 0.0;
-    store_slices(v, e, nz, r, j, k, tile, kpad, d);
-  }
+  store_row(row, map, k, e, r, 0, kpad, tile, kpad, d);
 }
 
 // Longer rows: two passes, the second from L2.
 __global__ void __launch_bounds__(256) k_split_rows_long(const double* __restrict__ src, int64_t k, int64_t ld,
                                                          int64_t kpad, int tile, const int* __restrict__ map,
                                                          uint16_t* __restrict__ d, int* __restrict__ expo) {
-  __shared__ uint64_t red[32];
+  __shared__ uint32_t red[32];
   const int64_t r = blockIdx.x;
   const double* x = src + r * ld;
   const bool vec = (ld & 1) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
-  uint64_t mx = 0;
-  bool nz;
+  uint32_t mx = 0;
   double v[8];
   for (int64_t j = 8 * (int64_t)threadIdx.x; j < k; j += 2048) {
     load8(x, j, k, vec, map, v);
     mx = max_mag(v, mx);
   }
-  const int e = row_exponent(mx, red, nz);
+  const int e = slice_exponent(block_max(mx, red));
+  const bool nz = e != kZeroRowExpo;
   if (threadIdx.x == 0) expo[r] = e;
   for (int64_t j = 8 * (int64_t)threadIdx.x; j < kpad; j += 2048) {
     load8(x, j, k, vec, map, v);
@@ -228,41 +226,27 @@ template <class Source>
 __global__ void __cluster_dims__(kSplitCluster, 1, 1) __launch_bounds__(256)
     k_split_rows_cluster(Source src, int64_t k, int64_t kpad, int tile, uint16_t* __restrict__ d,
                          int* __restrict__ expo) {
-  __shared__ uint64_t red[8];
-  __shared__ uint64_t share;
+  __shared__ uint32_t red[32];
+  __shared__ uint32_t share;
   cg::cluster_group cluster = cg::this_cluster();
   const unsigned rank = cluster.block_rank();
   const int64_t r = blockIdx.y;
   const int64_t per = (kpad / 8 + kSplitCluster - 1) / kSplitCluster * 8;
   const int64_t c0 = (int64_t)rank * per, c1 = min(kpad, c0 + per);
-  uint64_t mx = 0;
+  uint32_t mx = 0;
   double v[8];
   for (int64_t j = c0 + 8 * (int64_t)threadIdx.x; j < c1; j += 8 * (int64_t)blockDim.x) {
     src.load(r, j, k, v);
     mx = max_mag(v, mx);
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    const uint64_t other = __shfl_xor_sync(0xffffffffu, mx, o);
-    mx = other > mx ? other : mx;
-  }
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    uint64_t m = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = red[w] > m ? red[w] : m;
-    share = m;
-  }
+  mx = block_max(mx, red);
+  if (threadIdx.x == 0) share = mx;
   cluster.sync();  // every CTA's share is written
-  uint64_t all = 0;
-  for (int q = 0; q < kSplitCluster; ++q) {
-    const uint64_t o = *cluster.map_shared_rank(&share, q);
-    all = o > all ? o : all;
-  }
+  uint32_t all = 0;
+  for (int q = 0; q < kSplitCluster; ++q) all = max(all, *cluster.map_shared_rank(&share, q));
   cluster.sync();  // every CTA has read the shares before any of them exits
-  const double mxd = __longlong_as_double((long long)all);
-  int e = 0;
-  if (mxd > 0.0) frexp(mxd * (256.0 / 255.0), &e);
-  const bool nz = mxd > 0.0 && e >= -1000;
+  const int e = slice_exponent(all);
+  const bool nz = e != kZeroRowExpo;
   if (rank == 0 && threadIdx.x == 0) expo[r] = e;
   const bool once = per <= 8 * (int64_t)blockDim.x;
   for (int64_t j = c0 + 8 * (int64_t)threadIdx.x; j < c1; j += 8 * (int64_t)blockDim.x) {
@@ -273,46 +257,41 @@ __global__ void __cluster_dims__(kSplitCluster, 1, 1) __launch_bounds__(256)
 
 // ---- operands of the long-range exchange, sliced where they lie (no transposed or permuted FP64 copies)
 // Rows (mu, m) of MT, columns la: F_u(pair(mu, la), m), N_b <= 256 columns.  One CTA per mu and 32 columns m of
-// F_u: the rows of F_u are read along m into shared memory, the row maxima are taken, then the slices stored.  Blocks beyond the last column but one are not read by the products and stay
-// unwritten.  Gather and slicing of 2.5 M rows of 180 took 1.66 + 1.65 ms through a 3.6 GB copy.
+// F_u: the rows of F_u are read along m into shared memory, a column per lane, which also takes its maximum; then the
+// slices are stored.  Blocks beyond the last column but one are not read by the products and stay unwritten.
+// 2.5 M rows of 180: 3.3 ms through a gathered 3.6 GB copy, 1.67 with a warp per row maximum, 1.23 now (6.5 GB).
 __global__ void __launch_bounds__(256) k_split_MT(int nbf, int64_t n3, const double* __restrict__ F, int64_t ldF,
                                                   int64_t kpad, int kuse, int tile, uint16_t* __restrict__ d,
                                                   int* __restrict__ expo) {
   extern __shared__ double t[];  // [nbf][33]
+  __shared__ uint32_t top[8][32];
+  __shared__ int re[32];  // row exponents
   const int mu = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t m0 = (int64_t)blockIdx.x * 32;
+  const double* src = F + m0 + lane;
+  const bool in = m0 + lane < n3;
+  uint32_t mx = 0;
   for (int l0 = warp; l0 < nbf; l0 += 64) {  // eight rows' loads in flight per warp
     double v[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const int la = l0 + 8 * u, lo = mu < la ? mu : la, hi = mu < la ? la : mu;
-      const int64_t r = (int64_t)lo * nbf - (int64_t)lo * (lo - 1) / 2 + (hi - lo);
-      v[u] = la < nbf && m0 + lane < n3 ? F[r * ldF + m0 + lane] : 0.0;
+      const int la = l0 + 8 * u, lo = min(mu, la), hi = max(mu, la);
+      const int r = lo * nbf - lo * (lo - 1) / 2 + (hi - lo);
+      v[u] = la < nbf && in ? src[r * ldF] : 0.0;
     }
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
+    for (int u = 0; u < 8; ++u) {
+      mx = max(mx, magnitude(v[u]));
       if (l0 + 8 * u < nbf) t[(l0 + 8 * u) * 33 + lane] = v[u];
+    }
   }
+  top[warp][lane] = mx;
   __syncthreads();
-  __shared__ int re[32];  // row exponents; kZeroRow: nothing to slice
-  constexpr int kZeroRow = 1 << 20;
-  for (int q = warp; q < 32; q += 8) {
-    uint64_t mx = 0;
-    for (int la = lane; la < nbf; la += 32) {
-      const uint64_t a = (uint64_t)__double_as_longlong(t[la * 33 + q]) & 0x7FFFFFFFFFFFFFFFULL;
-      mx = a > mx ? a : mx;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      const uint64_t other = __shfl_xor_sync(0xffffffffu, mx, o);
-      mx = other > mx ? other : mx;
-    }
-    if (lane == 0) {
-      const double mxd = __longlong_as_double((long long)mx);
-      int e = 0;
-      if (mxd > 0.0) frexp(mxd * (256.0 / 255.0), &e);
-      re[q] = mxd > 0.0 && e >= -1000 ? e : kZeroRow;
-      if (m0 + q < n3) expo[(int64_t)mu * n3 + m0 + q] = e;
-    }
+  if (warp == 0) {
+#pragma unroll
+    for (int w = 1; w < 8; ++w) mx = max(mx, top[w][lane]);
+    re[lane] = slice_exponent(mx);
+    if (in) expo[(int64_t)mu * n3 + m0 + lane] = re[lane];
   }
   __syncthreads();
   // a warp takes 16 rows of one 16-column block, a lane half a row of it: 512 contiguous bytes per plane and store
@@ -324,35 +303,31 @@ __global__ void __launch_bounds__(256) k_split_MT(int nbf, int64_t n3, const dou
 #pragma unroll
     for (int u = 0; u < 8; ++u) v[u] = c0 + u < nbf ? t[(c0 + u) * 33 + q] : 0.0;
     const int e = re[q];
-    store_slices(v, e, e != kZeroRow, (int64_t)mu * n3 + m0 + q, c0, nbf, tile, kpad, d);
+    store_slices(v, e, e != kZeroRowExpo, (int64_t)mu * n3 + m0 + q, c0, nbf, tile, kpad, d);
   }
 }
 
-// Largest magnitude (bits) over the rows (j, mu), j < nj, of Z for each mu: the row maxima of Zp[mu][(j, m)].
+// Largest magnitude over the rows (j, mu), j < nj, of Z for each mu: the row maxima of Zp[mu][(j, m)].
 __global__ void __launch_bounds__(256) k_orbital_max(int nbf, int64_t cols, int64_t ld, const double* __restrict__ Z,
-                                                     unsigned long long* __restrict__ mx) {
+                                                     uint32_t* __restrict__ mx) {
+  __shared__ uint32_t red[32];
   const int64_t row = blockIdx.x;  // j nbf + mu
   const double* x = Z + row * ld;
-  unsigned long long v = 0;
-#pragma unroll 4
-  for (int64_t m = threadIdx.x; m < cols; m += 256) {
-    const unsigned long long a = (unsigned long long)__double_as_longlong(x[m]) & 0x7FFFFFFFFFFFFFFFULL;
-    v = a > v ? a : v;
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long other = __shfl_xor_sync(0xffffffffu, v, o);
-    v = other > v ? other : v;
-  }
-  if ((threadIdx.x & 31) == 0) atomicMax(mx + row % nbf, v);
+  uint32_t v = 0;
+#pragma unroll 8
+  for (int64_t m = threadIdx.x; m < cols; m += 256) v = max(v, magnitude(x[m]));
+  v = block_max(v, red);
+  if (threadIdx.x == 0) atomicMax(mx + row % nbf, v);
 }
 
 // Zp[mu][(j, m)] = Z[(j, mu)][map[m]] into slices (n3 a multiple of 8): one CTA per row (j, mu), staged by one
-// bulk copy, with the exponent of row mu.
-__global__ void __launch_bounds__(512) k_split_orbital_rows(int nbf, int64_t n3, int64_t cols, int64_t ld,
+// bulk copy, with the exponent of row mu: of its largest magnitude, or the largest of Z's row exponents (an exponent
+// grows with the magnitude; saves the pass for the maxima where Z's rows are sliced anyway).
+__global__ void __launch_bounds__(512) k_split_orbital_rows(int nbf, int64_t n3, int nj, int64_t cols, int64_t ld,
                                                             const double* __restrict__ Z, const int* __restrict__ map,
-                                                            const unsigned long long* __restrict__ mx, int64_t k,
-                                                            int64_t kpad, int tile, uint16_t* __restrict__ d,
-                                                            int* __restrict__ expo) {
+                                                            const uint32_t* __restrict__ mx,
+                                                            const int* __restrict__ row_expo, int64_t k, int64_t kpad,
+                                                            int tile, uint16_t* __restrict__ d, int* __restrict__ expo) {
   extern __shared__ __align__(16) double row[];
   __shared__ uint64_t bar;
   const int64_t i = blockIdx.x;
@@ -363,26 +338,20 @@ __global__ void __launch_bounds__(512) k_split_orbital_rows(int nbf, int64_t n3,
     mbar_arrive_expect_tx(&bar, (uint32_t)(cols * 8));
     bulk_load(row, Z + i * ld, (uint32_t)(cols * 8), &bar);
   }
-  const double mxd = __longlong_as_double((long long)mx[mu]);
-  int e = 0;
-  if (mxd > 0.0) frexp(mxd * (256.0 / 255.0), &e);
-  const bool nz = mxd > 0.0 && e >= -1000;
+  int e = kZeroRowExpo;
+  if (row_expo) {
+    for (int q = threadIdx.x & 31; q < nj; q += 32) e = max(e, row_expo[(int64_t)q * nbf + mu]);
+    e = __reduce_max_sync(0xffffffffu, e);
+  } else {
+    e = slice_exponent(mx[mu]);
+  }
   if (j == 0 && threadIdx.x == 0) expo[mu] = e;
   __syncthreads();
   for (long long t0 = clock64(); !mbar_try_wait(&bar, 0u) && clock64() - t0 < kWaitCycles;) {
   }
-  const int64_t c0 = (int64_t)j * n3;
-  for (int64_t m = 8 * (int64_t)threadIdx.x; m < n3; m += 8 * (int64_t)blockDim.x) {
-    double v[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = row[map ? map[m + u] : (int)m + u];
-    store_slices(v, e, nz, mu, c0 + m, k, tile, kpad, d);
-  }
-  if ((int64_t)(j + 1) * n3 == k) {  // the padding after the last orbital
-    double z[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int64_t c = k + 8 * (int64_t)threadIdx.x; c < kpad; c += 8 * (int64_t)blockDim.x)
-      store_slices(z, e, nz, mu, c, k, tile, kpad, d);
-  }
+  store_row(row, map, n3, e, mu, (int64_t)j * n3, n3, tile, kpad, d);
+  if ((int64_t)(j + 1) * n3 == k)  // the padding after the last orbital
+    store_row(row, nullptr, 0, e, mu, k, kpad - k, tile, kpad, d);
 }
 
 // Plain BF16 operands: one rounded copy per element, exponent 8 so that the epilogue scale
@@ -515,17 +484,20 @@ bool launch_split_MT(int nbf, int64_t n3, const double* d_F, int64_t ldF, const 
 }
 
 bool launch_split_orbitals(int nbf, int64_t n3, int nj, const double* d_Z, int64_t cols, const int* d_map,
-                           unsigned long long* d_max, const SplitMatrix& m, cudaStream_t st) {
+                           uint32_t* d_max, const int* d_row_expo, const SplitMatrix& m, cudaStream_t st) {
   if (m.plain || n3 % 8 != 0 || cols % 2 != 0 || cols > tc::kSplitCols || (reinterpret_cast<uintptr_t>(d_Z) & 15)) return false;
   static bool attr_set = false;
   if (!attr_set)
     attr_set = cudaFuncSetAttribute(tc::k_split_orbital_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)(sizeof(double) * tc::kSplitCols)) == cudaSuccess;
-  cudaMemsetAsync(d_max, 0, sizeof(unsigned long long) * (size_t)nbf, st);
-  count_launches(2);
-  tc::k_orbital_max<<<(unsigned)((int64_t)nj * nbf), 256, 0, st>>>(nbf, cols, cols, d_Z, d_max);
+  if (!d_row_expo) {
+    cudaMemsetAsync(d_max, 0, sizeof(uint32_t) * (size_t)nbf, st);
+    count_launch();
+    tc::k_orbital_max<<<(unsigned)((int64_t)nj * nbf), 256, 0, st>>>(nbf, cols, cols, d_Z, d_max);
+  }
+  count_launch();
   tc::k_split_orbital_rows<<<(unsigned)((int64_t)nj * nbf), cols > 8192 ? 512 : 256, sizeof(double) * (size_t)cols, st>>>(
-      nbf, n3, cols, cols, d_Z, d_map, d_max, m.k, m.kpad, m.tile, m.d, m.expo);
+      nbf, n3, nj, cols, cols, d_Z, d_map, d_max, d_row_expo, m.k, m.kpad, m.tile, m.d, m.expo);
   return true;
 }
 

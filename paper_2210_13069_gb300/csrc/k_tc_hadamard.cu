@@ -48,7 +48,6 @@ constexpr int QC = BN / (EPI / 4);  // columns per epilogue thread (16)
 constexpr uint32_t A_PLANE = BM * BK * 2;            // one T slice plane of a 32-deep step
 constexpr uint32_t A_STAGE = 3 * A_PLANE;            // 24 KB
 constexpr uint32_t B_PLANE = BN * BK * 2;            // one S slice plane of a 32-deep step
-constexpr int kZeroRowExpo = -30000;  // exponent of an all-zero slice row: its products vanish
 
 template <int KS>
 struct Cfg {
@@ -405,18 +404,9 @@ __global__ void k_slice_short_rows(const double* __restrict__ src, int64_t rows,
   if (row >= rows) return;
   const double* x = src + row * n;
   const double x0 = lane < n ? x[lane] : 0.0, x1 = lane + 32 < n ? x[lane + 32] : 0.0;
-  uint64_t mx = (uint64_t)__double_as_longlong(x0) & 0x7FFFFFFFFFFFFFFFULL;
-  const uint64_t m1 = (uint64_t)__double_as_longlong(x1) & 0x7FFFFFFFFFFFFFFFULL;
-  mx = m1 > mx ? m1 : mx;
-  for (int o = 16; o > 0; o >>= 1) {
-    const uint64_t other = __shfl_xor_sync(0xffffffffu, mx, o);
-    mx = other > mx ? other : mx;
-  }
-  const double m = __longlong_as_double((long long)mx);
-  int e = 0;
-  if (m > 0.0) frexp(m * (256.0 / 255.0), &e);
-  const bool nz = m > 0.0 && e >= -1000;
-  if (lane == 0) expo[row] = nz ? e : kZeroRowExpo;
+  const int e = slice_exponent(__reduce_max_sync(0xffffffffu, max(magnitude(x0), magnitude(x1))));
+  const bool nz = e != kZeroRowExpo;
+  if (lane == 0) expo[row] = e;
   if (lane < kpad) slice_store(x0, e, nz && lane < n, row * kpad + lane, s0, s1, s2, s1h);
   if (lane + 32 < kpad) slice_store(x1, e, nz && lane + 32 < n, row * kpad + lane + 32, s0, s1, s2, s1h);
 }

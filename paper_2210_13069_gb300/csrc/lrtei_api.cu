@@ -1839,7 +1839,7 @@ lrtei_status lrtei_exchange(lrtei_plan* plan, const double* d_Q, int norb, doubl
   LRTEI_TRY(sc.get(&Y, (size_t)ob * nbf * ycols));
   LRTEI_TRY(sc.get(&Kb, (size_t)nblk * nbf * nbf));
   if (tc) {
-    unsigned long long* dmax;
+    uint32_t* dmax;
     LRTEI_TRY(sc.get(&dmax, (size_t)nbf));
     SplitMatrix Qsp, MTsp, Xsp, Ypsp, Xpsp;
     LRTEI_TRY(scratch_split(sc, Qsp, norb, nbf, 128, plan));
@@ -1877,12 +1877,12 @@ lrtei_status lrtei_exchange(lrtei_plan* plan, const double* d_Q, int norb, doubl
       Xa.set_k((int64_t)nj * n3);
       {
         ProfScope ps("split", st);
-        if (!launch_split_orbitals(nbf, n3, nj, Y, ycols, plan->d_pos, dmax, Ya, st)) {
+        if (!launch_split_orbitals(nbf, n3, nj, Y, ycols, plan->d_pos, dmax, nullptr, Ya, st)) {
           LRTEI_TRY(need_copy(&Yp, (size_t)ob * rowlen));
           launch_perm_orbital_rows(nbf, n3, nj, Y, ycols, plan->d_pos, Yp, st);
           launch_split_rows(Yp, nbf, (int64_t)nj * n3, (int64_t)nj * n3, Ya, nullptr, st);
         }
-        if (!launch_split_orbitals(nbf, n3, nj, X, n3, nullptr, dmax, Xa, st)) {
+        if (!launch_split_orbitals(nbf, n3, nj, X, n3, nullptr, dmax, Xb.expo, Xa, st)) {
           LRTEI_TRY(need_copy(&Xp, (size_t)ob * rowlen));
           launch_perm_orbital_rows(nbf, n3, nj, X, n3, nullptr, Xp, st);
           launch_split_rows(Xp, nbf, (int64_t)nj * n3, (int64_t)nj * n3, Xa, nullptr, st);

@@ -374,10 +374,10 @@ lrtei_status tc_gemm_sym_band(const SplitMatrix& A, const SplitMatrix& B, int64_
                               double* d_C, int64_t ldc, int* d_status, cudaStream_t st);
 // The exchange's operands sliced without an FP64 copy of them; false where a size is not covered (nothing is
 // launched then).  MT: rows (mu, m), columns la of F_u(pair(mu, la), m).  Orbital rows: row mu, columns (j, m) of
-// Z[(j nbf + mu) cols + map[m]] (map NULL: m); d_max: nbf scratch words.
+// Z[(j nbf + mu) cols + map[m]] (map NULL: m); d_max: nbf scratch words, unless the exponents of Z's rows are given.
 bool launch_split_MT(int nbf, int64_t n3, const double* d_F, int64_t ldF, const SplitMatrix& m, cudaStream_t st);
 bool launch_split_orbitals(int nbf, int64_t n3, int nj, const double* d_Z, int64_t cols, const int* d_map,
-                           unsigned long long* d_max, const SplitMatrix& m, cudaStream_t st);
+                           uint32_t* d_max, const int* d_row_expo, const SplitMatrix& m, cudaStream_t st);
 void launch_transpose(const double* in, int64_t rows, int64_t cols, int64_t ldi, double* out, int64_t ldo,
                       cudaStream_t st);
 // out[i][j] = sum_q part[q * stride + i * ld + j] for i < rows, j < cols.
