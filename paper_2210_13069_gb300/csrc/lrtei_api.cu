@@ -1842,8 +1842,8 @@ lrtei_status lrtei_exchange(lrtei_plan* plan, const double* d_Q, int norb, doubl
     uint32_t* dmax;
     LRTEI_TRY(sc.get(&dmax, (size_t)nbf));
     SplitMatrix Qsp, MTsp, Xsp, Ypsp, Xpsp;
-    LRTEI_TRY(scratch_split(sc, Qsp, norb, nbf, 128, plan));
-    LRTEI_TRY(scratch_split(sc, MTsp, rowlen, nbf, split_tile(rowlen), plan));
+    LRTEI_TRY(scratch_split(sc, Qsp, ob, nbf, 128, plan));
+    LRTEI_TRY(scratch_split(sc, MTsp, rowlen, nbf, 128, plan));
     LRTEI_TRY(scratch_split(sc, Xsp, (int64_t)ob * nbf, n3, 128, plan));
     LRTEI_TRY(scratch_split(sc, Ypsp, nbf, (int64_t)ob * n3, 128, plan));
     LRTEI_TRY(scratch_split(sc, Xpsp, nbf, (int64_t)ob * n3, split_tile(nbf), plan));
@@ -1855,7 +1855,6 @@ lrtei_status lrtei_exchange(lrtei_plan* plan, const double* d_Q, int norb, doubl
     LRTEI_TRY(sc.get(&part, (size_t)sK * nbf * nbf));
     {
       ProfScope ps("split", st);
-      launch_split_rows(d_Q, norb, nbf, nbf, Qsp, nullptr, st);
       if (!launch_split_MT(nbf, n3, plan->d_F, n3, MTsp, st)) {
         LRTEI_TRY(need_copy(&MT, (size_t)rowlen * nbf));
         launch_gather_MT(nbf, n3, plan->d_F, n3, MT, st);
@@ -1864,7 +1863,13 @@ lrtei_status lrtei_exchange(lrtei_plan* plan, const double* d_Q, int norb, doubl
     }
     for (int b = 0; b < nblk; ++b) {
       const int j0 = b * ob, nj = std::min(ob, norb - j0);
-      LRTEI_TRY(tc_gemm(Qsp, j0, MTsp, nj, rowlen, 1.0, X, rowlen, false, false, 1, nullptr, plan->d_status, st));
+      SplitMatrix Qb = Qsp;
+      Qb.rows = nj;
+      {
+        ProfScope ps("split", st);
+        launch_split_rows(d_Q + (size_t)j0 * nbf, nj, nbf, nbf, Qb, nullptr, st);
+      }
+      LRTEI_TRY(tc_gemm_few(Qb, MTsp, nj, rowlen, X, rowlen, plan->d_status, st));
       SplitMatrix Xb = Xsp;
       Xb.rows = (int64_t)nj * nbf;
       {

@@ -355,6 +355,9 @@ bool launch_split_density(const PairTable& t, int nbf, int64_t R, const double* 
 lrtei_status tc_gemm(const SplitMatrix& A, int64_t a_row0, const SplitMatrix& B, int64_t M, int64_t N, double scale,
                      double* d_C, int64_t ldc, bool transpose_out, bool symmetric_upper, int splits, double* d_part,
                      int* d_status, cudaStream_t st);
+// The same C = A B^T, bit for bit, for few rows of A and many of B (tiles of 128 rows both): B on the left.
+lrtei_status tc_gemm_few(const SplitMatrix& A, const SplitMatrix& B, int64_t M, int64_t N, double* d_C, int64_t ldc,
+                         int* d_status, cudaStream_t st);
 // Products of rows [a_row0, + M) of A with rows [b_row0, + N) of B (b_row0 a multiple of 128), each at C + c_off.
 struct TcBlock {
   int64_t a_row0, b_row0, M, N, c_off;

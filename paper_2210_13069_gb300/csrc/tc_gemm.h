@@ -329,6 +329,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
       const int* eb = p.eb + sg.b_row0;
       double* C = p.C + sg.c_off + (int64_t)w.split * p.split_stride;
       const bool diag = p.symmetric && !w.mirror;  // the upper triangle only, mirrored below
+      if (n >= N) continue;
 #pragma unroll
       for (int j0 = 0; j0 < QC; j0 += 4) {
         T.template hold<4>(j0);  // one group of columns at a time (the sums fill the registers)

@@ -79,3 +79,20 @@ def test_exchange_operand_layouts(lib, prec, n, orbs):
     pl.status()
     assert rel_fro(K, ref) <= TOL[prec]
     pl.close()
+
+
+# 32-, 64- and 128-column tiles of orbitals, against the FP64 plan of the same molecule.
+@pytest.mark.parametrize("prec", ["split_f16", "split_f16_8"])
+@pytest.mark.parametrize("orbs", [32, 33, 65])
+def test_exchange_orbital_tiles(lib, prec, orbs):
+    import torch
+    m = molecule(8, 4, 5)
+    Q = torch.as_tensor(np.random.Generator(np.random.Philox(12)).normal(0.0, 1.0 / np.sqrt(m.nbf), size=(orbs, m.nbf)),
+                        device="cuda")
+    K = []
+    for p in ("fp64", prec):
+        pl = lib.Plan(m, p)
+        K.append(pl.exchange(Q).cpu().numpy())
+        pl.status()
+        pl.close()
+    assert rel_fro(K[1], K[0]) <= TOL[prec]
