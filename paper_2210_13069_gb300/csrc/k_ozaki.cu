@@ -24,6 +24,8 @@
 // functions, 32.7 -> 0.50 ms (6.2 ms with the FP64 kernels of k_jfp64.cu; its products read their
 // operand at 6.3 TB/s); the error against 64-bit
 // references is the same (1.8e-14) and slightly smaller (1.2e-14 -> 1.1e-14).
+#include <cuda_fp16.h>
+
 #include "tc_gemm.h"
 
 namespace lrtei {
@@ -124,54 +126,75 @@ struct Levels {
 // and block, and as shallow as the pipeline wants it.
 // Destination row i holds source row rowinv[i] (NULL: i), destination column j source column colinv[j]
 // (NULL: j for j < k); -1 gives zeros.  One block per row: the largest magnitude, then the digits.
-__global__ void k_oz_split(const double* __restrict__ src, int64_t k, int64_t ld, int64_t kpad, int tile,
-                           const int* __restrict__ rowinv, const int* __restrict__ colinv, uint16_t* __restrict__ d,
-                           int* __restrict__ expo) {
-  __shared__ unsigned long long red[32];
+// Bound by instructions, and by the conversion unit (16 a clock and SM) where the digits pass through it twice: 1830
+// rows of 13824 (0.5 GB) took 134 us so, 118 with FP16 integers made by an addition to 1536 and the row staged in
+// shared memory (`staged`; longer rows are read twice); the three operands of 16 densities of 120 functions 35 and 27 us.
+// q + 256 (1 + 512 + ... + 512^4) has the balanced digits plus 256 as its lowest 9-bit fields.
+constexpr unsigned long long kDigitBias = 256ULL * (1ULL + (1ULL << 9) + (1ULL << 18) + (1ULL << 27) + (1ULL << 36));
+
+// round(x 2^(54 - e)) + kDigitBias, |q| <= 2^53, of a row whose largest biased exponent is E.
+__device__ __forceinline__ unsigned long long biased_digits(unsigned long long b, int E) {
+  const int Ex = (int)((b >> 52) & 0x7FF), sh = E - Ex;
+  const unsigned long long m = (b & ((1ULL << 52) - 1)) | (1ULL << 52);
+  const unsigned long long q = (Ex == 0 || sh > 54) ? 0 : sh == 0 ? m : (m + (1ULL << (sh - 1))) >> sh;
+  return ((long long)b < 0 ? 0ULL - q : q) + kDigitBias;
+}
+
+// Plane s of two neighbouring elements: small integers as FP16, through 1536 + i (whose last place is 1).
+template <int S>
+__device__ __forceinline__ uint32_t digit_pair(unsigned long long u, unsigned long long v) {
+  constexpr int SH = 9 * (kOzSlices - 1 - S);
+  uint32_t w;
+  if constexpr (S == 0) w = 0x66006600u + (uint32_t)(int)((long long)u >> SH) + ((uint32_t)(int)((long long)v >> SH) << 16);
+  else w = 0x65006500u + ((uint32_t)(u >> SH) & 511u) + (((uint32_t)(v >> SH) & 511u) << 16);
+  const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&w), __half2half2(__ushort_as_half(0x6600)));
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+__global__ void __launch_bounds__(512) k_oz_split(const double* __restrict__ src, int64_t k, int64_t ld, int64_t kpad,
+                                                  int tile, int staged, const int* __restrict__ rowinv,
+                                                  const int* __restrict__ colinv, uint16_t* __restrict__ d,
+                                                  int* __restrict__ expo) {
+  extern __shared__ double row[];
+  __shared__ uint32_t red[32];
   const int64_t i = blockIdx.x;
   const int64_t r = rowinv ? rowinv[i] : i;
   const double* x = src + r * ld;
-  unsigned long long mx = 0;
-  if (r >= 0)
+  uint32_t mx = 0;  // the exponent's word is enough
+  if (r >= 0) {
+#pragma unroll 4
     for (int64_t j = threadIdx.x; j < k; j += blockDim.x) {
-      const unsigned long long a = (unsigned long long)__double_as_longlong(x[j]) & 0x7FFFFFFFFFFFFFFFULL;
-      mx = a > mx ? a : mx;
+      const double v = x[j];
+      if (staged) row[j] = v;
+      mx = max(mx, tc::magnitude(v));
     }
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long v = __shfl_xor_sync(0xffffffffu, mx, o);
-    mx = v > mx ? v : mx;
   }
+  mx = __reduce_max_sync(0xffffffffu, mx);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
   __syncthreads();
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) mx = red[w] > mx ? red[w] : mx;
-  const int E = (int)(mx >> 52);  // biased exponent of the largest magnitude; 0: zero row, 0x7FF: not finite
+  const unsigned lane = threadIdx.x & 31;
+  mx = __reduce_max_sync(0xffffffffu, lane < (blockDim.x >> 5) ? red[lane] : 0u);
+  const int E = (int)(mx >> 20);  // biased exponent of the largest magnitude; 0: zero row, 0x7FF: not finite
   const bool live = E > 0 && E < 0x7FF;
   if (threadIdx.x == 0) expo[i] = E == 0x7FF ? kOzBad : live ? E - 1021 : 0;
+  if (staged) x = row;
   for (int64_t j = 4 * (int64_t)threadIdx.x; j < kpad; j += 4 * (int64_t)blockDim.x) {
-    uint16_t h[4][kOzSlices];
+    unsigned long long q[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       const int64_t c = colinv ? colinv[j + e] : (j + e < k ? j + e : -1);
-      const unsigned long long b = (live && c >= 0) ? (unsigned long long)__double_as_longlong(x[c]) : 0ULL;
-      const int Ex = (int)((b >> 52) & 0x7FF), sh = E - Ex;
-      const unsigned long long m = (b & ((1ULL << 52) - 1)) | (1ULL << 52);
-      // q = round(x 2^(54 - e)), |q| <= 2^53
-      long long q = (Ex == 0 || sh > 54) ? 0 : sh == 0 ? (long long)m : (long long)((m + (1ULL << (sh - 1))) >> sh);
-      if (b >> 63) q = -q;
-#pragma unroll
-      for (int s = kOzSlices - 1; s > 0; --s) {
-        const int dg = (int)((q + 256) & 511) - 256;
-        q = (q - dg) >> 9;
-        h[e][s] = tc::f16_bits((float)dg);
-      }
-      h[e][0] = tc::f16_bits((float)(int)q);
+      q[e] = biased_digits((live && c >= 0) ? (unsigned long long)__double_as_longlong(x[c]) : 0ULL, E);
     }
     const int rr = (int)(i % tile), kk = (int)(j % KB) * 2;  // byte inside the 32-byte row; 16-byte pieces swizzled
     uint8_t* o = reinterpret_cast<uint8_t*>(d) + ((i / tile) * (kpad / KB) + j / KB) * (int64_t)(kOzSlices * tile * 32) +
                  rr * 32 + (kk ^ (((rr >> 2) & 1) << 4));
-#pragma unroll
-    for (int s = 0; s < kOzSlices; ++s)
-      *reinterpret_cast<ushort4*>(o + s * tile * 32) = make_ushort4(h[0][s], h[1][s], h[2][s], h[3][s]);
+    const int step = tile * 32;
+    *reinterpret_cast<uint2*>(o) = make_uint2(digit_pair<0>(q[0], q[1]), digit_pair<0>(q[2], q[3]));
+    *reinterpret_cast<uint2*>(o + step) = make_uint2(digit_pair<1>(q[0], q[1]), digit_pair<1>(q[2], q[3]));
+    *reinterpret_cast<uint2*>(o + 2 * step) = make_uint2(digit_pair<2>(q[0], q[1]), digit_pair<2>(q[2], q[3]));
+    *reinterpret_cast<uint2*>(o + 3 * step) = make_uint2(digit_pair<3>(q[0], q[1]), digit_pair<3>(q[2], q[3]));
+    *reinterpret_cast<uint2*>(o + 4 * step) = make_uint2(digit_pair<4>(q[0], q[1]), digit_pair<4>(q[2], q[3]));
+    *reinterpret_cast<uint2*>(o + 5 * step) = make_uint2(digit_pair<5>(q[0], q[1]), digit_pair<5>(q[2], q[3]));
   }
 }
 
@@ -252,9 +275,15 @@ static int pick_splits(int64_t items, int chunks, double store) {
 void launch_oz_split(const double* d_src, int64_t k, int64_t ld, const int* d_rowinv, const int* d_colinv, OzMatrix& m,
                      cudaStream_t st) {
   if (m.rows <= 0) return;
+  constexpr int64_t most = 28000;  // columns that fit shared memory
+  static bool attr_set = false;
+  if (!attr_set)
+    attr_set = cudaFuncSetAttribute(oz::k_oz_split, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)(sizeof(double) * most)) == cudaSuccess;
+  const int staged = k <= most ? 1 : 0;
   count_launch();
-  oz::k_oz_split<<<(unsigned)m.rows, m.rows < 2 * 152 ? 1024 : 256, 0, st>>>(d_src, k, ld, m.kpad, m.tile, d_rowinv, d_colinv,
-                                                                          m.d, m.expo);
+  oz::k_oz_split<<<(unsigned)m.rows, m.rows < 2 * 152 || k > 4096 ? 512 : 256, staged ? sizeof(double) * (size_t)k : 0, st>>>(
+      d_src, k, ld, m.kpad, m.tile, staged, d_rowinv, d_colinv, m.d, m.expo);
 }
 
 void launch_oz_build_K(int n, int P, bool parity, const ParityClasses& pc, const double* d_C, const double* d_w,
