@@ -186,15 +186,26 @@ def measured_peaks():
     return {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}, "fallback"
 
 
+def parity_steps(n: int) -> float:
+    """Share of K's 16-column blocks of the natural order that the products with K by parity class take: those that hold
+    a column of the row's class (A_d^(p)(a, b) = 0 for odd a + b), averaged over the rows.  A third at n = 24."""
+    blocks = (n ** 3 + 15) // 16
+    held = [set() for _ in range(8)]
+    for m in range(n ** 3):
+        held[(m // (n * n) % 2) * 4 + (m // n % n % 2) * 2 + m % n % 2].add(m // 16)
+    size = [((n + 1 - (c >> 2)) // 2) * ((n + 1 - (c >> 1 & 1)) // 2) * ((n + 1 - (c & 1)) // 2) for c in range(8)]
+    return sum(s * len(h) for s, h in zip(size, held)) / (n ** 3 * blocks)
+
+
 def jbuild_operand_bytes(nbf: int, n: int, precision: str) -> float:
     """Compulsory HBM reads of one factored J-build's three GEMMs (eq. coulapprox): F_u^T (for
-    X = F_u^T D), the dense K (Y = K X) and F_u (J_u = F_u Y), each read once as the GEMMs' A operand
-    in 16-bit planes (three planes for six products, four for eight, one for plain BF16); the
-    densities and the n^3-wide intermediates are negligible beside them."""
-    planes = {"split_f16_8": 4, "bf16": 1}.get(precision, 3)
+    X = F_u^T D), the stored blocks of K (Y = K X) and F_u (J_u = F_u Y), each read once as the GEMMs' A
+    operand in 16-bit planes (three, one for plain BF16); the densities and the n^3-wide intermediates
+    are negligible beside them."""
+    planes = 1 if precision == "bf16" else 3
     npair = nbf * (nbf + 1) // 2
     n3 = n ** 3
-    return 2.0 * planes * (2 * npair * n3 + n3 * n3)
+    return 2.0 * planes * (2 * npair * n3 + parity_steps(n) * n3 * n3)
 
 
 def kernel_source_hash(rel):
@@ -418,9 +429,9 @@ def run_ours(args, world, rank, local):
     # product plus 6 P n^4 N_b^2 for K applied by three mode products per node (eq. ig1), i.e.
     # 2 n^3 + 6 P n^4 / N_b^2 per entry over the N_b^4 entries a step writes.
     alg_flops_step = entries_per_step * (2.0 * n3 + 6.0 * mol.P * mol.n ** 4 / nb2)
-    # What the tensor-core kernel computes: unique pairs only, K dense (n^6 per row instead of
-    # 6 P n^4), the upper triangle of B_u (npair^2 n^3)
-    dense_flops_step = 2.0 * npair * n3 * n3 + 1.0 * npair * npair * n3
+    # What the tensor-core kernel computes: unique pairs only, K's stored blocks (parity_steps of n^6 per
+    # row instead of 6 P n^4), the upper triangle of B_u (npair^2 n^3)
+    dense_flops_step = 2.0 * npair * n3 * n3 * parity_steps(mol.n) + 1.0 * npair * npair * n3
     unique_flops_step = 6.0 * mol.P * mol.n ** 4 * npair + 1.0 * npair * npair * n3
     if args.precision in ("split_f16", "split_f16_8", "bf16"):
         kname, src = "tc_gemm", "paper_2210_13069_gb300/csrc/k_tcgen05.cu"
@@ -442,10 +453,11 @@ def run_ours(args, world, rank, local):
         flops_step = npair * npair * mol.P * Ibar2 * (6 * mol.n + 3)
         peak, unit, bound, k_slices = alu_peaks["fp64_tflops"], "TFLOP/s", "alu", 1
     else:
-        kname, src = "gemm_fp64", "paper_2210_13069_gb300/csrc/k_gemm.cu"
+        kname, src = "gemm_fp64", "paper_2210_13069_gb300/csrc/k_ozaki.cu"
         tot_ms, cnt = prof["gemm_fp64"]
-        flops_step = 2.0 * npair * npair * n3
-        peak, unit, bound, k_slices = alu_peaks["fp64_tflops"], "TFLOP/s", "alu", 1
+        dense_flops_step = 2.0 * npair * n3 * n3 / 8 + 1.0 * npair * npair * n3
+        flops_step, peak = alg_flops_step, peaks["bf16_tflops_sustained"]
+        unit, bound, k_slices = "TFLOP/s", "tensor", 21
     roofline = None
     if cnt > 0 and tot_ms > 0:
         per_launch_flops = flops_step * args.steps / cnt
@@ -465,24 +477,10 @@ def run_ours(args, world, rank, local):
                 # the same kernel judged on the work it does for the unique pairs (no credit for the
                 # pair and triangle symmetry), with the node sum counted as mode products
                 "frac_unique_work": per_launch_unique / (avg_ms / 1e3) / 1e12 / peak,
-                # dense K instead of mode products: flops executed per unique-work flop
+                # K's blocks instead of mode products: flops executed per unique-work flop
                 "dense_K_overhead": dense_flops_step / unique_flops_step,
-                # tensor-pipe issue: dense flops times the split products, against the same peak
+                # tensor-pipe issue: executed flops times the split products, against the same peak
                 "issued_frac": per_launch_dense * k_slices / (avg_ms / 1e3) / 1e12 / peak})
-        if args.precision == "split_f16":
-            # operand bytes the tensor-core GEMMs load per step (128 x 128 tiles, seven 16-bit planes
-            # of 128 rows per 64-deep K step), per SM and clock, against the per-SM TMA delivery
-            # measured with the MMAs switched off (65-68 B/clk/SM, independent of the SM count); an
-            # upper bound when the tuner keeps the CTA-pair kernel for G (5/7 of these bytes there)
-            tm = (npair + 127) // 128
-            kpad = (n3 + 255) // 256 * 256
-            tiles = tm * ((n3 + 127) // 128) + tm * (tm + 1) // 2
-            loaded = tiles * (kpad // 64) * 7 * 128 * 64 * 2
-            mhz = (clocks or {}).get("sm_mhz") or peaks.get("sm_max_mhz", 2070.0)
-            bpc = loaded * args.steps / (tot_ms / 1e3) / 152 / (mhz * 1e6)
-            roofline["operand_delivery"] = {"achieved_B_per_clk_per_sm": bpc, "ceiling_B_per_clk_per_sm": 66.0,
-                                            "frac": bpc / 66.0, "bytes_per_step": loaded,
-                                            "assumes": "one-SM 128 x 128 tiles for both products"}
 
     # ---- J-builds/s (32 densities), same plan
     jb = None
@@ -525,7 +523,7 @@ def run_ours(args, world, rank, local):
         centers, ls, nprim, exps, coefs = mol.packed()
         h2d = centers.nbytes + ls.nbytes + nprim.nbytes + exps.nbytes + coefs.nbytes
         times = []
-        for it in range(8):  # the first builds the tuning choices of every GEMM shape; median of the rest
+        for it in range(8):  # the first loads modules and fills the memory pool; median of the rest
             barrier(world)
             torch.cuda.synchronize()
             t0 = time.perf_counter()
@@ -581,11 +579,14 @@ def run_ours(args, world, rank, local):
         fp64 = {"entries_per_s": world * entries_per_step / (max_over_ranks(ms64, world, device="cuda") / 1e3),
                 "ms_per_step": ms64}
         if g_cnt > 0 and g_ms > 0:
-            # B_u = G F_u^T on the CUDA cores: 2 npair^2 n^3 flops per step
-            ach = 2.0 * npair * npair * n3 / (g_ms / 1e3) / 1e12
-            fp64["roofline"] = {"bound": "alu", "kernel": "gemm_fp64", "achieved": ach, "peak": alu_peaks["fp64_tflops"],
-                                "unit": "TFLOP/s", "frac": ach / alu_peaks["fp64_tflops"],
-                                "peak_kind": "nominal FP64 1.25 TF/s (FMA probe in cuda_core_peaks)", "share_of_step": g_ms / ms64}
+            # both products as 21 digit products on the tensor cores (K by parity class, an eighth of n^6; the
+            # triangle of B_u): the issued flops against the tensor peak
+            ach = 21 * (2.0 * npair * n3 * n3 / 8 + 1.0 * npair * npair * n3) / (g_ms / 1e3) / 1e12
+            fp64["roofline"] = {"bound": "tensor", "kernel": "gemm_fp64", "achieved": ach,
+                                "peak": peaks["bf16_tflops_sustained"], "unit": "TFLOP/s",
+                                "frac": ach / peaks["bf16_tflops_sustained"],
+                                "peak_kind": peak_kind + " (bf16_tflops_sustained), issued digit products",
+                                "share_of_step": g_ms / ms64}
         if not args.no_jbuild:
             R = 32
             D = torch.as_tensor(synth.random_densities(4242, nbf, R), device="cuda")

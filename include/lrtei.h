@@ -55,7 +55,9 @@ typedef enum {
 /* Arithmetic of the contractions (moments, nodes, Chebyshev coefficients and the node sum
  * are FP64 in every mode). */
 typedef enum {
-  LRTEI_FP64 = 0,        /* FP64 CUDA-core contractions */
+  LRTEI_FP64 = 0,        /* FP64 contractions: B and J-builds of enough work as exact products of 9-bit
+                            digits on the tensor cores (54 bits of each row's maximum), where their
+                            operands fit; the rest on the CUDA cores.  About 1e-14 either way */
   LRTEI_FP32 = 1,        /* FP32 CUDA-core contractions */
   LRTEI_SPLIT_F16 = 2,  /* tcgen05 tensor cores, split operands: per row a power-of-two scale and
                             three integer slices (8 + 12 + 12 bits) held exactly in 16-bit floats;
@@ -66,12 +68,11 @@ typedef enum {
                             FP32 accumulation */
   LRTEI_SPLIT_F16_8 = 4  /* as LRTEI_SPLIT_F16, plus the two next-order slice products (t1 t2 and
                             t2 t1), with the small terms in a third accumulator: 8 tensor-core
-                            products per K step instead of 6 and 128 x 64 tiles, an error several
-                            times smaller (1e-9 to 1.5e-8 measured) */
+                            products per K step instead of 6, an error several times smaller (1e-9 to 1.5e-8 measured) */
 } lrtei_precision;
 
-/* Which of the two equivalent forms of Theorem 1 assembles B.  On the FP64 and FP32 paths both
- * run on the CUDA cores.  With LRTEI_SPLIT_F16 the factored form runs on the tensor cores, and so
+/* Which of the two equivalent forms of Theorem 1 assembles B.  On the FP32 path both run on the
+ * CUDA cores, on the FP64 path the Hadamard form does.  With LRTEI_SPLIT_F16 the factored form runs on the tensor cores, and so
  * does the Hadamard form when every unique pair holds one primitive pair (an uncontracted basis,
  * n <= 64, no compression or adaptive boxes): per node and dimension the tile products
  * T_{d,p} S_d^T (depth n) on the tensor cores, the product over dimensions and the node sum in
@@ -277,8 +278,9 @@ lrtei_status lrtei_jbuild_apply_x(lrtei_plan* plan, const double* d_X, int R, in
  * LRTEI_EXCHANGE_BLOCK=<orbitals> in the environment sets the block).  Tensor-core
  * precisions run the three products on tcgen05 with split operands; FP64 / FP32 plans run FP64
  * CUDA-core GEMMs and apply K by mode products (eq. ig1).  A compressed plan gives eq.
- * approxepsilon's exchange.  Device scratch ~6 x min(norb, block) N_b n^3 doubles plus N_b^2 n^3
- * (and their slices).  LRTEI_ERR_ARG for NULL pointers or norb <= 0. */
+ * approxepsilon's exchange.  Device scratch: X and Y of a block, min(norb, block) N_b n^3 doubles
+ * each, and the 16-bit slices of both, of X and Y by orbitals and of N_b^2 n^3 elements of F_u
+ * (FP64 / FP32 plans, and orders whose n^3 is no multiple of 8: FP64 copies of these).  LRTEI_ERR_ARG for NULL pointers or norb <= 0. */
 lrtei_status lrtei_exchange(lrtei_plan* plan, const double* d_Q, int norb, double* d_K, void* stream);
 
 /* ---- batched J-builds (many molecules of uneven size in one graph-captured launch) -------
@@ -345,8 +347,9 @@ lrtei_status lrtei_selector_load(const char* path, lrtei_selector** out, char* m
  * J-build graph).  lrtei_profile_get synchronises those
  * events and returns the summed device time and the launch count of one kernel name.  Two
  * names are counters rather than kernels: "*" gives the number of kernels the library launched
- * since the last reset (time 0), and "alloc" the number of device allocations (cudaMalloc and
- * stream-ordered cudaMallocAsync) it has requested since it was loaded (time 0; never reset).
+ * since the last reset (time 0), and "alloc" the number of device allocations it has requested since it was loaded (time 0; never
+ * reset).  They come from one memory pool per device, which keeps up to 12 GiB of freed memory
+ * while plans exist and 2 GiB after the last one.
  * Off by default; process-wide; not thread-safe against concurrent enable/reset. */
 lrtei_status lrtei_profile_enable(int on);
 lrtei_status lrtei_profile_get(const char* kernel, double* total_ms, int64_t* launches);

@@ -424,9 +424,8 @@ cudaError_t launch_build_K(int n, int P, const double* d_C, const double* d_w, d
 
 // One block per unique pair r = (mu, nu); writes full rows mu*N_b+nu and nu*N_b+mu.
 // The column walk of one B row: col = t, t + step, ... with (ka, la) = (col / N_b, col % N_b)
-// advanced by additions (no 64-bit division per element), the non-finite test on the bit pattern
-// and the scale applied only when it is not 1 (this device's FP64 rate would otherwise make the
-// expansion ALU-bound rather than bound by its 12 GB of traffic).
+// advanced by additions (no 64-bit division per element) and the non-finite test on the bit pattern (an
+// FP64 operation per element would bound the expansion).
 struct ColWalk {
   int ka, la, dka, dla, nbf;
   __device__ ColWalk(int nbf_, int t, int step) : nbf(nbf_) {
