@@ -71,6 +71,47 @@ __device__ __forceinline__ double combine_pow2(int t0, float t12, int k, float t
   return __longlong_as_double((long long)bits);
 }
 
+// f = i + l / 2^21 for |f| < 2^23 by two additions to powers of two: i is even, |l| <= 2^21 rounded to nearest, halves
+// away from zero as f counts.
+__device__ __forceinline__ void split_2p21(float f, int& i, int& l) {
+  const float m = f + 25165824.f;  // 1.5 2^24: the last place is 2
+  i = 2 * (__float_as_int(m) - 0x4BC00000);
+  const float r = f - (m - 25165824.f), n = __fmaf_rn(r, 0x1p21f, 12582912.f);
+  l = __float_as_int(n) - 0x4B400000;
+  const float d = __fmaf_rn(r, 0x1p21f, -(n - 12582912.f));  // what the rounding (halves to even) left
+  l += d == copysignf(0.5f, f) ? (__float_as_int(f) >> 31) | 1 : 0;
+}
+
+// combine_pow2(t0, 4096 t1, k, 4096 t2) in 32-bit words, the same bits: X = S 2^21 + L with S = T0 + the whole parts
+// (|T0| <= 255^2 K, |T1| < 256 K, K <= 32768: within 32 bits).  For the products whose tiles are mostly epilogue (few
+// steps, or two launches): X of the exchange, 90 orbitals of 180 functions in two blocks, 1.77 -> 1.52 ms; the compressed
+// B of 180 functions unchanged to 0.8 % faster.  Not for the others: alike at 180 functions, 128.7 -> 131.4 us for the B of 45.
+__device__ __forceinline__ double combine_words(int t0, float t1, int k, float t2 = 0.f, bool two = false) {
+  int i, L;
+  split_2p21(t1, i, L);
+  int S = t0 + i;
+  if (two) {
+    int i2, l2;
+    split_2p21(t2, i2, l2);
+    S += i2;
+    L += l2;
+  }
+  S += L >> 21;
+  L &= 0x1FFFFF;
+  const int neg = S >> 31;  // -1: two's complement of the 53 bits
+  S = (S ^ neg) + (L == 0 ? neg & 1 : 0);
+  L = ((L ^ neg) - neg) & 0x1FFFFF;
+  const uint32_t low = (uint32_t)L << 11;  // S : low, the leading one moved to the top
+  const bool big = S != 0;
+  const uint32_t top = big ? (uint32_t)S : low, rest = big ? low : 0u;
+  const int lz = __clz((int)top);
+  const uint32_t h = __funnelshift_l(rest, top, lz), l = rest << (lz & 31);
+  const int E = (big ? 1023 + 52 - 21 : 1023 + 20 - 21) + k - lz;
+  const uint32_t hi = ((uint32_t)neg & 0x80000000u) | (uint32_t)min(E, 2046) << 20 | (h >> 11 & 0xFFFFFu);
+  const bool zero = E <= 0 || top == 0;
+  return __hiloint2double((int)(zero ? 0u : hi), (int)(zero ? 0u : __funnelshift_r(l, h, 11)));
+}
+
 // eight_hi and eight_lo: the two launches of eight products on 128 columns.
 enum class Scheme { six, eight, eight_hi, eight_lo, plain };
 
@@ -186,7 +227,10 @@ struct Split {
     // The planes' weights make T1 and T2 those of the sums of s0 t1 over 2^12.
     __device__ __forceinline__ double value(int j, int k, double scale) const {
       if constexpr (PLAIN) return scale * pow2(k - 16) * (double)T1[j];
-      const double v = combine_pow2(LO ? 0 : T0[ONE ? 0 : j], T1[j] * 4096.f, k - 16, P8 ? T2[P8 ? j : 0] * 4096.f : 0.f);
+      const int t0 = LO ? 0 : T0[ONE ? 0 : j];
+      const float t2 = P8 ? T2[P8 ? j : 0] : 0.f;
+      const double v = SWAP || HI || LO ? combine_words(t0, T1[j], k - 16, t2, P8)
+                                        : combine_pow2(t0, T1[j] * 4096.f, k - 16, t2 * 4096.f);
       return scale == 1.0 ? v : scale * v;
     }
   };
@@ -307,7 +351,7 @@ lrtei_status tc_gemm(const SplitMatrix& A, int64_t a_row0, const SplitMatrix& B,
 
 // C = A B^T for few rows A and many rows B, with B as the left operand of the tensor cores: its rows fill the 128 of
 // a tile and the few of A its columns, 32, 64 or 128 of them, so that the drains and the epilogue run over live
-// elements and a warp's stores along a row of C are one contiguous run.  53 rows by 2.5 M of 180: 1.5 ms with A on the left, 0.91 this
+// elements and a warp's stores along a row of C are one contiguous run.  53 rows by 2.5 M of 180: 1.5 ms with A on the left, 0.78 this
 // way (2.9 GB of B); 10 rows by 437 k of 75: 264 us, 84.
 lrtei_status tc_gemm_few(const SplitMatrix& A, const SplitMatrix& B, int64_t M, int64_t N, double* d_C, int64_t ldc,
                          int* d_status, cudaStream_t st) {
