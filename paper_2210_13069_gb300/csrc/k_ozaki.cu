@@ -17,13 +17,11 @@
 //
 // Wide products (B_u = G F_u^T and G = F_u K) run as three launches (levels 4-5, 2-3, 0-1; smallest
 // first, the later ones adding to C): 128 x 128 tiles, two FP32 accumulators double-buffered in the
-// 512 TMEM columns, and an epilogue register budget of one 64-bit sum per element allow two levels at
-// a time.  Skinny products (J-builds, N <= 32 columns a tile) keep all six levels in TMEM (2 x 6 x 32
+// 512 TMEM columns, and registers for one 64-bit sum per element allow two levels at a time.  Skinny products (J-builds, N <= 32 columns a tile) keep all six levels in TMEM (2 x 6 x 32
 // columns) and read their operand once.
-// Measured: FP64 B of 60 functions (n = 24, P = 32) 187 -> 3.0 ms; J-build of 16 densities, 120
-// functions, 32.7 -> 0.50 ms (6.2 ms with the FP64 kernels of k_jfp64.cu; its products read their
-// operand at 6.3 TB/s); the error against 64-bit
-// references is the same (1.8e-14) and slightly smaller (1.2e-14 -> 1.1e-14).
+// Measured: FP64 B of 60 functions (n = 24, P = 32) 187 -> 2.55 ms; J-build of 16 densities, 120 functions,
+// 32.7 -> 0.47 ms (6.2 ms with the FP64 kernels of k_jfp64.cu; its products read their operand at 6.3 TB/s); the
+// error against 64-bit references is the same (1.8e-14) and slightly smaller (1.2e-14 -> 1.1e-14).
 #include <cuda_fp16.h>
 
 #include "tc_gemm.h"
