@@ -9,7 +9,7 @@
 // about 2^-50 of the row maxima over K = 13 824, below the rounding of an FP64 dot product of that
 // length).  The FP32 sum of one level over a chunk of K is exact: at most (level + 1) 64 2^16 <= 2^24
 // for levels 0..3 and 64-deep chunks (levels 0 and 1: 128-deep ones too); levels 4 and 5 weigh 2^-36
-// and less.  Chunks are added in int32 (K is split before 128 of them), and two levels make one integer
+// and less.  Chunks are added in int32 (K is split before they could overflow, oz_splits.h), and two levels make one integer
 // X = 512 L_even + L_odd, so a result carries one rounding per pair of levels.  Rows holding a NaN or an infinity are marked in
 // their exponent and give NaN.
 //
@@ -24,6 +24,7 @@
 // error against 64-bit references is the same (1.8e-14) and slightly smaller (1.2e-14 -> 1.1e-14).
 #include <cuda_fp16.h>
 
+#include "oz_splits.h"
 #include "tc_gemm.h"
 
 namespace lrtei {
@@ -252,24 +253,9 @@ __global__ void k_oz_pack(int nbf, int R, int64_t npair, const int* __restrict__
     u[t] = mu == nu ? v : 2.0 * v;
   }
 }
-
-// ---------------------------------------------------------------- host side
-// Splits of K that shorten the last wave of `items` tiles on 152 SMs, each at least 8 pieces of 64; a
-// split more costs about `store` pieces (its tile's store and its share of the reduction).  At most 120
-// pieces each: the int32 sums of a chunk's at most 2^24 hold 127.
-static int pick_splits(int64_t items, int chunks, double store) {
-  int best = 1;
-  double cost = 1e30;
-  const int least = (chunks + 119) / 120;
-  for (int s = least; s <= std::max(16, least) && (s == least || chunks / s >= 8); ++s) {
-    const double c = (double)((items * s + 151) / 152) * ((double)chunks / s + store) * (1.0 + 0.01 * s);
-    if (c < cost) { cost = c; best = s; }
-  }
-  return best;
-}
-
 }  // namespace oz
 
+// ---------------------------------------------------------------- host side
 void launch_oz_split(const double* d_src, int64_t k, int64_t ld, const int* d_rowinv, const int* d_colinv, OzMatrix& m,
                      cudaStream_t st) {
   if (m.rows <= 0) return;
@@ -324,7 +310,9 @@ lrtei_status oz_gemm(const OzMatrix& A, const OzMatrix& B, const std::vector<OzS
   if (p.nitems == 0) return LRTEI_OK;
   p.blk0 = 0;
   p.blk1 = p.nb = p.seg[0].tiles_n;
-  p.splits = oz::pick_splits(p.nitems, max_units, BN == 32 ? 1.5 : 6.0);
+  // int32 sums: all six levels in the skinny product, levels 0 to 3 in the wide ones
+  p.splits = BN == 32 ? oz::pick_splits(p.nitems, max_units, 1.5, oz::max_pieces(5))
+                      : oz::pick_splits(p.nitems, max_units, 6.0, oz::max_pieces(3));
   double* part = nullptr;
   if (p.splits > 1) {
     cudaError_t e = scratch_alloc((void**)&part, sizeof(double) * (size_t)p.splits * c_rows * c_cols, st);
