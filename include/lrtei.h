@@ -56,8 +56,9 @@ typedef enum {
  * are FP64 in every mode). */
 typedef enum {
   LRTEI_FP64 = 0,        /* FP64 contractions: B and J-builds of enough work as exact products of 9-bit
-                            digits on the tensor cores (54 bits of each row's maximum), where their
-                            operands fit; the rest on the CUDA cores.  About 1e-14 either way */
+                            digits on the tensor cores (72 bits of each row's maximum), where their
+                            operands fit; the rest on the CUDA cores.  About 1e-14 in the norm, and
+                            FP64's accuracy in every element, either way */
   LRTEI_FP32 = 1,        /* FP32 CUDA-core contractions */
   LRTEI_SPLIT_F16 = 2,  /* tcgen05 tensor cores, split operands: per row a power-of-two scale and
                             three integer slices (8 + 12 + 12 bits) held exactly in 16-bit floats;

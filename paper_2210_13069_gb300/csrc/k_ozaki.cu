@@ -2,26 +2,32 @@
 // (Ozaki, Ogita, Oishi and Rump, "Error-free transformations of matrix multiplication", 2012).
 //
 // C = A B^T for FP64 matrices (rows x K, K contiguous).  Every row is scaled by a power of two and cut
-// into six balanced base-512 digits held exactly in FP16:
+// into eight balanced base-512 digits held exactly in FP16:
 //   x = 2^e sum_i d_i 2^(-9 (i + 1)),  |d_i| <= 256, |x| < 2^(e - 1),
-// 53 bits below the binade of the row's largest element, which is FP64's own resolution there.  The 21
-// digit products d_i d_j with level i + j <= 5 are formed on the tensor cores (the dropped ones are
-// about 2^-50 of the row maxima over K = 13 824, below the rounding of an FP64 dot product of that
-// length).  The FP32 sum of one level over a chunk of K is exact: at most (level + 1) 64 2^16 <= 2^24
-// for levels 0..3 and 64-deep chunks (levels 0 and 1: 128-deep ones too); levels 4 and 5 weigh 2^-36
-// and less.  Chunks are added in int32 (K is split before they could overflow, oz_splits.h), and two levels make one integer
-// X = 512 L_even + L_odd, so a result carries one rounding per pair of levels.  Rows holding a NaN or an infinity are marked in
-// their exponent and give NaN.
+// 71 bits below the binade of the row's largest element: an element down to 2^-18 of it is held as FP64 holds it.
+// The 36 digit products d_i d_j with level i + j <= 7 are formed on the tensor cores; the dropped ones are below
+// 2^-66 of the row maxima.  With six digits and 21 products the error had the size of FP64's in the norm only: small
+// elements of B, contractions of the small elements of two rows (the high multipoles of one charge distribution with
+// those of another), were off by up to 1e-9 where FP64 is by 1e-12.  Element by element, two atoms of s, p and d
+// functions, elements above 1e-10 of the largest, 99.9 % quantile / maximum of the relative error of B against 80-bit
+// sums from the same factors: FP64 8.9e-15 / 1.1e-13, six digits 1.6e-11 / 9.4e-10, seven 3.3e-14 / 8.3e-13, eight
+// 3.1e-15 / 7.3e-14; on a wider molecule FP64 8.8e-13 / 1.6e-11, seven 1.2e-12 / 9.3e-12, eight 4.1e-13 / 6.7e-12.
 //
-// Why: this device runs 1.2 TFLOP/s in FP64 and 1 900 in FP16; 21 products leave ~90.
+// The FP32 sum of one level over a chunk of K is exact, at most (level + 1) columns 2^16 <= 2^24: chunks of 128 columns
+// for levels 0 and 1, 64 for 2 and 3, 32 for 4 and 5 and for all eight of the skinny product.  In the wide products
+// levels 6 and 7, which weigh 2^-54 and less, stay FP32 sums.  Chunks are added in int32 (K is split before they could
+// overflow, oz_splits.h), and two levels make one integer X = 512 L_even + L_odd, so a result carries one rounding per
+// pair of levels.  Rows holding a NaN or an infinity are marked in their exponent and give NaN.
 //
-// Wide products (B_u = G F_u^T and G = F_u K) run as three launches (levels 4-5, 2-3, 0-1; smallest
+// Why: this device runs 1.2 TFLOP/s in FP64 and 1 900 in FP16; 36 products leave ~53.
+//
+// Wide products (B_u = G F_u^T and G = F_u K) run as four launches (levels 6-7, 4-5, 2-3, 0-1; smallest
 // first, the later ones adding to C): 128 x 128 tiles, two FP32 accumulators double-buffered in the
-// 512 TMEM columns, and registers for one 64-bit sum per element allow two levels at a time.  Skinny products (J-builds, N <= 32 columns a tile) keep all six levels in TMEM (2 x 6 x 32
-// columns) and read their operand once.
-// Measured: FP64 B of 60 functions (n = 24, P = 32) 187 -> 2.55 ms; J-build of 16 densities, 120 functions,
-// 32.7 -> 0.47 ms (6.2 ms with the FP64 kernels of k_jfp64.cu; its products read their operand at 6.3 TB/s); the
-// error against 64-bit references is the same (1.8e-14) and slightly smaller (1.2e-14 -> 1.1e-14).
+// 512 TMEM columns, and registers for one 64-bit sum per element allow two levels at a time.  Skinny products
+// (J-builds, N <= 32 columns a tile) keep all eight levels in TMEM (2 x 8 x 32 columns) and read their operand once.
+// Measured: FP64 B of 60 functions (n = 24, P = 32) 187 ms on the CUDA cores, 2.55 with six digits, 4.29 with eight;
+// J-build of 16 densities, 120 functions, 32.7 (6.2 with the kernels of k_jfp64.cu), 0.47 and 0.61 ms, the products
+// reading their operand at 6.5 TB/s.
 #include <cuda_fp16.h>
 
 #include "oz_splits.h"
@@ -37,12 +43,13 @@ template <int BN_, int LV0, int NLV>
 struct Levels {
   static constexpr int BN = BN_, NP = LV0 + NLV, PT = kOzSlices, NACC = NLV;
   static constexpr bool BF16 = false, ACCUM = NLV == 2, LIST = false;
-  static constexpr bool FLT = LV0 >= 4;  // FP32 running sums (level 4 weighs 2^-36)
+  static constexpr bool FLT = LV0 >= 6;  // FP32 running sums (level 6 weighs 2^-54)
   // K blocks per stage: one barrier round per 30 KB or more
   static constexpr int STEP = NP * (128 + BN) * 32, KS = STEP >= 30 * 1024 ? 1 : STEP >= 16 * 1024 ? 2 : 4;
   static constexpr int UNIT = 4;  // 64-deep split units
-  // chunk: exactness (top of the file); levels 4 and 5 need none
-  static constexpr int CHUNK = UNIT * (NLV == 6 ? 1 : LV0 == 0 ? 2 : LV0 == 4 ? 4 : 1);
+  // chunk, in 16-deep steps: exactness (top of the file), which levels 6 and 7 of the wide products do without
+  static constexpr int CHUNK = NLV == 8 || LV0 == 4 ? 2 : LV0 == 2 ? 4 : LV0 == 0 ? 8 : 16;
+  static_assert(FLT || (LV0 + NLV) * CHUNK * 16 * 65536 <= 1 << 24, "a chunk's sums are exact in FP32");
 
   static __device__ __forceinline__ void mma(uint32_t d0, uint64_t a, uint64_t b, uint32_t idesc, uint32_t first) {
 #pragma unroll
@@ -120,40 +127,61 @@ struct Levels {
 };
 
 // ---------------------------------------------------------------- slicing
-// Digit tiles: `tile` rows x 16 columns x 6 planes are contiguous (each plane's 32-byte rows in the 32-byte
+// Digit tiles: `tile` rows x 16 columns x 8 planes are contiguous (each plane's 32-byte rows in the 32-byte
 // swizzle of shared memory), K block after K block, so that a stage is one contiguous copy per operand
 // and block, and as shallow as the pipeline wants it.
 // Destination row i holds source row rowinv[i] (NULL: i), destination column j source column colinv[j]
-// (NULL: j for j < k); -1 gives zeros.  One block per row: the largest magnitude, then the digits.
-// Bound by instructions, and by the conversion unit (16 a clock and SM) where the digits pass through it twice: 1830
-// rows of 13824 (0.5 GB) took 134 us so, 118 with FP16 integers made by an addition to 1536 and the row staged in
-// shared memory (`staged`; longer rows are read twice); the three operands of 16 densities of 120 functions 35 and 27 us.
-// q + 256 (1 + 512 + ... + 512^4) has the balanced digits plus 256 as its lowest 9-bit fields.
-constexpr unsigned long long kDigitBias = 256ULL * (1ULL + (1ULL << 9) + (1ULL << 18) + (1ULL << 27) + (1ULL << 36));
+// (NULL: j for j < k); -1 gives zeros.  colexp (NULL: none): source column j comes times 2^-colexp[j].  One block per
+// row: the largest magnitude, then the digits.
+// Bound by instructions, and by the conversion unit (16 a clock and SM) where the digits pass through it twice: six
+// planes of 1830 rows of 13824 took 134 us so, 118 with FP16 integers made by an addition to 1536 and the row staged in
+// shared memory (`staged`; longer rows are read twice), and eight planes take 144 (0.6 GB); the three operands of 16
+// densities of 120 functions 35, 27 and, in eight planes, 34 us.
+// The digits of q = round(x 2^(72 - e)), |q| <= 2^71, as two words of four: q = hi 2^36 + lo with lo between -256 and
+// 255 times 1 + 512 + 512^2 + 512^3; a word plus 256 times its digits' weights (without the first digit's) has the
+// digits plus 256 as its 9-bit fields, the first one as it is.
+struct Digits {
+  long long hi, lo;
+};
+constexpr long long kBias3 = 256LL * (1 + (1LL << 9) + (1LL << 18)), kBias4 = kBias3 + (256LL << 27);
 
-// round(x 2^(54 - e)) + kDigitBias, |q| <= 2^53, of a row whose largest biased exponent is E.
-__device__ __forceinline__ unsigned long long biased_digits(unsigned long long b, int E) {
-  const int Ex = (int)((b >> 52) & 0x7FF), sh = E - Ex;
-  const unsigned long long m = (b & ((1ULL << 52) - 1)) | (1ULL << 52);
-  const unsigned long long q = (Ex == 0 || sh > 54) ? 0 : sh == 0 ? m : (m + (1ULL << (sh - 1))) >> sh;
-  return ((long long)b < 0 ? 0ULL - q : q) + kDigitBias;
+// The digits of an element of a row whose largest biased exponent is E.
+__device__ __forceinline__ Digits biased_digits(unsigned long long b, int E) {
+  const int Ex = (int)((b >> 52) & 0x7FF), sh = E - Ex;  // |q| = m 2^(18 - sh)
+  unsigned long long m = (b & ((1ULL << 52) - 1)) | (1ULL << 52);
+  if (sh > 18) m = sh > 72 ? 0 : (m + (1ULL << (sh - 19))) >> (sh - 18);
+  if (Ex == 0) m = 0;
+  const int up = max(18 - sh, 0);
+  const long long neg = (long long)b >> 63;  // 0 or -1
+  const long long h = (long long)(m >> (36 - up)), l = (long long)((m << up) & ((1ULL << 36) - 1));
+  const long long lo = ((l ^ neg) - neg) + kBias4;
+  return {((h ^ neg) - neg) + (lo >> 36) + kBias3, lo};
 }
 
 // Plane s of two neighbouring elements: small integers as FP16, through 1536 + i (whose last place is 1).
 template <int S>
-__device__ __forceinline__ uint32_t digit_pair(unsigned long long u, unsigned long long v) {
-  constexpr int SH = 9 * (kOzSlices - 1 - S);
+__device__ __forceinline__ uint32_t digit_pair(const Digits& u, const Digits& v) {
+  constexpr int SH = 9 * (3 - S % 4);
+  const long long x = S < 4 ? u.hi : u.lo, y = S < 4 ? v.hi : v.lo;
   uint32_t w;
-  if constexpr (S == 0) w = 0x66006600u + (uint32_t)(int)((long long)u >> SH) + ((uint32_t)(int)((long long)v >> SH) << 16);
-  else w = 0x65006500u + ((uint32_t)(u >> SH) & 511u) + (((uint32_t)(v >> SH) & 511u) << 16);
+  if constexpr (S == 0) w = 0x66006600u + (uint32_t)(int)(x >> SH) + ((uint32_t)(int)(y >> SH) << 16);
+  else w = 0x65006500u + ((uint32_t)(x >> SH) & 511u) + (((uint32_t)(y >> SH) & 511u) << 16);
   const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&w), __half2half2(__ushort_as_half(0x6600)));
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
+// x 2^-s for |x| < 2^s, zero below the normal range.
+__device__ __forceinline__ double scaled_down(double x, int s) {
+  const long long b = __double_as_longlong(x);
+  const int E = (int)((b >> 52) & 0x7FF) - s;
+  if (((b >> 52) & 0x7FF) == 0 || E <= 0) return 0.0;
+  return __longlong_as_double(b - ((long long)s << 52));
+}
+
 __global__ void __launch_bounds__(512) k_oz_split(const double* __restrict__ src, int64_t k, int64_t ld, int64_t kpad,
                                                   int tile, int staged, const int* __restrict__ rowinv,
-                                                  const int* __restrict__ colinv, uint16_t* __restrict__ d,
-                                                  int* __restrict__ expo) {
+                                                  const int* __restrict__ colinv, const int* __restrict__ colexp,
+                                                  uint16_t* __restrict__ d, int* __restrict__ expo) {
   extern __shared__ double row[];
   __shared__ uint32_t red[32];
   const int64_t i = blockIdx.x;
@@ -163,7 +191,7 @@ __global__ void __launch_bounds__(512) k_oz_split(const double* __restrict__ src
   if (r >= 0) {
 #pragma unroll 4
     for (int64_t j = threadIdx.x; j < k; j += blockDim.x) {
-      const double v = x[j];
+      const double v = colexp ? scaled_down(x[j], colexp[j]) : x[j];
       if (staged) row[j] = v;
       mx = max(mx, tc::magnitude(v));
     }
@@ -178,11 +206,13 @@ __global__ void __launch_bounds__(512) k_oz_split(const double* __restrict__ src
   if (threadIdx.x == 0) expo[i] = E == 0x7FF ? kOzBad : live ? E - 1021 : 0;
   if (staged) x = row;
   for (int64_t j = 4 * (int64_t)threadIdx.x; j < kpad; j += 4 * (int64_t)blockDim.x) {
-    unsigned long long q[4];
+    Digits q[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       const int64_t c = colinv ? colinv[j + e] : (j + e < k ? j + e : -1);
-      q[e] = biased_digits((live && c >= 0) ? (unsigned long long)__double_as_longlong(x[c]) : 0ULL, E);
+      double v = live && c >= 0 ? x[c] : 0.0;
+      if (colexp && !staged && c >= 0) v = scaled_down(v, colexp[c]);
+      q[e] = biased_digits((unsigned long long)__double_as_longlong(v), E);
     }
     const int rr = (int)(i % tile), kk = (int)(j % KB) * 2;  // byte inside the 32-byte row; 16-byte pieces swizzled
     uint8_t* o = reinterpret_cast<uint8_t*>(d) + ((i / tile) * (kpad / KB) + j / KB) * (int64_t)(kOzSlices * tile * 32) +
@@ -194,6 +224,8 @@ __global__ void __launch_bounds__(512) k_oz_split(const double* __restrict__ src
     *reinterpret_cast<uint2*>(o + 3 * step) = make_uint2(digit_pair<3>(q[0], q[1]), digit_pair<3>(q[2], q[3]));
     *reinterpret_cast<uint2*>(o + 4 * step) = make_uint2(digit_pair<4>(q[0], q[1]), digit_pair<4>(q[2], q[3]));
     *reinterpret_cast<uint2*>(o + 5 * step) = make_uint2(digit_pair<5>(q[0], q[1]), digit_pair<5>(q[2], q[3]));
+    *reinterpret_cast<uint2*>(o + 6 * step) = make_uint2(digit_pair<6>(q[0], q[1]), digit_pair<6>(q[2], q[3]));
+    *reinterpret_cast<uint2*>(o + 7 * step) = make_uint2(digit_pair<7>(q[0], q[1]), digit_pair<7>(q[2], q[3]));
   }
 }
 
@@ -242,22 +274,25 @@ __global__ void __launch_bounds__(256) k_oz_build_K(int n, int P, int par, Parit
   }
 }
 
-// Unique-pair densities, one row per density: u[q][r] = D_q(mu, nu) (2 - [mu == nu]).
+// Unique-pair densities, one row per density, in the units of the pairs' rows of F_u: u[q][r] =
+// D_q(mu, nu) (2 - [mu == nu]) 2^expo[r], to meet F_u^T with its columns scaled by 2^-expo.  Unscaled, a row of F_u^T
+// holds a pair of small overlap far below its largest one: a density on such pairs alone gave J off by 1e-12 of its terms.
 __global__ void k_oz_pack(int nbf, int R, int64_t npair, const int* __restrict__ pair_mu,
-                          const int* __restrict__ pair_nu, const double* __restrict__ D, double* __restrict__ u) {
+                          const int* __restrict__ pair_nu, const int* __restrict__ expo, const double* __restrict__ D,
+                          double* __restrict__ u) {
   const int64_t total = npair * R;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
     const int64_t r = t % npair, q = t / npair;
     const int mu = pair_mu[r], nu = pair_nu[r];
     const double v = D[q * nbf * nbf + (int64_t)mu * nbf + nu];
-    u[t] = mu == nu ? v : 2.0 * v;
+    u[t] = scalbn(v, expo[r] + (mu == nu ? 0 : 1));
   }
 }
 }  // namespace oz
 
 // ---------------------------------------------------------------- host side
-void launch_oz_split(const double* d_src, int64_t k, int64_t ld, const int* d_rowinv, const int* d_colinv, OzMatrix& m,
-                     cudaStream_t st) {
+void launch_oz_split(const double* d_src, int64_t k, int64_t ld, const int* d_rowinv, const int* d_colinv,
+                     const int* d_colexp, OzMatrix& m, cudaStream_t st) {
   if (m.rows <= 0) return;
   constexpr int64_t most = 28000;  // columns that fit shared memory
   static bool attr_set = false;
@@ -267,7 +302,7 @@ void launch_oz_split(const double* d_src, int64_t k, int64_t ld, const int* d_ro
   const int staged = k <= most ? 1 : 0;
   count_launch();
   oz::k_oz_split<<<(unsigned)m.rows, m.rows < 2 * 152 || k > 4096 ? 512 : 256, staged ? sizeof(double) * (size_t)k : 0, st>>>(
-      d_src, k, ld, m.kpad, m.tile, staged, d_rowinv, d_colinv, m.d, m.expo);
+      d_src, k, ld, m.kpad, m.tile, staged, d_rowinv, d_colinv, d_colexp, m.d, m.expo);
 }
 
 void launch_oz_build_K(int n, int P, bool parity, const ParityClasses& pc, const double* d_C, const double* d_w,
@@ -277,10 +312,10 @@ void launch_oz_build_K(int n, int P, bool parity, const ParityClasses& pc, const
                                                                              d_K, ldK);
 }
 
-void launch_oz_pack(const PairTable& t, int nbf, int R, const double* d_D, double* d_u, cudaStream_t st) {
+void launch_oz_pack(const PairTable& t, int nbf, int R, const double* d_D, const int* d_expo, double* d_u, cudaStream_t st) {
   count_launch();
   oz::k_oz_pack<<<(unsigned)std::min<int64_t>((t.npair * R + 255) / 256, 152 * 16), 256, 0, st>>>(
-      nbf, R, t.npair, t.pair_mu, t.pair_nu, d_D, d_u);
+      nbf, R, t.npair, t.pair_mu, t.pair_nu, d_expo, d_D, d_u);
 }
 
 // C = A B^T over the segments; C rows are A rows (transpose_out: C^T).  symmetric: one segment, C square,
@@ -310,9 +345,9 @@ lrtei_status oz_gemm(const OzMatrix& A, const OzMatrix& B, const std::vector<OzS
   if (p.nitems == 0) return LRTEI_OK;
   p.blk0 = 0;
   p.blk1 = p.nb = p.seg[0].tiles_n;
-  // int32 sums: all six levels in the skinny product, levels 0 to 3 in the wide ones
-  p.splits = BN == 32 ? oz::pick_splits(p.nitems, max_units, 1.5, oz::max_pieces(5))
-                      : oz::pick_splits(p.nitems, max_units, 6.0, oz::max_pieces(3));
+  // int32 sums: all eight levels in the skinny product, levels 0 to 5 in the wide ones
+  p.splits = BN == 32 ? oz::pick_splits(p.nitems, max_units, 1.5, oz::max_pieces(7))
+                      : oz::pick_splits(p.nitems, max_units, 6.0, oz::max_pieces(5));
   double* part = nullptr;
   if (p.splits > 1) {
     cudaError_t e = scratch_alloc((void**)&part, sizeof(double) * (size_t)p.splits * c_rows * c_cols, st);
@@ -342,10 +377,11 @@ lrtei_status oz_gemm(const OzMatrix& A, const OzMatrix& B, const std::vector<OzS
   {
     ProfScope ps("gemm_fp64", st);
     if (BN == 32) {
-      s = tcg::launch<oz::Levels<32, 0, 6>>(p, st);
+      s = tcg::launch<oz::Levels<32, 0, 8>>(p, st);
     } else {
-      s = tcg::launch<oz::Levels<128, 4, 2>>(p, st);
+      s = tcg::launch<oz::Levels<128, 6, 2>>(p, st);
       p.accumulate = 1;
+      if (s == LRTEI_OK) s = tcg::launch<oz::Levels<128, 4, 2>>(p, st);
       if (s == LRTEI_OK) s = tcg::launch<oz::Levels<128, 2, 2>>(p, st);
       p.mirror = (symmetric && !part) ? 1 : 0;
       if (s == LRTEI_OK) s = tcg::launch<oz::Levels<128, 0, 2>>(p, st);

@@ -1307,13 +1307,15 @@ lrtei_status ensure_ozF(lrtei_plan* pl, cudaStream_t st) {
   OzMatrix m;
   LRTEI_TRY(alloc_oz(pl, m, pl->t.npair, pl->pc.cols));
   ProfScope ps("split", st);
-  launch_oz_split(pl->d_F, n3, n3, nullptr, pl->d_perm, m, st);
+  launch_oz_split(pl->d_F, n3, n3, nullptr, pl->d_perm, nullptr, m, st);
   pl->ozF = m;
   return finish_launch("digits of F");
 }
+// F_u^T with its columns (pairs) scaled by their rows' powers of two in ozF; the densities carry the inverse
+// (launch_oz_pack).
 lrtei_status ensure_ozFT(lrtei_plan* pl, cudaStream_t st) {
   if (pl->ozFT.d) return LRTEI_OK;
-  LRTEI_TRY(ensure_classes(pl, st));
+  LRTEI_TRY(ensure_ozF(pl, st));
   LRTEI_TRY(ensure_F64(pl, st));
   const int64_t n3 = (int64_t)pl->n * pl->n * pl->n, npair = pl->t.npair;
   Scratch sc(st);
@@ -1323,7 +1325,7 @@ lrtei_status ensure_ozFT(lrtei_plan* pl, cudaStream_t st) {
   OzMatrix m;
   LRTEI_TRY(alloc_oz(pl, m, pl->pc.cols, (npair + 63) / 64 * 64));
   ProfScope ps("split", st);
-  launch_oz_split(FT, npair, npair, pl->d_perm, nullptr, m, st);
+  launch_oz_split(FT, npair, npair, pl->d_perm, nullptr, pl->ozF.expo, m, st);
   pl->ozFT = m;
   return finish_launch("digits of F^T");
 }
@@ -1343,7 +1345,7 @@ lrtei_status ensure_ozK(lrtei_plan* pl, cudaStream_t st) {
   OzMatrix m;
   LRTEI_TRY(alloc_oz(pl, m, pc.rows, pc.kmax));
   ProfScope ps("split", st);
-  launch_oz_split(K, pc.kmax, pc.kmax, nullptr, nullptr, m, st);
+  launch_oz_split(K, pc.kmax, pc.kmax, nullptr, nullptr, nullptr, m, st);
   pl->ozK = m;
   return finish_launch("digits of K");
 }
@@ -1360,9 +1362,9 @@ bool fits(double bytes) {
 }
 
 // Estimated seconds of the FP64 FMAs of a CUDA-core form (2 FMAs per clock and SM), of the K build, and
-// whether the digit products are cheaper for nr rows of B_u: 21 products at about half the FP16 peak plus
+// whether the digit products are cheaper for nr rows of B_u: 36 products at about half the FP16 peak plus
 // 0.4 ms of launches and slicing.  Measured at 60 functions, n = 24: 153 against 3 ms; the line lies near
-// 15 functions.  The memory they need decides too (digit planes are 12 bytes per element).
+// 15 functions.  The memory they need decides too (digit planes are 16 bytes per element).
 constexpr double kFmaRate = 0.6e12;
 double node_fmas(const lrtei_plan* pl, double rows) {
   const double n = pl->n;
@@ -1383,21 +1385,21 @@ bool oz_rows_ok(const lrtei_plan* pl, int64_t nr, cudaStream_t st) {
   const double n3 = (double)pl->n * pl->n * pl->n, np = (double)pl->t.npair;
   const double cuda = ((double)nr * np * n3 + node_fmas(pl, (double)nr)) / kFmaRate;
   const double build = pl->ozK.d ? 0.0 : K_elems(pl) * pl->P / kFmaRate;
-  if (cuda <= build + 42.0 * (double)nr * np * n3 / 0.9e15 + 4e-4) return false;
-  const double need = (pl->ozF.d ? 0.0 : 12 * np * n3) + (pl->d_F ? 0.0 : 8 * np * n3) +
-                      (pl->ozK.d ? 0.0 : 21 * K_elems(pl)) + nr * (20 * n3 + 8 * np);
+  if (cuda <= build + 72.0 * (double)nr * np * n3 / 0.9e15 + 4e-4) return false;
+  const double need = (pl->ozF.d ? 0.0 : 16 * np * n3) + (pl->d_F ? 0.0 : 8 * np * n3) +
+                      (pl->ozK.d ? 0.0 : 24 * K_elems(pl)) + nr * (24 * n3 + 8 * np);
   return fits(need);
 }
-// J-builds: R >= 2 densities (one is as fast through FP64 F_u, 8 bytes an element against 12), orders up
+// J-builds: R >= 2 densities (one is as fast through FP64 F_u, 8 bytes an element against 16), orders up
 // to 32 unless K is there (its build grows as n^6), and enough work to pay for a dozen launches.
 bool oz_jbuild_ok(const lrtei_plan* pl, int R, cudaStream_t st) {
   if (pl->prec != LRTEI_FP64 || pl->npart > 0 || R < 2 || (pl->n > 32 && !pl->ozK.d)) return false;
   const double n3 = (double)pl->n * pl->n * pl->n, np = (double)pl->t.npair;
   const double cuda = (2 * np * n3 * R + node_fmas(pl, R)) / kFmaRate;
-  if (cuda <= (24 * np * n3 + 12 * K_elems(pl)) / 5e12 + 8e-5) return false;
+  if (cuda <= (32 * np * n3 + 16 * K_elems(pl)) / 5e12 + 8e-5) return false;
   if (pl->ozF.d && pl->ozFT.d && pl->ozK.d) return true;
   if (capturing(st)) return false;
-  return fits(np * n3 * (pl->d_F ? 32 : 40) + 21 * K_elems(pl));
+  return fits(np * n3 * (pl->d_F ? 40 : 48) + 24 * K_elems(pl));
 }
 
 lrtei_status bu_rows_oz(lrtei_plan* pl, int64_t r0, int64_t r1, double* out, int64_t ld, cudaStream_t st) {
@@ -1418,7 +1420,7 @@ lrtei_status bu_rows_oz(lrtei_plan* pl, int64_t r0, int64_t r1, double* out, int
   LRTEI_TRY(scratch_oz(sc, Gs, nr, pc.cols, 128));
   {
     ProfScope ps("split", st);
-    launch_oz_split(G, pc.cols, pc.cols, nullptr, nullptr, Gs, st);
+    launch_oz_split(G, pc.cols, pc.cols, nullptr, nullptr, nullptr, Gs, st);
   }
   const bool sym = r0 == 0 && r1 == npair;
   return oz_gemm(Gs, pl->ozF, {{0, 0, nr, npair, 0, 0, 0, pc.cols}}, out, ld, false, sym, nr, npair, pl->d_status, st);
@@ -2308,18 +2310,18 @@ static lrtei_status jbuild_oz(lrtei_plan* plan, const double* d_D, int R, double
   LRTEI_TRY(scratch_oz(sc, us, R, plan->ozFT.kpad, tw));
   LRTEI_TRY(scratch_oz(sc, Xs, R, pc.cols, tw));
   LRTEI_TRY(scratch_oz(sc, Ys, R, pc.cols, tw));
-  launch_oz_pack(plan->t, nbf, R, d_D, u, st);
-  launch_oz_split(u, npair, npair, nullptr, nullptr, us, st);
+  launch_oz_pack(plan->t, nbf, R, d_D, plan->ozF.expo, u, st);
+  launch_oz_split(u, npair, npair, nullptr, nullptr, nullptr, us, st);
   LRTEI_TRY(oz_gemm(plan->ozFT, us, {{0, 0, pc.cols, R, 0, 0, 0, (int)us.kpad}}, X, pc.cols, true, false, R, pc.cols,
                     plan->d_status, st));
-  launch_oz_split(X, pc.cols, pc.cols, nullptr, nullptr, Xs, st);
+  launch_oz_split(X, pc.cols, pc.cols, nullptr, nullptr, nullptr, Xs, st);
   std::vector<OzSegment> seg;
   for (int c = 0; c < pc.nclass; ++c) {
     const int k = (pc.size[c] + 63) / 64 * 64;
     if (k > 0) seg.push_back({pc.row0[c], 0, k, R, pc.off[c], 0, pc.off[c], k});
   }
   LRTEI_TRY(oz_gemm(plan->ozK, Xs, seg, Y, pc.cols, true, false, R, pc.cols, plan->d_status, st));
-  launch_oz_split(Y, pc.cols, pc.cols, nullptr, nullptr, Ys, st);
+  launch_oz_split(Y, pc.cols, pc.cols, nullptr, nullptr, nullptr, Ys, st);
   LRTEI_TRY(oz_gemm(plan->ozF, Ys, {{0, 0, npair, R, 0, 0, 0, pc.cols}}, Ju, R, false, false, npair, R, plan->d_status, st));
   launch_unpack_J(nbf, R, Ju, 1.0, d_J, plan->d_status, st);
   return finish_launch("jbuild (digit products)");

@@ -288,21 +288,21 @@ void convert_f64_to_f32(const double* in, float* out, int64_t count, cudaStream_
 void convert_f32_to_f64(const float* in, double* out, int64_t count, cudaStream_t st);
 
 // ---------------------------------------------------------------- FP64 on the tensor cores (k_ozaki.cu)
-constexpr int kOzSlices = 6;      // base-512 digits of an FP64 element
+constexpr int kOzSlices = 8;      // base-512 digits of an FP64 element
 constexpr int kOzBad = 1 << 20;   // exponent of a row that holds a NaN or an infinity
 struct OzMatrix {                 // rows x kpad (a multiple of 64), kOzSlices digit planes, in tiles of
-  int64_t rows = 0, kpad = 0;     // `tile` rows x 32 columns (128; 32 for the B operand of skinny products)
+  int64_t rows = 0, kpad = 0;     // `tile` rows x 16 columns (128; 32 for the B operand of skinny products)
   int tile = 128;
   int64_t count() const { return (rows + tile - 1) / tile * tile * kpad * kOzSlices; }
   uint16_t* d = nullptr;
   int* expo = nullptr;
 };
-void launch_oz_split(const double* d_src, int64_t k, int64_t ld, const int* d_rowinv, const int* d_colinv, OzMatrix& m,
-                     cudaStream_t st);
+void launch_oz_split(const double* d_src, int64_t k, int64_t ld, const int* d_rowinv, const int* d_colinv,
+                     const int* d_colexp, OzMatrix& m, cudaStream_t st);
 // K (pc.rows x ldK, zero-filled by the caller) by parity class.
 void launch_oz_build_K(int n, int P, bool parity, const ParityClasses& pc, const double* d_C, const double* d_w,
                        double scale, double* d_K, int64_t ldK, cudaStream_t st);
-void launch_oz_pack(const PairTable& t, int nbf, int R, const double* d_D, double* d_u, cudaStream_t st);
+void launch_oz_pack(const PairTable& t, int nbf, int R, const double* d_D, const int* d_expo, double* d_u, cudaStream_t st);
 struct OzSegment {  // rows [a_row0, a_row0 + M) of A times rows [b_row0, b_row0 + N) of B over k (a multiple
   int64_t a_row0, b_row0, M, N, c_off;  // of 64) columns from a_k0 and b_k0, written at C + c_off
   int a_k0, b_k0, k;

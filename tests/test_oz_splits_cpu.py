@@ -1,7 +1,7 @@
 """The split of K of the FP64 digit products (csrc/oz_splits.h), compiled for the host.
 
 Each split's int32 sums must hold the largest sum that digits of magnitude 256 can give: (level + 1) 64 256^2 per piece,
-level 5 of the skinny product included.
+level 7 of the skinny product included.
 """
 import os
 import shutil
@@ -16,11 +16,11 @@ MAIN = r"""
 #include <cstdlib>
 #include "oz_splits.h"
 int main() {
-  for (int level : {3, 5})
+  for (int level : {5, 7})
     for (int pieces = 1; pieces <= 4096; ++pieces)
       for (int64_t items : {1LL, 7LL, 152LL, 153LL, 4000LL, 100000LL}) {
         const int most = lrtei::oz::max_pieces(level);
-        const int s = lrtei::oz::pick_splits(items, pieces, level == 3 ? 6.0 : 1.5, most);
+        const int s = lrtei::oz::pick_splits(items, pieces, level == 5 ? 6.0 : 1.5, most);
         const long long per = (pieces + s - 1) / s;  // as the kernel cuts them
         if (s < 1 || per * (level + 1) * 64 * 65536 > 0x7FFFFFFFLL) {
           std::printf("level %d, %d pieces in %d splits of %lld\n", level, pieces, s, per);
