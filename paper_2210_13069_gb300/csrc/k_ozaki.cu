@@ -345,9 +345,7 @@ lrtei_status oz_gemm(const OzMatrix& A, const OzMatrix& B, const std::vector<OzS
   if (p.nitems == 0) return LRTEI_OK;
   p.blk0 = 0;
   p.blk1 = p.nb = p.seg[0].tiles_n;
-  // int32 sums: all eight levels in the skinny product, levels 0 to 5 in the wide ones
-  p.splits = BN == 32 ? oz::pick_splits(p.nitems, max_units, 1.5, oz::max_pieces(7))
-                      : oz::pick_splits(p.nitems, max_units, 6.0, oz::max_pieces(5));
+  p.splits = oz::product_splits(p.nitems, max_units, BN == 32);
   double* part = nullptr;
   if (p.splits > 1) {
     cudaError_t e = scratch_alloc((void**)&part, sizeof(double) * (size_t)p.splits * c_rows * c_cols, st);

@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "lrtei_internal.h"
+#include "oz_splits.h"
 
 namespace lrtei {
 
@@ -719,12 +720,10 @@ lrtei_status ensure_F32(lrtei_plan* pl, cudaStream_t st) {
   return finish_launch("build_F32");
 }
 
-// Parity classes of the plan's columns: the permutation, its inverse and the step tables on the device.
-lrtei_status ensure_classes(lrtei_plan* pl, cudaStream_t st) {
-  if (pl->d_perm) return LRTEI_OK;
+// Sizes and places of the parity classes of the plan's columns.
+ParityClasses class_sizes(const lrtei_plan* pl) {
   ParityClasses pc;
   const int n = pl->n;
-  const int64_t n3 = (int64_t)n * n * n;
   pc.n = n;
   pc.par = has_parity(pl) ? 1 : 0;
   pc.cnt[0] = (n + 1) / 2;
@@ -739,6 +738,15 @@ lrtei_status ensure_classes(lrtei_plan* pl, cudaStream_t st) {
     pc.rows += (pc.size[c] + 127) / 128 * 128;
     pc.kmax = std::max(pc.kmax, k);
   }
+  return pc;
+}
+
+// Parity classes of the plan's columns: the permutation, its inverse and the step tables on the device.
+lrtei_status ensure_classes(lrtei_plan* pl, cudaStream_t st) {
+  if (pl->d_perm) return LRTEI_OK;
+  ParityClasses pc = class_sizes(pl);
+  const int n = pl->n;
+  const int64_t n3 = (int64_t)n * n * n;
   pc.units = (int)(kpad256(n3) / 128);
   const int nblk = pc.units * 8;
   std::vector<int> perm((size_t)pc.cols, -1), pos((size_t)n3), blk, tab;
@@ -1380,15 +1388,19 @@ bool capturing(cudaStream_t st) {
   if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
   return cap != cudaStreamCaptureStatusNone;
 }
-bool oz_rows_ok(const lrtei_plan* pl, int64_t nr, cudaStream_t st) {
+// out_too: the rows themselves are not allocated yet.
+bool oz_rows_ok(const lrtei_plan* pl, int64_t r0, int64_t r1, bool out_too, cudaStream_t st) {
+  const int64_t nr = r1 - r0;
   if (pl->prec != LRTEI_FP64 || pl->npart > 0 || (!(pl->ozF.d && pl->ozK.d) && capturing(st))) return false;
   const double n3 = (double)pl->n * pl->n * pl->n, np = (double)pl->t.npair;
   const double cuda = ((double)nr * np * n3 + node_fmas(pl, (double)nr)) / kFmaRate;
   const double build = pl->ozK.d ? 0.0 : K_elems(pl) * pl->P / kFmaRate;
   if (cuda <= build + 72.0 * (double)nr * np * n3 / 0.9e15 + 4e-4) return false;
-  const double need = (pl->ozF.d ? 0.0 : 16 * np * n3) + (pl->d_F ? 0.0 : 8 * np * n3) +
-                      (pl->ozK.d ? 0.0 : 24 * K_elems(pl)) + nr * (24 * n3 + 8 * np);
-  return fits(need);
+  const ParityClasses pc = class_sizes(pl);
+  const double cols = (double)pc.cols;
+  return fits((pl->ozF.d ? 0.0 : 16 * np * cols) + (pl->d_F ? 0.0 : 8 * np * n3) +
+              (pl->ozK.d ? 0.0 : 24.0 * pc.rows * pc.kmax) + nr * (24 * cols + (out_too ? 8 * np : 0.0)) +
+              oz::rows_partials(r0, r1, pl->t.npair, pc.size, pc.nclass, pc.cols));
 }
 // J-builds: R >= 2 densities (one is as fast through FP64 F_u, 8 bytes an element against 16), orders up
 // to 32 unless K is there (its build grows as n^6), and enough work to pay for a dozen launches.
@@ -1501,7 +1513,7 @@ lrtei_status bu_rows(lrtei_plan* pl, int form, int64_t r0, int64_t r1, double* o
     }
     return finish_launch("hadamard_rows");
   }
-  if (oz_rows_ok(pl, nr, st)) {
+  if (oz_rows_ok(pl, r0, r1, false, st)) {
     LRTEI_TRY(bu_rows_oz(pl, r0, r1, out, ld, st));
     return finish_launch("factored B rows (digit products)");
   }
@@ -1742,8 +1754,8 @@ lrtei_status lrtei_assemble_B(lrtei_plan* plan, lrtei_form form, double* d_B, in
   rb = std::min(rb, npair);
   if (is_split(plan)) rb = npair;  // one symmetric tensor-core pass over the whole B_u
   else if (f == LRTEI_FORM_FACTORED) {  // the same in digit products, or bands of 4096 rows, where they fit
-    if (oz_rows_ok(plan, npair, st)) rb = npair;
-    else if (npair > 4096 && oz_rows_ok(plan, 4096, st)) rb = 4096;
+    if (oz_rows_ok(plan, 0, npair, true, st)) rb = npair;
+    else if (npair > 4096 && oz_rows_ok(plan, 0, 4096, true, st)) rb = 4096;
   }
   Scratch sc(st);
   double* blk;

@@ -1,0 +1,62 @@
+"""Calls on a nearly full device: what a route allocates beyond its operands is part of the decision to take it.
+
+A tensor fills the device but for what the case names.  Each call has to end well where a route of less scratch exists.
+"""
+import numpy as np
+import pytest
+
+from paper_2210_13069_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lib():
+    import torch
+    from paper_2210_13069_gb300 import build_lib, lrtei
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    build_lib.build()
+    lrtei.load()
+    return lrtei
+
+
+def leave_free(nbytes):
+    """A tensor that leaves nbytes of the device's memory free."""
+    import torch
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    assert free > nbytes, "the device is not free enough for this case"
+    return torch.empty(free - nbytes, dtype=torch.uint8, device="cuda")
+
+
+def rel_fro(a, b):
+    return float(np.linalg.norm(a - b) / np.linalg.norm(b))
+
+
+@pytest.mark.parametrize("natoms,n,free", [(21, 24, 109_500_000_000), (15, 18, 21_000_000_000)])
+def test_fp64_B_where_the_split_partials_do_not_fit(lib, natoms, n, free):
+    """49 770 pairs of order 24: K of 216 pieces goes in three splits, 59 GB of partial sums beside the 53 GB of the
+    operands and B_u; 25 425 pairs of order 18: two splits, 10 beside 12 GB.  B has to come in bands of digit products
+    (1e-12 as in test_gpu_fp64_products.py)."""
+    import torch
+    m = synth.workload_spd(1002, natoms=natoms, n=n, P=20)
+    pl = lib.Plan(m, "fp64")
+    nb2 = m.nbf ** 2
+    B = torch.empty((nb2, nb2), dtype=torch.float64, device="cuda")
+    filler = leave_free(free)
+    lib.lrtei_profile_enable(True)
+    lib.lrtei_profile_reset()
+    pl.assemble_B("factored", out=B)
+    assert lib.lrtei_profile_get("kron")[1] == 0, "the CUDA-core route ran"
+    lib.lrtei_profile_enable(False)
+    pl.status()
+    del filler
+    r0 = 7
+    ref = pl.Bu_rows(r0, r0 + 2, "factored").cpu().numpy()  # two rows: the CUDA-core route
+    mu, nu = np.triu_indices(m.nbf)
+    cols = torch.as_tensor(mu * m.nbf + nu, device="cuda")
+    for i in range(2):
+        row = B[mu[r0 + i] * m.nbf + nu[r0 + i]][cols].cpu().numpy()
+        assert rel_fro(row, ref[i]) <= 1e-12
+    pl.close()
