@@ -2339,14 +2339,8 @@ static lrtei_status jbuild_oz(lrtei_plan* plan, const double* d_D, int R, double
   return finish_launch("jbuild (digit products)");
 }
 
-// One J-build launched kernel by kernel (also what a captured graph replays).
-static lrtei_status jbuild_direct(lrtei_plan* plan, const double* d_D, int R, double* d_J, cudaStream_t st) {
-  ProfScope ps_all("jbuild", st);
-  if (plan->npart > 0) return jbuild_adaptive(plan, d_D, R, d_J, st);
-  const int64_t rb = jbuild_stream_block(plan);
-  if (rb > 0) return jbuild_streamed(plan, d_D, R, d_J, rb, st);
-  if (is_split(plan)) return jbuild_tc(plan, d_D, R, d_J, st);
-  if (oz_jbuild_ok(plan, R, st)) return jbuild_oz(plan, d_D, R, d_J, st);
+// FP64 J-build on the CUDA cores.
+static lrtei_status jbuild_cores(lrtei_plan* plan, const double* d_D, int R, double* d_J, cudaStream_t st) {
   const int nbf = plan->basis.nbf, n = plan->n, P = plan->P;
   const int64_t npair = plan->t.npair, n3 = (int64_t)n * n * n;
   const double pref = plan->omega / sqrt(kPi);
@@ -2375,6 +2369,29 @@ static lrtei_status jbuild_direct(lrtei_plan* plan, const double* d_D, int R, do
     launch_jy(plan->t, nbf, n3, R, plan->d_F, Y, pref, d_J, plan->d_status, st);
   }
   return finish_launch("jbuild");
+}
+
+// One J-build launched kernel by kernel (also what a captured graph replays).
+static lrtei_status jbuild_direct(lrtei_plan* plan, const double* d_D, int R, double* d_J, cudaStream_t st) {
+  ProfScope ps_all("jbuild", st);
+  if (plan->npart > 0) return jbuild_adaptive(plan, d_D, R, d_J, st);
+  const int64_t rb = jbuild_stream_block(plan);
+  if (rb > 0) return jbuild_streamed(plan, d_D, R, d_J, rb, st);
+  if (is_split(plan)) return jbuild_tc(plan, d_D, R, d_J, st);
+  // Both FP64 forms take many densities in groups whose vectors, digits and partial sums stay within about 1 GiB
+  // (hundreds of densities for 180 functions): unbounded, a density more took up to ten times the scratch of its n^3.
+  const bool digits = oz_jbuild_ok(plan, R, st);
+  const int64_t npair = plan->t.npair, n3 = (int64_t)plan->n * plan->n * plan->n;
+  const double each = digits ? 72.0 * class_sizes(plan).cols + 56.0 * npair : 8.0 * (jx_splits(npair, n3) + 2) * n3;
+  const int most = 32 * (int)std::max(1.0, std::min(1e6, (double)(1 << 30) / (32 * each)));
+  const size_t nb2 = (size_t)plan->basis.nbf * plan->basis.nbf;
+  for (int q = 0; q < R; q += most) {
+    const int nq = std::min(most, R - q);
+    const double* D = d_D + (size_t)q * nb2;
+    double* J = d_J + (size_t)q * nb2;
+    LRTEI_TRY(digits ? jbuild_oz(plan, D, nq, J, st) : jbuild_cores(plan, D, nq, J, st));
+  }
+  return LRTEI_OK;
 }
 
 extern "C" {

@@ -2,6 +2,8 @@
 
 A tensor fills the device but for what the case names.  Each call has to end well where a route of less scratch exists.
 """
+import contextlib
+
 import numpy as np
 import pytest
 
@@ -20,14 +22,20 @@ def lib():
     return lrtei
 
 
+@contextlib.contextmanager
 def leave_free(nbytes):
-    """A tensor that leaves nbytes of the device's memory free."""
+    """Leaves nbytes of the device's memory free for a while."""
     import torch
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
     free, _ = torch.cuda.mem_get_info()
     assert free > nbytes, "the device is not free enough for this case"
-    return torch.empty(free - nbytes, dtype=torch.uint8, device="cuda")
+    filler = torch.empty(free - nbytes, dtype=torch.uint8, device="cuda")
+    try:
+        yield
+    finally:
+        del filler
+        torch.cuda.empty_cache()
 
 
 def rel_fro(a, b):
@@ -44,14 +52,13 @@ def test_fp64_B_where_the_split_partials_do_not_fit(lib, natoms, n, free):
     pl = lib.Plan(m, "fp64")
     nb2 = m.nbf ** 2
     B = torch.empty((nb2, nb2), dtype=torch.float64, device="cuda")
-    filler = leave_free(free)
     lib.lrtei_profile_enable(True)
     lib.lrtei_profile_reset()
-    pl.assemble_B("factored", out=B)
+    with leave_free(free):
+        pl.assemble_B("factored", out=B)
     assert lib.lrtei_profile_get("kron")[1] == 0, "the CUDA-core route ran"
     lib.lrtei_profile_enable(False)
     pl.status()
-    del filler
     r0 = 7
     ref = pl.Bu_rows(r0, r0 + 2, "factored").cpu().numpy()  # two rows: the CUDA-core route
     mu, nu = np.triu_indices(m.nbf)
@@ -59,4 +66,24 @@ def test_fp64_B_where_the_split_partials_do_not_fit(lib, natoms, n, free):
     for i in range(2):
         row = B[mu[r0 + i] * m.nbf + nu[r0 + i]][cols].cpu().numpy()
         assert rel_fro(row, ref[i]) <= 1e-12
+    pl.close()
+
+
+@pytest.mark.parametrize("precision,R,free", [("fp32", 8192, 3_000_000_000), ("fp64", 16384, 2_900_000_000)])
+def test_jbuild_of_many_densities_has_bounded_scratch(lib, precision, R, free):
+    """60 functions of order 16.  FP32 plans (CUDA cores, 38 partial sums of X) would take 10 GB for all densities at
+    once, FP64 ones (digits and their vectors) 6.6 GB."""
+    import torch
+    import oracle
+    m = synth.workload_spd(1002, natoms=4, cube=8.0, n=16, P=20)
+    pl = lib.Plan(m, precision)
+    few = torch.as_tensor(synth.random_densities(5, m.nbf, 7), device="cuda")
+    D = few[torch.arange(R, device="cuda") % 7].contiguous()
+    J = torch.empty_like(D)
+    with leave_free(free):
+        pl.jbuild(D, out=J)
+    pl.status()
+    ref = oracle.Oracle.from_molecule(m).jbuild_factored(few.cpu().numpy())
+    for q in (0, 31, 1023, R // 2 + 3, R - 1):
+        assert rel_fro(J[q].cpu().numpy(), ref[q % 7]) <= 1e-12
     pl.close()
