@@ -968,6 +968,17 @@ lrtei_status scratch_split(Scratch& sc, SplitMatrix& m, int64_t rows, int64_t k,
   return sc.get(&m.expo, rows);
 }
 
+// Whether `bytes` more fit in sixty percent of the free device memory (small needs are not asked about).
+bool fits(double bytes) {
+  if (bytes < 1e9) return true;
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return bytes <= 0.6 * (double)free_b;
+}
+
 // Positive integer from the environment (0 when unset): the host-output pipeline's band count
 // and copy chunk, for tests that need many bands on a small molecule.
 static int64_t env_count(const char* name) {
@@ -1167,8 +1178,10 @@ lrtei_status bu_adaptive(lrtei_plan* pl, double* Bu, cudaStream_t st) {
         most = std::max(most, ns);
       }
     // Small blocks B_st (fewer tiles than SMs) are formed in one launch for all pairs once every G is there: at
-    // 60 functions a block's 16 tiles took as long as all 160.  Large ones pair by pair, with one G.
-    const bool together = (most + 127) / 128 * ((maxr + 127) / 128) < 152;
+    // 60 functions a block's 16 tiles took as long as all 160.  Large ones, and where the G's, their slices and the
+    // blocks of all pairs do not fit, pair by pair with one G.
+    const bool together = (most + 127) / 128 * ((maxr + 127) / 128) < 152 &&
+                          fits((double)grows * (8.0 * pc.cols + 6.0 * kpad256(n3) + 8.0 * maxr));
     if (!together) grows = most;
     LRTEI_TRY(scratch_split(sc, Fsp, tile0.back(), n3, 128, pl));
     Ksp = split_shape(pl, pc.rows, K_cols(pl), K_kpad(pc), 128);
@@ -1356,17 +1369,6 @@ lrtei_status ensure_ozK(lrtei_plan* pl, cudaStream_t st) {
   launch_oz_split(K, pc.kmax, pc.kmax, nullptr, nullptr, nullptr, m, st);
   pl->ozK = m;
   return finish_launch("digits of K");
-}
-
-// Whether `bytes` more fit in sixty percent of the free device memory (small needs are not asked about).
-bool fits(double bytes) {
-  if (bytes < 1e9) return true;
-  size_t free_b = 0, total_b = 0;
-  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return bytes <= 0.6 * (double)free_b;
 }
 
 // Estimated seconds of the FP64 FMAs of a CUDA-core form (2 FMAs per clock and SM), of the K build, and

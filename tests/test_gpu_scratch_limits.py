@@ -87,3 +87,21 @@ def test_jbuild_of_many_densities_has_bounded_scratch(lib, precision, R, free):
     for q in (0, 31, 1023, R // 2 + 3, R - 1):
         assert rel_fro(J[q].cpu().numpy(), ref[q % 7]) <= 1e-12
     pl.close()
+
+
+def test_adaptive_B_where_the_blocks_of_all_pairs_do_not_fit(lib):
+    """150 functions in eight boxes of about 1400 pairs, order 13: G, its slices and the blocks of all 36 pairs of boxes
+    take 2.5 GB beside B_u (1.0 GB) and F_u (0.4 GB); one after the other 0.1."""
+    import torch
+    m = synth.workload_spd(1002, natoms=10, n=13, P=11)
+    pl = lib.Plan(m, "split_f16", adaptive=(1e-20, 8))
+    nb2 = m.nbf ** 2
+    B = torch.empty((nb2, nb2), dtype=torch.float64, device="cuda")
+    with leave_free(3_000_000_000):
+        pl.assemble_B(out=B)
+    pl.status()
+    tight = B.clone()
+    pl.assemble_B(out=B)
+    pl.status()
+    assert torch.equal(B, tight)  # the same products, tile by tile
+    pl.close()
