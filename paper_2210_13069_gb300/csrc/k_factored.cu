@@ -500,13 +500,7 @@ __global__ void __launch_bounds__(1024) k_expand_B_row(int nbf, int64_t npair, c
   const int nc = nbf * nbf / V;
   ColWalk w(nbf, V * (int)threadIdx.x, V * (int)blockDim.x);
   __syncthreads();
-  if (bulk) {
-    for (long long t0 = clock64(); !tc::mbar_try_wait(&bar, 0u);)
-      if (clock64() - t0 > tc::kWaitCycles) {
-        latch_status(status, (int)kDevTimeout);
-        break;
-      }
-  }
+  if (bulk) tc::wait_staged(&bar, status);
   bool bad = false;
   for (int c = threadIdx.x; c < nc; c += blockDim.x, w.next()) {
     double v[V];

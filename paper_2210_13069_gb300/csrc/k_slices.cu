@@ -4,6 +4,9 @@
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
+#include <stdlib.h>
+
+#include <algorithm>
 
 #include "lrtei_internal.h"
 #include "tc_common.h"
@@ -132,7 +135,8 @@ __global__ void __launch_bounds__(256) k_split_rows_warp(const double* __restric
 constexpr int64_t kSplitCols = 28000;
 __global__ void __launch_bounds__(512) k_split_rows(const double* __restrict__ src, int64_t cols, int64_t k, int64_t ld,
                                                     int64_t kpad, int tile, int bulk, const int* __restrict__ map,
-                                                    uint16_t* __restrict__ d, int* __restrict__ expo) {
+                                                    uint16_t* __restrict__ d, int* __restrict__ expo, int* status,
+                                                    long long stall) {
   extern __shared__ __align__(16) double row[];  // cols: the source row's columns (k without a map)
   __shared__ uint32_t red[32];
   __shared__ uint64_t bar;
@@ -148,8 +152,7 @@ __global__ void __launch_bounds__(512) k_split_rows(const double* __restrict__ s
       bulk_load(row, x, (uint32_t)(nc * 8), &bar);
     }
     __syncthreads();
-    for (long long t0 = clock64(); !mbar_try_wait(&bar, 0u) && clock64() - t0 < kWaitCycles;) {
-    }
+    wait_staged(&bar, status, stall);
 #pragma unroll 4
     for (int i = threadIdx.x; i < nc; i += blockDim.x) mx = max(mx, magnitude(row[i]));
   } else {
@@ -327,7 +330,8 @@ __global__ void __launch_bounds__(512) k_split_orbital_rows(int nbf, int64_t n3,
                                                             const double* __restrict__ Z, const int* __restrict__ map,
                                                             const uint32_t* __restrict__ mx,
                                                             const int* __restrict__ row_expo, int64_t k, int64_t kpad,
-                                                            int tile, uint16_t* __restrict__ d, int* __restrict__ expo) {
+                                                            int tile, uint16_t* __restrict__ d, int* __restrict__ expo,
+                                                            int* status, long long stall) {
   extern __shared__ __align__(16) double row[];
   __shared__ uint64_t bar;
   const int64_t i = blockIdx.x;
@@ -347,8 +351,7 @@ __global__ void __launch_bounds__(512) k_split_orbital_rows(int nbf, int64_t n3,
   }
   if (j == 0 && threadIdx.x == 0) expo[mu] = e;
   __syncthreads();
-  for (long long t0 = clock64(); !mbar_try_wait(&bar, 0u) && clock64() - t0 < kWaitCycles;) {
-  }
+  wait_staged(&bar, status, stall);
   store_row(row, map, n3, e, mu, (int64_t)j * n3, n3, tile, kpad, d);
   if ((int64_t)(j + 1) * n3 == k)  // the padding after the last orbital
     store_row(row, nullptr, 0, e, mu, k, kpad - k, tile, kpad, d);
@@ -425,6 +428,12 @@ __global__ void __launch_bounds__(256) k_reduce_many(const double* __restrict__ 
   }
 }
 
+// LRTEI_TEST_STALL_STAGED_CYCLES (tests only): the kernels that stage rows also wait that long for what never comes.
+static long long staged_stall_cycles() {
+  const char* v = getenv("LRTEI_TEST_STALL_STAGED_CYCLES");
+  return (v && *v) ? std::max(0LL, atoll(v)) : 0;
+}
+
 }  // namespace tc
 
 bool launch_split_density(const PairTable& t, int nbf, int64_t R, const double* d_D, const SplitMatrix& m,
@@ -437,7 +446,7 @@ bool launch_split_density(const PairTable& t, int nbf, int64_t R, const double* 
 }
 
 void launch_split_rows(const double* d_src, int64_t rows, int64_t k, int64_t ld, const SplitMatrix& m, const int* d_map,
-                       cudaStream_t st) {
+                       int* d_status, cudaStream_t st) {
   if (rows <= 0) return;
   count_launch();
   if (m.plain) {
@@ -467,7 +476,7 @@ void launch_split_rows(const double* d_src, int64_t rows, int64_t k, int64_t ld,
                                     (int)(sizeof(double) * tc::kSplitCols)) == cudaSuccess;
   const int bulk = (cols % 2 == 0 && ld % 2 == 0 && (reinterpret_cast<uintptr_t>(d_src) & 15) == 0) ? 1 : 0;
   tc::k_split_rows<<<(unsigned)rows, cols > 8192 ? 512 : 256, sizeof(double) * (size_t)cols, st>>>(
-      d_src, cols, k, ld, m.kpad, m.tile, bulk, d_map, m.d, m.expo);
+      d_src, cols, k, ld, m.kpad, m.tile, bulk, d_map, m.d, m.expo, d_status, tc::staged_stall_cycles());
 }
 
 bool launch_split_MT(int nbf, int64_t n3, const double* d_F, int64_t ldF, const SplitMatrix& m, cudaStream_t st) {
@@ -484,7 +493,7 @@ bool launch_split_MT(int nbf, int64_t n3, const double* d_F, int64_t ldF, const 
 }
 
 bool launch_split_orbitals(int nbf, int64_t n3, int nj, const double* d_Z, int64_t cols, const int* d_map,
-                           uint32_t* d_max, const int* d_row_expo, const SplitMatrix& m, cudaStream_t st) {
+                           uint32_t* d_max, const int* d_row_expo, const SplitMatrix& m, int* d_status, cudaStream_t st) {
   if (m.plain || n3 % 8 != 0 || cols % 2 != 0 || cols > tc::kSplitCols || (reinterpret_cast<uintptr_t>(d_Z) & 15)) return false;
   static bool attr_set = false;
   if (!attr_set)
@@ -497,7 +506,8 @@ bool launch_split_orbitals(int nbf, int64_t n3, int nj, const double* d_Z, int64
   }
   count_launch();
   tc::k_split_orbital_rows<<<(unsigned)((int64_t)nj * nbf), cols > 8192 ? 512 : 256, sizeof(double) * (size_t)cols, st>>>(
-      nbf, n3, nj, cols, cols, d_Z, d_map, d_max, d_row_expo, m.k, m.kpad, m.tile, m.d, m.expo);
+      nbf, n3, nj, cols, cols, d_Z, d_map, d_max, d_row_expo, m.k, m.kpad, m.tile, m.d, m.expo, d_status,
+      tc::staged_stall_cycles());
   return true;
 }
 

@@ -857,7 +857,7 @@ lrtei_status ensure_Fsp(lrtei_plan* pl, cudaStream_t st) {
   LRTEI_TRY(alloc_split(pl, pl->Fsp, pl->t.npair, n3, kpad256(n3)));
   {
     ProfScope ps("split", st);
-    launch_split_rows(pl->d_F, pl->t.npair, n3, n3, pl->Fsp, nullptr, st);
+    launch_split_rows(pl->d_F, pl->t.npair, n3, n3, pl->Fsp, nullptr, pl->d_status, st);
   }
   pl->have_Fsp = true;
   return finish_launch("split F");
@@ -918,7 +918,7 @@ lrtei_status slice_K(lrtei_plan* pl, const double* d_C, bool clear, double* K, c
     }
   }
   ProfScope ps("split", st);
-  launch_split_rows(K, pc.rows, ld, ld, m, nullptr, st);
+  launch_split_rows(K, pc.rows, ld, ld, m, nullptr, pl->d_status, st);
   return LRTEI_OK;
 }
 
@@ -945,7 +945,7 @@ lrtei_status ensure_FTsp(lrtei_plan* pl, cudaStream_t st) {
   LRTEI_TRY(alloc_split(pl, pl->FTsp, n3, npair, kpad256(npair)));
   {
     ProfScope ps("split", st);
-    launch_split_rows(FT, n3, npair, npair, pl->FTsp, nullptr, st);
+    launch_split_rows(FT, n3, npair, npair, pl->FTsp, nullptr, pl->d_status, st);
   }
   pl->have_FTsp = true;
   return finish_launch("split F^T");
@@ -1010,7 +1010,7 @@ lrtei_status bu_rows_tc(lrtei_plan* pl, int64_t r0, int64_t r1, double* out, int
   LRTEI_TRY(scratch_split(sc, Gs, nr, n3, 128, pl));
   {
     ProfScope ps("split", st);
-    launch_split_rows(G, nr, n3, pc.cols, Gs, pl->d_pos, st);  // back to the natural column order
+    launch_split_rows(G, nr, n3, pc.cols, Gs, pl->d_pos, pl->d_status, st);  // back to the natural column order
   }
   const bool sym = r0 == 0 && r1 == npair;
   return tc_gemm(Gs, 0, pl->Fsp, nr, npair, 1.0, out, ld, false, sym, 1, nullptr, pl->d_status, st);
@@ -1075,7 +1075,7 @@ static lrtei_status assemble_B_host_banded(lrtei_plan* pl, double* hB, int64_t l
     Gs.rows = nr;
     {
       ProfScope ps("split", st);
-      launch_split_rows(G, nr, n3, pc.cols, Gs, pl->d_pos, st);
+      launch_split_rows(G, nr, n3, pc.cols, Gs, pl->d_pos, pl->d_status, st);
     }
     if ((status = tc_gemm_sym_band(Gs, pl->Fsp, r0, r1, npair, Bu, npair, pl->d_status, st)) != LRTEI_OK) break;
     // basis functions a whose pairs (a, b >= a) all lie below r1: rows [a_done N_b, a_end N_b) of B
@@ -1196,7 +1196,7 @@ lrtei_status bu_adaptive(lrtei_plan* pl, double* Bu, cudaStream_t st) {
     {
       ProfScope ps("split", st);
       for (int s = 0; s < np; ++s)
-        launch_split_rows(ar.Fp + ar.off[s] * n3, ar.off[s + 1] - ar.off[s], n3, n3, rows_of(s), nullptr, st);
+        launch_split_rows(ar.Fp + ar.off[s] * n3, ar.off[s + 1] - ar.off[s], n3, n3, rows_of(s), nullptr, pl->d_status, st);
     }
     bool first = true;
     for (const Pair& q : pairs) {
@@ -1210,7 +1210,7 @@ lrtei_status bu_adaptive(lrtei_plan* pl, double* Bu, cudaStream_t st) {
       Gsp.rows = ns;
       {
         ProfScope ps("split", st);
-        launch_split_rows(G, ns, n3, pc.cols, Gsp, pl->d_pos, st);
+        launch_split_rows(G, ns, n3, pc.cols, Gsp, pl->d_pos, pl->d_status, st);
       }
       LRTEI_TRY(tc_gemm(Gsp, 0, rows_of(q.t), ns, nt, 1.0, blk, nt, false, false, 1, nullptr, pl->d_status, st));
       launch_scatter_block(blk, nt, ar.d_idx + ar.off[q.s], ns, ar.d_idx + ar.off[q.t], nt, Bu, npair, q.s != q.t, st);
@@ -1218,7 +1218,7 @@ lrtei_status bu_adaptive(lrtei_plan* pl, double* Bu, cudaStream_t st) {
     if (together) {
       {
         ProfScope ps("split", st);
-        launch_split_rows(G, grows, n3, pc.cols, Gsp, pl->d_pos, st);
+        launch_split_rows(G, grows, n3, pc.cols, Gsp, pl->d_pos, pl->d_status, st);
       }
       std::vector<TcBlock> blocks;
       for (const Pair& q : pairs)
@@ -1874,7 +1874,7 @@ lrtei_status lrtei_exchange(lrtei_plan* plan, const double* d_Q, int norb, doubl
       if (!launch_split_MT(nbf, n3, plan->d_F, n3, MTsp, st)) {
         LRTEI_TRY(need_copy(&MT, (size_t)rowlen * nbf));
         launch_gather_MT(nbf, n3, plan->d_F, n3, MT, st);
-        launch_split_rows(MT, rowlen, nbf, nbf, MTsp, nullptr, st);
+        launch_split_rows(MT, rowlen, nbf, nbf, MTsp, nullptr, plan->d_status, st);
       }
     }
     for (int b = 0; b < nblk; ++b) {
@@ -1883,14 +1883,14 @@ lrtei_status lrtei_exchange(lrtei_plan* plan, const double* d_Q, int norb, doubl
       Qb.rows = nj;
       {
         ProfScope ps("split", st);
-        launch_split_rows(d_Q + (size_t)j0 * nbf, nj, nbf, nbf, Qb, nullptr, st);
+        launch_split_rows(d_Q + (size_t)j0 * nbf, nj, nbf, nbf, Qb, nullptr, plan->d_status, st);
       }
       LRTEI_TRY(tc_gemm_few(Qb, MTsp, nj, rowlen, X, rowlen, plan->d_status, st));
       SplitMatrix Xb = Xsp;
       Xb.rows = (int64_t)nj * nbf;
       {
         ProfScope ps("split", st);
-        launch_split_rows(X, Xb.rows, n3, n3, Xb, nullptr, st);
+        launch_split_rows(X, Xb.rows, n3, n3, Xb, nullptr, plan->d_status, st);
       }
       LRTEI_TRY(tc_gemm_K(Xb, 0, plan->Ksp, plan->pc, Xb.rows, false, Y, 1, nullptr, plan->d_status, st));
       SplitMatrix Ya = Ypsp, Xa = Xpsp;
@@ -1898,15 +1898,15 @@ lrtei_status lrtei_exchange(lrtei_plan* plan, const double* d_Q, int norb, doubl
       Xa.set_k((int64_t)nj * n3);
       {
         ProfScope ps("split", st);
-        if (!launch_split_orbitals(nbf, n3, nj, Y, ycols, plan->d_pos, dmax, nullptr, Ya, st)) {
+        if (!launch_split_orbitals(nbf, n3, nj, Y, ycols, plan->d_pos, dmax, nullptr, Ya, plan->d_status, st)) {
           LRTEI_TRY(need_copy(&Yp, (size_t)ob * rowlen));
           launch_perm_orbital_rows(nbf, n3, nj, Y, ycols, plan->d_pos, Yp, st);
-          launch_split_rows(Yp, nbf, (int64_t)nj * n3, (int64_t)nj * n3, Ya, nullptr, st);
+          launch_split_rows(Yp, nbf, (int64_t)nj * n3, (int64_t)nj * n3, Ya, nullptr, plan->d_status, st);
         }
-        if (!launch_split_orbitals(nbf, n3, nj, X, n3, nullptr, dmax, Xb.expo, Xa, st)) {
+        if (!launch_split_orbitals(nbf, n3, nj, X, n3, nullptr, dmax, Xb.expo, Xa, plan->d_status, st)) {
           LRTEI_TRY(need_copy(&Xp, (size_t)ob * rowlen));
           launch_perm_orbital_rows(nbf, n3, nj, X, n3, nullptr, Xp, st);
-          launch_split_rows(Xp, nbf, (int64_t)nj * n3, (int64_t)nj * n3, Xa, nullptr, st);
+          launch_split_rows(Xp, nbf, (int64_t)nj * n3, (int64_t)nj * n3, Xa, nullptr, plan->d_status, st);
         }
       }
       const int sb = splits_for(nbf, (int64_t)nj * n3);
@@ -2064,19 +2064,19 @@ static lrtei_status jbuild_tc(lrtei_plan* plan, const double* d_D, int R, double
     launch_pack_density(nbf, R, d_D, Du, st);
     launch_transpose(Du, npair, R, R, DuT, npair, st);
     ProfScope ps("split", st);
-    launch_split_rows(DuT, R, npair, npair, Dsp, nullptr, st);
+    launch_split_rows(DuT, R, npair, npair, Dsp, nullptr, plan->d_status, st);
   }
   // X^T = (F^T D_u)^T : R x n^3
   LRTEI_TRY(tc_gemm(plan->FTsp, 0, Dsp, n3, R, 1.0, XT, n3, true, false, s1, part, plan->d_status, st));
   {
     ProfScope ps("split", st);
-    launch_split_rows(XT, R, n3, n3, Xsp, nullptr, st);
+    launch_split_rows(XT, R, n3, n3, Xsp, nullptr, plan->d_status, st);
   }
   // Y^T = (K X)^T (K symmetric), its columns in class order
   LRTEI_TRY(tc_gemm_K(Xsp, 0, plan->Ksp, pc, R, true, YT, s2, part, plan->d_status, st));
   {
     ProfScope ps("split", st);
-    launch_split_rows(YT, R, n3, pc.cols, Ysp, plan->d_pos, st);
+    launch_split_rows(YT, R, n3, pc.cols, Ysp, plan->d_pos, plan->d_status, st);
   }
   // J_u = F Y : npair x R
   LRTEI_TRY(tc_gemm(plan->Fsp, 0, Ysp, npair, R, 1.0, Ju, R, false, false, s3, part, plan->d_status, st));
@@ -2150,8 +2150,8 @@ static lrtei_status jbuild_streamed(lrtei_plan* plan, const double* d_D, int R, 
     Bm.set_k(nr);
     {
       ProfScope ps("split", st);
-      launch_split_rows(FbT, n3, nr, nr, A, nullptr, st);
-      launch_split_rows(DbT, R, nr, nr, Bm, nullptr, st);
+      launch_split_rows(FbT, n3, nr, nr, A, nullptr, plan->d_status, st);
+      launch_split_rows(DbT, R, nr, nr, Bm, nullptr, plan->d_status, st);
     }
     const int sb = splits_for(n3, nr);
     LRTEI_TRY(tc_gemm(A, 0, Bm, n3, R, 1.0, Xparts + b * R * n3, n3, true, false, sb, part, plan->d_status, st));
@@ -2163,7 +2163,7 @@ static lrtei_status jbuild_streamed(lrtei_plan* plan, const double* d_D, int R, 
   }
   {
     ProfScope ps("split", st);
-    launch_split_rows(Yt, R, n3, n3, Ysp, nullptr, st);
+    launch_split_rows(Yt, R, n3, n3, Ysp, nullptr, plan->d_status, st);
   }
   for (int64_t b = 0; b < nblk; ++b) {
     const int64_t r0 = b * rb, nr = std::min(npair, r0 + rb) - r0;
@@ -2172,7 +2172,7 @@ static lrtei_status jbuild_streamed(lrtei_plan* plan, const double* d_D, int R, 
     A.rows = nr;
     {
       ProfScope ps("split", st);
-      launch_split_rows(Fb, nr, n3, n3, A, nullptr, st);
+      launch_split_rows(Fb, nr, n3, n3, A, nullptr, plan->d_status, st);
     }
     LRTEI_TRY(tc_gemm(A, 0, Ysp, nr, R, 1.0, Ju + r0 * R, R, false, false, splits_for(nr, n3), part, plan->d_status, st));
   }
@@ -2229,8 +2229,8 @@ lrtei_status lrtei_jbuild_partial_x(lrtei_plan* plan, const double* d_D, int R, 
   launch_transpose(Du + pair_begin * R, nr, R, R, DbT, nr, st);
   {
     ProfScope ps("split", st);
-    launch_split_rows(FbT, n3, nr, nr, A, nullptr, st);
-    launch_split_rows(DbT, R, nr, nr, Bm, nullptr, st);
+    launch_split_rows(FbT, n3, nr, nr, A, nullptr, plan->d_status, st);
+    launch_split_rows(DbT, R, nr, nr, Bm, nullptr, plan->d_status, st);
   }
   LRTEI_TRY(tc_gemm(A, 0, Bm, n3, R, 1.0, d_X, n3, true, false, sb, part, plan->d_status, st));
   return finish_launch("partial X (tensor cores)");
@@ -2269,8 +2269,8 @@ lrtei_status lrtei_jbuild_apply_x(lrtei_plan* plan, const double* d_X, int R, in
     LRTEI_TRY(scratch_split(sc, Ysp, R, n3, split_tile(R), plan));
     {
       ProfScope ps("split", st);
-      launch_split_rows(Fb, nr, n3, n3, A, nullptr, st);
-      launch_split_rows(Y, R, n3, n3, Ysp, nullptr, st);
+      launch_split_rows(Fb, nr, n3, n3, A, nullptr, plan->d_status, st);
+      launch_split_rows(Y, R, n3, n3, Ysp, nullptr, plan->d_status, st);
     }
     LRTEI_TRY(tc_gemm(A, 0, Ysp, nr, R, 1.0, Ju, R, false, false, s3, part, plan->d_status, st));
   }

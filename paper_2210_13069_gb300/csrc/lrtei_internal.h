@@ -342,7 +342,7 @@ inline int split_tile(int64_t N) { return N <= 32 ? 32 : N <= 64 ? 64 : 128; }
 // Slice an FP64 row-major matrix (rows x k, ld) into a SplitMatrix (zero padded to kpad); column j is
 // source column d_map[j] (NULL: j).
 void launch_split_rows(const double* d_src, int64_t rows, int64_t k, int64_t ld, const SplitMatrix& m, const int* d_map,
-                       cudaStream_t st);
+                       int* d_status, cudaStream_t st);
 // R densities D as rows over the unique pairs (the off-diagonal ones doubled) into slices; false, and nothing
 // launched, where a plain operand or too many rows want the packed copy.
 bool launch_split_density(const PairTable& t, int nbf, int64_t R, const double* d_D, const SplitMatrix& m,
@@ -380,7 +380,7 @@ lrtei_status tc_gemm_sym_band(const SplitMatrix& A, const SplitMatrix& B, int64_
 // Z[(j nbf + mu) cols + map[m]] (map NULL: m); d_max: nbf scratch words, unless the exponents of Z's rows are given.
 bool launch_split_MT(int nbf, int64_t n3, const double* d_F, int64_t ldF, const SplitMatrix& m, cudaStream_t st);
 bool launch_split_orbitals(int nbf, int64_t n3, int nj, const double* d_Z, int64_t cols, const int* d_map,
-                           uint32_t* d_max, const int* d_row_expo, const SplitMatrix& m, cudaStream_t st);
+                           uint32_t* d_max, const int* d_row_expo, const SplitMatrix& m, int* d_status, cudaStream_t st);
 void launch_transpose(const double* in, int64_t rows, int64_t cols, int64_t ldi, double* out, int64_t ldo,
                       cudaStream_t st);
 // out[i][j] = sum_q part[q * stride + i * ld + j] for i < rows, j < cols.

@@ -76,6 +76,19 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return true;
 }
 
+// Waits, bounded, for a row's bulk copy into shared memory (phase 0 of `bar`); expiry raises the status word.  stall > 0
+// (tests only): then waits that many cycles for the next phase, which nothing completes.
+__device__ __forceinline__ void wait_staged(uint64_t* bar, int* status, long long stall = 0) {
+  for (uint32_t phase = 0; phase < (stall > 0 ? 2u : 1u); ++phase) {
+    const long long limit = phase ? stall : kWaitCycles;
+    for (long long t0 = clock64(); !mbar_try_wait(bar, phase);)
+      if (clock64() - t0 > limit) {
+        latch_status(status, (int)kDevTimeout);
+        break;
+      }
+  }
+}
+
 // True on one lane of the (converged) warp.  The MMA warps branch on it rather than on the lane number:
 // the compiler then knows that one thread runs the branch and issues MMAs without a per-thread loop.
 __device__ __forceinline__ bool elect_one() {
