@@ -41,6 +41,7 @@ struct Pool {
   cudaMemPool_t pool = nullptr;
   cudaStream_t st = nullptr;  // plan buffers are allocated and freed in its order, nothing else runs on it
   int plans = 0;              // plans alive on the device
+  void* token = nullptr;      // what device_idle frees
 };
 std::mutex g_pool_mu;
 std::map<int, Pool> g_pools;
@@ -67,6 +68,29 @@ cudaError_t current_pool(Pool** out, int dev = -1) {
   return cudaSuccess;
 }
 
+// Waits for all work of the current device, whose pool p is, as cudaFree does: by a cudaFree.  cudaDeviceSynchronize is
+// refused while any thread captures a stream, in whatever mode, and spoils that thread's capture (of a J-build, say).
+cudaError_t device_idle(Pool* p) {
+  void* t = nullptr;
+  {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    std::swap(t, p->token);
+  }
+  if (!t && cudaMalloc(&t, 16) != cudaSuccess) {  // no memory: the harder way
+    cudaGetLastError();
+    return cudaDeviceSynchronize();
+  }
+  const cudaError_t e = cudaFree(t);
+  if (e == cudaSuccess && cudaMalloc(&t, 16) != cudaSuccess) {
+    cudaGetLastError();
+    t = nullptr;
+  }
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  if (!p->token) std::swap(t, p->token);
+  if (t) cudaFree(t);  // two threads at once: one token is kept
+  return e;
+}
+
 // Plan buffers, usable on every stream when the call returns, as cudaMalloc's.
 cudaError_t plan_malloc(void** q, size_t bytes) {
   Pool* p = nullptr;
@@ -75,7 +99,7 @@ cudaError_t plan_malloc(void** q, size_t bytes) {
   e = cudaMallocFromPoolAsync(q, bytes, p->pool, p->st);
   if (e == cudaErrorMemoryAllocation) {  // what the pool keeps for scratch may be what is missing
     cudaGetLastError();
-    cudaDeviceSynchronize();
+    if (device_idle(p) != cudaSuccess) cudaGetLastError();
     cudaMemPoolTrimTo(p->pool, 0);
     e = cudaMallocFromPoolAsync(q, bytes, p->pool, p->st);
   }
@@ -191,8 +215,9 @@ struct lrtei_plan {
       allocs.erase(it);
       OnDevice on(dev);
       Pool* p = nullptr;
-      cudaDeviceSynchronize();  // kernels of any stream may still use it
-      if (current_pool(&p, dev) == cudaSuccess) cudaFreeAsync(q, p->st);
+      // kernels of any stream may still use it; where that cannot be waited for (a capture of this thread), it is not freed
+      if (current_pool(&p, dev) == cudaSuccess && device_idle(p) == cudaSuccess) cudaFreeAsync(q, p->st);
+      else cudaGetLastError();
       bytes -= b;
     }
   }
@@ -210,8 +235,15 @@ struct lrtei_plan {
     Pool* p = nullptr;
     if (dev < 0 || current_pool(&p, dev) != cudaSuccess) return;
     OnDevice on(dev);
-    if (!allocs.empty()) cudaDeviceSynchronize();
-    for (void* q : allocs) cudaFreeAsync(q, p->st);
+    if (!allocs.empty()) {
+      bool idle = cudaDeviceSynchronize() == cudaSuccess;  // 0.6 us where there is nothing to wait for, device_idle 60
+      if (!idle) {
+        cudaGetLastError();
+        idle = device_idle(p) == cudaSuccess;
+      }
+      if (idle) for (void* q : allocs) cudaFreeAsync(q, p->st);  // (else kept: as in release())
+      else cudaGetLastError();
+    }
     std::lock_guard<std::mutex> lk(g_pool_mu);
     if (--p->plans == 0) cudaMemPoolTrimTo(p->pool, kPoolIdle);
   }

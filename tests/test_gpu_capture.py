@@ -1,0 +1,69 @@
+"""Stream captures beside and around the library's calls.
+
+A plan that gives buffers back in one thread (compression, the FP64 F_u of a J-build) leaves another thread's capture
+alone (captures of the thread-local kind, as the library's own of its J-builds are).
+"""
+import threading
+
+import numpy as np
+import pytest
+
+from paper_2210_13069_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lib():
+    import torch
+    from paper_2210_13069_gb300 import build_lib, lrtei
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    build_lib.build()
+    lrtei.load()
+    return lrtei
+
+
+def molecule():
+    return synth.random_molecule(4301, natoms=2, cube=4.0, nprim=1, alpha_range=(0.15, 40.0), omega=0.45, n=8, P=6)
+
+
+@pytest.mark.parametrize("what", ["jbuild", "compress"])
+def test_plans_of_another_thread_leave_a_capture_alone(lib, what):
+    import torch
+    m = molecule()
+    x = torch.zeros(1000, device="cuda")
+    pl = lib.Plan(m, "split_f16")
+    ref = pl.assemble_B("factored")
+    D = torch.as_tensor(synth.random_densities(5, m.nbf, 2), device="cuda")
+    J = torch.empty_like(D)
+    errors = []
+
+    def other():
+        try:
+            if what == "compress":
+                pl.compress(0.0)  # full rank: releases the operands, B is the same
+            else:
+                pl.jbuild(D, out=J)  # F_u is sliced twice then, its FP64 copy goes
+        except Exception as e:  # reported below, in the test's thread
+            errors.append(e)
+
+    g = torch.cuda.CUDAGraph()
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=side, capture_error_mode="thread_local"):
+        x += 1.0
+        t = threading.Thread(target=other)
+        t.start()
+        t.join()
+        x += 1.0
+    assert not errors, errors
+    g.replay()
+    torch.cuda.synchronize()
+    assert (x == 2.0).all()
+    if what == "compress":
+        B = pl.assemble_B("factored")
+        assert torch.linalg.norm(B - ref) <= 1e-7 * torch.linalg.norm(ref)
+    else:
+        K = torch.einsum("rc,qc->qr", ref, D.reshape(2, -1)).reshape(D.shape)
+        assert torch.linalg.norm(J - K) <= 1e-7 * torch.linalg.norm(K)
+    pl.close()
