@@ -719,8 +719,33 @@ namespace {
 
 const double kPi = 3.14159265358979323846;
 
+// Whether the caller captures the stream.
+bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
+  return cap != cudaStreamCaptureStatusNone;
+}
+
+// An operand that is missing while the caller captures st is built at once on the pool's own stream: recorded into the
+// caller's graph, it would come into being with the graph's replay only, while the plan counts it as there.  As an
+// allocation, this is refused in capture modes other than the relaxed one.
+lrtei_status outside_capture(lrtei_plan* pl, cudaStream_t st, lrtei_status (*ensure)(lrtei_plan*, cudaStream_t)) {
+  Pool* p = nullptr;
+  cudaError_t e = current_pool(&p);
+  if (e == cudaSuccess) e = device_idle(p);  // what it is made of may be in work on other streams
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    set_error("the plan's operands cannot be built during this stream capture: %s", cudaGetErrorString(e));
+    return LRTEI_ERR_ALLOC;
+  }
+  const lrtei_status s = ensure(pl, p->st);
+  e = cudaStreamSynchronize(p->st);
+  return s == LRTEI_OK && e != cudaSuccess ? cuda_fail(e, "operands built during a stream capture") : s;
+}
+
 lrtei_status ensure_T(lrtei_plan* pl, cudaStream_t st) {
   if (pl->d_T) return LRTEI_OK;
+  if (capturing(st)) return outside_capture(pl, st, ensure_T);
   LRTEI_TRY(pl->alloc(&pl->d_T, (size_t)3 * pl->P * pl->t.nrows * pl->n));
   launch_tmat(pl->t.nrows, pl->n, pl->P, pl->d_S, pl->d_C, pl->d_T, st);
   return finish_launch("tmat");
@@ -733,6 +758,7 @@ bool has_parity(const lrtei_plan* pl) { return pl->kr_rank == 0; }
 
 lrtei_status ensure_F64(lrtei_plan* pl, cudaStream_t st) {
   if (pl->d_F) return LRTEI_OK;
+  if (capturing(st)) return outside_capture(pl, st, ensure_F64);
   const int64_t n3 = (int64_t)pl->n * pl->n * pl->n;
   LRTEI_TRY(pl->alloc(&pl->d_F, (size_t)pl->t.npair * n3));
   {
@@ -746,6 +772,7 @@ lrtei_status ensure_F64(lrtei_plan* pl, cudaStream_t st) {
 
 lrtei_status ensure_F32(lrtei_plan* pl, cudaStream_t st) {
   if (pl->d_F32) return LRTEI_OK;
+  if (capturing(st)) return outside_capture(pl, st, ensure_F32);
   const int64_t n3 = (int64_t)pl->n * pl->n * pl->n;
   LRTEI_TRY(pl->alloc(&pl->d_F32, (size_t)pl->t.npair * n3));
   launch_build_F<float>(pl->t, pl->n, pl->d_S, 0, pl->t.npair, pl->d_F32, n3, st);
@@ -776,6 +803,7 @@ ParityClasses class_sizes(const lrtei_plan* pl) {
 // Parity classes of the plan's columns: the permutation, its inverse and the step tables on the device.
 lrtei_status ensure_classes(lrtei_plan* pl, cudaStream_t st) {
   if (pl->d_perm) return LRTEI_OK;
+  if (capturing(st)) return outside_capture(pl, st, ensure_classes);
   ParityClasses pc = class_sizes(pl);
   const int n = pl->n;
   const int64_t n3 = (int64_t)n * n * n;
@@ -884,6 +912,7 @@ void release_split(lrtei_plan* pl, SplitMatrix& m) {
 // F_u slices, the left operand of J-builds and of G, the right one of B_u = G F_u^T.
 lrtei_status ensure_Fsp(lrtei_plan* pl, cudaStream_t st) {
   if (pl->have_Fsp) return LRTEI_OK;
+  if (capturing(st)) return outside_capture(pl, st, ensure_Fsp);
   const int64_t n3 = (int64_t)pl->n * pl->n * pl->n;
   LRTEI_TRY(ensure_F64(pl, st));
   LRTEI_TRY(alloc_split(pl, pl->Fsp, pl->t.npair, n3, kpad256(n3)));
@@ -897,7 +926,7 @@ lrtei_status ensure_Fsp(lrtei_plan* pl, cudaStream_t st) {
 
 // A split-precision plan keeps no FP64 copy of F_u once both slice layouts exist.
 void drop_F64_if_sliced(lrtei_plan* pl, cudaStream_t st) {
-  if (!is_split(pl) || !pl->d_F || !pl->have_Fsp || !pl->have_FTsp) return;
+  if (!is_split(pl) || !pl->d_F || !pl->have_Fsp || !pl->have_FTsp || capturing(st)) return;
   cudaStreamSynchronize(st);  // the slicing kernels read d_F
   const int64_t n3 = (int64_t)pl->n * pl->n * pl->n;
   forget_plan_graphs(pl);
@@ -956,6 +985,7 @@ lrtei_status slice_K(lrtei_plan* pl, const double* d_C, bool clear, double* K, c
 
 lrtei_status ensure_Ksp(lrtei_plan* pl, cudaStream_t st) {
   if (pl->have_Ksp) return LRTEI_OK;
+  if (capturing(st)) return outside_capture(pl, st, ensure_Ksp);
   LRTEI_TRY(ensure_classes(pl, st));
   Scratch sc(st);
   double* K;
@@ -968,6 +998,7 @@ lrtei_status ensure_Ksp(lrtei_plan* pl, cudaStream_t st) {
 
 lrtei_status ensure_FTsp(lrtei_plan* pl, cudaStream_t st) {
   if (pl->have_FTsp) return LRTEI_OK;
+  if (capturing(st)) return outside_capture(pl, st, ensure_FTsp);
   const int64_t n3 = (int64_t)pl->n * pl->n * pl->n, npair = pl->t.npair;
   LRTEI_TRY(ensure_F64(pl, st));
   Scratch sc(st);
@@ -1354,6 +1385,7 @@ lrtei_status scratch_oz(Scratch& sc, OzMatrix& m, int64_t rows, int64_t kpad, in
 
 lrtei_status ensure_ozF(lrtei_plan* pl, cudaStream_t st) {
   if (pl->ozF.d) return LRTEI_OK;
+  if (capturing(st)) return outside_capture(pl, st, ensure_ozF);
   LRTEI_TRY(ensure_classes(pl, st));
   LRTEI_TRY(ensure_F64(pl, st));
   const int64_t n3 = (int64_t)pl->n * pl->n * pl->n;
@@ -1368,6 +1400,7 @@ lrtei_status ensure_ozF(lrtei_plan* pl, cudaStream_t st) {
 // (launch_oz_pack).
 lrtei_status ensure_ozFT(lrtei_plan* pl, cudaStream_t st) {
   if (pl->ozFT.d) return LRTEI_OK;
+  if (capturing(st)) return outside_capture(pl, st, ensure_ozFT);
   LRTEI_TRY(ensure_ozF(pl, st));
   LRTEI_TRY(ensure_F64(pl, st));
   const int64_t n3 = (int64_t)pl->n * pl->n * pl->n, npair = pl->t.npair;
@@ -1385,6 +1418,7 @@ lrtei_status ensure_ozFT(lrtei_plan* pl, cudaStream_t st) {
 // K carries the prefactor omega / sqrt(pi).
 lrtei_status ensure_ozK(lrtei_plan* pl, cudaStream_t st) {
   if (pl->ozK.d) return LRTEI_OK;
+  if (capturing(st)) return outside_capture(pl, st, ensure_ozK);
   LRTEI_TRY(ensure_classes(pl, st));
   const ParityClasses& pc = pl->pc;
   Scratch sc(st);
@@ -1415,12 +1449,6 @@ double node_fmas(const lrtei_plan* pl, double rows) {
 double K_elems(const lrtei_plan* pl) {
   const double n = pl->n, n6 = n * n * n * n * n * n;
   return has_parity(pl) ? n6 / 8 : n6;
-}
-// Operands cannot be built while the caller captures the stream.
-bool capturing(cudaStream_t st) {
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
-  return cap != cudaStreamCaptureStatusNone;
 }
 // out_too: the rows themselves are not allocated yet.
 bool oz_rows_ok(const lrtei_plan* pl, int64_t r0, int64_t r1, bool out_too, cudaStream_t st) {
@@ -1495,6 +1523,7 @@ int choose_form(const lrtei_plan* pl, lrtei_form form) {
 // Slices of T_{d,p} and S'_d and the node tables of the tensor-core Hadamard form (once per plan).
 lrtei_status ensure_had(lrtei_plan* pl, cudaStream_t st) {
   if (pl->have_had) return LRTEI_OK;
+  if (capturing(st)) return outside_capture(pl, st, ensure_had);
   HadOperands& h = pl->had;
   h.nrows = pl->t.nrows;
   h.n = pl->n;

@@ -67,3 +67,41 @@ def test_plans_of_another_thread_leave_a_capture_alone(lib, what):
         K = torch.einsum("rc,qc->qr", ref, D.reshape(2, -1)).reshape(D.shape)
         assert torch.linalg.norm(J - K) <= 1e-7 * torch.linalg.norm(K)
     pl.close()
+
+
+CALLS = {
+    "B split factored": ("split_f16", lambda pl, D, Q: pl.assemble_B("factored")),
+    "B split Hadamard": ("split_f16", lambda pl, D, Q: pl.assemble_B("hadamard")),
+    "B fp64 factored": ("fp64", lambda pl, D, Q: pl.assemble_B("factored")),
+    "B fp64 Hadamard": ("fp64", lambda pl, D, Q: pl.assemble_B("hadamard")),
+    "B fp32": ("fp32", lambda pl, D, Q: pl.assemble_B("factored")),
+    "J split": ("split_f16_8", lambda pl, D, Q: pl.jbuild(D)),
+    "J fp64": ("fp64", lambda pl, D, Q: pl.jbuild(D)),
+    "K split": ("split_f16", lambda pl, D, Q: pl.exchange(Q)),
+}
+
+
+@pytest.mark.parametrize("name", sorted(CALLS))
+def test_operands_of_a_captured_first_call_exist_before_the_replay(lib, name):
+    """The first call of a plan inside a relaxed capture: its operands are there for plain calls, replayed or not."""
+    import torch
+    prec, call = CALLS[name]
+    m = molecule()
+    D = torch.as_tensor(synth.random_densities(5, m.nbf, 3), device="cuda")
+    Q = torch.as_tensor(np.random.default_rng(3).normal(size=(2, m.nbf)), device="cuda")
+    fresh = lib.Plan(m, prec)
+    ref = call(fresh, D, Q)
+    pl = lib.Plan(m, prec)
+    g = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=torch.cuda.Stream(), capture_error_mode="relaxed"):
+        out = call(pl, D, Q)
+    assert torch.equal(call(pl, D, Q), ref)
+    out.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, ref)
+    pl.status()
+    del g
+    pl.close()
+    fresh.close()
