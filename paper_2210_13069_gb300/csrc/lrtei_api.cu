@@ -46,6 +46,10 @@ struct Pool {
 std::mutex g_pool_mu;
 std::map<int, Pool> g_pools;
 
+cudaError_t pool_keeps(cudaMemPool_t pool, uint64_t bytes) {
+  return cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &bytes);
+}
+
 // The pool of the current device, `dev` (created on first use).
 cudaError_t current_pool(Pool** out, int dev = -1) {
   cudaError_t e = cudaSuccess;
@@ -59,8 +63,7 @@ cudaError_t current_pool(Pool** out, int dev = -1) {
     props.location.type = cudaMemLocationTypeDevice;
     props.location.id = dev;
     if ((e = cudaMemPoolCreate(&p.pool, &props)) != cudaSuccess) return e;
-    uint64_t keep = kPoolKeep;
-    if ((e = cudaMemPoolSetAttribute(p.pool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) return e;
+    if ((e = pool_keeps(p.pool, kPoolIdle)) != cudaSuccess) return e;
     if ((e = cudaStreamCreateWithFlags(&p.st, cudaStreamNonBlocking)) != cudaSuccess) return e;
     it = g_pools.emplace(dev, p).first;
   }
@@ -229,7 +232,7 @@ struct lrtei_plan {
       return;
     }
     std::lock_guard<std::mutex> lk(g_pool_mu);
-    ++p->plans;
+    if (p->plans++ == 0) pool_keeps(p->pool, kPoolKeep);
   }
   ~lrtei_plan() {
     Pool* p = nullptr;
@@ -245,7 +248,11 @@ struct lrtei_plan {
       else cudaGetLastError();
     }
     std::lock_guard<std::mutex> lk(g_pool_mu);
-    if (--p->plans == 0) cudaMemPoolTrimTo(p->pool, kPoolIdle);
+    if (--p->plans == 0) {
+      pool_keeps(p->pool, kPoolIdle);
+      // what was freed above counts as free once its stream has come to it
+      if (cudaStreamSynchronize(p->st) != cudaSuccess || cudaMemPoolTrimTo(p->pool, kPoolIdle) != cudaSuccess) cudaGetLastError();
+    }
   }
   lrtei_plan(const lrtei_plan&) = delete;
   lrtei_plan& operator=(const lrtei_plan&) = delete;
