@@ -1038,16 +1038,23 @@ lrtei_status scratch_split(Scratch& sc, SplitMatrix& m, int64_t rows, int64_t k,
   return sc.get(&m.expo, rows);
 }
 
-// Whether `bytes` more fit in sixty percent of the free device memory (small needs are not asked about).
-bool fits(double bytes) {
-  if (bytes < 1e9) return true;
+// Memory that the library can still have: the device's free memory and what its pool holds for reuse.  < 0: not known.
+double free_memory() {
   size_t free_b = 0, total_b = 0;
-  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return bytes <= 0.6 * (double)free_b;
+  uint64_t held = 0, used = 0;
+  Pool* p = nullptr;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // the pool's figures are refused inside other captures
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  const bool known = cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && current_pool(&p) == cudaSuccess &&
+                     cudaMemPoolGetAttribute(p->pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
+                     cudaMemPoolGetAttribute(p->pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (!known) cudaGetLastError();
+  return known ? (double)free_b + (double)held - (double)used : -1.0;
 }
+
+// Whether `bytes` more fit in sixty percent of it (small needs are not asked about).
+bool fits(double bytes) { return bytes < 1e9 || bytes <= 0.6 * free_memory(); }
 
 // Positive integer from the environment (0 when unset): the host-output pipeline's band count
 // and copy chunk, for tests that need many bands on a small molecule.
@@ -2354,18 +2361,15 @@ static int64_t jbuild_stream_block(const lrtei_plan* plan) {
   // operands already resident: the one-pass J-build needs nothing more
   if (is_split(plan) ? (plan->have_FTsp && plan->have_Fsp && plan->have_Ksp) : plan->d_F != nullptr) return 0;
   const int64_t npair = plan->t.npair, n3 = (int64_t)plan->n * plan->n * plan->n;
-  size_t free_b = 0, total_b = 0;
-  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
+  const double free_b = free_memory();
+  if (free_b < 0) return 0;
   const double f = (double)npair * n3, k = (double)n3 * n3;
   // split: F (FP64) + F^T (FP64, transient) + F^T and F slices + K (FP64) and its slices;
   // FP64: F.  Already-built operands are counted as if they had to be built.
   const double need = is_split(plan) ? f * (8 + 8 + 6 + 8) + k * (8 + 6) : f * 8;
-  if (need <= 0.5 * (double)free_b) return 0;
+  if (need <= 0.5 * free_b) return 0;
   const double per_row = (double)n3 * (is_split(plan) ? 8 + 8 + 8 + 8 : 8);
-  int64_t rb = (int64_t)(0.15 * (double)free_b / per_row);
+  int64_t rb = (int64_t)(0.15 * free_b / per_row);
   rb = std::max<int64_t>(128, rb / 128 * 128);
   return std::min(rb, npair);
 }

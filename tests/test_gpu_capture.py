@@ -105,3 +105,22 @@ def test_operands_of_a_captured_first_call_exist_before_the_replay(lib, name):
     del g
     pl.close()
     fresh.close()
+
+
+@pytest.mark.parametrize("mode", ["global", "thread_local"])
+def test_a_B_that_asks_for_the_free_memory_can_be_captured(lib, mode):
+    """105 functions of order 18 in digit products: 1.6 GB of scratch, which the call looks for."""
+    import torch
+    m = synth.workload_spd(1002, natoms=7, n=18, P=20)
+    pl = lib.Plan(m, "fp64")
+    ref = pl.assemble_B("factored")
+    out = torch.empty_like(ref)
+    g = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=torch.cuda.Stream(), capture_error_mode=mode):
+        pl.assemble_B("factored", out=out)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, ref)
+    del g
+    pl.close()

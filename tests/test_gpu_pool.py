@@ -15,7 +15,7 @@ def test_pool_keeps_at_most_2_GiB_after_the_last_plan():
     lrtei.load()
     gc.collect()  # plans that other tests left
     torch.cuda.synchronize()
-    m = synth.workload_spd(natoms=10, n=20, P=20)
+    m = synth.workload_spd()
     small = lrtei.Plan(synth.workload_small_s(), "fp64")
     small.close()  # modules and the like are loaded now
     nb2 = m.nbf ** 2

@@ -105,3 +105,25 @@ def test_adaptive_B_where_the_blocks_of_all_pairs_do_not_fit(lib):
     pl.status()
     assert torch.equal(B, tight)  # the same products, tile by tile
     pl.close()
+
+
+def test_the_idle_pool_counts_as_free_memory(lib):
+    """150 functions of order 18: a B in digit products needs 4.8 GB of scratch and leaves about 3.9 in the pool.  With
+    5 GB free beside that it is formed whole again, not in bands."""
+    import torch
+    m = synth.workload_spd(1002, natoms=10, n=18, P=20)
+    pl = lib.Plan(m, "fp64")
+    nb2 = m.nbf ** 2
+    B = torch.empty((nb2, nb2), dtype=torch.float64, device="cuda")
+    pl.assemble_B("factored", out=B)  # its operands are built
+    first = B.clone()
+    with leave_free(5_000_000_000):
+        lib.lrtei_profile_enable(True)
+        lib.lrtei_profile_reset()
+        pl.assemble_B("factored", out=B)
+        products = lib.lrtei_profile_get("gemm_fp64")[1]
+        lib.lrtei_profile_enable(False)
+    pl.status()
+    assert products == 2, "G and B_u: the rows came in bands"
+    assert torch.equal(B, first)
+    pl.close()
