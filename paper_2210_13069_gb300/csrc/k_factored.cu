@@ -530,12 +530,8 @@ void launch_expand_B(const PairTable& t, int nbf, int64_t npair, const double* d
     return;
   }
   const size_t smem = sizeof(double) * (size_t)(npair + 2);
-  static bool attr_set = false;
-  if (!attr_set) {
-    const int most = (int)(sizeof(double) * (kExpandPairs + 2));
-    attr_set = cudaFuncSetAttribute(k_expand_B_row<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess &&
-               cudaFuncSetAttribute(k_expand_B_row<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess;
-  }
+  shared_opt_in<&k_expand_B_row<1>>(sizeof(double) * (kExpandPairs + 2));  // a refusal shows at the launch
+  shared_opt_in<&k_expand_B_row<4>>(sizeof(double) * (kExpandPairs + 2));
   // a row alone on its SM takes all its threads; several short ones share it
   const int threads = npair >= 8192 ? 1024 : npair >= 2048 ? 512 : 256;
   const int bulk = (ldu % 2 == 0 && ldu >= (npair + 1) / 2 * 2 && (reinterpret_cast<uintptr_t>(d_Bu) & 15) == 0) ? 1 : 0;

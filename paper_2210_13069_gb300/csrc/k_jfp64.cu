@@ -126,13 +126,7 @@ cudaError_t launch_kron_apply(int n, int P, const double* d_C, const double* d_w
   cudaError_t e = scratch_alloc((void**)&Z, sizeof(double) * (size_t)rows * P * n3, st);
   if (e != cudaSuccess) return e;
   const size_t smem = sizeof(double) * 2 * ((size_t)n * n + (size_t)n * (n + 1));
-  static bool attr_set = false;
-  if (!attr_set) {
-    const int most = (int)(sizeof(double) * 2 * (kMaxN * kMaxN + kMaxN * (kMaxN + 1)));
-    e = cudaFuncSetAttribute(k_node_modes, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  shared_opt_in<&k_node_modes>(sizeof(double) * 2 * (kMaxN * kMaxN + kMaxN * (kMaxN + 1)));  // a refusal shows below
   const int par = parity ? 1 : 0;
   for (int64_t r0 = 0; r0 < ncol; r0 += rows) {
     const int64_t nr = std::min(rows, ncol - r0);

@@ -295,10 +295,7 @@ void launch_oz_split(const double* d_src, int64_t k, int64_t ld, const int* d_ro
                      const int* d_colexp, OzMatrix& m, cudaStream_t st) {
   if (m.rows <= 0) return;
   constexpr int64_t most = 28000;  // columns that fit shared memory
-  static bool attr_set = false;
-  if (!attr_set)
-    attr_set = cudaFuncSetAttribute(oz::k_oz_split, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)(sizeof(double) * most)) == cudaSuccess;
+  shared_opt_in<&oz::k_oz_split>(sizeof(double) * most);  // a refusal shows at the launch
   const int staged = k <= most ? 1 : 0;
   count_launch();
   oz::k_oz_split<<<(unsigned)m.rows, m.rows < 2 * 152 || k > 4096 ? 512 : 256, staged ? sizeof(double) * (size_t)k : 0, st>>>(

@@ -470,10 +470,7 @@ void launch_split_rows(const double* d_src, int64_t rows, int64_t k, int64_t ld,
     tc::k_split_rows_long<<<(unsigned)rows, 256, 0, st>>>(d_src, k, ld, m.kpad, m.tile, d_map, m.d, m.expo);
     return;
   }
-  static bool attr_set = false;
-  if (!attr_set)
-    attr_set = cudaFuncSetAttribute(tc::k_split_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)(sizeof(double) * tc::kSplitCols)) == cudaSuccess;
+  shared_opt_in<&tc::k_split_rows>(sizeof(double) * tc::kSplitCols);  // a refusal shows at the launch
   const int bulk = (cols % 2 == 0 && ld % 2 == 0 && (reinterpret_cast<uintptr_t>(d_src) & 15) == 0) ? 1 : 0;
   tc::k_split_rows<<<(unsigned)rows, cols > 8192 ? 512 : 256, sizeof(double) * (size_t)cols, st>>>(
       d_src, cols, k, ld, m.kpad, m.tile, bulk, d_map, m.d, m.expo, d_status, tc::staged_stall_cycles());
@@ -482,10 +479,7 @@ void launch_split_rows(const double* d_src, int64_t rows, int64_t k, int64_t ld,
 bool launch_split_MT(int nbf, int64_t n3, const double* d_F, int64_t ldF, const SplitMatrix& m, cudaStream_t st) {
   const size_t smem = sizeof(double) * 33 * (size_t)nbf;
   if (m.plain || nbf > 256 || m.kpad > 256) return false;
-  static bool attr_set = false;
-  if (!attr_set)
-    attr_set = cudaFuncSetAttribute(tc::k_split_MT, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)(sizeof(double) * 33 * 256)) == cudaSuccess;
+  shared_opt_in<&tc::k_split_MT>(sizeof(double) * 33 * 256);
   count_launch();
   tc::k_split_MT<<<dim3((unsigned)((n3 + 31) / 32), (unsigned)nbf), 256, smem, st>>>(
       nbf, n3, d_F, ldF, m.kpad, (m.steps() + 1) / 2 * 32, m.tile, m.d, m.expo);
@@ -495,10 +489,7 @@ bool launch_split_MT(int nbf, int64_t n3, const double* d_F, int64_t ldF, const 
 bool launch_split_orbitals(int nbf, int64_t n3, int nj, const double* d_Z, int64_t cols, const int* d_map,
                            uint32_t* d_max, const int* d_row_expo, const SplitMatrix& m, int* d_status, cudaStream_t st) {
   if (m.plain || n3 % 8 != 0 || cols % 2 != 0 || cols > tc::kSplitCols || (reinterpret_cast<uintptr_t>(d_Z) & 15)) return false;
-  static bool attr_set = false;
-  if (!attr_set)
-    attr_set = cudaFuncSetAttribute(tc::k_split_orbital_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)(sizeof(double) * tc::kSplitCols)) == cudaSuccess;
+  shared_opt_in<&tc::k_split_orbital_rows>(sizeof(double) * tc::kSplitCols);
   if (!d_row_expo) {
     cudaMemsetAsync(d_max, 0, sizeof(uint32_t) * (size_t)nbf, st);
     count_launch();

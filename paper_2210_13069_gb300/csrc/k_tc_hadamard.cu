@@ -480,16 +480,9 @@ static lrtei_status launch_had_kernel(const HadOperands& h, const tch::Params& p
     set_error("cuTensorMapEncodeTiled failed for the Hadamard operands");
     return LRTEI_ERR_CUDA;
   }
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_tc_hadamard<KS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)Cfg<KS>::SMEM);
-    if (e != cudaSuccess) return cuda_fail(e, "tensor-core Hadamard smem attribute");
-    attr_set = true;
-  }
-  int dev = 0, nsm = 152;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  LRTEI_CUDA(shared_opt_in<&k_tc_hadamard<KS>>(Cfg<KS>::SMEM));
+  int nsm = 0;
+  LRTEI_CUDA(sm_count(&nsm));
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(p.ntiles, nsm));
   count_launch();
   k_tc_hadamard<KS><<<(unsigned)grid, THREADS, Cfg<KS>::SMEM, st>>>(m[0], m[1], m[2], m[3], m[4], m[5], m[6], p);

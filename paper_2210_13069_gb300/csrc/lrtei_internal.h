@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/lrtei.h"
+#include "device_once.h"
 
 namespace lrtei {
 

@@ -375,18 +375,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
 // ------------------------------------------------------------------ host side
 template <class S>
 lrtei_status launch(const Params& p, cudaStream_t st) {
-  static bool attr_set = false;  // once per instantiation (also keeps it out of stream capture)
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_tc_gemm<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo<S>::SMEM);
-    if (e != cudaSuccess) return cuda_fail(e, "tensor-core GEMM shared-memory attribute");
-    attr_set = true;
-  }
-  static int nsm = 0;  // persistent grid: one CTA per SM (shared memory and TMEM allow one)
-  if (nsm <= 0) {
-    int dev = 0;
-    LRTEI_CUDA(cudaGetDevice(&dev));
-    LRTEI_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  }
+  LRTEI_CUDA(shared_opt_in<&k_tc_gemm<S>>(Geo<S>::SMEM));
+  int nsm = 0;  // persistent grid: one CTA per SM (shared memory and TMEM allow one)
+  LRTEI_CUDA(sm_count(&nsm));
   const int64_t items = p.nitems * p.splits;
   if (items <= 0) return LRTEI_OK;
   count_launch();
