@@ -1470,8 +1470,8 @@ bool oz_rows_ok(const lrtei_plan* pl, int64_t r0, int64_t r1, bool out_too, cuda
   if (pl->prec != LRTEI_FP64 || pl->npart > 0 || (!(pl->ozF.d && pl->ozK.d) && capturing(st))) return false;
   const double n3 = (double)pl->n * pl->n * pl->n, np = (double)pl->t.npair;
   const double cuda = ((double)nr * np * n3 + node_fmas(pl, (double)nr)) / kFmaRate;
-  const double build = pl->ozK.d ? 0.0 : K_elems(pl) * pl->P / kFmaRate;
-  if (cuda <= build + 72.0 * (double)nr * np * n3 / 0.9e15 + 4e-4) return false;
+  const double build = K_elems(pl) * pl->P / kFmaRate;  // counted also where K is there: a call's route, and so its last
+  if (cuda <= build + 72.0 * (double)nr * np * n3 / 0.9e15 + 4e-4) return false;  // bits, do not depend on what was called before
   const ParityClasses pc = class_sizes(pl);
   const double cols = (double)pc.cols;
   return fits((pl->ozF.d ? 0.0 : 16 * np * cols) + (pl->d_F ? 0.0 : 8 * np * n3) +
@@ -1479,9 +1479,9 @@ bool oz_rows_ok(const lrtei_plan* pl, int64_t r0, int64_t r1, bool out_too, cuda
               oz::rows_partials(r0, r1, pl->t.npair, pc.size, pc.nclass, pc.cols));
 }
 // J-builds: R >= 2 densities (one is as fast through FP64 F_u, 8 bytes an element against 16), orders up
-// to 32 unless K is there (its build grows as n^6), and enough work to pay for a dozen launches.
+// to 32 (the build of K grows as n^6), and enough work to pay for a dozen launches.
 bool oz_jbuild_ok(const lrtei_plan* pl, int R, cudaStream_t st) {
-  if (pl->prec != LRTEI_FP64 || pl->npart > 0 || R < 2 || (pl->n > 32 && !pl->ozK.d)) return false;
+  if (pl->prec != LRTEI_FP64 || pl->npart > 0 || R < 2 || pl->n > 32) return false;
   const double n3 = (double)pl->n * pl->n * pl->n, np = (double)pl->t.npair;
   const double cuda = (2 * np * n3 * R + node_fmas(pl, R)) / kFmaRate;
   if (cuda <= (32 * np * n3 + 16 * K_elems(pl)) / 5e12 + 8e-5) return false;
