@@ -69,12 +69,13 @@ typedef enum {
                             FP32 accumulation */
   LRTEI_SPLIT_F16_8 = 4  /* as LRTEI_SPLIT_F16, plus the two next-order slice products (t1 t2 and
                             t2 t1), with the small terms in a third accumulator: 8 tensor-core
-                            products per K step instead of 6, an error several times smaller (1e-9 to 1.5e-8 measured) */
+                            products per K step instead of 6, an error several times smaller
+                            (1e-9 to 1.5e-8 measured) */
 } lrtei_precision;
 
 /* Which of the two equivalent forms of Theorem 1 assembles B.  On the FP32 path both run on the
- * CUDA cores, on the FP64 path the Hadamard form does.  With LRTEI_SPLIT_F16 the factored form runs on the tensor cores, and so
- * does the Hadamard form when every unique pair holds one primitive pair (an uncontracted basis,
+ * CUDA cores, on the FP64 path the Hadamard form does.  With LRTEI_SPLIT_F16 the factored form
+ * runs on the tensor cores, and so does the Hadamard form when every unique pair holds one primitive pair (an uncontracted basis,
  * n <= 64, no compression or adaptive boxes): per node and dimension the tile products
  * T_{d,p} S_d^T (depth n) on the tensor cores, the product over dimensions and the node sum in
  * pairs of FP32 numbers; elsewhere the tensor-core precisions take the factored form whatever
@@ -239,7 +240,7 @@ lrtei_status lrtei_dense_K(lrtei_plan* plan, double* d_K, void* stream);
  * d_D: R symmetric N_b x N_b densities (FP64, row-major, consecutive); d_J: same shape.
  * J_r(mu, nu) = sum_{ka, la} B(mu nu, ka la) D_r(ka, la), through the factored form, never
  * forming B.  Uses the plan's precision for the two M-contractions.  When the resident operands
- * (F_u, F_u^T and the dense n^3 x n^3 K, with their slices) would take more than half of the free
+ * (F_u, F_u^T and K, counted as dense, n^3 x n^3, with their slices) would take more than half of the free
  * device memory, F_u is instead built in blocks of unique pairs, twice per call, and the node sum
  * runs as FP64 mode products (eq. ig1); LRTEI_JBUILD_BLOCK=<pairs> in the environment forces this
  * streamed form with that block size.  A call repeating an earlier one-pass call's plan, d_D, d_J
@@ -247,7 +248,9 @@ lrtei_status lrtei_dense_K(lrtei_plan* plan, double* d_K, void* stream);
  * at replay time; up to 32 graphs are kept, least recently used dropped first, each holding its
  * scratch memory; a plan's graphs are dropped when its operands are rebuilt or it is destroyed).
  * Streamed calls, calls on a stream the caller is capturing, and LRTEI_JBUILD_GRAPH=0 launch
- * kernel by kernel.  The environment switches are read when a call is made; a replayed graph
+ * kernel by kernel; a first call inside a relaxed capture builds its operands at once, outside the
+ * graph (other capture modes refuse it).  FP64 and FP32 plans take many densities in groups of
+ * about 1 GiB of scratch.  The environment switches are read when a call is made; a replayed graph
  * keeps the choices of the call it was captured from. */
 lrtei_status lrtei_jbuild(lrtei_plan* plan, const double* d_D, int R, double* d_J, void* stream);
 
@@ -281,7 +284,8 @@ lrtei_status lrtei_jbuild_apply_x(lrtei_plan* plan, const double* d_X, int R, in
  * CUDA-core GEMMs and apply K by mode products (eq. ig1).  A compressed plan gives eq.
  * approxepsilon's exchange.  Device scratch: X and Y of a block, min(norb, block) N_b n^3 doubles
  * each, and the 16-bit slices of both, of X and Y by orbitals and of N_b^2 n^3 elements of F_u
- * (FP64 / FP32 plans, and orders whose n^3 is no multiple of 8: FP64 copies of these).  LRTEI_ERR_ARG for NULL pointers or norb <= 0. */
+ * (FP64 / FP32 plans, and orders whose n^3 is no multiple of 8: FP64 copies of these).
+ * LRTEI_ERR_ARG for NULL pointers or norb <= 0. */
 lrtei_status lrtei_exchange(lrtei_plan* plan, const double* d_Q, int norb, double* d_K, void* stream);
 
 /* ---- batched J-builds (many molecules of uneven size in one graph-captured launch) -------
@@ -348,9 +352,9 @@ lrtei_status lrtei_selector_load(const char* path, lrtei_selector** out, char* m
  * J-build graph).  lrtei_profile_get synchronises those
  * events and returns the summed device time and the launch count of one kernel name.  Two
  * names are counters rather than kernels: "*" gives the number of kernels the library launched
- * since the last reset (time 0), and "alloc" the number of device allocations it has requested since it was loaded (time 0; never
- * reset).  They come from one memory pool per device, which keeps up to 12 GiB of freed memory
- * while plans exist and 2 GiB after the last one.
+ * since the last reset (time 0), and "alloc" the number of device allocations it has requested
+ * since it was loaded (time 0; never reset).  They come from one memory pool per device, which
+ * keeps up to 12 GiB of freed memory while plans exist and 2 GiB after the last one.
  * Off by default; process-wide; not thread-safe against concurrent enable/reset. */
 lrtei_status lrtei_profile_enable(int on);
 lrtei_status lrtei_profile_get(const char* kernel, double* total_ms, int64_t* launches);

@@ -1,12 +1,13 @@
 // k_jfp64.cu -- the FP64 CUDA-core J-build and node sum.
 //   X = F_u^T u, Y = sum_p w_p (A_x^p (x) A_y^p (x) A_z^p) X (eq. ig1), J_u = F_u Y (eq. coulapprox)
 // This device runs about two FP64 FMAs per clock and SM, so every kernel here is bound by its FMA
-// count once the chip is full; below that, by launches.  Hence four launches per J-build, whatever
-// n and P, and the node sum skips the zeros of the Chebyshev coefficients: A^(p)(a, b) = 0 for odd
+// count once the chip is full; below that, by launches.  Hence as few of them as there are products, whatever n and
+// P (k_jx and k_jy once per eight densities, two kernels of the node sum per 128 MB of its intermediate, a reduction
+// where X comes in more than eight parts: five for the molecule below), and the node sum skips the zeros of the Chebyshev coefficients: A^(p)(a, b) = 0 for odd
 // a + b, because the kernel exp(-s^2 (x - y)^2) on two boxes about one centre is unchanged by
 // (x, y) -> (-x, -y).
 // One density of the 20-function molecule (n = 16, P = 20), a CUDA graph replay: 4 810 us with the
-// 64 x 64-tile GEMM and 4 P mode-product launches before.
+// 64 x 64-tile GEMM and 4 P mode-product launches before, 30 here.
 #include <algorithm>
 
 #include "lrtei_internal.h"

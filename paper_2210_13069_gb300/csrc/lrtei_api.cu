@@ -179,7 +179,7 @@ struct lrtei_plan {
   double* d_T = nullptr;      // Hadamard: 3 * P * nrows * n
   double* d_F = nullptr;      // factored: npair * n^3 (FP64)
   float* d_F32 = nullptr;     // factored: npair * n^3 (FP32)
-  SplitMatrix Fsp, Ksp, FTsp; // tensor-core operands: F_u, K, F_u^T as BF16 slices
+  SplitMatrix Fsp, Ksp, FTsp; // tensor-core operands: slices of F_u, K and F_u^T
   bool have_Fsp = false, have_Ksp = false, have_FTsp = false;
   HadOperands had;            // tensor-core Hadamard form (one primitive pair per unique pair)
   bool have_had = false;
@@ -1724,8 +1724,7 @@ lrtei_status batched_graph_run(lrtei_plan* const* plans, int nmol, const double*
       return LRTEI_OK;
     }
   }
-  // First call for this set: run it directly (this also settles the GEMM tuning choices for
-  // every shape), then capture the same work into a graph for the calls that follow.
+  // First call for this set: run it directly, then capture the same work into a graph for the calls that follow.
   for (int m = 0; m < nmol; ++m) LRTEI_TRY(jbuild_direct(plans[m], d_D[m], R[m], d_J[m], st));
   BatchGraph g;
   LRTEI_TRY(capture_batch(plans, nmol, d_D, R, d_J, st, &g));
