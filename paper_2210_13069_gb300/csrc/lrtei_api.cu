@@ -42,6 +42,8 @@ struct Pool {
   cudaStream_t st = nullptr;  // plan buffers are allocated and freed in its order, nothing else runs on it
   int plans = 0;              // plans alive on the device
   void* token = nullptr;      // what device_idle frees
+  size_t total = 0;           // the device's memory
+  size_t digits = 0;          // bytes that FP64 plans hold as digit operands
 };
 std::mutex g_pool_mu;
 std::map<int, Pool> g_pools;
@@ -64,6 +66,8 @@ cudaError_t current_pool(Pool** out, int dev = -1) {
     props.location.id = dev;
     if ((e = cudaMemPoolCreate(&p.pool, &props)) != cudaSuccess) return e;
     if ((e = pool_keeps(p.pool, kPoolIdle)) != cudaSuccess) return e;
+    size_t free_b = 0;
+    if ((e = cudaMemGetInfo(&free_b, &p.total)) != cudaSuccess) return e;
     if ((e = cudaStreamCreateWithFlags(&p.st, cudaStreamNonBlocking)) != cudaSuccess) return e;
     it = g_pools.emplace(dev, p).first;
   }
@@ -192,7 +196,17 @@ struct lrtei_plan {
   OzMatrix ozF, ozFT, ozK;
   std::vector<void*> allocs;
   size_t bytes = 0;
+  size_t digits = 0;  // of them, in digit operands
   int dev = -1;  // the device current at creation
+
+  // The device's account of digit operands.
+  void count_digits(int64_t more) {
+    Pool* p = nullptr;
+    if (dev < 0 || current_pool(&p, dev) != cudaSuccess) return;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    digits += more;
+    p->digits += more;
+  }
 
   template <typename T>
   lrtei_status alloc(T** p, size_t count) {
@@ -248,6 +262,7 @@ struct lrtei_plan {
       else cudaGetLastError();
     }
     std::lock_guard<std::mutex> lk(g_pool_mu);
+    p->digits -= digits;
     if (--p->plans == 0) {
       pool_keeps(p->pool, kPoolIdle);
       // what was freed above counts as free once its stream has come to it
@@ -1381,10 +1396,12 @@ lrtei_status alloc_oz(lrtei_plan* pl, OzMatrix& m, int64_t rows, int64_t kpad) {
   q.kpad = kpad;
   LRTEI_TRY(pl->alloc(&q.d, (size_t)q.count()));
   LRTEI_TRY(pl->alloc(&q.expo, (size_t)rows));
+  pl->count_digits((int64_t)sizeof(uint16_t) * q.count());
   m = q;
   return LRTEI_OK;
 }
 void release_oz(lrtei_plan* pl, OzMatrix& m) {
+  if (m.d) pl->count_digits(-(int64_t)sizeof(uint16_t) * m.count());
   pl->release(m.d, sizeof(uint16_t) * (size_t)m.count());
   pl->release(m.expo, sizeof(int) * (size_t)m.rows);
   m = OzMatrix();
@@ -1464,6 +1481,15 @@ double K_elems(const lrtei_plan* pl) {
   const double n = pl->n, n6 = n * n * n * n * n * n;
   return has_parity(pl) ? n6 / 8 : n6;
 }
+// Digit operands take 16 bytes an element and copy where F_u itself takes 8.  All plans of a device hold at most a third of
+// its memory in them, so that those that come later find room for their F_u: a batch of sixty molecules of 180 functions
+// ended for want of memory, and plans one after the other turned to streamed J-builds.
+bool digits_fit(double bytes) {
+  Pool* p = nullptr;
+  if (current_pool(&p) != cudaSuccess) return false;
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  return (double)p->digits + bytes <= (double)p->total / 3;
+}
 // out_too: the rows themselves are not allocated yet.
 bool oz_rows_ok(const lrtei_plan* pl, int64_t r0, int64_t r1, bool out_too, cudaStream_t st) {
   const int64_t nr = r1 - r0;
@@ -1474,8 +1500,10 @@ bool oz_rows_ok(const lrtei_plan* pl, int64_t r0, int64_t r1, bool out_too, cuda
   if (cuda <= build + 72.0 * (double)nr * np * n3 / 0.9e15 + 4e-4) return false;  // bits, do not depend on what was called before
   const ParityClasses pc = class_sizes(pl);
   const double cols = (double)pc.cols;
-  return fits((pl->ozF.d ? 0.0 : 16 * np * cols) + (pl->d_F ? 0.0 : 8 * np * n3) +
-              (pl->ozK.d ? 0.0 : 24.0 * pc.rows * pc.kmax) + nr * (24 * cols + (out_too ? 8 * np : 0.0)) +
+  const double digits = (pl->ozF.d ? 0.0 : 16 * np * cols) + (pl->ozK.d ? 0.0 : 16.0 * pc.rows * pc.kmax);
+  if (digits > 0 && !digits_fit(digits)) return false;
+  return fits(digits + (pl->d_F ? 0.0 : 8 * np * n3) + (pl->ozK.d ? 0.0 : 8.0 * pc.rows * pc.kmax) +
+              nr * (24 * cols + (out_too ? 8 * np : 0.0)) +
               oz::rows_partials(r0, r1, pl->t.npair, pc.size, pc.nclass, pc.cols));
 }
 // J-builds: R >= 2 densities (one is as fast through FP64 F_u, 8 bytes an element against 16), orders up
@@ -1487,7 +1515,12 @@ bool oz_jbuild_ok(const lrtei_plan* pl, int R, cudaStream_t st) {
   if (cuda <= (32 * np * n3 + 16 * K_elems(pl)) / 5e12 + 8e-5) return false;
   if (pl->ozF.d && pl->ozFT.d && pl->ozK.d) return true;
   if (capturing(st)) return false;
-  return fits(np * n3 * (pl->d_F ? 40 : 48) + 24 * K_elems(pl));
+  const ParityClasses pc = class_sizes(pl);
+  const double cols = (double)pc.cols, kk = (double)pc.rows * pc.kmax;
+  const double digits =
+      (pl->ozF.d ? 0.0 : 16 * np * cols) + (pl->ozFT.d ? 0.0 : 16 * np * cols) + (pl->ozK.d ? 0.0 : 16 * kk);
+  // beside them for a while: the FP64 F_u^T and K
+  return digits_fit(digits) && fits(digits + (pl->d_F ? 0.0 : 8 * np * n3) + std::max(8 * np * n3, 8 * kk));
 }
 
 lrtei_status bu_rows_oz(lrtei_plan* pl, int64_t r0, int64_t r1, double* out, int64_t ld, cudaStream_t st) {
@@ -1693,18 +1726,15 @@ lrtei_status capture_batch(lrtei_plan* const* plans, int nmol, const double* con
 
 lrtei_status batched_graph_run(lrtei_plan* const* plans, int nmol, const double* const* d_D, const int* R,
                                double* const* d_J, cudaStream_t st) {
-  // operands of every molecule exist before capture (their set-up allocates and synchronises)
-  for (int m = 0; m < nmol; ++m) {
-    if (is_split(plans[m])) LRTEI_TRY(ensure_jbuild_operands(plans[m], st));
-    else {
-      LRTEI_TRY(ensure_F64(plans[m], st));
-      if (oz_jbuild_ok(plans[m], R[m], st)) {
-        LRTEI_TRY(ensure_ozFT(plans[m], st));
-        LRTEI_TRY(ensure_ozF(plans[m], st));
-        LRTEI_TRY(ensure_ozK(plans[m], st));
-      }
+  // operands of every molecule exist before capture (their set-up allocates and synchronises): those that no form does
+  // without, then digits where they fit beside all of them
+  for (int m = 0; m < nmol; ++m)
+    LRTEI_TRY(is_split(plans[m]) ? ensure_jbuild_operands(plans[m], st) : ensure_F64(plans[m], st));
+  for (int m = 0; m < nmol; ++m)
+    if (!is_split(plans[m]) && oz_jbuild_ok(plans[m], R[m], st)) {
+      LRTEI_TRY(ensure_ozFT(plans[m], st));
+      LRTEI_TRY(ensure_ozK(plans[m], st));
     }
-  }
   std::vector<uintptr_t> key;
   key.push_back((uintptr_t)nmol);
   for (int m = 0; m < nmol; ++m) {

@@ -127,3 +127,25 @@ def test_the_idle_pool_counts_as_free_memory(lib):
     assert products == 2, "G and B_u: the rows came in bands"
     assert torch.equal(B, first)
     pl.close()
+
+
+@pytest.mark.parametrize("batched", [False, True])
+def test_many_fp64_plans_share_the_device(lib, batched):
+    """Sixty plans of 180 functions: 108 GB of F_u in FP64, which fit, and 430 GB as digit operands, which do not."""
+    import torch
+    m = synth.workload_spd()
+    D = torch.as_tensor(synth.random_densities(5, m.nbf, 4), device="cuda")
+    plans = [lib.Plan(m, "fp64") for _ in range(60)]
+    J = [torch.empty_like(D) for _ in plans]
+    if batched:
+        lib.lrtei_jbuild_batched([p.plan for p in plans], [D] * 60, [4] * 60, J)
+    else:
+        for p, j in zip(plans, J):
+            p.jbuild(D, out=j)
+    torch.cuda.synchronize()
+    for p in (plans[0], plans[59]):
+        p.status()
+    a, b = J[0].cpu().numpy(), J[59].cpu().numpy()  # digit products, CUDA cores
+    assert rel_fro(a, b) <= 1e-12
+    for p in plans:
+        p.close()
