@@ -175,7 +175,7 @@ __device__ __forceinline__ double scaled_down(double x, int s) {
   const long long b = __double_as_longlong(x);
   const int E = (int)((b >> 52) & 0x7FF) - s;
   if (((b >> 52) & 0x7FF) == 0 || E <= 0) return 0.0;
-  return __longlong_as_double(b - ((long long)s << 52));
+  return __longlong_as_double(b - s * (1LL << 52));
 }
 
 __global__ void __launch_bounds__(512) k_oz_split(const double* __restrict__ src, int64_t k, int64_t ld, int64_t kpad,
