@@ -248,6 +248,16 @@ static int tile_of_waves(int BN, int64_t tiles128, int64_t tiles64) {
   return 72 * w64 < 100 * w128 ? 64 : 128;
 }
 
+// The same for eight products of M rows and N columns, which are one launch in 64-column tiles and two in 128-column
+// ones.  Up to 128 columns the left operand's bytes count: three planes once (the second tile finds them in L2) against
+// two and three.  J-builds of 100 densities, 120 functions, n = 16: 495 us in two launches, 309 in one; of 65 densities, 90
+// functions, n = 12: 178, 115; exchange of 180 functions and 90 orbitals, n = 10: 1.07 ms, 0.85.
+static int tile_of_rows(int BN, int64_t M, int64_t N, int64_t splits) {
+  if (BN == 128 && N <= 128) return 64;
+  const int64_t tiles = (M + 127) / 128 * splits;
+  return tile_of_waves(BN, tiles * ((N + 127) / 128), tiles * ((N + 63) / 64));
+}
+
 template <bool LIST, bool SWAP>
 static lrtei_status run_as(const tcg::Params& p, int BN, bool plain, bool eight, cudaStream_t st) {
   if (plain)
@@ -335,7 +345,9 @@ lrtei_status tc_gemm(const SplitMatrix& A, int64_t a_row0, const SplitMatrix& B,
     return LRTEI_ERR_ARG;
   }
   if (symmetric_upper) return tc_gemm_sym_band(A, B, 0, N, N, d_C, ldc, d_status, st);
-  const int BN = tc::tile_n(N, A.plain), m_lo = (int)(a_row0 % 128), units = (int)(A.kpad / 128);
+  const int m_lo = (int)(a_row0 % 128), units = (int)(A.kpad / 128);
+  int BN = tc::tile_n(N, A.plain);
+  if (A.eight) BN = tc::tile_of_rows(BN, M + m_lo, N, splits);
   tcg::Params p{};
   const int64_t c_rows = transpose_out ? N : M, c_cols = transpose_out ? M : N;
   lrtei_status s = tc::fill(p, A, B, BN, units, scale, d_C, ldc, transpose_out, splits, c_rows, c_cols, d_part, d_status);
@@ -359,8 +371,9 @@ lrtei_status tc_gemm_few(const SplitMatrix& A, const SplitMatrix& B, int64_t M, 
     set_error("tc_gemm_few: operands must share a K padded to a multiple of 128");
     return LRTEI_ERR_ARG;
   }
-  const int BN = tc::tile_n(M, A.plain), units = (int)(A.kpad / 128);
-  int splits = 1;
+  const int units = (int)(A.kpad / 128);
+  int splits = 1, BN = tc::tile_n(M, A.plain);
+  if (A.eight) BN = tc::tile_of_rows(BN, N, M, 1);
   tcg::Params p{};
   lrtei_status s = tc::fill(p, B, A, BN, units, 1.0, d_C, ldc, true, splits, M, N, nullptr, d_status);
   if (s != LRTEI_OK) return s;
@@ -432,7 +445,9 @@ lrtei_status tc_gemm_K(const SplitMatrix& X, int64_t x_row0, const SplitMatrix& 
   const SplitMatrix &A = k_is_a ? K : X, &B = k_is_a ? X : K;
   const int m_lo = k_is_a ? 0 : (int)(x_row0 % 128);
   int BN = tc::tile_n(rows, A.plain);
-  if (!k_is_a) {
+  if (k_is_a) {
+    if (A.eight) BN = tc::tile_of_rows(BN, pc.rows, rows, splits);
+  } else {
     int64_t nmax = 0, t128 = 0, t64 = 0;
     for (int c = 0; c < pc.nclass; ++c) {
       nmax = std::max<int64_t>(nmax, pc.size[c]);

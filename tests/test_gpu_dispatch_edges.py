@@ -25,12 +25,14 @@ def rel_fro(a, b):
     return float(np.linalg.norm(a - b) / np.linalg.norm(b))
 
 
+@pytest.mark.parametrize("prec", ["split_f16", "split_f16_8", "bf16"])
 @pytest.mark.parametrize("natoms", [3, 4, 5])
-def test_tile_widths_give_equal_bits(lib, natoms):
+def test_tile_widths_give_equal_bits(lib, natoms, prec):
     """B_u of 1035 pairs goes in 64-column tiles, of 1830 and 2850 pairs in 128-column ones; its first 128 rows by
-    themselves, with tile widths of their own for G, are the same bits from the diagonal on."""
+    themselves, with tile widths of their own, are the same bits from the diagonal on.  With eight products 128-column
+    tiles are two launches (the smaller terms added to C), 64-column ones a single launch."""
     m = synth.workload_spd(1002, natoms=natoms, n=13, P=7)
-    pl = lib.Plan(m, "split_f16")
+    pl = lib.Plan(m, prec)
     whole = pl.Bu_rows(0, pl.npair, "factored").cpu().numpy()
     band = pl.Bu_rows(0, 128, "factored").cpu().numpy()
     pl.status()
@@ -38,15 +40,16 @@ def test_tile_widths_give_equal_bits(lib, natoms):
     pl.close()
 
 
-def test_eight_products_in_one_and_in_two_launches_give_equal_bits(lib):
-    """64 densities take one launch a product, 65 and more two (the smaller terms added to C)."""
+def test_eight_products_of_few_and_many_columns_give_equal_bits(lib):
+    """J-builds of 64, 100 and 300 densities: one 64-column tile, two, and launches by the waves they take."""
     import torch
-    m = synth.workload_spd(1002, natoms=2, n=12, P=6)
-    D = torch.as_tensor(synth.random_densities(5, m.nbf, 100), device="cuda")
+    m = synth.workload_spd(1002, natoms=5, n=12, P=6)
+    D = torch.as_tensor(synth.random_densities(5, m.nbf, 300), device="cuda")
     pl = lib.Plan(m, "split_f16_8")
-    J64, J100 = pl.jbuild(D[:64]), pl.jbuild(D)
+    J = pl.jbuild(D)
+    for R in (64, 100):
+        assert torch.equal(pl.jbuild(D[:R].contiguous()), J[:R])
     pl.status()
-    assert torch.equal(J64, J100[:64])
     pl.close()
 
 
