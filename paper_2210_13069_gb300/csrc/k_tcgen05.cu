@@ -31,9 +31,11 @@
 namespace lrtei {
 namespace tc {
 
-__device__ __forceinline__ double pow2(int k) {  // 2^k, exponent clamped to the normal range
-  k = max(-1022, min(1023, k));
-  return __longlong_as_double((long long)(k + 1023) << 52);
+// f in FP64 from its bits: conversions to FP64 run at two a clock and SM.
+__device__ __forceinline__ double widen(float f) {
+  const uint32_t b = __float_as_uint(f), E = (b >> 23) & 0xFFu;
+  if (E == 0 || E == 0xFFu) return (double)f;  // zero, subnormal, infinity, NaN
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + (896u << 20))), (int)(b << 29));
 }
 
 // (T0 + T12 / 2^12) 2^k in integer arithmetic (this device's FP64 rate would make an FP64
@@ -120,8 +122,9 @@ template <int BN_, Scheme M, bool LIST_, bool SWAP = false>
 struct Split {
   static constexpr bool P8 = M == Scheme::eight, PLAIN = M == Scheme::plain, HI = M == Scheme::eight_hi,
                         LO = M == Scheme::eight_lo, ONE = PLAIN || LO;  // ONE: a single FP32 accumulator
-  static constexpr int BN = BN_, NP = PLAIN ? 1 : HI ? 2 : 3, PT = PLAIN ? 1 : 3, NACC = ONE ? 1 : P8 ? 3 : 2, KS = 2;
-  // KS: two steps a stage, half the barrier rounds
+  static constexpr int BN = BN_, NP = PLAIN ? 1 : HI ? 2 : 3, PT = PLAIN ? 1 : 3, NACC = ONE ? 1 : P8 ? 3 : 2, KS = PLAIN ? 8 : 2;
+  // KS: two steps a stage, half the barrier rounds; plain operands, whose step is one MMA, a whole chunk (ten rows
+  // of B_u of 60 functions, n = 11: G 21 -> 13 us, B_u 24 -> 16, together with an epilogue without FP64)
   static constexpr int UNIT = 8, CHUNK = 8;  // 128 deep
   static constexpr bool BF16 = PLAIN, ACCUM = LO, LIST = LIST_;
 
@@ -226,7 +229,7 @@ struct Split {
     }
     // The planes' weights make T1 and T2 those of the sums of s0 t1 over 2^12.
     __device__ __forceinline__ double value(int j, int k, double scale) const {
-      if constexpr (PLAIN) return scale * pow2(k - 16) * (double)T1[j];
+      if constexpr (PLAIN) return scale == 1.0 ? widen(T1[j]) : scale * widen(T1[j]);  // k is 16 (k_plain_rows)
       const int t0 = LO ? 0 : T0[ONE ? 0 : j];
       const float t2 = P8 ? T2[P8 ? j : 0] : 0.f;
       const double v = SWAP || HI || LO ? combine_words(t0, T1[j], k - 16, t2, P8)

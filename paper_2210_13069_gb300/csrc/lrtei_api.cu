@@ -858,9 +858,10 @@ lrtei_status ensure_classes(lrtei_plan* pl, cudaStream_t st) {
             blk[(size_t)c * nblk + b] = (int)list.size();
             list.push_back(b);
           }
-        for (size_t i = before; i < list.size(); i += 2) {
-          if (i + 1 < list.size()) list[i] |= 1 << 29;   // two steps in one stage
-          if (i + 2 >= list.size()) list[i] |= 1 << 30;  // the chunk's last stage
+        const size_t per = pl->prec == LRTEI_BF16 ? 8 : 2;  // steps of a stage (k_tcgen05.cu)
+        for (size_t i = before; i < list.size(); i += per) {
+          list[i] |= (int)(std::min(per, list.size() - i) - 1) << 26;
+          if (i + per >= list.size()) list[i] |= 1 << 30;  // the chunk's last stage
         }
         if (list.size() > before) ++nonempty;
       }

@@ -185,8 +185,8 @@ struct ParityClasses {
   // Step tables of the split-precision products, whose K runs in the natural order (device; NULL without
   // parity): per class, at tab + tab_off[c], [units + 1] the first list entry of each 128-deep chunk,
   // [units + 1] the number of chunks with entries before it, and the list of the 16-deep K blocks that
-  // hold columns of the class, two to a stage where a chunk allows (2^29 on the first), the stage that
-  // ends a chunk flagged with 2^30.
+  // hold columns of the class, in stages of up to two (plain operands: eight) where a chunk allows (their number less
+  // one times 2^26 on the first), the stage that ends a chunk flagged with 2^30.
   const int* tab = nullptr;
   int tab_off[8] = {};
   int units = 0;           // chunks of the padded n^3

@@ -36,9 +36,10 @@ constexpr int EPI = 16;      // epilogue warps: four per TMEM lane quadrant
 constexpr int THREADS = 64 + 32 * EPI;
 constexpr int kGroupM = 16;  // M tiles walked together (operand slabs shared in L2)
 constexpr int kGroupRows = 8;
-// Flags of a step table's entries (K block numbers): the entry opens a stage that ends its chunk; the entry and
-// the next one share a stage.
-constexpr int kLast = 1 << 30, kTwo = 1 << 29;
+// Flags of a step table's entries (K block numbers below 2^26): the entry opens a stage that ends its chunk; how many
+// entries share a stage that it opens, less one.
+constexpr int kLast = 1 << 30, kCountBit = 26, kBlock = (1 << kCountBit) - 1;
+__host__ __device__ constexpr int stage_entries(int e) { return ((e >> kCountBit) & 7) + 1; }
 
 // One block of the product: rows a_row0 + [0, M) of A, b_row0 + [0, N) of B, `units` split units of K from
 // block a_blk and b_blk, written at C + c_off.  Rows below m_lo belong to the first tile only (a_row0 is a
@@ -216,14 +217,14 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
         for (int t = w.t0; t < w.t1; ++it) {
           const int s = (int)(it % STAGES);
           const int e = S::LIST ? list[t] : 0;
-          const int cnt = S::LIST ? ((e & kTwo) ? 2 : 1) : KS;  // steps of this stage
+          const int cnt = S::LIST ? stage_entries(e) : KS;  // steps of this stage
           if (!mbar_wait(&empty[s], ((it / STAGES) & 1u) ^ 1u, abort_flag, p.status, 32)) { stop = true; break; }
           mbar_arrive_expect_tx(&full[s], (uint32_t)cnt * G::STEP);
           uint8_t* st = smem + (size_t)s * G::STAGE;
 #pragma unroll
           for (int q = 0; q < KS; ++q) {
             if (q >= cnt) break;
-            const int pos = t + q, nat = S::LIST ? (q == 0 ? e : list[pos]) & (kTwo - 1) : pos;
+            const int pos = t + q, nat = S::LIST ? (q == 0 ? e : list[pos]) & kBlock : pos;
             const int ka = S::LIST && p.list_is_a ? nat : pos, kb = S::LIST && !p.list_is_a ? nat : pos;
             bulk_load(st + q * G::STEP, a + (int64_t)ka * (S::PT * G::A_BYTES), NP * G::A_BYTES, &full[s]);
             uint8_t* sb = st + q * G::STEP + NP * G::A_BYTES;
@@ -269,7 +270,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
         int in_chunk = 0;  // steps of the current chunk so far
         int next = S::LIST && w.t0 < w.t1 ? list[w.t0] : 0;
         for (int t = w.t0; t < w.t1;) {
-          const int e = next, cnt = S::LIST ? ((e & kTwo) ? 2 : 1) : KS;
+          const int e = next, cnt = S::LIST ? stage_entries(e) : KS;
           t += cnt;
           // the chunk ends with a flagged stage, after CHUNK steps, or with the item
           const bool last = (S::LIST ? (e & kLast) != 0 : in_chunk + cnt >= S::CHUNK) || t >= w.t1;
@@ -329,7 +330,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
       const int* eb = p.eb + sg.b_row0;
       double* C = p.C + sg.c_off + (int64_t)w.split * p.split_stride;
       const bool diag = p.symmetric && !w.mirror;  // the upper triangle only, mirrored below
-      if (n >= N) continue;
+      if (n >= N || !__any_sync(0xffffffffu, mlive)) continue;  // a warp without rows to store
 #pragma unroll
       for (int j0 = 0; j0 < QC; j0 += 4) {
         T.template hold<4>(j0);  // one group of columns at a time (the sums fill the registers)
