@@ -25,7 +25,7 @@
 // first, the later ones adding to C): 128 x 128 tiles, two FP32 accumulators double-buffered in the
 // 512 TMEM columns, and registers for one 64-bit sum per element allow two levels at a time.  Skinny products
 // (J-builds, N <= 32 columns a tile) keep all eight levels in TMEM (2 x 8 x 32 columns) and read their operand once.
-// Measured: FP64 B of 60 functions (n = 24, P = 32) 187 ms on the CUDA cores, 2.55 with six digits, 4.29 with eight;
+// Measured: FP64 B of 60 functions (n = 24, P = 32) 187 ms on the CUDA cores, 2.55 with six digits, 4.23 with eight;
 // J-build of 16 densities, 120 functions, 32.7 (6.2 with the kernels of k_jfp64.cu), 0.47 and 0.61 ms, the products
 // reading their operand at 6.5 TB/s.
 #include <cuda_fp16.h>
