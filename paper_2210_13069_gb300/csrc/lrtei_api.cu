@@ -92,8 +92,10 @@ cudaError_t device_idle(Pool* p) {
     cudaGetLastError();
     t = nullptr;
   }
-  std::lock_guard<std::mutex> lk(g_pool_mu);
-  if (!p->token) std::swap(t, p->token);
+  {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (!p->token) std::swap(t, p->token);
+  }
   if (t) cudaFree(t);  // two threads at once: one token is kept
   return e;
 }
